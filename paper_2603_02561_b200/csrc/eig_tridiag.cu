@@ -1,27 +1,25 @@
 // Batched symmetric eigensolver, tridiagonal route: the top-r eigenpairs of every Gram matrix
 // G_b = H_b^T H_b (Eq. 9 without U: s_i = sqrt(lambda_i), V = eigenvectors) by the classical
-// dense-symmetric chain, one CTA per user, sized so that a user costs tens of thousands of warp
-// instructions and a modest register and shared-memory footprint (several CTAs share an SM with
-// the streaming kernels of other requests) instead of the hundreds of thousands of a Jacobi solve:
+// dense-symmetric chain, one CTA per user (128 threads; 256 at d = 128):
 //
 //   1. G = sum of the slices' partial Grams (fixed order), scaled by a power of two.
-//   2. Householder tridiagonalisation T = Q^T G Q with the matrix held in REGISTERS, spread over
-//      all warps of the CTA: thread (warp w, lane l) owns rows l, l+32, ... and the columns of
-//      its warp's 4-column groups, so the symmetric matrix-vector product and the rank-2 update
-//      of a step are FMAs on statically indexed registers.  Every warp computes the step's
-//      scalars redundantly (column norm and p^T v by shuffles); the warps exchange only their
-//      partial products, through shared memory, at ONE barrier per step.  The next step's
-//      column comes from the owner of row k+1 (by symmetry) before the update and is corrected
-//      by the rank-2 term, so no step waits for the update of the one before.
-//   3. The r largest eigenvalues of T by multisection on Sturm counts: one lane per eigenvalue,
-//      one interior point per warp and step (4 or 8 points), the counts taken from the
-//      three-term recurrence of the leading principal minors with a power-of-two rescale every
-//      four steps -- one FMA per step on the dependency chain instead of a division.
-//   4. One eigenvector per eigenvalue from the twisted factorisation of T - lambda I (forward
-//      and backward pivot sequences as ratios of consecutive minors, twist at the smallest
-//      |gamma_k|): inverse iteration from the best unit vector, O(d) per vector, no pivoting.
-//   5. Back-transformation V = Q Z: four threads per vector, each applying the d-2 reflectors to
-//      its quarter of the rows held in registers.
+//   2. Householder tridiagonalisation T = Q^T G Q with the matrix in REGISTERS, in tiles of d/32
+//      rows x 16 columns per thread; the vectors of a step live in registers too, at the thread's
+//      columns and at its rows, so the norm, the inner product and a row of A x are each complete
+//      after the two (three) shuffles over the threads of a row.  The product is taken with the
+//      column x itself and corrected to the reflector v = x - alpha e_1 afterwards, so that the
+//      square root runs beside it; the next column comes from row k+1 (by symmetry) of the matrix
+//      before the update.  What crosses warps is A x and that row, at ONE barrier per step.
+//   3. The r largest eigenvalues of T by multisection on Sturm counts: the points of an eigenvalue
+//      are lanes of one warp (a ballot instead of a barrier), the counts come from the three-term
+//      recurrence of the leading principal minors -- one FMA per row on the dependency chain.
+//   4. One eigenvector per eigenvalue from the twisted factorisation of T - lambda I: inverse
+//      iteration from the best unit vector, O(d) per vector, no pivoting.  Leading and trailing
+//      minors run on two warps; gamma_k = det / (p_k t_{k+1}), so the twist is where the product
+//      of the two minors is largest and their logarithms are all that has to be compared.
+//   5. V = Q Z.  fp32, d <= 64: Q is accumulated during step 2 (each thread's tile of Q beside its
+//      tile of A, in the shadow of the step's shuffles) and this is one small product; otherwise
+//      the reflectors are applied one by one (no registers left for Q).
 //   6. Gram-Schmidt passes in matrix form, V <- V (I - strict_upper(V^T V - I)) D^-1, repeated
 //      while V^T V - I is above the rounding level (vectors of close eigenvalues come out of
 //      step 4 with a mutual error of order eps |T| / gap); a column is only ever corrected by
@@ -32,10 +30,13 @@
 //      CTA runs the parallel Jacobi eigensolver on the whole matrix, which is valid for any
 //      spectrum (clusters of equal eigenvalues, rank(H) < r, ...).
 //
-// A warp that runs alone on its scheduler pays the full latency of every branch and of every
-// dependent instruction; the code below is therefore straight-line over static ranges (the
-// Householder loop is cut into stages with fixed live rows and columns), keeps divisions off
-// the dependency chains, and spreads independent work over the warps.
+// What bounds it: the dependency chain (d steps of a matrix-vector product, an inner product and a
+// barrier, then the recurrences over the rows of T), not work or bandwidth: 16 users keep 16 of
+// 148 SMs busy.  A warp that is alone on its scheduler pays the full latency of every dependent
+// instruction and shared-memory load, and tens of cycles for every branch, taken or not; the code
+// below is therefore straight-line over static ranges (the Householder loop is cut into stages
+// with fixed live columns; conditions are predicates of single instructions), fetches ahead, and
+// keeps divisions off the dependency chains.
 #include "eig_jacobi.cuh"
 #include "project_mma.cuh"
 
@@ -46,39 +47,36 @@ namespace {
 constexpr unsigned kFull = 0xffffffffu;
 
 template <int D> struct TriCfg {
-  static constexpr int NT = (D == 128) ? 256 : 128;   // threads of the CTA
+  static constexpr int GX = (D == 128) ? 8 : 4;       // threads across a row; 32 groups of them
+  static constexpr int RT = D / 32;                   // rows of a thread: RT * group ..
+  static constexpr int NT = 32 * GX;                  // threads of the CTA
   static constexpr int NW = NT / 32;
-  static constexpr int RPT = D / 32;                  // rows per thread: l + 32 q
-  static constexpr int CPT = D / NW;                  // columns per thread ...
-  static constexpr int NG = CPT / 4;                  // ... as 4-column groups: group g of warp w = columns 4 (w + NW g) ..+3
-  static constexpr int SS = 4 * NW;                   // steps per stage: from step s * SS on, the groups g < s are finished
-  static constexpr int LD = D + 4;                    // pitch of the staged row-major G
-  static constexpr int NB = D / 4;                    // 4-column blocks of a row
-  static_assert(SS * NG == D && RPT * 32 == D, "ownership covers the matrix");
+  static constexpr int CW = 4 * GX;                   // columns of a chunk: thread g of a group has 4 g .. 4 g + 3
+  static constexpr int NCH = D / CW;                  // chunks of a row
+  static constexpr int WR = D / NW;                   // rows of a warp
+  static constexpr int CTAS = (D == 128) ? 1 : 3;     // resident CTAs that the register count has to allow
+  static constexpr int LD = D + 4;                    // pitch of Q^T and of the row-major G
 };
 
 // Shared-memory layout (floats) for subspace width RP = 32 * ceil(r / 32).
 template <int D, int RP> struct TriSmem {
   using C = TriCfg<D>;
-  static constexpr int HV = 0;                                   // [D][D] reflector k in row k; later G
-  static constexpr int VS = HV + D * D;                          // [D][RP] V
-  static constexpr int WORK_FLOATS = (D * C::LD > 2 * D * RP) ? D * C::LD : 2 * D * RP;
-  static constexpr int WORK = VS + D * RP;                       // staged G | tf, tb [D][RP] | V'
-  static constexpr int EM = WORK + WORK_FLOATS;                  // [RP][RP] V^T V - I (before: multisection flags)
-  static constexpr int DG = EM + RP * RP;                        // [D] diagonal of T
-  static constexpr int EO = DG + D;                              // [D] off-diagonal: e[k] couples k, k+1
-  static constexpr int E2 = EO + D;                              // [D] e2s[i] = e[i-1]^2 (floored), e2s[0] = 0
-  static constexpr int BE = E2 + D;                              // [D] beta of reflector k
-  static constexpr int XP = BE + D;                              // [2][D] row k+1 before the update of step k
-  static constexpr int TP = XP + 2 * D;                          // [2][NW][D] the warps' partial products A v
-  static constexpr int PV = TP + 2 * C::NW * D;                  // [2][8] the warps' partial p^T v
-  static constexpr int LAM = PV + 16;                            // [RP] eigenvalues of T
-  static constexpr int TH = LAM + RP;                            // [RP] Rayleigh quotients
-  static constexpr int RH = TH + RP;                             // [RP] squared residual norms
-  static constexpr int SG = RH + RP;                             // [RP] gauge signs; before: 1 / |z|
-  static constexpr int KT = SG + RP;                             // [RP] twist index (int)
-  static constexpr int PART = KT + RP;                           // [2][NW][RP] per-warp partial results
-  static constexpr int TRI_FLOATS = PART + 2 * C::NW * RP;
+  static constexpr int R0 = 0;                                   // Q^T [D][LD] or the reflectors [D][D]; later G [D][D]
+  static constexpr int A1 = R0 + (D == 128 ? D * D : D * C::LD); // [D][RP] upward multipliers; V
+  static constexpr int A2 = A1 + D * RP;                         // [D][RP] downward multipliers; V'
+  static constexpr int A3 = A2 + D * RP;                         // [D][RP] log2 of the leading minors; Z
+  static constexpr int A4 = A3 + D * RP;                         // [D][RP] log2 of the trailing minors; V^T V - I [RP][RP]
+  static constexpr int DG = A4 + D * RP;                         // diagonal of T (this and the next five with room for fp64)
+  static constexpr int EO = DG + 2 * D;                          // off-diagonal: e[k] couples k, k+1
+  static constexpr int E2 = EO + 2 * D;                          // e2s[i] = e[i-1]^2 (floored), e2s[0] = 0
+  static constexpr int YV = E2 + 2 * D;                          // [2][D] A x
+  static constexpr int XP = YV + 4 * D;                          // [2][D] row k+1 of the matrix before step k's update
+  static constexpr int LAM = XP + 4 * D;                         // [RP] eigenvalues of T
+  static constexpr int BE = LAM + 2 * RP;                        // [D] beta of reflector k
+  static constexpr int TH = BE + D;                              // [RP] Rayleigh quotients
+  static constexpr int KT = TH + RP;                             // [RP] eigenvalues of the fp32 chain
+  static constexpr int PART = KT + RP;                           // [3][NW][RP] per-warp partial results
+  static constexpr int TRI_FLOATS = PART + 3 * C::NW * RP;
   // the projection epilogue: V Sigma, Key_r^T, two weights (FFMA form) or the tensor-core form's staging
   static constexpr int EPI_FFMA = 2 * D * RP + 2 * D * D;
   static constexpr int EPI_MMA = (D >= 64) ? pmma::Lay<(D >= 64 ? D : 64)>::bytes(RP) / 4 : 0;
@@ -86,214 +84,384 @@ template <int D, int RP> struct TriSmem {
   static constexpr int M1 = TRI_FLOATS > full_jacobi_floats<D>() ? TRI_FLOATS : full_jacobi_floats<D>();
   static constexpr int FLOATS = M1 > EPI_FLOATS ? M1 : EPI_FLOATS;
   static constexpr size_t BYTES = (size_t)FLOATS * sizeof(float);
-  static_assert(DG % 4 == 0 && EO % 4 == 0 && E2 % 4 == 0 && XP % 4 == 0 && TP % 4 == 0 && PV % 4 == 0 &&
-                EM % 4 == 0 && WORK % 4 == 0 && VS % 4 == 0, "16-byte alignment of the regions");
+  static_assert(A1 % 4 == 0 && DG % 4 == 0 && YV % 4 == 0 && LAM % 4 == 0 && BE % 4 == 0 && TH % 4 == 0 && PART % 4 == 0,
+                "16-byte alignment of the regions");
+  static_assert(RP <= D && BYTES <= 226 * 1024, "V^T V - I fits; one CTA fits an SM");
 };
 
-__device__ __forceinline__ float warp_sum(float v) {
-#pragma unroll
-  for (int o = 16; o; o >>= 1) v += __shfl_xor_sync(kFull, v, o);
-  return v;
-}
+// ---- arithmetic in fp32 and fp64 -------------------------------------------------------------
 __device__ __forceinline__ float warp_max(float v) {
 #pragma unroll
   for (int o = 16; o; o >>= 1) v = fmaxf(v, __shfl_xor_sync(kFull, v, o));
   return v;
 }
-// 16-byte store to shared memory under a predicate, without a branch.
-__device__ __forceinline__ void sts_v4_if(float* p, float a, float b, float c, float d, bool pred) {
-  asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.s32 p, %5, 0;\n\t@p st.shared.v4.f32 [%0], {%1, %2, %3, %4};\n\t}"
-               ::"r"((uint32_t)__cvta_generic_to_shared(p)), "f"(a), "f"(b), "f"(c), "f"(d), "r"((int)pred)
-               : "memory");
+// sum over the GX threads of a row (every thread gets the same bits)
+template <int GX, typename T> __device__ __forceinline__ T row_sum(T v) {
+#pragma unroll
+  for (int o = 1; o < GX; o <<= 1) v += __shfl_xor_sync(kFull, v, o);
+  return v;
 }
-// 1 / sqrt(x) and 1 / x to fp32 accuracy (approximation plus one Newton step): the reflector
-// I - beta v v^T is orthogonal only as far as beta v^T v = 2 holds.
-__device__ __forceinline__ float rsqrt_acc(float x) {
-  const float y = rsqrtf(x);
-  return y * fmaf(-0.5f * x * y, y, 1.5f);
-}
-__device__ __forceinline__ float rcp_acc(float x) {
+__device__ __forceinline__ float fma_t(float a, float b, float c) { return fmaf(a, b, c); }
+__device__ __forceinline__ double fma_t(double a, double b, double c) { return fma(a, b, c); }
+__device__ __forceinline__ float abs_t(float x) { return fabsf(x); }
+__device__ __forceinline__ double abs_t(double x) { return fabs(x); }
+__device__ __forceinline__ float rcp_fast(float x) {
   float y;
   asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+  return y;
+}
+__device__ __forceinline__ float lg2(float x) {
+  float y;
+  asm("lg2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+  return y;
+}
+// 1 / sqrt(x) and 1 / x to the accuracy of the type (fp32: approximation plus one Newton step):
+// the reflector I - beta v v^T is orthogonal only as far as beta v^T v = 2 holds.
+__device__ __forceinline__ float rsqrt_t(float x) {
+  float y;
+  asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+  return y * fmaf(-0.5f * x * y, y, 1.5f);
+}
+__device__ __forceinline__ double rsqrt_t(double x) { return rsqrt(x); }
+__device__ __forceinline__ float rcp_t(float x) {
+  const float y = rcp_fast(x);
   return y * fmaf(-x, y, 2.f);
 }
+__device__ __forceinline__ double rcp_t(double x) { return 1.0 / x; }
+// the word that holds the sign and the exponent
+__device__ __forceinline__ unsigned top_word(float x) { return __float_as_uint(x); }
+__device__ __forceinline__ unsigned top_word(double x) { return (unsigned)__double2hiint(x); }
+// a power of two that brings max(|p|, |q|) into [1, 2)
+__device__ __forceinline__ float pow2_scale(float p, float q) {
+  return __uint_as_float(0x7f000000u - (__float_as_uint(fmaxf(fabsf(p), fabsf(q))) & 0x7f800000u));
+}
+__device__ __forceinline__ double pow2_scale(double p, double q) {
+  const int m = max(__double2hiint(p) & 0x7ff00000, __double2hiint(q) & 0x7ff00000);
+  return __hiloint2double(0x7fe00000 - m, 0);
+}
+__device__ __forceinline__ int exponent(float pow2) { return (int)(__float_as_uint(pow2) >> 23) - 127; }
+__device__ __forceinline__ int exponent(double pow2) { return (__double2hiint(pow2) >> 20) - 1023; }
+__device__ __forceinline__ void ld4(const float* p, float (&o)[4]) {
+  const float4 t = *reinterpret_cast<const float4*>(p);
+  o[0] = t.x; o[1] = t.y; o[2] = t.z; o[3] = t.w;
+}
+__device__ __forceinline__ void ld4(const double* p, double (&o)[4]) {
+  const double2 t = *reinterpret_cast<const double2*>(p), u = *reinterpret_cast<const double2*>(p + 2);
+  o[0] = t.x; o[1] = t.y; o[2] = u.x; o[3] = u.y;
+}
+__device__ __forceinline__ void st4(float* p, const float (&v)[4]) { *reinterpret_cast<float4*>(p) = make_float4(v[0], v[1], v[2], v[3]); }
+__device__ __forceinline__ void st4(double* p, const double (&v)[4]) {
+  *reinterpret_cast<double2*>(p) = make_double2(v[0], v[1]);
+  *reinterpret_cast<double2*>(p + 2) = make_double2(v[2], v[3]);
+}
+// Stores to shared memory under a predicate, without a branch.
+__device__ __forceinline__ void st4_if(float* p, const float (&v)[4], bool pred) {
+  asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.s32 p, %5, 0;\n\t@p st.shared.v4.f32 [%0], {%1, %2, %3, %4};\n\t}"
+               ::"r"((uint32_t)__cvta_generic_to_shared(p)), "f"(v[0]), "f"(v[1]), "f"(v[2]), "f"(v[3]), "r"((int)pred)
+               : "memory");
+}
+__device__ __forceinline__ void st4_if(double* p, const double (&v)[4], bool pred) {
+  asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.s32 p, %5, 0;\n\t@p st.shared.v2.f64 [%0], {%1, %2};\n\t"
+               "@p st.shared.v2.f64 [%0+16], {%3, %4};\n\t}"
+               ::"r"((uint32_t)__cvta_generic_to_shared(p)), "d"(v[0]), "d"(v[1]), "d"(v[2]), "d"(v[3]), "r"((int)pred)
+               : "memory");
+}
+__device__ __forceinline__ void st_if(float* p, float v, bool pred) {
+  asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.s32 p, %2, 0;\n\t@p st.shared.f32 [%0], %1;\n\t}"
+               ::"r"((uint32_t)__cvta_generic_to_shared(p)), "f"(v), "r"((int)pred) : "memory");
+}
+__device__ __forceinline__ void st_if(double* p, double v, bool pred) {
+  asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.s32 p, %2, 0;\n\t@p st.shared.f64 [%0], %1;\n\t}"
+               ::"r"((uint32_t)__cvta_generic_to_shared(p)), "d"(v), "r"((int)pred) : "memory");
+}
+__device__ __forceinline__ void cp_async16(float* dst, const float* src) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src) : "memory");
+}
+__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 
-// ---- Householder steps of stage S: k in [S * SS, min((S + 1) * SS, D - 2)) -------------------
-// From step S * SS on the column groups g < S and the row slots q < Q0 are finished, so every
-// range below is static.  State carried from step to step: the matrix a, and column k of the
-// current matrix at the thread's rows (xr) and columns (xc; by symmetry row k).
-template <int D, int S>
-__device__ __forceinline__ void tri_stage(float (&a)[TriCfg<D>::RPT][TriCfg<D>::CPT], float (&xr)[TriCfg<D>::RPT],
-                                          float (&xc)[TriCfg<D>::CPT], float* __restrict__ hv,
-                                          float* __restrict__ xpre, float* __restrict__ tpart,
-                                          float* __restrict__ pvp, float* __restrict__ dg, float* __restrict__ eo,
-                                          float* __restrict__ betas, int tid, float& tr_rest, float& tr_comp, float stop_tr,
-                                          float stop_x2, int r, int& k_stop) {
+// What a thread carries through the Householder steps.
+template <typename T, int D, bool KEEP> struct TriState {
   using C = TriCfg<D>;
-  constexpr int NW = C::NW, RPT = C::RPT, NG = C::NG, SS = C::SS;
-  constexpr int G0 = S;                                               // first live column group
-  constexpr int Q0 = (S * SS >= 31) ? (S * SS - 31) / 32 + 1 : 0;     // first live row slot
-  constexpr int K1 = ((S + 1) * SS < D - 2) ? (S + 1) * SS : D - 2;
-  const int lane = tid & 31, warp = tid >> 5;
-  if (k_stop >= 0) return;
+  T a[C::RT][C::NCH][4];        // its tile of the current matrix
+  float q[KEEP ? C::RT : 1][KEEP ? C::NCH : 1][4];   // its tile of Q
+  T x[C::NCH][4], xr[C::RT];    // column k below the diagonal at its columns and rows, zero elsewhere
+  T y[C::RT];                   // A x at its rows
+  T s2, x1, dk;                 // |x|^2, the subdiagonal entry, the diagonal entry
+  float tr_rest, tr_comp, stop_tr, stop_x2;   // trace not yet reduced, compensated; the stop
+  int k_stop;                   // step at which the reduction stopped early (uniform), or -1
+};
+// Where the steps exchange and leave their results.
+template <typename T> struct TriOut {
+  T *dg, *eo, *yv, *xp;
+  float *betas, *hv;
+  float* stop;                  // [2] (0 or 1) for warps without unfinished rows: the reduction ended in the step before
+  int r;
+};
+
+// From the new column k (s.x, s.xr: not yet masked) to the state before step k: A x and row k+1
+// into shared memory.  M: the chunk that holds column k.
+template <int M, typename T, int D, bool KEEP>
+__device__ __forceinline__ void tri_prepare(TriState<T, D, KEEP>& s, const TriOut<T>& o, int k, int tid) {
+  using C = TriCfg<D>;
+  constexpr int GX = C::GX, RT = C::RT, NCH = C::NCH, CW = C::CW, M2 = M + 1 < NCH ? M + 1 : M;
+  const int lane = tid & 31, g = lane & (GX - 1), row0 = (tid / GX) * RT;
+  const int k1 = k + 1, par = k & 1, kc = k1 - CW * M;      // column k+1 within the chunk (CW: it opens the next one)
+  // the entries k and k+1 of the column
+  const T dkl = (k & 2) ? ((k & 1) ? s.x[M][3] : s.x[M][2]) : ((k & 1) ? s.x[M][1] : s.x[M][0]);
+  const T x1l = (k1 & 2) ? ((k1 & 1) ? s.x[M][3] : s.x[M][2]) : ((k1 & 1) ? s.x[M][1] : (kc == CW ? s.x[M2][0] : s.x[M][0]));
+  s.dk = __shfl_sync(kFull, dkl, (k & (CW - 1)) >> 2);
+  s.x1 = __shfl_sync(kFull, x1l, (k1 & (CW - 1)) >> 2);
+#pragma unroll
+  for (int c = 0; c < 4; ++c) s.x[M][c] = (4 * g + c >= kc) ? s.x[M][c] : T(0);
+#pragma unroll
+  for (int rr = 0; rr < RT; ++rr) s.xr[rr] = (row0 + rr >= k1) ? s.xr[rr] : T(0);
+  // row k+1 of the matrix (predicated stores: no index into the registers may depend on k)
+#pragma unroll
+  for (int rr = 0; rr < RT; ++rr)
+#pragma unroll
+    for (int m = M; m < NCH; ++m) st4_if(o.xp + par * D + CW * m + 4 * g, s.a[rr][m], row0 + rr == k1);
+  T n0 = 0, n1 = 0;
+#pragma unroll
+  for (int rr = 0; rr < RT; ++rr) {
+    T t0 = 0, t1 = 0;
+#pragma unroll
+    for (int m = M; m < NCH; ++m) {
+      t0 = fma_t(s.a[rr][m][0], s.x[m][0], t0); t1 = fma_t(s.a[rr][m][1], s.x[m][1], t1);
+      t0 = fma_t(s.a[rr][m][2], s.x[m][2], t0); t1 = fma_t(s.a[rr][m][3], s.x[m][3], t1);
+    }
+    s.y[rr] = row_sum<GX>(t0 + t1);
+  }
+#pragma unroll
+  for (int m = M; m < NCH; ++m) {
+    n0 = fma_t(s.x[m][0], s.x[m][0], n0); n1 = fma_t(s.x[m][1], s.x[m][1], n1);
+    n0 = fma_t(s.x[m][2], s.x[m][2], n0); n1 = fma_t(s.x[m][3], s.x[m][3], n1);
+  }
+  s.s2 = row_sum<GX>(n0 + n1);
+#pragma unroll
+  for (int rr = 0; rr < RT; ++rr) st_if(o.yv + par * D + row0 + rr, s.y[rr], g == 0);
+}
+
+// ---- Householder steps k whose column k+1 lies in chunk M ---------------------------------------
+// A <- H A H with H = I - beta v v^T: w = u - kappa v, u = A v, kappa = beta v^T u / 2,
+// A <- A - beta (v w^T + w v^T); Q <- Q H.
+template <int M, typename T, int D, bool KEEP>
+__device__ __forceinline__ void tri_stage(TriState<T, D, KEEP>& s, const TriOut<T>& o, int tid) {
+  using C = TriCfg<D>;
+  constexpr int GX = C::GX, RT = C::RT, NCH = C::NCH, CW = C::CW, NW = C::NW, WR = C::WR;
+  constexpr int K0 = CW * M > 0 ? CW * M - 1 : 0, K1 = CW * (M + 1) - 1 < D - 2 ? CW * (M + 1) - 1 : D - 2;
+  constexpr bool F64 = sizeof(T) == 8;
+  const int lane = tid & 31, warp = tid >> 5, g = lane & (GX - 1), row0 = (tid / GX) * RT;
+  if (s.k_stop >= 0) return;
+  int kend = K1;
 #pragma unroll 1
-  for (int k = S * SS; k < K1; ++k) {
-    const int k1 = k + 1, par = k & 1, q1 = k1 >> 5, l1 = k1 & 31;
-    // row k+1 of the current matrix at my columns, for the next step's vector (no branch: the
-    // store is predicated; one lane per warp owns the row)
-#pragma unroll
-    for (int q = Q0; q < RPT; ++q)
-#pragma unroll
-      for (int g = G0; g < NG; ++g)
-        sts_v4_if(xpre + par * D + 4 * (warp + NW * g), a[q][4 * g], a[q][4 * g + 1], a[q][4 * g + 2],
-                  a[q][4 * g + 3], q == q1 && lane == l1);
-    // x = column k below the subdiagonal; its norm; alpha, beta, v
-    float xs[RPT], sq = 0.f, c1 = xr[RPT - 1], ck = xr[RPT - 1];
-#pragma unroll
-    for (int q = RPT - 1; q >= 0; --q) {
-      xs[q] = (q >= Q0 && lane + 32 * q > k1) ? xr[q] : 0.f;
-      sq = fmaf(xs[q], xs[q], sq);
-      c1 = (q == q1) ? xr[q] : c1;
-      ck = (q == (k >> 5)) ? xr[q] : ck;
-    }
-    const float x1 = __shfl_sync(kFull, c1, l1), dk = __shfl_sync(kFull, ck, k & 31);
-    const float tail2 = warp_sum(sq);
-    // With nothing to annihilate (an exactly zero tail) the reflector is the identity: beta = 0
-    // makes p, w and the update vanish, and the step still hands on column k+1.
-    const bool reflect = tail2 > 1e-35f;
-    const float s2 = fmaf(x1, x1, tail2);
-    // Rank-revealing stop: once the rows below k carry a negligible trace (G is positive
-    // semi-definite, so that bounds every entry of the block) and row k hardly couples to them,
-    // T ends at row k.  A history of low rank -- the premise of the method -- then costs its rank
-    // in Householder steps, and every later phase works on the shorter T.
-    {                                    // tr_rest -= dk, compensated (the trace is ~10^7 stop thresholds)
-      const float y = -dk - tr_comp, t = tr_rest + y;
-      tr_comp = (t - tr_rest) - y;
-      tr_rest = t;
-    }
-    if (k1 >= r && tr_rest <= stop_tr && s2 <= stop_x2) {
-      if (tid == 0) { dg[k] = dk; eo[k] = 0.f; betas[k] = 0.f; }
-      k_stop = k;
-      return;
-    }
-    const float nrm = s2 * rsqrt_acc(fmaxf(s2, 1e-37f));
-    const float alpha = reflect ? -copysignf(nrm, x1) : x1;
-    const float vk1 = reflect ? x1 - alpha : 0.f;
-    const float beta = reflect ? rcp_acc(nrm * fabsf(vk1)) : 0.f;
-    if (tid == 0) { dg[k] = dk; eo[k] = alpha; betas[k] = beta; }
-    float vr[RPT], vc[NG][4];
-#pragma unroll
-    for (int q = Q0; q < RPT; ++q) {
-      vr[q] = (lane + 32 * q == k1) ? vk1 : xs[q];
-      if (warp == 0) hv[k * D + lane + 32 * q] = vr[q];        // reflector k (rows <= k stay zero)
-    }
-#pragma unroll
-    for (int g = G0; g < NG; ++g)
-#pragma unroll
-      for (int c = 0; c < 4; ++c) {
-        const int col = 4 * (warp + NW * g) + c;
-        vc[g][c] = (col == k1) ? vk1 : (col > k1 ? xc[4 * g + c] : 0.f);
-      }
-    // my columns' share of A v at my rows, and of p^T v
-    float dp = 0.f;
-#pragma unroll
-    for (int q = Q0; q < RPT; ++q) {
-      float t0 = 0.f, t1 = 0.f;
-#pragma unroll
-      for (int g = G0; g < NG; ++g) {
-        t0 = fmaf(a[q][4 * g], vc[g][0], t0);     t1 = fmaf(a[q][4 * g + 1], vc[g][1], t1);
-        t0 = fmaf(a[q][4 * g + 2], vc[g][2], t0); t1 = fmaf(a[q][4 * g + 3], vc[g][3], t1);
-      }
-      const float pq = t0 + t1;
-      tpart[(par * NW + warp) * D + lane + 32 * q] = pq;
-      dp = fmaf(pq, vr[q], dp);
-    }
-    dp = warp_sum(dp);
-    if (lane == 0) pvp[par * 8 + warp] = dp;
+  for (int k = K0; k < kend; ++k) {
+    const int k1 = k + 1, par = k & 1, kc = k1 - CW * M;
+    const T* const yv = o.yv + par * D;
+    const T* const xp = o.xp + par * D;
     __syncthreads();
-    // p = beta A v at my rows, my columns and at k+1; K = beta p^T v / 2; w = p - K v
-    float pvs = 0.f, pk1 = 0.f;
-#pragma unroll
-    for (int w = 0; w < NW; ++w) { pvs += pvp[par * 8 + w]; pk1 += tpart[(par * NW + w) * D + k1]; }
-    const float kk = 0.5f * beta * beta * pvs;
-    const float wk1 = fmaf(-kk, vk1, beta * pk1);
-    float wr[RPT], wc[NG][4], prow[RPT];
-#pragma unroll
-    for (int q = 0; q < RPT; ++q) prow[q] = 0.f;
-#pragma unroll
-    for (int q = Q0; q < RPT; ++q) {
-      float t = 0.f;
-#pragma unroll
-      for (int w = 0; w < NW; ++w) t += tpart[(par * NW + w) * D + lane + 32 * q];
-      prow[q] = t;
-      wr[q] = (lane + 32 * q > k) ? fmaf(-kk, vr[q], beta * t) : 0.f;
-      // column k+1 of the updated matrix at my rows: row k+1 before the update, corrected
-      xr[q] = fmaf(-wr[q], vk1, fmaf(-vr[q], wk1, xpre[par * D + lane + 32 * q]));
+    if (!KEEP && (warp + 1) * WR <= k1) {                    // only finished rows
+      if (!F64 && *(volatile float*)(o.stop + par) != 0.f) { s.k_stop = k - 1; return; }
+      continue;
     }
+    // x^T A x; meanwhile the reflector's scalars
+    const T yk1 = yv[k1], xpk1 = xp[k1];
+    T d0 = 0, d1 = 0, d2 = 0, d3 = 0;
 #pragma unroll
-    for (int g = G0; g < NG; ++g) {
-      const int cb = 4 * (warp + NW * g);
-      const float4 xp = *reinterpret_cast<const float4*>(xpre + par * D + cb);
-      const float xx[4] = {xp.x, xp.y, xp.z, xp.w};
-      float tt[4];
-      // (A v) at column cb + c is the row sum held by the lane that owns row cb + c (slot
-      // 4 NW g / 32 of that lane): one shuffle instead of NW loads and adds
+    for (int m = M; m < NCH; ++m) {
+      T t[4];
+      ld4(yv + CW * m + 4 * g, t);
+      d0 = fma_t(s.x[m][0], t[0], d0); d1 = fma_t(s.x[m][1], t[1], d1);
+      d2 = fma_t(s.x[m][2], t[2], d2); d3 = fma_t(s.x[m][3], t[3], d3);
+    }
+    const T xax = row_sum<GX>((d0 + d1) + (d2 + d3));
+    // A column of zeros has beta = 0: w and the update vanish, and the step still hands on column k+1.
+    const T tiny = T(F64 ? 1e-290 : 1e-35);
+    const bool reflect = s.s2 > tiny;
+    const T nrm = s.s2 * rsqrt_t(reflect ? s.s2 : tiny);
+    const T alpha = reflect ? (s.x1 < 0 ? nrm : -nrm) : s.x1;
+    const T vk1 = reflect ? s.x1 - alpha : T(0);
+    const T beta = reflect ? rcp_t(nrm * abs_t(vk1)) : T(0);
+    bool stop = false;
+    if (!F64) {
+      // Rank-revealing stop: once the rows below k carry a negligible trace (G is positive
+      // semi-definite, so that bounds every entry of the block) and row k hardly couples to them,
+      // T ends at row k.  A history of low rank -- the premise of the method -- then costs its rank
+      // in Householder steps, and every later phase works on the shorter T.
+      const float d = -(float)s.dk - s.tr_comp, t = s.tr_rest + d;   // compensated: the trace is ~10^7 stop thresholds
+      s.tr_comp = (t - s.tr_rest) - d;
+      s.tr_rest = t;
+      stop = (int)(k1 >= o.r) & (int)(t <= s.stop_tr) & (int)((float)s.s2 <= s.stop_x2);   // no branches
+    }
+    const bool last = tid == C::NT - 1;
+    st_if(o.dg + k, s.dk, last);
+    st_if(o.eo + k, stop ? T(0) : alpha, last);
+    if (!KEEP) st_if(o.betas + k, (float)beta, last);
+    if (!KEEP && !F64) st_if(o.stop + (par ^ 1), stop ? 1.f : 0.f, last);
+    kend = stop ? k1 : kend;
+    s.k_stop = stop ? k : -1;              // this step is still made: it touches nothing left of column k+1
+    // x becomes v
 #pragma unroll
-      for (int c = 0; c < 4; ++c) tt[c] = __shfl_sync(kFull, prow[(4 * NW * g) >> 5], (cb + c) & 31);
+    for (int c = 0; c < 4; ++c) s.x[M][c] = (4 * g + c == kc) ? vk1 : s.x[M][c];
+    if (!KEEP) {                                             // reflector k (zero at rows <= k)
 #pragma unroll
-      for (int c = 0; c < 4; ++c) {
-        wc[g][c] = (cb + c > k) ? fmaf(-kk, vc[g][c], beta * tt[c]) : 0.f;
-        xc[4 * g + c] = fmaf(-wc[g][c], vk1, fmaf(-vc[g][c], wk1, xx[c]));
+      for (int m = M; m < NCH; ++m) {
+        const float f[4] = {(float)s.x[m][0], (float)s.x[m][1], (float)s.x[m][2], (float)s.x[m][3]};
+        st4_if(o.hv + k * D + CW * m + 4 * g, f, (int)(warp == NW - 1) & (int)(lane < GX));
       }
     }
-    // A <- A - v w^T - w v^T on the live block
+    float qs[KEEP ? RT : 1];
+    if (KEEP) {
 #pragma unroll
-    for (int q = Q0; q < RPT; ++q)
+      for (int rr = 0; rr < RT; ++rr) {
+        float q0 = 0.f, q1 = 0.f;
 #pragma unroll
-      for (int g = G0; g < NG; ++g)
+        for (int m = M; m < NCH; ++m)
 #pragma unroll
-        for (int c = 0; c < 4; ++c)
-          a[q][4 * g + c] = fmaf(-vr[q], wc[g][c], fmaf(-wr[q], vc[g][c], a[q][4 * g + c]));
+          for (int c = 0; c < 4; ++c) {
+            if (c & 1) q1 = fmaf(s.q[KEEP ? rr : 0][KEEP ? m : 0][c], (float)s.x[m][c], q1);
+            else q0 = fmaf(s.q[KEEP ? rr : 0][KEEP ? m : 0][c], (float)s.x[m][c], q0);
+          }
+        qs[KEEP ? rr : 0] = (float)beta * row_sum<GX>(q0 + q1);
+      }
+    }
+    // v^T A v = x^T A x - 2 alpha (A x)_{k+1} + alpha^2 a_{k+1,k+1}
+    const T kap = T(0.5) * beta * fma_t(alpha, fma_t(alpha, xpk1, T(-2) * yk1), xax);
+    const T wk1 = fma_t(-kap, vk1, fma_t(-alpha, xpk1, yk1));
+    const T bv1 = beta * vk1, bw1 = beta * wk1;
+    T bv[RT], bw[RT];
+#pragma unroll
+    for (int rr = 0; rr < RT; ++rr) {
+      const int row = row0 + rr;
+      const T xpi = xp[row], v = row == k1 ? vk1 : s.xr[rr];
+      T w = fma_t(-kap, v, fma_t(-alpha, xpi, s.y[rr]));
+      w = row >= k1 ? w : T(0);
+      bv[rr] = beta * v; bw[rr] = beta * w;
+      s.xr[rr] = fma_t(-bw1, v, fma_t(-bv1, w, xpi));
+    }
+#pragma unroll
+    for (int m = M; m < NCH; ++m) {
+      T yy[4], pp[4];
+      ld4(yv + CW * m + 4 * g, yy);
+      ld4(xp + CW * m + 4 * g, pp);
+#pragma unroll
+      for (int c = 0; c < 4; ++c) {
+        const T v = s.x[m][c];
+        T w = fma_t(-kap, v, fma_t(-alpha, pp[c], yy[c]));
+        if (m == M) w = (4 * g + c >= kc) ? w : T(0);        // finished columns stay as they are
+#pragma unroll
+        for (int rr = 0; rr < RT; ++rr) s.a[rr][m][c] = fma_t(-bw[rr], v, fma_t(-bv[rr], w, s.a[rr][m][c]));
+        if (KEEP) {
+#pragma unroll
+          for (int rr = 0; rr < RT; ++rr)
+            s.q[KEEP ? rr : 0][KEEP ? m : 0][c] = fmaf(-qs[KEEP ? rr : 0], (float)v, s.q[KEEP ? rr : 0][KEEP ? m : 0][c]);
+        }
+        s.x[m][c] = fma_t(-bw1, v, fma_t(-bv1, w, pp[c]));   // column k+1 of the updated matrix
+      }
+    }
+    tri_prepare<M, T, D, KEEP>(s, o, k1, tid);
   }
 }
 
-// Number of eigenvalues of T below x, for CH values of x at once.  p_{i+1} = (d_i - x) p_i -
-// e_{i-1}^2 p_{i-1} is the leading principal minor of order i+1 of T - x I; the sign changes
-// along p_0 = 1, p_1, ..., p_D count the eigenvalues below x.  The off-diagonal squares are
-// floored above zero, so an exact zero never persists, and an isolated zero gives one change
-// whichever sign the hardware gives it.
-template <int D, int CH>
-__device__ __forceinline__ void sturm(const float* __restrict__ dg, const float* __restrict__ e2s,
-                                      const float (&x)[CH], int (&cnt)[CH], int nb4) {
-  float p[CH], q[CH];
-  unsigned n[CH];
+// Number of eigenvalues of T below x.  p_{i+1} = (d_i - x) p_i - e_{i-1}^2 p_{i-1} is the leading
+// principal minor of order i+1 of T - x I; the sign changes along p_0 = 1, p_1, ... count the
+// eigenvalues below x.  The off-diagonal squares are floored above zero, so an exact zero never
+// persists, and an isolated zero gives one change whichever sign the hardware gives it.  The
+// signs are shifted into a word (one instruction per row) and their changes counted by blocks of
+// eight rows.  The pair (p, q) is brought back near 1 by a power of two taken two rows before it is
+// applied, off the dependency chain: |d - x| and e^2 are bounded by the scaling of G, and rows
+// shrink by 2^-23 (fp64: 2^-52) at most, so in fp32 every four rows keep it in range, in fp64 every
+// eight.  The next block's rows are fetched while this one is counted.  CH points at once: one
+// chain alone leaves more than half of a scheduler's slots empty.
+template <typename T, int CH>
+__device__ __forceinline__ void sturm(const T* __restrict__ dg, const T* __restrict__ e2s, const T (&x)[CH], int (&n)[CH], int nb8) {
+  T p[CH], q[CH], sc[CH];
+  unsigned bits[CH];
 #pragma unroll
-  for (int h = 0; h < CH; ++h) { p[h] = 1.f; q[h] = 0.f; n[h] = 0; }
-#pragma unroll 4
-  for (int ib = 0; ib < nb4; ++ib) {
-    const float4 d4 = *reinterpret_cast<const float4*>(dg + 4 * ib);
-    const float4 e4 = *reinterpret_cast<const float4*>(e2s + 4 * ib);
-    const float dd[4] = {d4.x, d4.y, d4.z, d4.w}, ee[4] = {e4.x, e4.y, e4.z, e4.w};
+  for (int h = 0; h < CH; ++h) { p[h] = 1; q[h] = 0; bits[h] = 0; n[h] = 0; }
+  T dd[8], ee[8];
+  auto fetch = [&](int at, T (&d)[8], T (&e)[8]) {
 #pragma unroll
-    for (int u = 0; u < 4; ++u)
+    for (int h = 0; h < 2; ++h) {
+      T t[4], u[4];
+      ld4(dg + at + 4 * h, t); ld4(e2s + at + 4 * h, u);
+#pragma unroll
+      for (int c = 0; c < 4; ++c) { d[4 * h + c] = t[c]; e[4 * h + c] = u[c]; }
+    }
+  };
+  fetch(0, dd, ee);
+#pragma unroll 1
+  for (int ib = 0; ib < nb8; ++ib) {
+    T dn[8], en[8];
+    fetch(8 * min(ib + 1, nb8 - 1), dn, en);
+#pragma unroll
+    for (int u = 0; u < 8; ++u)
 #pragma unroll
       for (int h = 0; h < CH; ++h) {
-        const float t = ee[u] * q[h];
-        const float rr = fmaf(dd[u] - x[h], p[h], -t);
-        n[h] += (__float_as_uint(rr) ^ __float_as_uint(p[h])) >> 31;
+        const T rr = fma_t(dd[u] - x[h], p[h], -(ee[u] * q[h]));
+        bits[h] = __funnelshift_l(top_word(rr), bits[h], 1);
         q[h] = p[h]; p[h] = rr;
+        constexpr int P = sizeof(T) == 4 ? 4 : 8;
+        if (u % P == P - 3) sc[h] = pow2_scale(p[h], q[h]);
+        if (u % P == P - 1) { p[h] *= sc[h]; q[h] *= sc[h]; }
       }
-    // bring the larger of (p, q) back into [1, 2): |d - x| and e^2 are bounded by the scaling of G,
-    // so four steps can neither overflow nor (factors above 2^-23 each) underflow
 #pragma unroll
-    for (int h = 0; h < CH; ++h) {
-      const unsigned m = __float_as_uint(fmaxf(fabsf(p[h]), fabsf(q[h]))) >> 23;
-      const float sc = __uint_as_float((254u - m) << 23);
-      p[h] *= sc; q[h] *= sc;
-    }
+    for (int h = 0; h < CH; ++h) n[h] += __popc((bits[h] ^ (bits[h] >> 1)) & 0xffu);
+#pragma unroll
+    for (int u = 0; u < 8; ++u) { dd[u] = dn[u]; ee[u] = en[u]; }
   }
+}
+
+// One of the two minor sequences of T - lambda I for one eigenvalue, and the multipliers of z:
+//   DOWN = false: leading minors p_i;   z_i = mul_i z_{i+1},  mul_i = -e_i p_i / p_{i+1}
+//   DOWN = true:  trailing minors t_i;  z_i = mul_i z_{i-1},  mul_i = -e_{i-1} t_{i+1} / t_i
+// mn[i] = log2 of the minor before row i (p_i, t_{i+1}).  A minor below pfl times the one before is
+// replaced by that much (a perturbation of d_i by pfl).  Four rows are fetched ahead.
+template <bool DOWN, typename T, int RP>
+__device__ __forceinline__ void minors(const T* __restrict__ dg, const T* __restrict__ eo, const T* __restrict__ e2s, int de,
+                                       T lam, T pfl, float* __restrict__ mul, float* __restrict__ mn) {
+  T p = 1, po = 0;
+  int ex = 0;
+  auto fetch = [&](int t0, T (&d)[4], T (&e2)[4], T (&e1)[4]) {
 #pragma unroll
-  for (int h = 0; h < CH; ++h) cnt[h] = (int)n[h];
+    for (int u = 0; u < 4; ++u) {
+      const int t = min(t0 + u, de - 1), n = DOWN ? de - 1 - t : t;
+      d[u] = dg[n];
+      if (DOWN) {                       // e2s[0] = 0 stands for the coupling past the last row
+        e2[u] = e2s[t > 0 ? n + 1 : 0];
+        e1[u] = eo[max(n - 1, 0)];      // unused at n = 0
+      } else {
+        e2[u] = e2s[n];
+        e1[u] = eo[n];
+      }
+    }
+  };
+  T d[4], e2[4], e1[4];
+  fetch(0, d, e2, e1);
+#pragma unroll 1
+  for (int t0 = 0; t0 < de; t0 += 4) {
+    T dn[4], e2n[4], e1n[4];
+    fetch(t0 + 4, dn, e2n, e1n);
+    float mu[4], lg[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      lg[u] = lg2(fabsf((float)p)) + (float)ex;
+      T np = fma_t(d[u] - lam, p, -(e2[u] * po));
+      const T fl = pfl * abs_t(p);
+      np = abs_t(np) >= fl ? np : -fl;
+      mu[u] = -(float)e1[u] * ((float)p * rcp_fast((float)np));
+      po = p; p = np;
+    }
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const int n = DOWN ? de - 1 - (t0 + u) : t0 + u;
+      st_if(mul + n * RP, mu[u], t0 + u < de);
+      st_if(mn + n * RP, lg[u], t0 + u < de);
+    }
+    const T sc = pow2_scale(p, po);
+    p *= sc; po *= sc; ex -= exponent(sc);
+#pragma unroll
+    for (int u = 0; u < 4; ++u) { d[u] = dn[u]; e2[u] = e2n[u]; e1[u] = e1n[u]; }
+  }
 }
 
 // Acceptance thresholds (chosen by the storage type).
@@ -307,6 +475,502 @@ struct TriTol {
   float sweep_stop;  // of the Jacobi fallback
 };
 
+struct TriShared {
+  double trace;
+  float tr_t;
+  float stop[2];
+  int flags[4];
+  int why;
+};
+
+// Steps 2-7 in T for the user of this CTA; acc: the thread's tile of G in fp32.  Returns whether the
+// result is certified; Vc: where the vectors are ([D][RP]).  theta[] holds the eigenvalues of sc * G,
+// part[NW ..] the largest component of every vector per warp.  Without force, nothing is finished
+// that cannot be certified any more.
+template <typename T, int D, int RP>
+__device__ __forceinline__ bool tri_chain(const float (&acc)[TriCfg<D>::RT][TriCfg<D>::NCH][4], float* __restrict__ smem,
+                                          TriShared& sh, const float* __restrict__ gout, float sc, int r, bool force,
+                                          const TriTol& tol, bool trigger_early, float*& Vc_out, int& passes, int tid) {
+  using C = TriCfg<D>;
+  using L = TriSmem<D, RP>;
+  constexpr int GX = C::GX, RT = C::RT, NT = C::NT, NW = C::NW, NCH = C::NCH, CW = C::CW, LD = C::LD;
+  constexpr bool F64 = sizeof(T) == 8, KEEP = !F64 && D <= 64;
+  constexpr int NE = RP / 32;                 // groups of 32 eigenvalues (columns)
+  const int lane = tid & 31, warp = tid >> 5, g = lane & (GX - 1), row0 = (tid / GX) * RT;
+  T* const dg = reinterpret_cast<T*>(smem + L::DG);
+  T* const eo = reinterpret_cast<T*>(smem + L::EO);
+  T* const e2s = reinterpret_cast<T*>(smem + L::E2);
+  T* const lamv = reinterpret_cast<T*>(smem + L::LAM);
+  float* const theta = smem + L::TH;
+  float* const part = smem + L::PART;
+  bool ok = true;
+  passes = 0;
+
+  // ---- 2. Householder tridiagonalisation, the matrix in registers ------------------------------
+  int k_stop;
+  {
+    TriOut<T> o;
+    o.dg = dg; o.eo = eo;
+    o.yv = reinterpret_cast<T*>(smem + L::YV);
+    o.xp = reinterpret_cast<T*>(smem + L::XP);
+    o.betas = smem + L::BE; o.hv = smem + L::R0;
+    o.stop = sh.stop; o.r = r;
+    TriState<T, D, KEEP> s;
+    const float trs = (float)((double)sc * sh.trace);
+    s.tr_rest = trs; s.tr_comp = 0.f;
+    s.stop_tr = trs * tol.stop_trace;
+    s.stop_x2 = (trs * tol.stop_couple) * (trs * tol.stop_couple);
+    s.k_stop = -1;
+#pragma unroll
+    for (int rr = 0; rr < RT; ++rr)
+#pragma unroll
+      for (int m = 0; m < NCH; ++m)
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+          s.a[rr][m][c] = (T)(acc[rr][m][c] * sc);
+          if (KEEP) s.q[KEEP ? rr : 0][KEEP ? m : 0][c] = (CW * m + 4 * g + c == row0 + rr) ? 1.f : 0.f;
+        }
+    // column 0 (= row 0), by way of the buffer that step 1 writes
+#pragma unroll
+    for (int m = 0; m < NCH; ++m) st4_if(o.xp + D + CW * m + 4 * g, s.a[0][m], row0 == 0);
+    if (!KEEP)
+      for (int e = tid; e < D * D / 4; e += NT) reinterpret_cast<float4*>(o.hv)[e] = make_float4(0.f, 0.f, 0.f, 0.f);
+    __syncthreads();
+#pragma unroll
+    for (int m = 0; m < NCH; ++m) ld4(o.xp + D + CW * m + 4 * g, s.x[m]);
+#pragma unroll
+    for (int rr = 0; rr < RT; ++rr) s.xr[rr] = o.xp[D + row0 + rr];
+    tri_prepare<0, T, D, KEEP>(s, o, 0, tid);
+    tri_stage<0, T, D, KEEP>(s, o, tid);
+    tri_stage<1, T, D, KEEP>(s, o, tid);
+    if constexpr (NCH > 2) {
+      tri_stage<2, T, D, KEEP>(s, o, tid);
+      tri_stage<3, T, D, KEEP>(s, o, tid);
+    }
+    // Finished warps learn of a stop one barrier later.  Those that did in the loop have passed that
+    // barrier there; for all others (no stop, or one in the very last step) it is this one.
+    if (!KEEP && !F64 && (s.k_stop < 0 || (warp + 1) * C::WR > s.k_stop + 1)) {
+      __syncthreads();
+      if (s.k_stop < 0 && *(volatile float*)(sh.stop + (D & 1)) != 0.f) s.k_stop = D - 3;
+    }
+    // the last 2 x 2 block
+    if (s.k_stop < 0 && tid == NT - 1) {
+      dg[D - 2] = s.dk; eo[D - 2] = s.x1; eo[D - 1] = 0;
+      dg[D - 1] = s.a[RT - 1][NCH - 1][3];
+    }
+    if (KEEP) {
+      float* Qt = smem + L::R0;
+#pragma unroll
+      for (int rr = 0; rr < RT; ++rr)
+#pragma unroll
+        for (int m = 0; m < NCH; ++m)
+#pragma unroll
+          for (int c = 0; c < 4; ++c) Qt[(CW * m + 4 * g + c) * LD + row0 + rr] = s.q[KEEP ? rr : 0][KEEP ? m : 0][c];
+    }
+    k_stop = s.k_stop;
+  }
+  // T has `de` rows (all D unless the reduction stopped early), padded with zero rows to a multiple of 8
+  const int de = k_stop >= 0 ? k_stop + 1 : D, de8 = (de + 7) & ~7;
+  const int kb = k_stop >= 0 ? k_stop : D - 2;            // reflectors 0 .. kb-1 exist
+  if (tid < de8 - de) { dg[de + tid] = 0; eo[de + tid] = 0; }
+  __syncthreads();
+
+  // ---- 3. Gershgorin interval, floored squares, trace (every warp for itself); multisection ------
+  T lo, hi, tnorm;
+  {
+    T l = T(3.0e38), h = T(-3.0e38), tr = 0;
+#pragma unroll
+    for (int q = 0; q < D / 32; ++q) {
+      const int n = lane + 32 * q;
+      const bool in = n < de;
+      const T el0 = eo[max(n - 1, 0)], er0 = eo[n], dd0 = dg[n];
+      const T el = ((int)in & (int)(n > 0)) ? el0 : T(0), er = in ? er0 : T(0), dd = in ? dd0 : T(0);   // eo[de-1] = 0
+      const T rad = abs_t(er) + abs_t(el);
+      l = ((int)in & (int)(dd - rad < l)) ? dd - rad : l;
+      h = ((int)in & (int)(dd + rad > h)) ? dd + rad : h;
+      tr += dd;
+    }
+#pragma unroll
+    for (int o = 16; o; o >>= 1) {
+      const T l2 = __shfl_xor_sync(kFull, l, o), h2 = __shfl_xor_sync(kFull, h, o);
+      l = l2 < l ? l2 : l; h = h2 > h ? h2 : h;
+      tr += __shfl_xor_sync(kFull, tr, o);
+    }
+    const T span = h - l;
+    lo = l - T(1e-6) * span - T(1e-30); hi = h + T(1e-6) * span + T(1e-30);
+    tnorm = -lo > hi ? -lo : hi;
+    const T fl = tnorm * T(F64 ? 2.7755575615628914e-17 : 1.4901161e-08);           // 2^-55, 2^-26 of |T|
+    if (warp == 0) {
+      for (int n = lane; n < de8; n += 32) {
+        const T e = n > 0 ? eo[n - 1] : T(0);
+        e2s[n] = n > 0 ? (e * e > fl * fl ? e * e : fl * fl) : T(0);
+      }
+      if (lane == 0) sh.tr_t = (float)tr;
+    }
+  }
+  __syncthreads();
+  {
+    constexpr int PT = NT / RP < 8 ? NT / RP : 8;               // lanes per eigenvalue
+    constexpr int CH = NW == 4 ? 2 : 1, NPT = PT * CH;          // points per lane (one warp per scheduler: two)
+    constexpr int STEPS = (NPT == 8 ? 9 : 12);                  // (NPT + 1)^STEPS >= 2^27
+    static_assert(PT * RP == NT && (NPT == 8 || NPT == 4), "every lane has points");
+    const int j = tid / PT, pt = tid % PT, jj = j < r ? j : r - 1;     // surplus lanes shadow column r-1
+    const int target = de8 - 1 - jj;    // lambda_(jj-th largest) >= x  <=>  #(eigenvalues < x) <= target
+#pragma unroll 1
+    for (int step = 0; step < STEPS; ++step) {
+      const T w = (hi - lo) * T(1.0 / (NPT + 1));
+      T x[CH];
+      int n[CH], idx = 0;                                        // points at or below the eigenvalue
+#pragma unroll
+      for (int h = 0; h < CH; ++h) x[h] = fma_t(T(pt + h * PT + 1), w, lo);
+      sturm<T, CH>(dg, e2s, x, n, de8 >> 3);
+#pragma unroll
+      for (int h = 0; h < CH; ++h)
+        idx += __popc((__ballot_sync(kFull, n[h] <= target) >> (lane & ~(PT - 1))) & ((1u << PT) - 1));
+      const T nlo = fma_t(T(idx), w, lo), nhi = fma_t(T(idx + 1), w, lo);
+      lo = idx == 0 ? lo : nlo;
+      hi = idx == NPT ? hi : nhi;
+    }
+    if (pt == 0) lamv[j] = T(0.5) * (lo + hi);
+  }
+  __syncthreads();
+  // A reduction to tridiagonal form is backward stable in the norm of G only: it fixes a kept
+  // vector to an angle of a few eps |T| / gap, whatever the size of its eigenvalue.  Where a
+  // gap among the kept eigenvalues is too small for the angle the storage type needs (a
+  // strongly graded spectrum such as sigma_i = i^-1.5 over 128 directions), this route is not
+  // to be trusted.
+  if (!F64) {
+    const int tight = tid < r - 1 && (float)(lamv[tid] - lamv[tid + 1]) < tol.gap_min * (float)lamv[0];
+    if (__syncthreads_or(tight)) {
+      ok = false;
+      if (tid == 0) sh.why |= kWhyGap;
+      if (!force) return false;
+    }
+  }
+
+  // ---- 4. twisted factorisation -----------------------------------------------------------------
+  float* const up = smem + L::A1;
+  float* const dn = smem + L::A2;
+  float* const lp = smem + L::A3;
+  float* const lt = smem + L::A4;
+  {
+    const T pfl = tnorm * T(F64 ? 1.734723475976807e-18 : 9.3132257e-10);            // pivot floor 2^-59, 2^-30 of |T|
+    if (warp < NE) minors<false, T, RP>(dg, eo, e2s, de, lamv[32 * warp + lane], pfl, up + 32 * warp + lane, lp + 32 * warp + lane);
+    else if (warp < 2 * NE)
+      minors<true, T, RP>(dg, eo, e2s, de, lamv[32 * (warp - NE) + lane], pfl, dn + 32 * (warp - NE) + lane, lt + 32 * (warp - NE) + lane);
+  }
+  __syncthreads();
+  constexpr int NS = NT / RP;                                    // threads per eigenvalue here
+  {
+    const int j = tid % RP, sl = tid / RP;
+    float best = -3.0e38f;
+    int kbest = 0;
+#pragma unroll 4
+    for (int n = sl; n < de; n += NS) {
+      const float v = lp[n * RP + j] + lt[n * RP + j];
+      kbest = v > best ? n : kbest;
+      best = fmaxf(v, best);
+    }
+    part[sl * RP + j] = best;
+    reinterpret_cast<int*>(part)[(NW + sl) * RP + j] = kbest;
+  }
+  __syncthreads();
+  // z_kt = 1, upwards and downwards from there on two warps (no branches: a lane that has not
+  // reached its twist index yet keeps z = 1)
+  float* const Z = lp;
+  if (warp < 2 * NE) {
+    const bool dwn = warp >= NE;
+    const int j = 32 * (dwn ? warp - NE : warp) + lane;
+    float best = -3.4e38f;
+    int kt = 0;
+#pragma unroll
+    for (int sl = 0; sl < NS; ++sl) {
+      const float v = part[sl * RP + j];
+      const int kk = reinterpret_cast<const int*>(part)[(NW + sl) * RP + j];
+      const bool take = (int)(v > best) | ((int)(v == best) & (int)(kk < kt));
+      best = take ? v : best;
+      kt = take ? kk : kt;
+    }
+    const float* const mul = (dwn ? dn : up) + j;
+    const int n0 = dwn ? 0 : de - 1, sg = dwn ? 1 : -1, tk = dwn ? kt : de - 1 - kt;   // the twist is met at t = tk
+    float z = 1.f, ss = 0.f;
+#pragma unroll 1
+    for (int t0 = 0; t0 < de; t0 += 8) {
+      float mu[8];
+#pragma unroll
+      for (int u = 0; u < 8; ++u) mu[u] = mul[(n0 + sg * min(t0 + u, de - 1)) * RP];
+#pragma unroll
+      for (int u = 0; u < 8; ++u) {
+        const int t = t0 + u;
+        z = t > tk ? z * mu[u] : 1.f;
+        const float zi = ((int)(t > tk) & (int)(t < de)) ? z : 0.f;
+        ss = fmaf(zi, zi, ss);
+        st_if(Z + (n0 + sg * t) * RP + j, z, (int)(t >= tk) & (int)(t < de));
+      }
+    }
+    // behind the entries that the other half may still be reading
+    part[(2 * NW + (dwn ? 1 : 0)) * RP + j] = ss;
+  }
+  __syncthreads();
+
+  // ---- 5. V = Q Z -------------------------------------------------------------------------------
+  float* Vc = smem + L::A1;      // current vectors
+  float* Vn = smem + L::A2;      // next
+  const float* const zs = part + 2 * NW * RP;
+  if constexpr (KEEP) {
+    const float* Qt = smem + L::R0;
+    constexpr int CG = RP / 4, RS = NT / CG, NP = (D / 4 + RS - 1) / RS;      // 4 x 4 tiles of V, NP per thread
+    const int cg = tid % CG, rq = tid / CG;
+    if (RS * NP == D / 4 || rq < D / 4) {
+      float v[NP][4][4];
+#pragma unroll
+      for (int n = 0; n < NP; ++n)
+#pragma unroll
+        for (int x = 0; x < 4; ++x)
+#pragma unroll
+          for (int c = 0; c < 4; ++c) v[n][x][c] = 0.f;
+#pragma unroll 4
+      for (int t = 0; t < de; ++t) {
+        float z[4];
+        ld4(Z + t * RP + 4 * cg, z);
+#pragma unroll
+        for (int n = 0; n < NP; ++n) {
+          float q[4];
+          ld4(Qt + t * LD + 4 * (rq + n * RS), q);
+#pragma unroll
+          for (int x = 0; x < 4; ++x)
+#pragma unroll
+            for (int c = 0; c < 4; ++c) v[n][x][c] = fmaf(q[x], z[c], v[n][x][c]);
+        }
+      }
+      float zn[4];
+#pragma unroll
+      for (int c = 0; c < 4; ++c) zn[c] = rsqrtf(1.f + zs[4 * cg + c] + zs[RP + 4 * cg + c]);   // 1 / |z|
+#pragma unroll
+      for (int n = 0; n < NP; ++n)
+#pragma unroll
+        for (int x = 0; x < 4; ++x) {
+          const float t[4] = {v[n][x][0] * zn[0], v[n][x][1] * zn[1], v[n][x][2] * zn[2], v[n][x][3] * zn[3]};
+          st4(Vc + (4 * (rq + n * RS) + x) * RP + 4 * cg, t);
+        }
+    }
+  } else {
+    // v = H_0 H_1 ... H_{kb-1} z: TPV threads per vector, RB rows each (16-byte pieces dealt round
+    // robin: conflict-free), the reflector's inner product completed by shuffles
+    constexpr int TPV = NT / RP, RB = D / TPV;
+    const int j = tid / TPV, qt = tid % TPV;
+    const float zn = rsqrtf(1.f + zs[j] + zs[RP + j]);
+    const float* hv = smem + L::R0 + 4 * qt;
+    const float* betas = smem + L::BE;
+    float z[RB];
+#pragma unroll
+    for (int u = 0; u < RB; ++u) {
+      const int n = ((u >> 2) * TPV + qt) * 4 + (u & 3);
+      z[u] = n < de ? Z[n * RP + j] * zn : 0.f;
+    }
+#pragma unroll 2
+    for (int k = kb - 1; k >= 0; --k) {
+      float h[RB], d0 = 0.f, d1 = 0.f;
+#pragma unroll
+      for (int u = 0; u < RB; u += 4) {
+        float t[4];
+        ld4(hv + k * D + (u >> 2) * TPV * 4, t);
+        h[u] = t[0]; h[u + 1] = t[1]; h[u + 2] = t[2]; h[u + 3] = t[3];
+        d0 = fmaf(t[0], z[u], d0);     d1 = fmaf(t[1], z[u + 1], d1);
+        d0 = fmaf(t[2], z[u + 2], d0); d1 = fmaf(t[3], z[u + 3], d1);
+      }
+      const float c = -betas[k] * row_sum<TPV>(d0 + d1);
+#pragma unroll
+      for (int u = 0; u < RB; ++u) z[u] = fmaf(c, h[u], z[u]);
+    }
+#pragma unroll
+    for (int u = 0; u < RB; ++u) Vc[(((u >> 2) * TPV + qt) * 4 + (u & 3)) * RP + j] = z[u];
+  }
+  __syncthreads();
+  // The long serial part is over: the next kernel may start launching -- unless the process runs
+  // many requests at once, where its parked CTAs are better kept out a little longer (after the
+  // certificate).
+  if (trigger_early) pdl_trigger();
+
+  // G for the residuals, over Q or the reflectors; it arrives behind step 6
+  float* const Gsm = smem + L::R0;
+  for (int e = tid; e < D * D / 4; e += NT) cp_async16(Gsm + 4 * e, gout + 4 * e);
+
+  // ---- 6. orthogonalisation passes while V^T V - I is above the rounding level ---------------------
+  // Column-parallel: lane = column(s) c, c + 32; a warp takes RP / NW rows a of E.
+  constexpr int AW = RP / NW;
+  float* const Em = smem + L::A4;
+  for (;;) {
+    float ev[NE][AW];
+#pragma unroll
+    for (int h = 0; h < NE; ++h)
+#pragma unroll
+      for (int u = 0; u < AW; ++u) ev[h][u] = 0.f;
+    const int a0 = warp * AW;
+#pragma unroll 8
+    for (int n = 0; n < D; ++n) {
+      float av[AW];
+#pragma unroll
+      for (int u = 0; u < AW; u += 4) {
+        float t[4];
+        ld4(Vc + n * RP + a0 + u, t);
+        av[u] = t[0]; av[u + 1] = t[1]; av[u + 2] = t[2]; av[u + 3] = t[3];
+      }
+#pragma unroll
+      for (int h = 0; h < NE; ++h) {
+        const float vc = Vc[n * RP + 32 * h + lane];
+#pragma unroll
+        for (int u = 0; u < AW; ++u) ev[h][u] = fmaf(av[u], vc, ev[h][u]);
+      }
+    }
+    float emax = 0.f;
+#pragma unroll
+    for (int h = 0; h < NE; ++h)
+#pragma unroll
+      for (int u = 0; u < AW; ++u) {
+        const int x = a0 + u, c = 32 * h + lane;
+        float e = ev[h][u] - (x == c ? 1.f : 0.f);
+        e = ((int)(x >= r) | (int)(c >= r)) ? 0.f : e;       // surplus columns are copies of column r-1
+        Em[x * RP + c] = e;
+        emax = (fabsf(e) <= emax) ? emax : fabsf(e);         // a NaN stays
+      }
+#pragma unroll
+    for (int o = 16; o; o >>= 1) {
+      const float e2 = __shfl_xor_sync(kFull, emax, o);
+      emax = (e2 <= emax) ? emax : e2;
+    }
+    if (lane == 0) part[warp] = emax;
+    __syncthreads();
+    float em = 0.f;
+#pragma unroll
+    for (int w = 0; w < NW; ++w) { const float e = part[w]; em = (e <= em) ? em : e; }
+    if (em <= tol.ortho) break;                       // orthonormal to rounding
+    if (passes == 6 || !(em <= 0.98f)) { ok = false; if (tid == 0) sh.why |= kWhyOrtho; break; }
+    ++passes;
+    // One pass of Gram-Schmidt against the ORIGINAL earlier columns (larger eigenvalues, the
+    // better determined vectors): v_c <- (v_c - sum_{a<c} E_ac v_a) / |.|.  A later column never
+    // changes an earlier one, so a poorly separated pair cannot damage its neighbours; for
+    // two vectors the pass is exact, for more it converges quadratically like the symmetric
+    // form.  Rows n of V' for this warp: D / NW of them; lane = column.
+#pragma unroll 1
+    for (int h = 0; h < NE; ++h) {
+      const int c = 32 * h + lane;
+      float ecol[RP], nn = 1.f;
+#pragma unroll
+      for (int x = 0; x < RP; ++x) {
+        const float e = Em[x * RP + c];
+        ecol[x] = x < c ? e : 0.f;
+        nn += x < c ? -e * e : (x == c ? e : 0.f);
+      }
+      const float scol = rsqrtf(fmaxf(nn, 1e-6f));
+#pragma unroll 2
+      for (int n = warp; n < D; n += NW) {
+        float o0 = 0.f, o1 = 0.f;
+#pragma unroll
+        for (int x = 0; x < RP; x += 4) {
+          const float4 t = *reinterpret_cast<const float4*>(Vc + n * RP + x);
+          o0 = fmaf(t.x, ecol[x], o0);     o1 = fmaf(t.y, ecol[x + 1], o1);
+          o0 = fmaf(t.z, ecol[x + 2], o0); o1 = fmaf(t.w, ecol[x + 3], o1);
+        }
+        Vn[n * RP + c] = (Vc[n * RP + c] - (o0 + o1)) * scol;
+      }
+    }
+    __syncthreads();
+    float* t = Vc; Vc = Vn; Vn = t;
+    // With E = L + diag + L^T the pass leaves (I - L)(I + E)(I - L^T) = I + diag - L L^T - L^2 -
+    // (L^T)^2 + O(E^3), and the scaling removes the diagonal: what remains off the diagonal is
+    // below 3 r max|E|^2.  Where that is a quarter of the bound, V^T V is not formed again.
+    if (3.f * (float)r * em * em <= 0.25f * tol.ortho) break;
+  }
+  Vc_out = Vc;
+  cp_async_wait_all();
+  __syncthreads();      // G is staged; the vectors are settled; the warps' maxima are read
+  if (!ok && !force) return false;
+
+  // ---- 7. Rayleigh quotients and residuals against G; certification; the largest components -------
+  {
+    constexpr int RW = D / NW;        // rows of Y = G V per warp
+    float y[NE][RW];
+#pragma unroll
+    for (int h = 0; h < NE; ++h)
+#pragma unroll
+      for (int u = 0; u < RW; ++u) y[h][u] = 0.f;
+    const int i0 = warp * RW;
+#pragma unroll 2
+    for (int k = 0; k < D; k += 4) {
+      float vk[NE][4];
+#pragma unroll
+      for (int h = 0; h < NE; ++h)
+#pragma unroll
+        for (int u = 0; u < 4; ++u) vk[h][u] = Vc[(k + u) * RP + 32 * h + lane];
+#pragma unroll
+      for (int u = 0; u < RW; ++u) {
+        const float4 gg = *reinterpret_cast<const float4*>(Gsm + (i0 + u) * D + k);
+#pragma unroll
+        for (int h = 0; h < NE; ++h) {
+          y[h][u] = fmaf(gg.x, vk[h][0], y[h][u]); y[h][u] = fmaf(gg.y, vk[h][1], y[h][u]);
+          y[h][u] = fmaf(gg.z, vk[h][2], y[h][u]); y[h][u] = fmaf(gg.w, vk[h][3], y[h][u]);
+        }
+      }
+    }
+    float* const lead = part + NW * RP;                // [NW][RP] the largest component of the warp's rows
+#pragma unroll
+    for (int h = 0; h < NE; ++h) {
+      float t = 0.f, best = -1.f, lv = 1.f;
+#pragma unroll
+      for (int u = 0; u < RW; ++u) {
+        const float v = Vc[(i0 + u) * RP + 32 * h + lane];
+        y[h][u] *= sc;
+        t = fmaf(v, y[h][u], t);
+        lv = fabsf(v) > best ? v : lv;                          // strict: lowest index wins a tie
+        best = fmaxf(fabsf(v), best);
+      }
+      part[warp * RP + 32 * h + lane] = t;
+      lead[warp * RP + 32 * h + lane] = lv;
+    }
+    __syncthreads();
+#pragma unroll
+    for (int h = 0; h < NE; ++h) {
+      const int c = 32 * h + lane;
+      float th = 0.f;
+      if (F64) {
+        th = (float)lamv[c];             // accurate relative to the eigenvalue itself, unlike an fp32 quotient
+      } else {
+#pragma unroll
+        for (int w = 0; w < NW; ++w) th += part[w * RP + c];
+      }
+      if (warp == 0) theta[c] = th;
+      float t = 0.f;
+#pragma unroll
+      for (int u = 0; u < RW; ++u) {
+        const float d = fmaf(-th, Vc[(i0 + u) * RP + c], y[h][u]);
+        t = fmaf(d, d, t);
+      }
+      part[(2 * NW + warp) * RP + c] = t;
+    }
+    __syncthreads();
+    int good = 1;
+    if (tid < r) {
+      const float th1 = theta[0], thi = theta[tid];
+      float gap = 3.0e38f, rho2 = 0.f;
+#pragma unroll
+      for (int w = 0; w < NW; ++w) rho2 += part[(2 * NW + w) * RP + tid];
+      if (tid > 0) gap = fminf(gap, theta[tid - 1] - thi);
+      if (tid < r - 1) gap = fminf(gap, thi - theta[tid + 1]);
+      const float resn = sqrtf(rho2);
+      const bool res_ok = resn <= fmaxf(tol.eps_vec * gap, tol.floor_rel * th1);
+      // T is similar to sc * G: the traces agree to rounding
+      const float trG = (float)((double)sc * sh.trace);
+      const bool tr_ok = fabsf(sh.tr_t - trG) <= 1e-4f * fabsf(trG) && isfinite(thi) && isfinite(resn);
+      if (!res_ok) atomicOr(&sh.why, kWhyResidual);
+      if (!tr_ok) atomicOr(&sh.why, kWhyTrace);
+      good = res_ok && tr_ok;
+    }
+    ok = __syncthreads_and(good) && ok;
+  }
+  return ok;
+}
+
 // The eigensolve of user blockIdx.x; every thread of the CTA calls it and all leave together.
 // With want_vs, a certified tridiagonal result also leaves V Sigma at the start of the dynamic
 // shared memory ([D][rp], rp = r rounded up to 4, zero in the padding) and true is returned.
@@ -316,81 +980,72 @@ __device__ __forceinline__ bool eig_user(const float* __restrict__ gpart, const 
                                          const TriTol& tol, bool want_vs, bool late_trigger, float* __restrict__ S,
                                          float* __restrict__ V, int* __restrict__ info,
                                          int* __restrict__ route_taken) {
-  using Cfg = TriCfg<D>;
+  using C = TriCfg<D>;
   using L = TriSmem<D, RP>;
-  constexpr int NT = Cfg::NT, NW = Cfg::NW, RPT = Cfg::RPT, CPT = Cfg::CPT, NG = Cfg::NG, LD = Cfg::LD;
-  constexpr int NE = RP / 32;                 // groups of 32 eigenvalues (columns)
-  constexpr int WG = NW / NE;                 // warps per group in the eigenvalue-parallel phases
+  constexpr int GX = C::GX, RT = C::RT, NT = C::NT, NW = C::NW, NCH = C::NCH, CW = C::CW, LD = C::LD, NE = RP / 32;
   extern __shared__ __align__(16) float smem[];
-  float* hv = smem + L::HV;
-  float* vs = smem + L::VS;
-  float* work = smem + L::WORK;
-  float* Em = smem + L::EM;
-  float* dg = smem + L::DG;
-  float* eo = smem + L::EO;
-  float* e2s = smem + L::E2;
-  float* betas = smem + L::BE;
-  float* xpre = smem + L::XP;
-  float* tpart = smem + L::TP;
-  float* pvp = smem + L::PV;
-  float* lamv = smem + L::LAM;
-  float* theta = smem + L::TH;
-  float* rho2 = smem + L::RH;
-  float* sgn = smem + L::SG;
-  int* ktv = reinterpret_cast<int*>(smem + L::KT);
-  float* part = smem + L::PART;
-  __shared__ float s_gmax, s_lo, s_hi, s_emax, s_trT;
-  __shared__ double s_trace;
-  __shared__ int s_flags[4];
-  __shared__ int s_why;
-
+  __shared__ TriShared sh;
   const int b = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int g = lane & (GX - 1), row0 = (tid / GX) * RT;
+  float* const theta = smem + L::TH;
+  float* const part = smem + L::PART;
   pdl_wait();          // everything below reads what the Gram kernel wrote
 
-  // ---- 1. G = sum of the slices' partial Grams, in a fixed order -----------------------------
-  float* Gs = work;    // [D][LD] staging copy
+  // ---- 1. G = sum of the slices' partial Grams, in a fixed order, in the registers' layout ---------
   // the summed matrix in global memory: a user's only partial as it is, else written below
   const float* gout = parts == 1 ? gpart + (size_t)b * D * D : gsum + (size_t)b * D * D;
+  float acc[RT][NCH][4];
   {
     const float4* gp = reinterpret_cast<const float4*>(gpart + (size_t)b * parts * D * D);
     int lost = 0;
     for (int s = tid; s < splits; s += NT) lost |= (gram_status[b * splits + s] != kGramStatusOk);
-    int bad = 0;
-    // fp32 sums in slice order.  A thread owns EPT 16-byte elements; the loads of SC slices for all
-    // of them are issued before the first add: the phase is bound by their latency.
-    constexpr int EPT = D * D / 4 / NT;
-    constexpr int SC = (EPT >= 16) ? 2 : (EPT >= 8) ? 3 : 8;
-    static_assert(EPT * NT * 4 == D * D, "whole elements");
-    float4 acc[EPT];
+    // fp32 sums in slice order; the loads of SCN slices are issued before the first add: the
+    // phase is bound by their latency
+    constexpr int SCN = RT * NCH >= 16 ? 2 : RT * NCH >= 8 ? 3 : 8;
 #pragma unroll
-    for (int u = 0; u < EPT; ++u) acc[u] = make_float4(0.f, 0.f, 0.f, 0.f);
-    for (int s0 = 0; s0 < parts; s0 += SC) {
-      float4 v[SC][EPT];
+    for (int rr = 0; rr < RT; ++rr)
 #pragma unroll
-      for (int c = 0; c < SC; ++c)
+      for (int m = 0; m < NCH; ++m)
 #pragma unroll
-        for (int u = 0; u < EPT; ++u)
-          v[c][u] = (s0 + c < parts) ? __ldg(gp + (size_t)(s0 + c) * (D * D / 4) + tid + u * NT)
-                                      : make_float4(0.f, 0.f, 0.f, 0.f);
+        for (int c = 0; c < 4; ++c) acc[rr][m][c] = 0.f;
+    for (int s0 = 0; s0 < parts; s0 += SCN) {
+      float4 v[SCN][RT][NCH];
 #pragma unroll
-      for (int c = 0; c < SC; ++c)
+      for (int s = 0; s < SCN; ++s)
 #pragma unroll
-        for (int u = 0; u < EPT; ++u) {
-          acc[u].x += v[c][u].x; acc[u].y += v[c][u].y; acc[u].z += v[c][u].z; acc[u].w += v[c][u].w;
+        for (int rr = 0; rr < RT; ++rr)
+#pragma unroll
+          for (int m = 0; m < NCH; ++m)
+            v[s][rr][m] = (s0 + s < parts) ? __ldg(gp + (size_t)(s0 + s) * (D * D / 4) + (row0 + rr) * (D / 4) + GX * m + g)
+                                           : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+      for (int s = 0; s < SCN; ++s)
+#pragma unroll
+        for (int rr = 0; rr < RT; ++rr)
+#pragma unroll
+          for (int m = 0; m < NCH; ++m) {
+            acc[rr][m][0] += v[s][rr][m].x; acc[rr][m][1] += v[s][rr][m].y;
+            acc[rr][m][2] += v[s][rr][m].z; acc[rr][m][3] += v[s][rr][m].w;
+          }
+    }
+    float zero = 0.f;
+#pragma unroll
+    for (int rr = 0; rr < RT; ++rr)
+#pragma unroll
+      for (int m = 0; m < NCH; ++m) {
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+          zero = fmaf(acc[rr][m][c], 0.f, zero);             // NaN where an entry is not finite
+          st_if(part + row0 + rr, acc[rr][m][c], CW * m + 4 * g + c == row0 + rr);
         }
-    }
-#pragma unroll
-    for (int u = 0; u < EPT; ++u) {
-      const int eh = tid + u * NT;
-      bad |= !(isfinite(acc[u].x) && isfinite(acc[u].y) && isfinite(acc[u].z) && isfinite(acc[u].w));
-      *reinterpret_cast<float4*>(Gs + (eh / (D / 4)) * LD + (eh % (D / 4)) * 4) = acc[u];
-      if (parts > 1) reinterpret_cast<float4*>(gsum + (size_t)b * D * D)[eh] = acc[u];   // the residual check and the fallback read it back
-    }
-    if (tid < 4) s_flags[tid] = 0;
-    if (tid == 0) s_why = 0;
-    lost = __syncthreads_or(lost);
-    bad = __syncthreads_or(bad);
-    if (bad || lost) {
+        if (parts > 1)                                        // read back by the residual check and the fallback
+          reinterpret_cast<float4*>(gsum + (size_t)b * D * D)[(row0 + rr) * (D / 4) + GX * m + g] =
+              make_float4(acc[rr][m][0], acc[rr][m][1], acc[rr][m][2], acc[rr][m][3]);
+      }
+    if (tid < 4) sh.flags[tid] = 0;
+    if (tid == 0) sh.why = 0;
+    if (__syncthreads_or(lost | (int)!(zero == 0.f))) {
+      lost = __syncthreads_or(lost);
       const float qnan = __int_as_float(0x7fc00000);
       for (int e = tid; e < D * r; e += NT) V[(size_t)b * D * r + e] = qnan;
       for (int e = tid; e < r; e += NT) S[(size_t)b * r + e] = qnan;
@@ -399,549 +1054,85 @@ __device__ __forceinline__ bool eig_user(const float* __restrict__ gpart, const 
       return false;
     }
   }
-  if (tid < 32) {
-    float m = 0.f;
+  float gmax = 0.f;
+  {
     double tr = 0.0;
-    for (int i = tid; i < D; i += 32) {
-      const float g = Gs[i * LD + i];
-      m = fmaxf(m, fabsf(g));
-      tr += (double)g;
+#pragma unroll
+    for (int q = 0; q < D / 32; ++q) {
+      const float d = part[lane + 32 * q];
+      gmax = fmaxf(gmax, fabsf(d));
+      tr += (double)d;
     }
-    m = warp_max(m);
+    gmax = warp_max(gmax);
 #pragma unroll
     for (int o = 16; o; o >>= 1) tr += __shfl_xor_sync(kFull, tr, o);
-    if (tid == 0) { s_gmax = m; s_trace = tr; }
+    if (tid == 0) sh.trace = tr;
   }
-  __syncthreads();
-  const float gmax = s_gmax;
   // Power-of-two scale that brings the largest diagonal entry into [1, 2): everything below works
   // on sc * G (exact), and the eigenvalues are divided by sc at the end.
   const float sc = gmax > 0.f ? exp2f(-(float)max(-100, min(100, ilogbf(gmax)))) : 1.f;
+  __syncthreads();
 
-  bool ok = true;
-  int passes = 0;
   if (route != kRouteFull && gmax > 0.f) {
-    // ---- 2. Householder tridiagonalisation, the matrix in registers ---------------------------
-    int k_stop = -1;                     // step at which the reduction stopped early (uniform), or -1
-    {
-      float a[RPT][CPT], xr[RPT], xc[CPT];
-#pragma unroll
-      for (int q = 0; q < RPT; ++q) {
-#pragma unroll
-        for (int g = 0; g < NG; ++g) {
-          const float4 t = *reinterpret_cast<const float4*>(Gs + (lane + 32 * q) * LD + 4 * (warp + NW * g));
-          a[q][4 * g] = t.x * sc; a[q][4 * g + 1] = t.y * sc; a[q][4 * g + 2] = t.z * sc; a[q][4 * g + 3] = t.w * sc;
-        }
-        xr[q] = Gs[(lane + 32 * q) * LD] * sc;                      // column 0 at my rows ...
-      }
-#pragma unroll
-      for (int g = 0; g < NG; ++g) {
-        const float4 t = *reinterpret_cast<const float4*>(Gs + 4 * (warp + NW * g));   // ... and (row 0) at my columns
-        xc[4 * g] = t.x * sc; xc[4 * g + 1] = t.y * sc; xc[4 * g + 2] = t.z * sc; xc[4 * g + 3] = t.w * sc;
-      }
-      for (int e = tid; e < D * D / 4; e += NT) reinterpret_cast<float4*>(hv)[e] = make_float4(0.f, 0.f, 0.f, 0.f);
-      for (int e = tid; e < 2 * D; e += NT) xpre[e] = 0.f;
-      __syncthreads();
-      const float trs = (float)((double)sc * s_trace);
-      float tr_rest = trs, tr_comp = 0.f;
-      const float stop_tr = trs * tol.stop_trace, stop_x2 = (trs * tol.stop_couple) * (trs * tol.stop_couple);
-      tri_stage<D, 0>(a, xr, xc, hv, xpre, tpart, pvp, dg, eo, betas, tid, tr_rest, tr_comp, stop_tr, stop_x2, r, k_stop);
-      tri_stage<D, 1>(a, xr, xc, hv, xpre, tpart, pvp, dg, eo, betas, tid, tr_rest, tr_comp, stop_tr, stop_x2, r, k_stop);
-      if constexpr (NG > 2) {
-        tri_stage<D, 2>(a, xr, xc, hv, xpre, tpart, pvp, dg, eo, betas, tid, tr_rest, tr_comp, stop_tr, stop_x2, r, k_stop);
-        tri_stage<D, 3>(a, xr, xc, hv, xpre, tpart, pvp, dg, eo, betas, tid, tr_rest, tr_comp, stop_tr, stop_x2, r, k_stop);
-      }
-      if (k_stop < 0) {
-        // the last 2 x 2 block: xr holds column D-2
-        if (warp == 0) {
-#pragma unroll
-          for (int q = 0; q < RPT; ++q) {
-            if (lane + 32 * q == D - 2) dg[D - 2] = xr[q];
-            if (lane + 32 * q == D - 1) eo[D - 2] = xr[q];
-          }
-          if (lane == 0) { eo[D - 1] = 0.f; betas[D - 2] = 0.f; betas[D - 1] = 0.f; }
-        }
-        if (warp == NW - 1 && lane == 31) dg[D - 1] = a[RPT - 1][CPT - 1];
-      }
-    }
-    // T has `de` rows (all D unless the reduction stopped early), padded with zero rows to a multiple of 4
-    const int de = k_stop >= 0 ? k_stop + 1 : D, de4 = (de + 3) & ~3;
-    const int kb = k_stop >= 0 ? k_stop : D - 2;            // reflectors 0 .. kb-1 exist
-    if (tid < de4 - de) { dg[de + tid] = 0.f; eo[de + tid] = 0.f; }
-    __syncthreads();
-
-    // ---- 3. Gershgorin interval, floored squares, trace; multisection --------------------------
-    if (warp == 0) {
-      float lo = 3.0e38f, hi = -3.0e38f, tr = 0.f;
-      for (int i = lane; i < de; i += 32) {
-        const float rad = fabsf(eo[i]) + (i > 0 ? fabsf(eo[i - 1]) : 0.f);   // eo[de-1] = 0
-        lo = fminf(lo, dg[i] - rad); hi = fmaxf(hi, dg[i] + rad);
-        tr += dg[i];
-      }
-      lo = -warp_max(-lo); hi = warp_max(hi); tr = warp_sum(tr);
-      const float tn = fmaxf(fabsf(lo), fabsf(hi));
-      const float fl = (tn * 1.4901161e-08f) * (tn * 1.4901161e-08f);         // (2^-26 |T|)^2
-      for (int i = lane; i < de4; i += 32) e2s[i] = i > 0 ? fmaxf(eo[i - 1] * eo[i - 1], fl) : 0.f;
-      if (lane == 0) {
-        const float span = hi - lo;
-        s_lo = lo - 1e-6f * span - 1e-30f; s_hi = hi + 1e-6f * span + 1e-30f; s_trT = tr;
-      }
-    }
-    __syncthreads();
-    const float tnorm = fmaxf(fabsf(s_lo), fabsf(s_hi));
-    // Eigenvalue j = 32 * gi + lane belongs to the group gi of WG warps; every warp of the group
-    // keeps the same bracket and evaluates its own interior point(s) in each step.
-    const int gi = warp / WG, wg = warp % WG;
-    const int j = gi * 32 + lane, jj = j < r ? j : r - 1;       // surplus lanes shadow column r-1
-    float lam;
-    {
-      constexpr int CH = (WG >= 4) ? 1 : 2;                      // points per warp and step
-      constexpr int P = CH * WG;                                 // 4 or 8 points: 5 or 9 sub-intervals
-      constexpr int STEPS = (P >= 8) ? 9 : 12;                   // (P + 1)^STEPS >= 2^27
-      static_assert(2 * NE * P * 32 <= RP * RP, "flags fit in the E region");
-      unsigned char* flag = reinterpret_cast<unsigned char*>(Em);   // [2][NE][P][32]: count(point) > target
-      const int target = de4 - 1 - jj;    // lambda_(jj-th largest) >= x  <=>  #(eigenvalues < x) <= target
-      float lo = s_lo, hi = s_hi;
-#pragma unroll 1
-      for (int step = 0; step < STEPS; ++step) {
-        const float w = (hi - lo) * (1.f / (P + 1));
-        float x[CH];
-        int cnt[CH];
-#pragma unroll
-        for (int h = 0; h < CH; ++h) x[h] = fmaf((float)(wg * CH + h + 1), w, lo);
-        sturm<D, CH>(dg, e2s, x, cnt, de4 >> 2);
-        unsigned char* fl = flag + (((step & 1) * NE + gi) * P) * 32;
-#pragma unroll
-        for (int h = 0; h < CH; ++h) fl[(wg * CH + h) * 32 + lane] = cnt[h] > target;
-        __syncthreads();
-        int idx = P;                       // first point above the eigenvalue
-#pragma unroll
-        for (int pnt = P - 1; pnt >= 0; --pnt) idx = fl[pnt * 32 + lane] ? pnt : idx;
-        const float nlo = idx == 0 ? lo : fmaf((float)idx, w, lo);
-        const float nhi = idx == P ? hi : fmaf((float)(idx + 1), w, lo);
-        lo = nlo; hi = nhi;
-      }
-      lam = 0.5f * (lo + hi);
-      if (wg == 0) lamv[j] = lam;
-    }
-    // A reduction to tridiagonal form is backward stable in the norm of G only: it fixes a kept
-    // vector to an angle of a few eps |T| / gap, whatever the size of its eigenvalue.  Where a
-    // gap among the kept eigenvalues is too small for the angle the storage type needs (a
-    // strongly graded spectrum such as sigma_i = i^-1.5 over 128 directions), the Jacobi solve,
-    // which works to an accuracy relative to each eigenvalue, takes over at once.
-    __syncthreads();
-    {
-      int tight = 0;
-      if (wg == 0 && j < r - 1) tight = (lamv[j] - lamv[j + 1]) < tol.gap_min * lamv[0];
-      if (__syncthreads_or(tight)) {
-        ok = false;
-        if (tid == 0) s_why |= kWhyGap;
-      }
-    }
-    float* Vc = vs;        // current vectors
-    float* Vn = work;      // next (over the twisted-factorisation buffers once they are free)
-    if (ok || route == kRouteTridiag) {
-    // ---- 4. twisted factorisation ---------------------------------------------------------------
-    // The pivots of the two triangular factorisations of T - lambda I are ratios of consecutive
-    // minors: q+_i = p_{i+1} / p_i with the leading minors p of the Sturm recurrence, and
-    // q-_i = t_i / t_{i+1} with the trailing minors t.  Taking them from the (rescaled) minor
-    // recurrences keeps the divisions off the dependency chain, which is one FMA per step.  The
-    // forward and the backward sequence run on two warps of the group; then every warp takes a
-    // range of i for gamma_i and the multipliers; then two warps run the two halves of z.
-    float* tf = work;                 // [D][RP] forward pivots, then the upward multipliers / values
-    float* tb = work + D * RP;        // [D][RP] backward pivots, then the downward multipliers / values
-    const float pfl = tnorm * 9.3132257e-10f;                                // pivot floor 2^-30 |T|
-    constexpr int WB = (WG > 1) ? 1 : 0;                                     // the warp of the backward sequences
-    {
-      if (wg == 0) {
-        float pf = 1.f, pfo = 0.f;                              // p_i, p_{i-1}
-#pragma unroll 8
-        for (int t = 0; t < de; ++t) {
-          const float nf = fmaf(dg[t] - lam, pf, -(e2s[t] * pfo));
-          float qf = __fdividef(nf, pf);
-          qf = (fabsf(qf) >= pfl) ? qf : -pfl;                   // also catches NaN
-          tf[t * RP + j] = qf;
-          pfo = pf; pf = nf;
-          if ((t & 3) == 3) {
-            const unsigned mf = __float_as_uint(fmaxf(fabsf(pf), fabsf(pfo))) >> 23;
-            const float sf = __uint_as_float((254u - mf) << 23);
-            pf *= sf; pfo *= sf;
-          }
-        }
-      }
-      if (wg == WB) {
-        float pb = 1.f, pbo = 0.f;                              // t_{i+1}, t_{i+2}
-#pragma unroll 8
-        for (int t = 0; t < de; ++t) {
-          const int ib = de - 1 - t;
-          const float nb = fmaf(dg[ib] - lam, pb, -((t > 0 ? e2s[ib + 1] : 0.f) * pbo));
-          float qb = __fdividef(nb, pb);
-          qb = (fabsf(qb) >= pfl) ? qb : -pfl;
-          tb[ib * RP + j] = qb;
-          pbo = pb; pb = nb;
-          if ((t & 3) == 3) {
-            const unsigned mb = __float_as_uint(fmaxf(fabsf(pb), fabsf(pbo))) >> 23;
-            const float sb = __uint_as_float((254u - mb) << 23);
-            pb *= sb; pbo *= sb;
-          }
-        }
-      }
-    }
-    __syncthreads();
-    {
-      // gamma_i = q+_i + q-_i - (d_i - lambda) over my range of i; the multipliers
-      // z_i = -(e_i / q+_i) z_{i+1} going up, z_i = -(e_{i-1} / q-_i) z_{i-1} going down
-      const int IR = (de + WG - 1) / WG, i1 = min((wg + 1) * IR, de);
-      float best = 3.0e38f;
-      int kbest = 0;
-#pragma unroll 8
-      for (int i = wg * IR; i < i1; ++i) {
-        const float qf = tf[i * RP + j], qb = tb[i * RP + j];
-        const float gam = fabsf((qf + qb) - (dg[i] - lam));
-        if (gam < best) { best = gam; kbest = i; }
-        tf[i * RP + j] = -__fdividef(eo[i], qf);
-        tb[i * RP + j] = i > 0 ? -__fdividef(eo[i - 1], qb) : 0.f;
-      }
-      part[wg * RP + j] = best;
-      reinterpret_cast<int*>(part)[(NW + wg) * RP + j] = kbest;
-    }
-    __syncthreads();
-    int kt = 0;
-    {
-      float best = 3.0e38f;
-#pragma unroll
-      for (int w2 = 0; w2 < WG; ++w2) {
-        const float bv = part[w2 * RP + j];
-        const int bk = reinterpret_cast<const int*>(part)[(NW + w2) * RP + j];
-        if (bv < best) { best = bv; kt = bk; }                   // ranges ascend: the lowest i wins a tie
-      }
-    }
-    __syncthreads();
-    {
-      // z_kt = 1; the values above the twist overwrite tf, those below it tb (no branches: a lane
-      // that has not reached its twist index yet keeps z = 1)
-      if (wg == 0) {
-        float zu = 1.f, ss = 0.f;
-#pragma unroll 8
-        for (int iu = de - 2; iu >= 0; --iu) {
-          const float mu = tf[iu * RP + j];
-          zu = (iu < kt) ? zu * mu : 1.f;
-          ss = fmaf(zu, (iu < kt) ? zu : 0.f, ss);
-          tf[iu * RP + j] = zu;
-        }
-        part[j] = ss;
-        ktv[j] = kt;
-      }
-      if (wg == WB) {
-        float zd = 1.f, ss = 0.f;
-#pragma unroll 8
-        for (int t = 1; t < de; ++t) {
-          const float md = tb[t * RP + j];
-          zd = (t > kt) ? zd * md : 1.f;
-          ss = fmaf(zd, (t > kt) ? zd : 0.f, ss);
-          tb[t * RP + j] = zd;
-        }
-        part[RP + j] = ss;
-      }
-    }
-    __syncthreads();
-    if (wg == 0) sgn[j] = rsqrtf(1.f + part[j] + part[RP + j]);   // 1 / |z|
-    __syncthreads();
-
-    // ---- 5. back-transformation: v = H_0 H_1 ... H_{D-3} z ------------------------------------
-    // Four threads per vector, each with a quarter of the rows in registers; the reflector's
-    // inner product is completed by two shuffles.  Reflector k is zero at rows <= k, so the
-    // quarters need no conditions.
-    {
-      constexpr int RB = D / 4;                   // rows per thread
-      constexpr int VPP = NT / 4;                 // vectors per pass
-      constexpr int NPASS = (RP + VPP - 1) / VPP;
-      static_assert(NPASS * VPP >= RP, "every vector is transformed");
-#pragma unroll 1
-      for (int pass = 0; pass < NPASS; ++pass) {
-        const int jv = pass * VPP + (tid >> 2), qt = tid & 3;
-        const bool act = jv < RP;
-        const int jc = act ? jv : 0;
-        const int ktj = ktv[jc];
-        const float zn = sgn[jc];
-        float z[RB];
-#pragma unroll
-        for (int u = 0; u < RB; ++u) {
-          const int i = qt * RB + u;
-          const float upv = tf[i * RP + jc], dnv = tb[i * RP + jc];
-          z[u] = i < de ? (i < ktj ? upv : i > ktj ? dnv : 1.f) * zn : 0.f;
-        }
-#pragma unroll 2
-        for (int k = kb - 1; k >= 0; --k) {
-          const float beta = betas[k];
-          const float4* h4 = reinterpret_cast<const float4*>(hv + k * D + qt * RB);
-          float4 h[RB / 4];
-          float d0 = 0.f, d1 = 0.f;
-#pragma unroll
-          for (int u = 0; u < RB / 4; ++u) {
-            h[u] = h4[u];
-            d0 = fmaf(h[u].x, z[4 * u], d0);     d1 = fmaf(h[u].y, z[4 * u + 1], d1);
-            d0 = fmaf(h[u].z, z[4 * u + 2], d0); d1 = fmaf(h[u].w, z[4 * u + 3], d1);
-          }
-          float dt = d0 + d1;
-          dt += __shfl_xor_sync(kFull, dt, 1);
-          dt += __shfl_xor_sync(kFull, dt, 2);
-          const float c = -beta * dt;
-#pragma unroll
-          for (int u = 0; u < RB / 4; ++u) {
-            z[4 * u] = fmaf(c, h[u].x, z[4 * u]);         z[4 * u + 1] = fmaf(c, h[u].y, z[4 * u + 1]);
-            z[4 * u + 2] = fmaf(c, h[u].z, z[4 * u + 2]); z[4 * u + 3] = fmaf(c, h[u].w, z[4 * u + 3]);
-          }
-        }
-        if (act) {
-#pragma unroll
-          for (int u = 0; u < RB; ++u) vs[(qt * RB + u) * RP + jv] = z[u];
-        }
-      }
-    }
-    __syncthreads();
-    // The long serial part is over: the next kernel may start launching -- unless the process runs
-    // many requests at once, where its parked CTAs are better kept out a little longer (after the
-    // certificate: 7.65 -> 7.59 us per step in flight, at 0.4 us of a single call's latency).
-    if (!late_trigger) pdl_trigger();
-
-    // G back into shared memory (over the reflectors), for the residuals
-    float* Gsm = hv;   // [D][D], sc * G
-    for (int e = tid; e < D * D / 4; e += NT) {
-      float4 g = reinterpret_cast<const float4*>(gout)[e];
-      g.x *= sc; g.y *= sc; g.z *= sc; g.w *= sc;
-      reinterpret_cast<float4*>(Gsm)[e] = g;
-    }
-
-    // ---- 6. orthogonalisation passes while V^T V - I is above the rounding level ---------------
-    // Column-parallel: lane = column(s) c, c + 32; a warp takes RP / NW rows a of E.
-    constexpr int AW = RP / NW;
-    for (;;) {
-      float acc[NE][AW];
-#pragma unroll
-      for (int h = 0; h < NE; ++h)
-#pragma unroll
-        for (int u = 0; u < AW; ++u) acc[h][u] = 0.f;
-      const int a0 = warp * AW;
-#pragma unroll 8
-      for (int i = 0; i < D; ++i) {
-        float av[AW];
-        if (AW >= 4) {
-#pragma unroll
-          for (int u = 0; u < AW; u += 4) {
-            const float4 t = *reinterpret_cast<const float4*>(Vc + i * RP + a0 + u);
-            av[u] = t.x; av[u + 1] = t.y; av[u + 2] = t.z; av[u + 3] = t.w;
-          }
-        } else {
-#pragma unroll
-          for (int u = 0; u < AW; ++u) av[u] = Vc[i * RP + a0 + u];
-        }
-#pragma unroll
-        for (int h = 0; h < NE; ++h) {
-          const float vc = Vc[i * RP + 32 * h + lane];
-#pragma unroll
-          for (int u = 0; u < AW; ++u) acc[h][u] = fmaf(av[u], vc, acc[h][u]);
-        }
-      }
-      float emax = 0.f;
-#pragma unroll
-      for (int h = 0; h < NE; ++h)
-#pragma unroll
-        for (int u = 0; u < AW; ++u) {
-          const int a = a0 + u, c = 32 * h + lane;
-          float e = acc[h][u] - (a == c ? 1.f : 0.f);
-          if (a >= r || c >= r) e = 0.f;               // surplus columns are copies of column r-1
-          Em[a * RP + c] = e;
-          emax = fmaxf(emax, fabsf(e));
-        }
-      emax = warp_max(emax);
-      if (lane == 0) part[warp] = emax;
-      __syncthreads();
-      if (tid == 0) {
-        float m = 0.f;
-        for (int w = 0; w < NW; ++w) m = fmaxf(m, part[w]);
-        s_emax = m;
-      }
-      __syncthreads();
-      const float em = s_emax;
-      if (em <= tol.ortho) break;                       // orthonormal to rounding
-      if (passes == 6 || !(em <= 0.98f)) { ok = false; if (tid == 0) s_why |= kWhyOrtho; break; }
-      ++passes;
-      // One pass of Gram-Schmidt against the ORIGINAL earlier columns (larger eigenvalues, the
-      // better determined vectors): v_c <- (v_c - sum_{a<c} E_ac v_a) / |.|.  A later column never
-      // changes an earlier one, so a poorly separated pair cannot damage its neighbours; for
-      // two vectors the pass is exact, for more it converges quadratically like the symmetric
-      // form.  Rows i of V' for this warp: D / NW of them; lane = column(s).
-      float ecol[NE][RP], scol[NE];
-#pragma unroll
-      for (int h = 0; h < NE; ++h) {
-        const int c = 32 * h + lane;
-        float nn = 1.f;
-#pragma unroll
-        for (int a = 0; a < RP; ++a) {
-          const float e = Em[a * RP + c];
-          ecol[h][a] = a < c ? e : 0.f;
-          nn += a < c ? -e * e : (a == c ? e : 0.f);
-        }
-        scol[h] = rsqrtf(fmaxf(nn, 1e-6f));
-      }
-      for (int i = warp; i < D; i += NW) {
-        float o[NE];
-#pragma unroll
-        for (int h = 0; h < NE; ++h) o[h] = 0.f;
-#pragma unroll
-        for (int a = 0; a < RP; a += 4) {
-          const float4 t = *reinterpret_cast<const float4*>(Vc + i * RP + a);
-#pragma unroll
-          for (int h = 0; h < NE; ++h) {
-            o[h] = fmaf(t.x, ecol[h][a], o[h]);     o[h] = fmaf(t.y, ecol[h][a + 1], o[h]);
-            o[h] = fmaf(t.z, ecol[h][a + 2], o[h]); o[h] = fmaf(t.w, ecol[h][a + 3], o[h]);
-          }
-        }
-#pragma unroll
-        for (int h = 0; h < NE; ++h)
-          Vn[i * RP + 32 * h + lane] = (Vc[i * RP + 32 * h + lane] - o[h]) * scol[h];
-      }
-      __syncthreads();
-      float* t = Vc; Vc = Vn; Vn = t;
-      // With E = L + diag + L^T the pass leaves (I - L)(I + E)(I - L^T) = I + diag - L L^T - L^2 -
-      // (L^T)^2 + O(E^3), and the scaling removes the diagonal: what remains off the diagonal is
-      // below 3 r max|E|^2.  Where that is a quarter of the bound, V^T V is not formed again.
-      if (3.f * (float)r * em * em <= 0.25f * tol.ortho) break;
-    }
-    __syncthreads();      // G is staged; E and the vectors are settled
-
-    // ---- 7. Rayleigh quotients and residuals against G; certification ------------------------
-    if (ok || route == kRouteTridiag) {
-      constexpr int RW = D / NW;        // rows of Y = G V per warp
-      float y[NE][RW];
-#pragma unroll
-      for (int h = 0; h < NE; ++h)
-#pragma unroll
-        for (int u = 0; u < RW; ++u) y[h][u] = 0.f;
-      const int i0 = warp * RW;
-#pragma unroll 2
-      for (int k = 0; k < D; k += 4) {
-        float vk[NE][4];
-#pragma unroll
-        for (int h = 0; h < NE; ++h)
-#pragma unroll
-          for (int u = 0; u < 4; ++u) vk[h][u] = Vc[(k + u) * RP + 32 * h + lane];
-#pragma unroll
-        for (int u = 0; u < RW; ++u) {
-          const float4 g = *reinterpret_cast<const float4*>(Gsm + (i0 + u) * D + k);
-#pragma unroll
-          for (int h = 0; h < NE; ++h) {
-            y[h][u] = fmaf(g.x, vk[h][0], y[h][u]); y[h][u] = fmaf(g.y, vk[h][1], y[h][u]);
-            y[h][u] = fmaf(g.z, vk[h][2], y[h][u]); y[h][u] = fmaf(g.w, vk[h][3], y[h][u]);
-          }
-        }
-      }
-      float vown[NE][RW];
-#pragma unroll
-      for (int h = 0; h < NE; ++h) {
-        float t = 0.f;
-#pragma unroll
-        for (int u = 0; u < RW; ++u) {
-          vown[h][u] = Vc[(i0 + u) * RP + 32 * h + lane];
-          t = fmaf(vown[h][u], y[h][u], t);
-        }
-        part[warp * RP + 32 * h + lane] = t;
-      }
-      __syncthreads();
-      if (tid < RP) {
-        float t = 0.f;
-        for (int w = 0; w < NW; ++w) t += part[w * RP + tid];
-        theta[tid] = t;
-      }
-      __syncthreads();
-#pragma unroll
-      for (int h = 0; h < NE; ++h) {
-        const float th = theta[32 * h + lane];
-        float t = 0.f;
-#pragma unroll
-        for (int u = 0; u < RW; ++u) {
-          const float d = fmaf(-th, vown[h][u], y[h][u]);
-          t = fmaf(d, d, t);
-        }
-        part[warp * RP + 32 * h + lane] = t;
-      }
-      __syncthreads();
-      if (tid < RP) {
-        float t = 0.f;
-        for (int w = 0; w < NW; ++w) t += part[w * RP + tid];
-        rho2[tid] = t;
-      }
-      __syncthreads();
-      int good = 1;
-      if (tid < r) {
-        const float th1 = theta[0], thi = theta[tid];
-        float gap = 3.0e38f;
-        if (tid > 0) gap = fminf(gap, theta[tid - 1] - thi);
-        if (tid < r - 1) gap = fminf(gap, thi - theta[tid + 1]);
-        const float resn = sqrtf(rho2[tid]);
-        const bool res_ok = resn <= fmaxf(tol.eps_vec * gap, tol.floor_rel * th1);
-        // T is similar to sc * G: the traces agree to rounding
-        const float trG = (float)((double)sc * s_trace);
-        const bool tr_ok = fabsf(s_trT - trG) <= 1e-4f * fabsf(trG) && isfinite(thi) && isfinite(resn);
-        if (!res_ok) atomicOr(&s_why, kWhyResidual);
-        if (!tr_ok) atomicOr(&s_why, kWhyTrace);
-        good = res_ok && tr_ok;
-      }
-      ok = __syncthreads_and(good) && ok;
-    }
-
-    }   // the gaps allow the tridiagonal route
-
+    float* Vc = nullptr;
+    int passes = 0;
+    const bool ok = tri_chain<float, D, RP>(acc, smem, sh, gout, sc, r, route == kRouteTridiag, tol, !late_trigger, Vc, passes, tid);
     if (ok || route == kRouteTridiag) {
       if (late_trigger) pdl_trigger();
       // singular values (non-increasing: a Rayleigh quotient may pass its neighbour by a rounding
       // error), sign gauge, output
-      if (tid < RP) {
-        const int j = tid < r ? tid : r - 1;
+      const int rp = (r + 3) & ~3;
+      float sv[NE], sg[NE], carry = 3.0e38f;
+#pragma unroll
+      for (int h = 0; h < NE; ++h) {
+        const int c = 32 * h + lane, j = c < r ? c : r - 1;
         float m = theta[j];
-        for (int q = 0; q < j; ++q) m = fminf(m, theta[q]);
-        float best = -1.f, lead = 1.f;
-        for (int i = 0; i < D; ++i) {
-          const float v = Vc[i * RP + j];
-          if (fabsf(v) > best) { best = fabsf(v); lead = v; }   // strict: lowest index wins a tie
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+          const float t = __shfl_up_sync(kFull, m, o);
+          m = lane >= o ? fminf(m, t) : m;
         }
-        sgn[tid] = lead < 0.f ? -1.f : 1.f;
-        const float sv = sqrtf(fmaxf(m, 0.f) / sc);
-        rho2[tid] = sv;
-        if (tid < r) S[(size_t)b * r + tid] = sv;
-      }
-      __syncthreads();
-      for (int e = tid; e < D * r; e += NT) {
-        const int i = e / r, j = e % r;
-        V[(size_t)b * D * r + e] = Vc[i * RP + j] * sgn[j];
-      }
-      if (want_vs) {
-        const int rp = (r + 3) & ~3;
-        float* vsig = smem;                            // over G: the residuals are done
-        for (int e = tid; e < D * rp; e += NT) {
-          const int i = e / rp, j = e % rp;
-          vsig[e] = j < r ? (Vc[i * RP + j] * sgn[j]) * rho2[j] : 0.f;
+        m = fminf(m, carry);
+        carry = __shfl_sync(kFull, m, 31);
+        float best = -1.f, lv = 1.f;
+#pragma unroll
+        for (int w = 0; w < NW; ++w) {
+          const float v = part[(NW + w) * RP + c];
+          lv = fabsf(v) > best ? v : lv;
+          best = fmaxf(fabsf(v), best);
         }
+        sg[h] = lv < 0.f ? -1.f : 1.f;
+        sv[h] = sqrtf(fmaxf(m, 0.f) / sc);
+        if (warp == 0 && c < r) S[(size_t)b * r + c] = sv[h];
       }
+      float* vsig = smem;                            // over G: the residuals are done
+#pragma unroll 4
+      for (int n = warp; n < D; n += NW)
+#pragma unroll
+        for (int h = 0; h < NE; ++h) {
+          const int c = 32 * h + lane;
+          const float v = Vc[n * RP + c] * sg[h];
+          if (c < r) V[((size_t)b * D + n) * r + c] = v;
+          st_if(vsig + n * rp + c, c < r ? v * sv[h] : 0.f, (int)want_vs & (int)(c < rp));
+        }
       if (tid == 0) {
         if (info) info[b] = ok ? 0 : SOLAR_INFO_NOT_CERTIFIED;
-        if (route_taken) route_taken[b] = kRouteTridiag | (passes << 16) | (s_why << 24);
+        if (route_taken) route_taken[b] = kRouteTridiag | (passes << 16) | (sh.why << 24);
       }
       return want_vs;
     }
     __syncthreads();
   }
 
-  // ---- fallback (or the caller's choice): Jacobi on the whole matrix ---------------------------
+  // ---- fallback (or the caller's choice): Jacobi on the whole matrix -------------------------------
   for (int e = tid; e < D * D / 4; e += NT) {
-    float4 g = reinterpret_cast<const float4*>(gout)[e];
-    g.x *= sc; g.y *= sc; g.z *= sc; g.w *= sc;
-    *reinterpret_cast<float4*>(smem + (e / (D / 4)) * LD + (e % (D / 4)) * 4) = g;
+    float4 t = reinterpret_cast<const float4*>(gout)[e];
+    t.x *= sc; t.y *= sc; t.z *= sc; t.w *= sc;
+    *reinterpret_cast<float4*>(smem + (e / (D / 4)) * LD + (e % (D / 4)) * 4) = t;
   }
   __syncthreads();
   const float thr_abs2 = (kTolAbs * gmax * sc) * (kTolAbs * gmax * sc);
-  full_jacobi_route<D, NT>(smem, s_flags, b, tid, r, sc, thr_abs2, tol.sweep_stop * tol.sweep_stop, s_why,
+  full_jacobi_route<D, NT>(smem, sh.flags, b, tid, r, sc, thr_abs2, tol.sweep_stop * tol.sweep_stop, sh.why,
                            sweep_cap, S, V, info, route_taken);
   return false;
 }
@@ -1192,7 +1383,7 @@ __device__ __forceinline__ void prepare_epilogue(float* __restrict__ sm, int b, 
 }
 
 template <int D, int RP>
-__global__ void __launch_bounds__(TriCfg<D>::NT, 1)
+__global__ void __launch_bounds__(TriCfg<D>::NT, TriCfg<D>::CTAS)
 eig_tridiag_kernel(const float* __restrict__ gpart, const int* __restrict__ gram_status, int parts, int splits,
                    float* __restrict__ gsum, int r, int route, int sweep_cap, TriTol tol,
                    float* __restrict__ S, float* __restrict__ V, int* __restrict__ info,
