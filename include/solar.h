@@ -68,7 +68,8 @@ enum {
  * matrix, the r largest eigenvalues by Sturm-count multisection, their vectors by the
  * twisted factorisation, back-transformation; accepted per user only when the residuals
  * G v - theta v against the Gram matrix itself, V^T V = I and the trace certify the r
- * pairs, else the parallel Jacobi eigensolver on the whole matrix runs for that user.
+ * pairs, else the same chain in double precision, and where that cannot be certified either (equal
+ * eigenvalues) the parallel Jacobi eigensolver on the whole matrix, runs for that user.
  * SUBSPACE: Algorithm 1 (randomized range finder with power iteration) applied to the
  * d x d Gram matrix, then a Rayleigh-Ritz solve, alone; users whose residual and trace
  * bounds do not certify the result are flagged in info[].  FULL: the Jacobi eigensolver for every user (Eq. 9's exact
@@ -215,7 +216,7 @@ solar_status_t solar_eig_from_partials(int B, int N, int d, int r, solar_dtype_t
 
 /* As above with the route chosen by the caller.  route_taken (device, [B] ints, or
  * NULL) receives per user: route used (1 subspace, 2 full, 3 tridiagonal; 0 = non-finite
- * input) | power steps << 8 | Jacobi sweeps (route 3: orthogonalisation passes) << 16 |
+ * input) | power steps << 8 (route 2: 1 if it was the double-precision tridiagonal chain) | Jacobi sweeps (tridiagonal chains: orthogonalisation passes) << 16 |
  * reason << 24, where reason says why the first route tried was not certified: 1 no gap
  * at the cut, 2 residual too large for its gap, 4 a kept eigenvalue not positive, 8 sweep
  * cap, 16 non-finite pivot, 32 vectors of a cluster not independent, 64 trace mismatch

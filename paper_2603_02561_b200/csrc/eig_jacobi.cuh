@@ -22,6 +22,7 @@ constexpr float kUnit = 5.9604645e-08f;    // 2^-24, fp32 unit roundoff
 
 // route_taken[b] = route | detail << 8 | sweeps or passes << 16 | kWhy* bits << 24
 constexpr int kRouteSubspace = 1, kRouteFull = 2, kRouteTridiag = 3;
+constexpr int kDetailWide = 1;      // route 2: the tridiagonal chain in double precision answered, not the Jacobi solve
 // Why a route's result was not certified (0 = it was, or it was not tried):
 constexpr int kWhyCut = 1;          // the trace bound does not separate theta_r from the rest
 constexpr int kWhyResidual = 2;     // a residual is too large for its gap
@@ -30,7 +31,7 @@ constexpr int kWhySweepCap = 8;     // the Ritz Jacobi hit its sweep cap
 constexpr int kWhyCholesky = 16;    // non-finite pivot in the Cholesky-QR
 constexpr int kWhyOrtho = 32;       // tridiagonal route: vectors of a cluster came out dependent
 constexpr int kWhyTrace = 64;       // tridiagonal route: trace of T differs from trace of G, or not finite
-constexpr int kWhyGap = 128;        // tridiagonal route: a gap between kept eigenvalues is too small for its accuracy
+constexpr int kWhyGap = 128;        // tridiagonal route: a gap between kept eigenvalues is too small for fp32
 
 // Rotation J = [[c, s], [-s, c]] that annihilates g_pq of the 2x2 symmetric block
 // [[a, g], [g, b]]; identity when g is negligible (or not a number).  Returned

@@ -26,9 +26,17 @@
 //      the columns of larger eigenvalues.
 //   7. Rayleigh quotients theta_i = v_i^T G v_i and residuals G v_i - theta_i v_i against the
 //      ORIGINAL G: the result is accepted only if every residual is small against its gap (or
-//      at the rounding floor), V^T V = I to rounding, and trace(T) = trace(G); otherwise the
-//      CTA runs the parallel Jacobi eigensolver on the whole matrix, which is valid for any
-//      spectrum (clusters of equal eigenvalues, rank(H) < r, ...).
+//      at the rounding floor), V^T V = I to rounding, and trace(T) = trace(G).
+//
+// The chain runs in fp32 first.  A reduction to tridiagonal form is backward stable in the norm of
+// G only: it fixes a kept vector to an angle of a few eps |T| / gap, whatever the size of its
+// eigenvalue.  Where a gap among the kept eigenvalues is too small for that (sigma_i = i^-1 over 128
+// directions), or the certificate fails, the CTA runs the same chain with steps 2-4 in fp64, where
+// the angle is eps_64 |T| / gap; the fp32 eigenvalues are its starting brackets.  Only what that
+// cannot certify either (vectors of equal eigenvalues) goes to the parallel Jacobi solve on the
+// whole matrix, which is valid for any spectrum.  Forward pass of 8 users, d = 128, r = 64 of a power
+// law (every user takes the fp64 chain): 3075 us with Jacobi in its place, 384 now; 64 users, d = r =
+// 64, one or none of them: 440 and 134 us.
 //
 // What bounds it: the dependency chain (d steps of a matrix-vector product, an inner product and a
 // barrier, then the recurrences over the rows of T), not work or bandwidth: 16 users keep 16 of
@@ -74,8 +82,8 @@ template <int D, int RP> struct TriSmem {
   static constexpr int LAM = XP + 4 * D;                         // [RP] eigenvalues of T
   static constexpr int BE = LAM + 2 * RP;                        // [D] beta of reflector k
   static constexpr int TH = BE + D;                              // [RP] Rayleigh quotients
-  static constexpr int KT = TH + RP;                             // [RP] eigenvalues of the fp32 chain
-  static constexpr int PART = KT + RP;                           // [3][NW][RP] per-warp partial results
+  static constexpr int L32 = TH + RP;                            // [RP] eigenvalues of the fp32 chain
+  static constexpr int PART = L32 + RP;                          // [3][NW][RP] per-warp partial results
   static constexpr int TRI_FLOATS = PART + 3 * C::NW * RP;
   // the projection epilogue: V Sigma, Key_r^T, two weights (FFMA form) or the tensor-core form's staging
   static constexpr int EPI_FFMA = 2 * D * RP + 2 * D * D;
@@ -502,6 +510,7 @@ __device__ __forceinline__ bool tri_chain(const float (&acc)[TriCfg<D>::RT][TriC
   T* const e2s = reinterpret_cast<T*>(smem + L::E2);
   T* const lamv = reinterpret_cast<T*>(smem + L::LAM);
   float* const theta = smem + L::TH;
+  float* const lam32 = smem + L::L32;
   float* const part = smem + L::PART;
   bool ok = true;
   passes = 0;
@@ -613,11 +622,27 @@ __device__ __forceinline__ bool tri_chain(const float (&acc)[TriCfg<D>::RT][TriC
     constexpr int PT = NT / RP < 8 ? NT / RP : 8;               // lanes per eigenvalue
     constexpr int CH = NW == 4 ? 2 : 1, NPT = PT * CH;          // points per lane (one warp per scheduler: two)
     constexpr int STEPS = (NPT == 8 ? 9 : 12);                  // (NPT + 1)^STEPS >= 2^27
+    constexpr int STEPS64 = (NPT == 8 ? 14 : 19);               // ... >= 2^44, from the Gershgorin interval in fp64
     static_assert(PT * RP == NT && (NPT == 8 || NPT == 4), "every lane has points");
     const int j = tid / PT, pt = tid % PT, jj = j < r ? j : r - 1;     // surplus lanes shadow column r-1
     const int target = de8 - 1 - jj;    // lambda_(jj-th largest) >= x  <=>  #(eigenvalues < x) <= target
+    int steps = STEPS;
+    if (F64) {
+      // bracket: the fp32 chain's eigenvalue +- 2^-15 |T| where the counts confirm it
+      const T c0 = (T)lam32[j], dl = tnorm * T(3.0517578125e-05);
+      T x[CH];
+      int n[CH];
+      if (CH == 2) { x[0] = c0 - dl; x[CH - 1] = c0 + dl; }
+      else x[0] = (pt & 1) ? c0 + dl : c0 - dl;
+      sturm<T, CH>(dg, e2s, x, n, de8 >> 3);
+      const bool in = CH == 2 ? (int)(n[0] <= target) & (int)(n[CH - 1] > target) : ((pt & 1) ? n[0] > target : n[0] <= target);
+      const unsigned all = __ballot_sync(kFull, in);
+      const bool mine = ((~all >> (lane & ~(PT - 1))) & ((1u << PT) - 1)) == 0;
+      lo = mine ? c0 - dl : lo; hi = mine ? c0 + dl : hi;
+      steps = all == kFull ? STEPS : STEPS64;
+    }
 #pragma unroll 1
-    for (int step = 0; step < STEPS; ++step) {
+    for (int step = 0; step < steps; ++step) {
       const T w = (hi - lo) * T(1.0 / (NPT + 1));
       T x[CH];
       int n[CH], idx = 0;                                        // points at or below the eigenvalue
@@ -632,14 +657,10 @@ __device__ __forceinline__ bool tri_chain(const float (&acc)[TriCfg<D>::RT][TriC
       hi = idx == NPT ? hi : nhi;
     }
     if (pt == 0) lamv[j] = T(0.5) * (lo + hi);
+    if (!F64 && pt == 0) lam32[j] = (float)(T(0.5) * (lo + hi));
   }
   __syncthreads();
-  // A reduction to tridiagonal form is backward stable in the norm of G only: it fixes a kept
-  // vector to an angle of a few eps |T| / gap, whatever the size of its eigenvalue.  Where a
-  // gap among the kept eigenvalues is too small for the angle the storage type needs (a
-  // strongly graded spectrum such as sigma_i = i^-1.5 over 128 directions), this route is not
-  // to be trusted.
-  if (!F64) {
+  if (!F64) {                            // gaps too small for the angle the storage type needs
     const int tight = tid < r - 1 && (float)(lamv[tid] - lamv[tid + 1]) < tol.gap_min * (float)lamv[0];
     if (__syncthreads_or(tight)) {
       ok = false;
@@ -1075,10 +1096,19 @@ __device__ __forceinline__ bool eig_user(const float* __restrict__ gpart, const 
 
   if (route != kRouteFull && gmax > 0.f) {
     float* Vc = nullptr;
-    int passes = 0;
-    const bool ok = tri_chain<float, D, RP>(acc, smem, sh, gout, sc, r, route == kRouteTridiag, tol, !late_trigger, Vc, passes, tid);
+    int passes = 0, wide = 0;            // wide: the fp64 chain gave the result
+    bool ok = tri_chain<float, D, RP>(acc, smem, sh, gout, sc, r, route == kRouteTridiag, tol, !late_trigger, Vc, passes, tid);
+    if (!ok && route != kRouteTridiag) {
+      __syncthreads();
+#pragma unroll
+      for (int rr = 0; rr < RT; ++rr)
+#pragma unroll
+        for (int m = 0; m < NCH; ++m) ld4(gout + (row0 + rr) * D + CW * m + 4 * g, acc[rr][m]);
+      wide = 1;
+      ok = tri_chain<double, D, RP>(acc, smem, sh, gout, sc, r, false, tol, false, Vc, passes, tid);
+    }
     if (ok || route == kRouteTridiag) {
-      if (late_trigger) pdl_trigger();
+      if (late_trigger || wide) pdl_trigger();
       // singular values (non-increasing: a Rayleigh quotient may pass its neighbour by a rounding
       // error), sign gauge, output
       const int rp = (r + 3) & ~3;
@@ -1117,14 +1147,14 @@ __device__ __forceinline__ bool eig_user(const float* __restrict__ gpart, const 
         }
       if (tid == 0) {
         if (info) info[b] = ok ? 0 : SOLAR_INFO_NOT_CERTIFIED;
-        if (route_taken) route_taken[b] = kRouteTridiag | (passes << 16) | (sh.why << 24);
+        if (route_taken) route_taken[b] = (wide ? kRouteFull | (kDetailWide << 8) : kRouteTridiag) | (passes << 16) | (sh.why << 24);
       }
       return want_vs;
     }
     __syncthreads();
   }
 
-  // ---- fallback (or the caller's choice): Jacobi on the whole matrix -------------------------------
+  // ---- last resort (or the caller's choice): Jacobi on the whole matrix ----------------------------
   for (int e = tid; e < D * D / 4; e += NT) {
     float4 t = reinterpret_cast<const float4*>(gout)[e];
     t.x *= sc; t.y *= sc; t.z *= sc; t.w *= sc;
