@@ -1037,7 +1037,7 @@ __device__ __forceinline__ bool eig_user(const float* __restrict__ gpart, const 
         for (int rr = 0; rr < RT; ++rr)
 #pragma unroll
           for (int m = 0; m < NCH; ++m)
-            v[s][rr][m] = (s0 + s < parts) ? __ldg(gp + (size_t)(s0 + s) * (D * D / 4) + (row0 + rr) * (D / 4) + GX * m + g)
+            v[s][rr][m] = (s0 + s < parts) ? ld_dep(gp + (size_t)(s0 + s) * (D * D / 4) + (row0 + rr) * (D / 4) + GX * m + g)
                                            : make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
       for (int s = 0; s < SCN; ++s)

@@ -116,7 +116,9 @@ gram_umma_kernel(const __grid_constant__ CUtensorMap tmap, float* __restrict__ g
 
   // ---- epilogue: tensor memory -> shared memory -> sum over the cluster -> global ----------
   const bool done = ptx::mbar_wait(&accum_bar, 0, err, kErrEpilogue);
-  pdl_trigger();       // only the epilogue is left: the next kernel may start launching
+  // The next kernel is not released here: the eigensolver's few CTAs would be packed, up to three, onto
+  // the SMs that this grid leaves free and slow each other down (16 x 10240 x 64: 52.9 us per forward
+  // pass with an early release, 52.0 without; 128 users of one tile each: 70 and 53.5).
   __syncwarp();
   ptx::tc_fence_after_sync();
   // the accumulator as a row-major fp32 matrix over the ring (every tile has been consumed);

@@ -50,7 +50,7 @@ solar_status_t attn_apply_impl(int B, int M, int d, int r, solar_dtype_t dt, con
                                void* O, const char* ws, bool early_c, cudaStream_t st) {
   if (attn_umma_supported(d, dt))
     return from_cuda(launch_attn_umma(B, M, d, r, C, flags, O, ws, attn_ws_layout(d, r), early_c, st));
-  return from_cuda(launch_attn_simt(B, M, d, r, dt, C, flags, O, ws, attn_ws_layout(d, r), st));
+  return from_cuda(launch_attn_simt(B, M, d, r, dt, C, flags, O, ws, attn_ws_layout(d, r), early_c, st));
 }
 
 // Workspace of the fused forward call: the factorization's, then the attention's.

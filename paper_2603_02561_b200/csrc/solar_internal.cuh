@@ -228,7 +228,7 @@ cudaError_t launch_attn_prepare(int B, int d, int r, solar_dtype_t dt, const flo
                                 const float* V, const void* Wq, const void* Wk, const void* Wv,
                                 float scale, char* ws, const AttnWs& lay, cudaStream_t st);
 cudaError_t launch_attn_simt(int B, int M, int d, int r, solar_dtype_t dt, const void* C,
-                             unsigned flags, void* O, const char* ws, const AttnWs& lay,
+                             unsigned flags, void* O, const char* ws, const AttnWs& lay, bool early_c,
                              cudaStream_t st);
 bool flash_factored_supported(int d, int r, solar_dtype_t dt);
 cudaError_t launch_flash_factored(int B, int M, int N, int d, int r, const void* C, const void* US, void* O,
@@ -284,6 +284,19 @@ inline cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, s
 }
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
+// Loads of what the kernel before wrote, after pdl_wait(): volatile, because a load that the compiler
+// takes for a read of constant memory (__ldg, a const __restrict__ pointer) may be moved above the wait.
+__device__ __forceinline__ float ld_dep(const float* p) {
+  float v;
+  asm volatile("ld.global.f32 %0, [%1];" : "=f"(v) : "l"(p) : "memory");
+  return v;
+}
+__device__ __forceinline__ float4 ld_dep(const float4* p) {
+  float4 v;
+  asm volatile("ld.global.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "l"(p) : "memory");
+  return v;
+}
 
 // ---- device helpers ----------------------------------------------------------
 template <typename T> __device__ __forceinline__ float to_f32(T x);
