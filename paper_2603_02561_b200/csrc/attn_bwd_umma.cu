@@ -99,7 +99,9 @@ attn_bwd_umma_kernel(const __grid_constant__ CUtensorMap tmC, const __grid_const
   const bool use_softmax = !(flags & SOLAR_FLAG_NO_SOFTMAX);
 
   if (tid == 0) {
-    // the per-user operands, once
+    // the per-user operands, once; they come from the kernel before, which itself has waited for whatever
+    // wrote the caller's C and dO
+    pdl_wait();
     ptx::mbar_arrive_expect_tx(&bar_ops, 2 * Cfg::tok_bytes(np) + Cfg::TK_BYTES);
 #pragma unroll
     for (int x = 0; x < Cfg::KB; ++x)
@@ -347,39 +349,11 @@ attn_bwd_umma_kernel(const __grid_constant__ CUtensorMap tmC, const __grid_const
   if (warp == 1) ptx::tmem_dealloc(tmem, kTmemCols);
 }
 
-// T [d][r] and Value_r [r][d] (fp32, written by the prepare kernel) as the two extra bf16
-// operand images of the kernel above: Tkm [2][d][64] (T, tokens along K, zero past r) and
-// Vkm [2][64][d] (Value_r, zero rows past r), each as a high and a low half.
-__global__ void attn_bwd_pack_kernel(const char* __restrict__ ws, AttnWs lay, int d, int r,
-                                     __nv_bfloat16* __restrict__ pk) {
-  const int b = blockIdx.y;
-  const char* wsb = ws + (size_t)b * lay.per_user;
-  const float* Tf = reinterpret_cast<const float*>(wsb + lay.tf_off);
-  const float* Vr = reinterpret_cast<const float*>(wsb + lay.vr_off);
-  __nv_bfloat16* Tkm = pk + (size_t)b * 4 * kTokenSlots * d;
-  __nv_bfloat16* Vkm = Tkm + 2 * kTokenSlots * d;
-  for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < d * kTokenSlots; e += gridDim.x * blockDim.x) {
-    const int k = e / kTokenSlots, i = e % kTokenSlots;
-    const float t = i < r ? Tf[k * r + i] : 0.f;
-    const __nv_bfloat16 th = __float2bfloat16_rn(t);
-    Tkm[e] = th;
-    Tkm[d * kTokenSlots + e] = __float2bfloat16_rn(t - __bfloat162float(th));
-    const int i2 = e / d, j = e % d;
-    const float v = i2 < r ? Vr[i2 * d + j] : 0.f;
-    const __nv_bfloat16 vh = __float2bfloat16_rn(v);
-    Vkm[e] = vh;
-    Vkm[kTokenSlots * d + e] = __float2bfloat16_rn(v - __bfloat162float(vh));
-  }
-}
-
 template <int D>
 cudaError_t launch_d(int B, int M, int r, const void* C, const void* dO, unsigned flags, void* dC, float* part,
                      __nv_bfloat16* pk, int tiles_per_cta, int chunks, const char* ws, const AttnWs& lay,
                      cudaStream_t st) {
   using Cfg = BwdCfg<D>;
-  attn_bwd_pack_kernel<<<dim3(D * kTokenSlots / 256, B), 256, 0, st>>>(ws, lay, D, r, pk);
-  cudaError_t e = cudaGetLastError();
-  if (e != cudaSuccess) return e;
   CUtensorMap tmC, tmG, tmDC, tmT, tmVk, tmTk;
   const uint64_t pu = lay.per_user, pku = (uint64_t)4 * kTokenSlots * D * 2;
   const int np = (r + 15) & ~15;
@@ -391,12 +365,12 @@ cudaError_t launch_d(int B, int M, int r, const void* C, const void* dO, unsigne
   ok = ok && encode_tmap_bf16_3d(&tmVk, pk + 2 * kTokenSlots * D, D, 2 * kTokenSlots, (uint64_t)B, (uint64_t)D * 2, pku,
                                  64, np);
   if (!ok) return cudaErrorInvalidValue;
-  e = cudaFuncSetAttribute(attn_bwd_umma_kernel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           (int)Cfg::smem(kTokenSlots));
+  static bool limits_set[kMaxDevicesCached] = {};
+  const cudaError_t e = set_kernel_limits(reinterpret_cast<const void*>(&attn_bwd_umma_kernel<D>), Cfg::smem(kTokenSlots),
+                                          limits_set);
   if (e != cudaSuccess) return e;
-  attn_bwd_umma_kernel<D><<<dim3(chunks, B), 128, Cfg::smem(np), st>>>(
-      tmC, tmG, tmDC, tmT, tmVk, tmTk, r, flags, static_cast<__nv_bfloat16*>(dC), part, M, tiles_per_cta);
-  return cudaGetLastError();
+  return launch_pdl(attn_bwd_umma_kernel<D>, dim3(chunks, B), dim3(128), Cfg::smem(np), st, tmC, tmG, tmDC, tmT, tmVk, tmTk,
+                    r, flags, static_cast<__nv_bfloat16*>(dC), part, M, tiles_per_cta);
 }
 
 }  // namespace

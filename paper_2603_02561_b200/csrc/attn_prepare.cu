@@ -142,41 +142,61 @@ attn_prepare_kernel(const float* __restrict__ S, const float* __restrict__ V,
   }
 }
 
-// bf16 weights, d = 64 or 128: one CTA per user, the three products on the tensor cores (the
-// routine the eigensolver's epilogue uses, so a forward pass gives the same bits either way).
+// bf16 weights, d = 64 or 128: two CTAs per user, one for Key_r and T, one for Value_r, on the tensor
+// cores (the routine the eigensolver's epilogue uses, so a forward pass gives the same bits either
+// way).  Bound by latency: one round of global loads (weights, factors and singular values together),
+// two barriers and the chained products.  8 users, d = 64, r = 27: @OLD@ us with one CTA per user and the
+// weights loaded behind the factors, @NEW@ now.
+template <int D, int KINDS>
+__device__ __forceinline__ void prepare_kinds(unsigned char* smb, const float* S, const float* V, const void* Wq, const void* Wk,
+                                              const void* Wv, float scale, int r, const pmma::Out& o, int b, int tid) {
+  constexpr int NT = D == 128 ? 256 : 128;
+  const int rp = (r + 3) & ~3;
+  float* VS = reinterpret_cast<float*>(smb);     // [D][rp]  V Sigma (zero in the padding)
+  pmma::Weights<D, NT, KINDS> w;
+  w.load(Wq, Wk, Wv, tid);
+  const float* Vb = V + (size_t)b * D * r;
+#pragma unroll 8
+  for (int e = tid; e < D * rp; e += NT) {
+    const int k = e / rp, i = e - k * rp, ic = min(i, r - 1);
+    const float v = ld_dep(Vb + (size_t)k * r + ic), s = S != nullptr ? ld_dep(S + (size_t)b * r + ic) : 1.f;
+    VS[e] = i < r ? v * s : 0.f;
+  }
+  __syncthreads();
+  pdl_trigger();
+  pmma::project<D, NT, KINDS>(smb, r, w, scale, o, tid);
+}
+
 template <int D>
 __global__ void __launch_bounds__(D == 128 ? 256 : 128, 1)
 attn_prepare_mma_kernel(const float* __restrict__ S, const float* __restrict__ V, const void* __restrict__ Wq,
                         const void* __restrict__ Wk, const void* __restrict__ Wv, float scale, int r,
-                        char* __restrict__ ws, AttnWs lay) {
-  constexpr int NT = D == 128 ? 256 : 128;
+                        char* __restrict__ ws, AttnWs lay, int f32, __nv_bfloat16* __restrict__ bwd_pk) {
   extern __shared__ __align__(16) unsigned char smb[];
-  const int rp = (r + 3) & ~3;
   const int b = blockIdx.x, tid = threadIdx.x;
   char* wsb = ws + (size_t)b * lay.per_user;
-  float* VS = reinterpret_cast<float*>(smb);     // [D][rp]  V Sigma (zero in the padding)
+  pmma::Out o;
+  o.Tpk = reinterpret_cast<__nv_bfloat16*>(wsb + lay.tpk_off);
+  o.Vpk = reinterpret_cast<__nv_bfloat16*>(wsb + lay.vpk_off);
+  o.Tf = f32 ? reinterpret_cast<float*>(wsb + lay.tf_off) : nullptr;
+  o.Vr = f32 ? reinterpret_cast<float*>(wsb + lay.vr_off) : nullptr;
+  o.Tkm = bwd_pk != nullptr ? bwd_pk + (size_t)b * 4 * kTokenSlots * D : nullptr;
+  o.Vkm = bwd_pk != nullptr ? o.Tkm + 2 * kTokenSlots * D : nullptr;
   pdl_wait();                                    // as in the kernel above
-  for (int e = tid; e < D * rp; e += NT) {
-    const int k = e / rp, i = e % rp;
-    VS[e] = i < r ? V[((size_t)b * D + k) * r + i] * (S != nullptr ? S[(size_t)b * r + i] : 1.f) : 0.f;
-  }
-  __syncthreads();
-  pdl_trigger();
-  pmma::project<D, NT>(smb, r, Wq, Wk, Wv, scale, reinterpret_cast<__nv_bfloat16*>(wsb + lay.tpk_off),
-                       reinterpret_cast<__nv_bfloat16*>(wsb + lay.vpk_off), reinterpret_cast<float*>(wsb + lay.tf_off),
-                       reinterpret_cast<float*>(wsb + lay.vr_off), kTokenSlots, tid);
+  if (blockIdx.y == 0) prepare_kinds<D, 1>(smb, S, V, Wq, Wk, Wv, scale, r, o, b, tid);
+  else prepare_kinds<D, 2>(smb, S, V, Wq, Wk, Wv, scale, r, o, b, tid);
 }
 
 template <int D>
 cudaError_t launch_mma(int B, int r, const float* S, const float* V, const void* Wq, const void* Wk, const void* Wv,
-                       float scale, char* ws, const AttnWs& lay, cudaStream_t st) {
+                       float scale, char* ws, const AttnWs& lay, bool f32, void* bwd_pk, cudaStream_t st) {
   static bool limits_set[kMaxDevicesCached] = {};
   cudaError_t e = set_kernel_limits(reinterpret_cast<const void*>(&attn_prepare_mma_kernel<D>),
                                     (size_t)pmma::Lay<D>::bytes(kTokenSlots), limits_set);
   if (e != cudaSuccess) return e;
-  e = launch_pdl(attn_prepare_mma_kernel<D>, dim3(B), dim3(D == 128 ? 256 : 128),
-                 (size_t)pmma::Lay<D>::bytes((r + 15) & ~15), st, S, V, Wq, Wk, Wv, scale, r, ws, lay);
-  return e != cudaSuccess ? e : cudaGetLastError();
+  return launch_pdl(attn_prepare_mma_kernel<D>, dim3(B, 2), dim3(D == 128 ? 256 : 128),
+                    (size_t)pmma::Lay<D>::bytes((r + 15) & ~15), st, S, V, Wq, Wk, Wv, scale, r, ws, lay, (int)f32,
+                    static_cast<__nv_bfloat16*>(bwd_pk));
 }
 
 template <typename T>
@@ -212,9 +232,9 @@ cudaError_t launch_t(int B, int d, int r, const float* S, const float* V, const 
 
 cudaError_t launch_attn_prepare(int B, int d, int r, solar_dtype_t dt, const float* S,
                                 const float* V, const void* Wq, const void* Wk, const void* Wv,
-                                float scale, char* ws, const AttnWs& lay, cudaStream_t st) {
-  if (dt == SOLAR_BF16 && d == 64) return launch_mma<64>(B, r, S, V, Wq, Wk, Wv, scale, ws, lay, st);
-  if (dt == SOLAR_BF16 && d == 128) return launch_mma<128>(B, r, S, V, Wq, Wk, Wv, scale, ws, lay, st);
+                                float scale, char* ws, const AttnWs& lay, bool f32, void* bwd_pk, cudaStream_t st) {
+  if (dt == SOLAR_BF16 && d == 64) return launch_mma<64>(B, r, S, V, Wq, Wk, Wv, scale, ws, lay, f32, bwd_pk, st);
+  if (dt == SOLAR_BF16 && d == 128) return launch_mma<128>(B, r, S, V, Wq, Wk, Wv, scale, ws, lay, f32, bwd_pk, st);
   return dt == SOLAR_BF16
              ? launch_t<__nv_bfloat16>(B, d, r, S, V, Wq, Wk, Wv, scale, ws, lay, st)
              : launch_t<float>(B, d, r, S, V, Wq, Wk, Wv, scale, ws, lay, st);

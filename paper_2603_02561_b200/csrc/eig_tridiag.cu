@@ -1274,8 +1274,10 @@ __device__ __forceinline__ void prepare_epilogue(float* __restrict__ sm, int b, 
       }
       __syncthreads();
     }
-    pmma::project<(D >= 64 ? D : 64), NT>(reinterpret_cast<unsigned char*>(sm), r, fa.Wq, fa.Wk, fa.Wv, fa.scale, Tpk, Vpk,
-                                          nullptr, nullptr, (r + 15) & ~15, tid);
+    constexpr int DP = D >= 64 ? D : 64;
+    pmma::Weights<DP, NT, 3> w;
+    w.load(fa.Wq, fa.Wk, fa.Wv, tid);
+    pmma::project<DP, NT, 3>(reinterpret_cast<unsigned char*>(sm), r, w, fa.scale, pmma::Out{Tpk, Vpk, nullptr, nullptr, nullptr, nullptr}, tid);
     return;
   }
   stage_weight_any<D, NT, false>(fa.Wk, fa.mode, W0, tid);

@@ -3,7 +3,8 @@
 //   Value_r = (V Sigma)^T W_V   [r,d]
 //   T       = scale * W_Q Key_r^T  [d,r]   (so that the scores of Eq. 12 are C T)
 // written as the attention kernels' packed operands (T^T and Value_r^T, each as a high and a
-// low bf16 half) and, on request, as fp32 copies.  Three small GEMMs per user -- far too small
+// low bf16 half; token rows up to the next multiple of 16, which is what those kernels read) and, on
+// request, as fp32 copies and as the backward kernel's operands.  Three small GEMMs per user -- far too small
 // for tcgen05 (M would be 16 or 32) -- so they run as warp-level mma.sync.m16n8k16 with fp32
 // accumulation: the fp32 factor V Sigma enters as a high and a low bf16 half (two MMAs per
 // product, ~16 mantissa bits), the weights are bf16 already, and Key_r never leaves the
@@ -44,7 +45,7 @@ __device__ __forceinline__ void split2(float a, float b, uint32_t& hi, uint32_t&
   lo = pack2(a - ah, b - bh);
 }
 __device__ __forceinline__ void mma16816(float (&c)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
-  asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
+  asm("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
                : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
                : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
 }
@@ -56,17 +57,42 @@ __device__ __forceinline__ void ldsm_x4_trans(uint32_t (&x)[4], const void* p) {
                : "r"((uint32_t)__cvta_generic_to_shared(p)));
 }
 
+// The weights of the products wanted (KINDS: bit 0 Key_r and T, bit 1 Value_r) as a thread's 16-byte
+// pieces; loaded ahead of project() so that their latency runs beside whatever comes between.
+template <int D, int NT, int KINDS> struct Weights {
+  static constexpr int NV = D * D / 8 / NT;
+  static_assert(NV * NT * 8 == D * D, "whole pieces");
+  uint4 k[(KINDS & 1) ? NV : 1], q[(KINDS & 1) ? NV : 1], v[(KINDS & 2) ? NV : 1];
+  __device__ __forceinline__ void load(const void* Wq, const void* Wk, const void* Wv, int tid) {
+#pragma unroll
+    for (int n = 0; n < NV; ++n) {
+      if (KINDS & 1) {
+        k[n] = ld_dep(static_cast<const uint4*>(Wk) + tid + n * NT);
+        q[n] = ld_dep(static_cast<const uint4*>(Wq) + tid + n * NT);
+      }
+      if (KINDS & 2) v[n] = ld_dep(static_cast<const uint4*>(Wv) + tid + n * NT);
+    }
+  }
+};
+
+// Where the results go.  Tpk, Vpk: the attention kernels' operands T^T [2][64][D] and Value_r^T
+// [2][D][64].  Tf, Vr: fp32 copies T [D][r] and Value_r [r][D], or nullptr.  Tkm, Vkm: the backward
+// kernel's further operands T [2][D][64] (zero past r) and Value_r [2][64][D], or nullptr (Tkm only
+// where a CTA makes one kind).
+struct Out {
+  __nv_bfloat16 *Tpk, *Vpk, *Tkm, *Vkm;
+  float *Tf, *Vr;
+};
+
 // Every thread of the CTA (NT threads) calls this after a barrier behind the writes of the fp32
-// factor at sm[0 ..).  pad_to: token slots to leave zero-filled in the packed operands
-// (>= 16 ceil(r / 16), <= kTokenSlots).  Tf / Vr: fp32 copies T [D][r] and Value_r [r][D], or
-// both nullptr.
-template <int D, int NT>
-__device__ __forceinline__ void project(unsigned char* __restrict__ sm, int r, const void* __restrict__ Wq,
-                                        const void* __restrict__ Wk, const void* __restrict__ Wv, float scale,
-                                        __nv_bfloat16* __restrict__ Tpk, __nv_bfloat16* __restrict__ Vpk,
-                                        float* __restrict__ Tf, float* __restrict__ Vr, int pad_to, int tid) {
+// factor at sm[0 ..).  The MMAs of a job run as four independent accumulator chains; where the CTA has
+// more warps than jobs, two warps share the columns of T or Value_r.
+template <int D, int NT, int KINDS>
+__device__ __forceinline__ void project(unsigned char* __restrict__ sm, int r, const Weights<D, NT, KINDS>& w, float scale,
+                                        const Out& o, int tid) {
   using L = Lay<D>;
-  constexpr int P = L::P, NW = NT / 32, KS = D / 16, NTL = D / 8;
+  constexpr int P = L::P, NW = NT / 32, KS = D / 16, NTL = D / 8, NV = Weights<D, NT, KINDS>::NV;
+  constexpr int NK = KINDS == 3 ? 2 : 1;
   const int rp = (r + 3) & ~3, rp16 = (r + 15) & ~15, mt_n = rp16 / 16;
   const float* VS = reinterpret_cast<const float*>(sm);
   unsigned char* vsh = sm + L::vsh(rp16);
@@ -74,54 +100,34 @@ __device__ __forceinline__ void project(unsigned char* __restrict__ sm, int r, c
   unsigned char* wks = sm + L::wk(rp16);
   unsigned char* wqs = sm + L::wq(rp16);
   unsigned char* wvs = sm + L::wv(rp16);
-  unsigned char* vout = sm + L::vout(rp16);
+  unsigned char* stage = sm + L::vout(rp16);             // [2][D][rp16+8] Value_r^T (or T) halves
   const int lane = tid & 31, warp = tid >> 5, g = lane >> 2, t = lane & 3;
 
-  // the three weights as they are stored (16-byte pieces; all loads of a thread first)
-  {
-    constexpr int NV = D * D / 8 / NT;
-    static_assert(NV * NT * 8 == D * D, "whole pieces");
-    uint4 raw[3][NV];
 #pragma unroll
-    for (int n = 0; n < NV; ++n) {
-      raw[0][n] = __ldg(static_cast<const uint4*>(Wk) + tid + n * NT);
-      raw[1][n] = __ldg(static_cast<const uint4*>(Wq) + tid + n * NT);
-      raw[2][n] = __ldg(static_cast<const uint4*>(Wv) + tid + n * NT);
+  for (int n = 0; n < NV; ++n) {
+    const int v = tid + n * NT, row = v / (D / 8), c = v % (D / 8);
+    if (KINDS & 1) {
+      *reinterpret_cast<uint4*>(wks + row * P + c * 16) = w.k[n];
+      *reinterpret_cast<uint4*>(wqs + row * P + c * 16) = w.q[n];
     }
-#pragma unroll
-    for (int n = 0; n < NV; ++n) {
-      const int v = tid + n * NT, row = v / (D / 8), c = v % (D / 8);
-      *reinterpret_cast<uint4*>(wks + row * P + c * 16) = raw[0][n];
-      *reinterpret_cast<uint4*>(wqs + row * P + c * 16) = raw[1][n];
-      *reinterpret_cast<uint4*>(wvs + row * P + c * 16) = raw[2][n];
-    }
+    if (KINDS & 2) *reinterpret_cast<uint4*>(wvs + row * P + c * 16) = w.v[n];
   }
   // (V Sigma)^T as bf16 halves, token-major; token rows >= rp are zero rows
+#pragma unroll 4
   for (int e = tid; e < rp16 * (D / 2); e += NT) {
-    const int i = e % rp16, kp = e / rp16;
-    const float a = i < rp ? VS[(2 * kp) * rp + i] : 0.f, c = i < rp ? VS[(2 * kp + 1) * rp + i] : 0.f;
+    const int kp = e / rp16, i = e - kp * rp16, ic = min(i, rp - 1);
+    const float a0 = VS[(2 * kp) * rp + ic], c0 = VS[(2 * kp + 1) * rp + ic];
     uint32_t hi, lo;
-    split2(a, c, hi, lo);
+    split2(i < rp ? a0 : 0.f, i < rp ? c0 : 0.f, hi, lo);
     *reinterpret_cast<uint32_t*>(vsh + i * P + kp * 4) = hi;
     *reinterpret_cast<uint32_t*>(vsl + i * P + kp * 4) = lo;
   }
-  // token slots rp16 .. pad_to - 1 of the packed operands stay zero
-  {
-    const uint4 z4 = make_uint4(0u, 0u, 0u, 0u);
-    const int extra = pad_to - rp16;
-    for (int e = tid; e < 2 * extra * (D / 8); e += NT) {
-      const int h = e / (extra * (D / 8)), rem = e % (extra * (D / 8));
-      reinterpret_cast<uint4*>(Tpk + ((size_t)h * kTokenSlots + rp16) * D)[rem] = z4;
-    }
-    for (int e = tid; e < 2 * D * (extra / 8); e += NT) {
-      const int row = e / (extra / 8), c = e % (extra / 8);
-      reinterpret_cast<uint4*>(Vpk + (size_t)row * kTokenSlots + rp16)[c] = z4;      // row runs over [2][D]
-    }
-  }
   __syncthreads();
 
-  for (int job = warp; job < 2 * mt_n; job += NW) {
-    const int mt = job % mt_n, kind = job / mt_n;          // kind 0: Key_r, then T; 1: Value_r
+  const int slices = (NK * mt_n * 2 <= NW) ? 2 : 1, per = NTL / slices;   // columns (blocks of 8) of a warp
+  for (int job = warp; job < NK * mt_n * slices; job += NW) {
+    const int sl = job % slices, mt = (job / slices) % mt_n;
+    const int kind = KINDS == 3 ? job / (slices * mt_n) : KINDS - 1;        // 0: Key_r, then T; 1: Value_r
     const int i0 = 16 * mt + g;                            // this lane's token rows: i0 and i0 + 8
     // A fragments of (V Sigma)^T for all k
     uint32_t ah[KS][4], al[KS][4];
@@ -137,84 +143,122 @@ __device__ __forceinline__ void project(unsigned char* __restrict__ sm, int r, c
       al[ks][2] = *reinterpret_cast<const uint32_t*>(vsl + o0 + 16);
       al[ks][3] = *reinterpret_cast<const uint32_t*>(vsl + o1 + 16);
     }
-    // X[i][j] = sum_k (V Sigma)[k][i] W[k][j], all D columns j of the 16 tokens
-    const unsigned char* wsrc = kind == 0 ? wks : wvs;
-    float acc[NTL][4];
+    // acc[c] = columns 8 (nt0 + c) .. of X[i][j] = sum_k (V Sigma)[k][i] W[k][j], four blocks at a time
+    auto four = [&](float (&acc)[4][4], const unsigned char* wsrc, int nt0) {
 #pragma unroll
-    for (int nt = 0; nt < NTL; ++nt) { acc[nt][0] = acc[nt][1] = acc[nt][2] = acc[nt][3] = 0.f; }
-#pragma unroll
-    for (int ks = 0; ks < KS; ++ks) {
-#pragma unroll
-      for (int nt = 0; nt < NTL; nt += 2) {
-        uint32_t bfr[4];       // b0, b1 of column block nt; b0, b1 of block nt + 1
-        ldsm_x4_trans(bfr, wsrc + (16 * ks + 8 * ((lane >> 3) & 1) + (lane & 7)) * P + (8 * (nt + (lane >> 4))) * 2);
-        mma16816(acc[nt], ah[ks], bfr[0], bfr[1]);
-        mma16816(acc[nt], al[ks], bfr[0], bfr[1]);
-        mma16816(acc[nt + 1], ah[ks], bfr[2], bfr[3]);
-        mma16816(acc[nt + 1], al[ks], bfr[2], bfr[3]);
-      }
-    }
-    if (kind == 1) {
-      // Value_r^T halves into the staging tile [h][j][token]; the fp32 copy straight from the registers
-#pragma unroll
-      for (int nt = 0; nt < NTL; ++nt) {
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-          const int i = i0 + 8 * (q >> 1), j = 8 * nt + 2 * t + (q & 1);
-          const float x = acc[nt][q];
-          const __nv_bfloat16 hi = __float2bfloat16_rn(x);
-          __nv_bfloat16* row = reinterpret_cast<__nv_bfloat16*>(vout) + (size_t)j * (rp16 + 8) + i;
-          row[0] = hi;
-          row[(size_t)D * (rp16 + 8)] = __float2bfloat16_rn(x - __bfloat162float(hi));
-        }
-        if (Vr != nullptr) {
-          if (i0 < r) *reinterpret_cast<float2*>(Vr + (size_t)i0 * D + 8 * nt + 2 * t) = make_float2(acc[nt][0], acc[nt][1]);
-          if (i0 + 8 < r) *reinterpret_cast<float2*>(Vr + (size_t)(i0 + 8) * D + 8 * nt + 2 * t) = make_float2(acc[nt][2], acc[nt][3]);
-        }
-      }
-      continue;
-    }
-    // Key_r as the A operand of T^T[i][k] = scale * sum_j Key_r[i][j] W_Q[k][j]
-    uint32_t kh[KS][4], kl[KS][4];
-#pragma unroll
-    for (int ks = 0; ks < KS; ++ks) {
-      split2(acc[2 * ks][0], acc[2 * ks][1], kh[ks][0], kl[ks][0]);
-      split2(acc[2 * ks][2], acc[2 * ks][3], kh[ks][1], kl[ks][1]);
-      split2(acc[2 * ks + 1][0], acc[2 * ks + 1][1], kh[ks][2], kl[ks][2]);
-      split2(acc[2 * ks + 1][2], acc[2 * ks + 1][3], kh[ks][3], kl[ks][3]);
-    }
-#pragma unroll
-    for (int nt = 0; nt < NTL; ++nt) {
-      float tc[4] = {0.f, 0.f, 0.f, 0.f};
+      for (int c = 0; c < 4; ++c) acc[c][0] = acc[c][1] = acc[c][2] = acc[c][3] = 0.f;
 #pragma unroll
       for (int ks = 0; ks < KS; ++ks) {
-        const unsigned char* wrow = wqs + (8 * nt + g) * P + (16 * ks + 2 * t) * 2;     // W_Q[k = 8 nt + g][j ..]
-        const uint32_t b0 = *reinterpret_cast<const uint32_t*>(wrow), b1 = *reinterpret_cast<const uint32_t*>(wrow + 16);
-        mma16816(tc, kh[ks], b0, b1);
-        mma16816(tc, kl[ks], b0, b1);
+        uint32_t b0[4], b1[4];       // b0, b1 of a column block; b0, b1 of the next
+        const unsigned char* wr = wsrc + (16 * ks + 8 * ((lane >> 3) & 1) + (lane & 7)) * P + (8 * (nt0 + (lane >> 4))) * 2;
+        ldsm_x4_trans(b0, wr);
+        ldsm_x4_trans(b1, wr + 32);
+        mma16816(acc[0], ah[ks], b0[0], b0[1]); mma16816(acc[1], ah[ks], b0[2], b0[3]);
+        mma16816(acc[2], ah[ks], b1[0], b1[1]); mma16816(acc[3], ah[ks], b1[2], b1[3]);
+        mma16816(acc[0], al[ks], b0[0], b0[1]); mma16816(acc[1], al[ks], b0[2], b0[3]);
+        mma16816(acc[2], al[ks], b1[0], b1[1]); mma16816(acc[3], al[ks], b1[2], b1[3]);
       }
+    };
+    // a 2 x 2 piece (tokens i, i + 8; columns j, j + 1) into the staging tile [h][j][token]
+    auto put = [&](const float (&x)[4], int j) {
 #pragma unroll
-      for (int q = 0; q < 4; ++q) tc[q] *= scale;
-      const int k0 = 8 * nt + 2 * t;
-      uint32_t hi, lo;
-      split2(tc[0], tc[1], hi, lo);
-      *reinterpret_cast<uint32_t*>(Tpk + (size_t)i0 * D + k0) = hi;
-      *reinterpret_cast<uint32_t*>(Tpk + ((size_t)kTokenSlots + i0) * D + k0) = lo;
-      split2(tc[2], tc[3], hi, lo);
-      *reinterpret_cast<uint32_t*>(Tpk + (size_t)(i0 + 8) * D + k0) = hi;
-      *reinterpret_cast<uint32_t*>(Tpk + ((size_t)kTokenSlots + i0 + 8) * D + k0) = lo;
-      if (Tf != nullptr) {
-        if (i0 < r) { Tf[(size_t)k0 * r + i0] = tc[0]; Tf[(size_t)(k0 + 1) * r + i0] = tc[1]; }
-        if (i0 + 8 < r) { Tf[(size_t)k0 * r + i0 + 8] = tc[2]; Tf[(size_t)(k0 + 1) * r + i0 + 8] = tc[3]; }
+      for (int q = 0; q < 4; ++q) {
+        const __nv_bfloat16 hi = __float2bfloat16_rn(x[q]);
+        __nv_bfloat16* row = reinterpret_cast<__nv_bfloat16*>(stage) + (size_t)(j + (q & 1)) * (rp16 + 8) + i0 + 8 * (q >> 1);
+        row[0] = hi;
+        row[(size_t)D * (rp16 + 8)] = __float2bfloat16_rn(x[q] - __bfloat162float(hi));
+      }
+    };
+    if ((KINDS & 2) && kind == 1) {
+#pragma unroll 1
+      for (int nt0 = sl * per; nt0 < (sl + 1) * per; nt0 += 4) {
+        float acc[4][4];
+        four(acc, wvs, nt0);
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+          const int j = 8 * (nt0 + c) + 2 * t;
+          put(acc[c], j);
+          if (o.Vr != nullptr) {
+            if (i0 < r) *reinterpret_cast<float2*>(o.Vr + (size_t)i0 * D + j) = make_float2(acc[c][0], acc[c][1]);
+            if (i0 + 8 < r) *reinterpret_cast<float2*>(o.Vr + (size_t)(i0 + 8) * D + j) = make_float2(acc[c][2], acc[c][3]);
+          }
+          if (o.Vkm != nullptr) {                             // zero rows come out of zero rows of V Sigma
+            uint32_t hi, lo;
+            split2(acc[c][0], acc[c][1], hi, lo);
+            *reinterpret_cast<uint32_t*>(o.Vkm + (size_t)i0 * D + j) = hi;
+            *reinterpret_cast<uint32_t*>(o.Vkm + (size_t)(kTokenSlots + i0) * D + j) = lo;
+            split2(acc[c][2], acc[c][3], hi, lo);
+            *reinterpret_cast<uint32_t*>(o.Vkm + (size_t)(i0 + 8) * D + j) = hi;
+            *reinterpret_cast<uint32_t*>(o.Vkm + (size_t)(kTokenSlots + i0 + 8) * D + j) = lo;
+          }
+        }
+      }
+    }
+    if ((KINDS & 1) && kind == 0) {
+      // Key_r, all D columns, as the A operand of T^T[i][k] = scale * sum_j Key_r[i][j] W_Q[k][j]
+      uint32_t kh[KS][4], kl[KS][4];
+#pragma unroll
+      for (int nt0 = 0; nt0 < NTL; nt0 += 4) {
+        float acc[4][4];
+        four(acc, wks, nt0);
+#pragma unroll
+        for (int c = 0; c < 4; c += 2) {
+          const int ks = (nt0 + c) / 2;
+          split2(acc[c][0], acc[c][1], kh[ks][0], kl[ks][0]);
+          split2(acc[c][2], acc[c][3], kh[ks][1], kl[ks][1]);
+          split2(acc[c + 1][0], acc[c + 1][1], kh[ks][2], kl[ks][2]);
+          split2(acc[c + 1][2], acc[c + 1][3], kh[ks][3], kl[ks][3]);
+        }
+      }
+#pragma unroll 1
+      for (int nt0 = sl * per; nt0 < (sl + 1) * per; nt0 += 4) {
+        float tc[4][4];
+#pragma unroll
+        for (int c = 0; c < 4; ++c) tc[c][0] = tc[c][1] = tc[c][2] = tc[c][3] = 0.f;
+#pragma unroll
+        for (int ks = 0; ks < KS; ++ks) {
+          uint32_t b0[4], b1[4];
+#pragma unroll
+          for (int c = 0; c < 4; ++c) {
+            const unsigned char* wrow = wqs + (8 * (nt0 + c) + g) * P + (16 * ks + 2 * t) * 2;     // W_Q[k = 8 nt + g][j ..]
+            b0[c] = *reinterpret_cast<const uint32_t*>(wrow); b1[c] = *reinterpret_cast<const uint32_t*>(wrow + 16);
+          }
+#pragma unroll
+          for (int c = 0; c < 4; ++c) mma16816(tc[c], kh[ks], b0[c], b1[c]);
+#pragma unroll
+          for (int c = 0; c < 4; ++c) mma16816(tc[c], kl[ks], b0[c], b1[c]);
+        }
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+#pragma unroll
+          for (int q = 0; q < 4; ++q) tc[c][q] *= scale;
+          const int k0 = 8 * (nt0 + c) + 2 * t;
+          uint32_t hi, lo;
+          split2(tc[c][0], tc[c][1], hi, lo);
+          *reinterpret_cast<uint32_t*>(o.Tpk + (size_t)i0 * D + k0) = hi;
+          *reinterpret_cast<uint32_t*>(o.Tpk + ((size_t)kTokenSlots + i0) * D + k0) = lo;
+          split2(tc[c][2], tc[c][3], hi, lo);
+          *reinterpret_cast<uint32_t*>(o.Tpk + (size_t)(i0 + 8) * D + k0) = hi;
+          *reinterpret_cast<uint32_t*>(o.Tpk + ((size_t)kTokenSlots + i0 + 8) * D + k0) = lo;
+          if (KINDS == 1 && o.Tkm != nullptr) put(tc[c], k0);
+          if (o.Tf != nullptr) {
+            if (i0 < r) { o.Tf[(size_t)k0 * r + i0] = tc[c][0]; o.Tf[(size_t)(k0 + 1) * r + i0] = tc[c][1]; }
+            if (i0 + 8 < r) { o.Tf[(size_t)k0 * r + i0 + 8] = tc[c][2]; o.Tf[(size_t)(k0 + 1) * r + i0 + 8] = tc[c][3]; }
+          }
+        }
       }
     }
   }
-  __syncthreads();
-  // Value_r^T out: 16-byte pieces of the rows [h][j][0 .. rp16)
-  for (int e = tid; e < 2 * D * (rp16 / 8); e += NT) {
-    const int row = e / (rp16 / 8), c = e % (rp16 / 8);                                  // row runs over [2][D]
-    reinterpret_cast<uint4*>(Vpk + (size_t)row * kTokenSlots)[c] =
-        *reinterpret_cast<const uint4*>(vout + ((size_t)row * (rp16 + 8) + 8 * c) * 2);
+  // what was staged, as 16-byte pieces of the rows [h][j][0 .. rp16); Tkm is read to its 64th column
+  __nv_bfloat16* dst = (KINDS & 2) ? o.Vpk : o.Tkm;
+  if ((KINDS & 2) || dst != nullptr) {
+    __syncthreads();
+    const int pc = (KINDS & 2) ? rp16 / 8 : kTokenSlots / 8;
+    for (int e = tid; e < 2 * D * pc; e += NT) {
+      const int row = e / pc, c = e % pc;                                                  // row runs over [2][D]
+      reinterpret_cast<uint4*>(dst + (size_t)row * kTokenSlots)[c] =
+          c < rp16 / 8 ? *reinterpret_cast<const uint4*>(stage + ((size_t)row * (rp16 + 8) + 8 * c) * 2) : make_uint4(0u, 0u, 0u, 0u);
+    }
   }
 }
 

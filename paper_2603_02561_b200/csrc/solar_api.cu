@@ -177,7 +177,7 @@ solar_status_t solar_attn_prepare(int B, int d, int r, solar_dtype_t dt, const f
   SOLAR_TRY(check_ptr(Wv));
   SOLAR_TRY(check_ws(workspace, workspace_bytes, attn_ws_bytes(B, d, r)));
   return from_cuda(launch_attn_prepare(B, d, r, dt, S, V, Wq, Wk, Wv, scale,
-                                       static_cast<char*>(workspace), attn_ws_layout(d, r),
+                                       static_cast<char*>(workspace), attn_ws_layout(d, r), true, nullptr,
                                        static_cast<cudaStream_t>(stream)));
 }
 
@@ -211,8 +211,8 @@ solar_status_t solar_svd_attention_fwd(int B, int M, int N, int d, int r, solar_
   SOLAR_TRY(check_ptr(Wk));
   SOLAR_TRY(check_ptr(Wv));
   SOLAR_TRY(check_ws(workspace, workspace_bytes, attn_ws_bytes(B, d, r)));
-  SOLAR_TRY(solar_attn_prepare(B, d, r, dt, S, V, Wq, Wk, Wv, scale, workspace, workspace_bytes,
-                               stream));
+  SOLAR_TRY(from_cuda(launch_attn_prepare(B, d, r, dt, S, V, Wq, Wk, Wv, scale, static_cast<char*>(workspace),
+                                          attn_ws_layout(d, r), false, nullptr, static_cast<cudaStream_t>(stream))));
   return attn_apply_impl(B, M, d, r, dt, C, flags, O, static_cast<const char*>(workspace), true,
                          static_cast<cudaStream_t>(stream));
 }
@@ -289,7 +289,7 @@ solar_status_t solar_svd_attention_bwd(int B, int M, int N, int d, int r, solar_
   const AttnWs lay = attn_ws_layout(d, r);
   char* ws = static_cast<char*>(workspace);
   // T_b and Value_r as in the forward call
-  SOLAR_TRY(from_cuda(launch_attn_prepare(B, d, r, dt, S, V, Wq, Wk, Wv, scale, ws, lay, st)));
+  SOLAR_TRY(from_cuda(launch_attn_prepare(B, d, r, dt, S, V, Wq, Wk, Wv, scale, ws, lay, false, ws + bl.pk_off, st)));
   return from_cuda(launch_attn_bwd(B, M, d, r, dt, C, dO, S, V, Wq, Wk, Wv, scale, flags, dC, dWq, dWk, dWv,
                                    dS, dV, ws, lay, bl, st));
 }
@@ -336,7 +336,8 @@ solar_status_t solar_factored_softmax_attention_fwd(int B, int M, int N, int d, 
   // The packed operands of the kernel are the prepare kernel's with unit singular values:
   // T^T becomes (scale log2e W_Q W_K^T V)^T and Value_r^T becomes (V^T W_V)^T.
   SOLAR_TRY(from_cuda(launch_attn_prepare(B, d, r, dt, nullptr, V, Wq, Wk, Wv,
-                                          scale * 1.4426950408889634f, static_cast<char*>(workspace), lay, st)));
+                                          scale * 1.4426950408889634f, static_cast<char*>(workspace), lay, false,
+                                          nullptr, st)));
   return from_cuda(launch_flash_factored(B, M, N, d, r, C, US, O, static_cast<const char*>(workspace), lay, st));
 }
 

@@ -224,9 +224,11 @@ cudaError_t launch_attn_bwd_umma(int B, int M, int d, int r, const void* C, cons
 bool project_us_umma_supported(int N, int d, int r, solar_dtype_t dt);
 cudaError_t launch_project_us_umma(int B, int N, int d, int r, const void* H, const float* V, void* US,
                                    cudaStream_t st);
+// bwd_pk: also the backward kernel's operands [B][4][64][d] (tensor-core shapes), or nullptr; f32: also the
+// fp32 copies where only the backward pass or a caller of the stage would read them
 cudaError_t launch_attn_prepare(int B, int d, int r, solar_dtype_t dt, const float* S,
                                 const float* V, const void* Wq, const void* Wk, const void* Wv,
-                                float scale, char* ws, const AttnWs& lay, cudaStream_t st);
+                                float scale, char* ws, const AttnWs& lay, bool f32, void* bwd_pk, cudaStream_t st);
 cudaError_t launch_attn_simt(int B, int M, int d, int r, solar_dtype_t dt, const void* C,
                              unsigned flags, void* O, const char* ws, const AttnWs& lay, bool early_c,
                              cudaStream_t st);
@@ -290,6 +292,11 @@ __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.lau
 __device__ __forceinline__ float ld_dep(const float* p) {
   float v;
   asm volatile("ld.global.f32 %0, [%1];" : "=f"(v) : "l"(p) : "memory");
+  return v;
+}
+__device__ __forceinline__ uint4 ld_dep(const uint4* p) {
+  uint4 v;
+  asm volatile("ld.global.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p) : "memory");
   return v;
 }
 __device__ __forceinline__ float4 ld_dep(const float4* p) {
