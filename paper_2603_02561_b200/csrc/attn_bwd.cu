@@ -8,8 +8,8 @@
 //   dW_K = A^T dKey_r,   dW_V = A^T dValue_r,   dSigma_i = sum_k dA_ik V_ki,   dV_ki = dA_ik sigma_i.
 // Four kernels: the streaming one (one CTA per chunk of candidate rows; recomputes S and P,
 // writes dC and a partial of dT and dValue_r^T), the sum of the partials in chunk order, a
-// per-user one (the small chain; writes dSigma, dV and this user's dW contributions) and a
-// sum over users in user order.  The streaming kernel here is the FFMA one (fp32 storage,
+// per-user one (the small chain on four CTAs; writes dSigma, dV and this user's dW contributions)
+// and a sum over users in user order.  The streaming kernel here is the FFMA one (fp32 storage,
 // d = 32); bf16 storage with d = 64 or 128 takes the tensor-core kernel instead.
 #include <math.h>
 
@@ -21,7 +21,7 @@ namespace {
 
 constexpr int kThreads = 256;
 constexpr int kWarps = kThreads / 32;
-constexpr int kUserThreads = 1024;   // the per-user chain is latency-bound: many warps per scheduler
+constexpr int kUserThreads = 256;
 constexpr int kUserWarps = kUserThreads / 32;
 constexpr int kBatch = 32;            // candidate rows per inner batch
 constexpr int kRP = kTokenSlots;      // 64 token slots, zero padded
@@ -190,9 +190,12 @@ __device__ __forceinline__ void small_gemm(int rows, int K, FA a, FB b, FS store
   }
 }
 
-// Per-user chain from dT and dValue_r to dSigma, dV and this user's dW contributions.
-// Each weight matrix is staged in shared memory (fp32, odd pitch) when it is needed: W_K for
-// Key_r, W_Q for dKey_r, then W_K and W_V again for dA, where they are read along their rows.
+// Per-user chain from dT and dValue_r to dSigma, dV and this user's dW contributions, on four CTAs per
+// user: 0 Key_r -> dW_Q; 1 dKey_r -> dW_K; 2 dKey_r -> dA -> dSigma, dV; 3 dW_V (dKey_r is formed twice).
+// Bound by latency: a round of global loads, then two small products (three for role 2) with a barrier
+// each; a weight that is needed later is fetched into registers while the product before runs.  Weights
+// sit in shared memory as fp32 at odd pitch, dT and dValue_r^T are read along both indices.
+// 16 users, d = 64, r = 32: 24 us as one chain on one CTA of 1024 threads, 12 now.
 template <typename T, int D>
 __global__ void __launch_bounds__(kUserThreads)
 attn_bwd_user_kernel(const float* __restrict__ part, int chunks, const float* __restrict__ S,
@@ -200,90 +203,134 @@ attn_bwd_user_kernel(const float* __restrict__ part, int chunks, const float* __
                      const T* __restrict__ Wv, float scale, int r, float* __restrict__ dS,
                      float* __restrict__ dV, float* __restrict__ dw) {
   extern __shared__ __align__(16) float sm[];
-  constexpr int LR = kRP + 1;           // odd pitch: dT and dValue_r^T are read along both indices
-  constexpr int LW = D + 1;             // odd pitch of the staged weight matrix
+  constexpr int LR = kRP + 1;           // odd pitch
+  constexpr int LW = D + 1;
   float* dT = sm;                       // [D][LR]    dT[k][i]
   float* dVT = dT + D * LR;             // [D][LR]    dValue_r^T[j][i]
-  float* A = dVT + D * LR;              // [kRP][D]   Sigma V^T (rows past r zero), at the end dA
-  float* X = A + kRP * D;               // [kRP][D]   Key_r, then dKey_r (rows past r zero)
+  float* A = dVT + D * LR;              // [kRP][D]   Sigma V^T; role 2: dA
+  float* X = A + kRP * D;               // [kRP][D]   Key_r or dKey_r
   float* Ws = X + kRP * D;              // [D][LW]    the weight matrix in use
-  const int b = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int b = blockIdx.x, role = blockIdx.y, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  constexpr int VE = Vec16<T>::kElems, PCS = D * D / VE, NV = (PCS + kUserThreads - 1) / kUserThreads;
 
-  auto stage = [&](const T* __restrict__ W) {
-    constexpr int VE = Vec16<T>::kElems;
-    for (int v = tid; v < D * D / VE; v += kUserThreads) {
+  float4 wreg[NV];                      // 16-byte pieces of the weight that comes next
+  auto fetch = [&](const T* W) {
+#pragma unroll
+    for (int n = 0; n < NV; ++n) wreg[n] = ld_dep(reinterpret_cast<const float4*>(W) + min(tid + n * kUserThreads, PCS - 1));
+  };
+  auto stage = [&]() {
+#pragma unroll
+    for (int n = 0; n < NV; ++n) {
+      const int v = min(tid + n * kUserThreads, PCS - 1), k = (v * VE) / D, j = (v * VE) % D;
       float tmp[VE];
-      Vec16<T>::load(W + (size_t)v * VE, tmp);
-      const int k = (v * VE) / D, j = (v * VE) % D;
+      Vec16<T>::load(reinterpret_cast<const T*>(&wreg[n]), tmp);
 #pragma unroll
       for (int e = 0; e < VE; ++e) Ws[k * LW + j + e] = tmp[e];
     }
   };
-
-  stage(Wk);
-  // the partials, summed into the first chunk's slot by sum_chunks_kernel
-  for (int e = tid; e < 2 * D * kRP; e += kUserThreads)
-    dT[(e / kRP) * LR + e % kRP] = part[(size_t)b * chunks * 2 * D * kRP + e];   // dVT follows dT in shared memory
-  for (int e = tid; e < kRP * D; e += kUserThreads) {
-    const int k = e / kRP, i = e % kRP;   // V is read along its rows
-    A[i * D + k] = i < r ? S[(size_t)b * r + i] * V[((size_t)b * D + k) * r + i] : 0.f;
-    X[e] = 0.f;
-  }
-  __syncthreads();
-  // Key_r[i][j] = sum_k A[i][k] W_K[k][j]
-  small_gemm<D>(r, D, [&](int i, int k) { return A[i * D + k]; }, [&](int k, int j) { return Ws[k * LW + j]; },
-                [&](int i, int j, float v) { X[i * D + j] = v; }, warp, lane, kUserWarps);
-  __syncthreads();
-  stage(Wq);
+  // a [D][64] matrix of the partials, summed into the first chunk's slot by sum_chunks_kernel
+  auto load_sum = [&](float* dst, int which) {
+    const float4* src = reinterpret_cast<const float4*>(part + (size_t)b * chunks * 2 * D * kRP + (size_t)which * D * kRP);
+#pragma unroll 4
+    for (int e = tid; e < D * kRP / 4; e += kUserThreads) {
+      const float4 x = ld_dep(src + e);
+      float* row = dst + (e / (kRP / 4)) * LR + (e % (kRP / 4)) * 4;
+      row[0] = x.x; row[1] = x.y; row[2] = x.z; row[3] = x.w;
+    }
+  };
+  auto load_a = [&]() {
+#pragma unroll 8
+    for (int e = tid; e < D * r; e += kUserThreads) {          // V is read along its rows
+      const int k = e / r, i = e - k * r;
+      A[i * D + k] = ld_dep(S + (size_t)b * r + i) * ld_dep(V + (size_t)b * D * r + e);
+    }
+  };
   float* dWq = dw + (size_t)b * 3 * D * D;
   float* dWk = dWq + D * D;
   float* dWv = dWk + D * D;
-  // dW_Q[k][j] = scale sum_i dT[k][i] Key_r[i][j]
-  small_gemm<D>(D, r, [&](int k, int i) { return dT[k * LR + i]; }, [&](int i, int j) { return X[i * D + j]; },
-                [&](int k, int j, float v) { dWq[k * D + j] = scale * v; }, warp, lane, kUserWarps);
+
+  pdl_wait();
+  if (role == 3) {
+    // dW_V[k][j] = sum_i A[i][k] dValue_r[i][j]
+    load_a();
+    load_sum(dVT, 1);
+    __syncthreads();
+    pdl_trigger();
+    small_gemm<D>(D, r, [&](int k, int i) { return A[i * D + k]; }, [&](int i, int j) { return dVT[j * LR + i]; },
+                  [&](int k, int j, float v) { dWv[k * D + j] = v; }, warp, lane, kUserWarps);
+    return;
+  }
+  fetch(role == 0 ? Wk : Wq);
+  load_sum(dT, 0);
+  if (role == 2) load_sum(dVT, 1); else load_a();
+  stage();
+  if (role == 2) fetch(Wk);
+  // rows past r that a tile of four reads
+  for (int e = tid; e < kRP * D - r * D; e += kUserThreads) { X[r * D + e] = 0.f; A[r * D + e] = 0.f; }
   __syncthreads();
-  // dKey_r[i][j] = scale sum_k dT[k][i] W_Q[k][j]   (over Key_r)
+  if (role == 0) {
+    // Key_r[i][j] = sum_k A[i][k] W_K[k][j];  dW_Q[k][j] = scale sum_i dT[k][i] Key_r[i][j]
+    small_gemm<D>(r, D, [&](int i, int k) { return A[i * D + k]; }, [&](int k, int j) { return Ws[k * LW + j]; },
+                  [&](int i, int j, float v) { X[i * D + j] = v; }, warp, lane, kUserWarps);
+    __syncthreads();
+    pdl_trigger();
+    small_gemm<D>(D, r, [&](int k, int i) { return dT[k * LR + i]; }, [&](int i, int j) { return X[i * D + j]; },
+                  [&](int k, int j, float v) { dWq[k * D + j] = scale * v; }, warp, lane, kUserWarps);
+    return;
+  }
+  // dKey_r[i][j] = scale sum_k dT[k][i] W_Q[k][j]
   small_gemm<D>(r, D, [&](int i, int k) { return dT[k * LR + i]; }, [&](int k, int j) { return Ws[k * LW + j]; },
                 [&](int i, int j, float v) { X[i * D + j] = scale * v; }, warp, lane, kUserWarps);
   __syncthreads();
-  stage(Wk);
-  // dW_K[k][j] = sum_i A[i][k] dKey_r[i][j],  dW_V[k][j] = sum_i A[i][k] dValue_r[i][j]
-  small_gemm<D>(D, r, [&](int k, int i) { return A[i * D + k]; }, [&](int i, int j) { return X[i * D + j]; },
-                [&](int k, int j, float v) { dWk[k * D + j] = v; }, warp, lane, kUserWarps);
-  small_gemm<D>(D, r, [&](int k, int i) { return A[i * D + k]; }, [&](int i, int j) { return dVT[j * LR + i]; },
-                [&](int k, int j, float v) { dWv[k * D + j] = v; }, warp, lane, kUserWarps);
+  if (role == 1) {
+    pdl_trigger();
+    // dW_K[k][j] = sum_i A[i][k] dKey_r[i][j]
+    small_gemm<D>(D, r, [&](int k, int i) { return A[i * D + k]; }, [&](int i, int j) { return X[i * D + j]; },
+                  [&](int k, int j, float v) { dWk[k * D + j] = v; }, warp, lane, kUserWarps);
+    return;
+  }
+  // dA[i][k] = sum_j dKey_r[i][j] W_K[k][j] + dValue_r[i][j] W_V[k][j]
+  stage();
+  fetch(Wv);
   __syncthreads();
-  // dA[i][k] = sum_j dKey_r[i][j] W_K[k][j] + dValue_r[i][j] W_V[k][j]; dA takes the place of A
   small_gemm<D>(r, D, [&](int i, int j) { return X[i * D + j]; }, [&](int j, int k) { return Ws[k * LW + j]; },
                 [&](int i, int k, float v) { A[i * D + k] = v; }, warp, lane, kUserWarps);
   __syncthreads();
-  stage(Wv);
+  stage();
   __syncthreads();
+  pdl_trigger();
   small_gemm<D>(r, D, [&](int i, int j) { return dVT[j * LR + i]; }, [&](int j, int k) { return Ws[k * LW + j]; },
                 [&](int i, int k, float v) { A[i * D + k] += v; }, warp, lane, kUserWarps);
   __syncthreads();
   const float* dA = A;
   // dSigma_i = sum_k dA[i][k] V[k][i],  dV[k][i] = dA[i][k] sigma_i
+#pragma unroll 2
   for (int i = warp; i < r; i += kUserWarps) {
     float acc = 0.f;
+#pragma unroll
     for (int k = lane; k < D; k += 32) acc = fmaf(dA[i * D + k], V[((size_t)b * D + k) * r + i], acc);
 #pragma unroll
     for (int o = 16; o; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
     if (lane == 0) dS[(size_t)b * r + i] = acc;
   }
+#pragma unroll 4
   for (int e = tid; e < D * r; e += kUserThreads) {
-    const int k = e / r, i = e % r;
+    const int k = e / r, i = e - k * r;
     dV[(size_t)b * D * r + e] = dA[i * D + k] * S[(size_t)b * r + i];
   }
 }
 
-// part[b][0][e] = sum over the chunks (in chunk order) of part[b][c][e]
+// part[b][0][e] = sum over the chunks (in chunk order) of part[b][c][e].  One element per thread: as
+// 16-byte pieces there are too few threads to hide the loads (4.4 -> 6.3 us at 16 x 16 chunks of 32 KB).
 __global__ void sum_chunks_kernel(float* __restrict__ part, int chunks, int n) {
   const int e = blockIdx.x * blockDim.x + threadIdx.x;
+  pdl_wait();
+  pdl_trigger();
   if (e >= n) return;
   float* p = part + (size_t)blockIdx.y * chunks * n + e;
   float acc = 0.f;
-  for (int c = 0; c < chunks; ++c) acc += p[(size_t)c * n];
+#pragma unroll 8
+  for (int c = 0; c < chunks; ++c) acc += ld_dep(p + (size_t)c * n);
   p[0] = acc;
 }
 
@@ -292,9 +339,11 @@ __global__ void sum_users_kernel(const float* __restrict__ dw, int B, int n, flo
                                  float* __restrict__ o1, float* __restrict__ o2) {
   const int e = blockIdx.x * blockDim.x + threadIdx.x;
   const int w = blockIdx.y;
+  pdl_wait();
   if (e >= n) return;
   float acc = 0.f;
-  for (int b = 0; b < B; ++b) acc += dw[((size_t)b * 3 + w) * n + e];
+#pragma unroll 16
+  for (int b = 0; b < B; ++b) acc += ld_dep(dw + ((size_t)b * 3 + w) * n + e);
   (w == 0 ? o0 : w == 1 ? o1 : o2)[e] = acc;
 }
 
@@ -328,20 +377,18 @@ cudaError_t launch_td(int B, int M, int r, const void* C, const void* dO, const 
     if (e != cudaSuccess) return e;
   }
   if (chunks > 1) {
-    sum_chunks_kernel<<<dim3((2 * D * kRP + 255) / 256, B), 256, 0, st>>>(part, chunks, 2 * D * kRP);
-    e = cudaGetLastError();
+    constexpr int n = 2 * D * kRP;
+    e = launch_pdl(sum_chunks_kernel, dim3(n / 256, B), dim3(256), 0, st, part, chunks, n);
     if (e != cudaSuccess) return e;
   }
-  const size_t smem_user = (size_t)(2 * D * (kRP + 1) + 2 * kRP * D + D * (D + 1)) * sizeof(float);
-  e = cudaFuncSetAttribute(attn_bwd_user_kernel<T, D>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_user);
+  constexpr size_t smem_user = (size_t)(2 * D * (kRP + 1) + 2 * kRP * D + D * (D + 1)) * sizeof(float);
+  static bool limits_set[kMaxDevicesCached] = {};
+  e = set_kernel_limits(reinterpret_cast<const void*>(&attn_bwd_user_kernel<T, D>), smem_user, limits_set);
   if (e != cudaSuccess) return e;
-  attn_bwd_user_kernel<T, D><<<B, kUserThreads, smem_user, st>>>(part, chunks, S, V, static_cast<const T*>(Wq),
-                                                            static_cast<const T*>(Wk), static_cast<const T*>(Wv),
-                                                            scale, r, dS, dV, dw);
-  e = cudaGetLastError();
+  e = launch_pdl(attn_bwd_user_kernel<T, D>, dim3(B, 4), dim3(kUserThreads), smem_user, st, part, chunks, S, V,
+                 static_cast<const T*>(Wq), static_cast<const T*>(Wk), static_cast<const T*>(Wv), scale, r, dS, dV, dw);
   if (e != cudaSuccess) return e;
-  sum_users_kernel<<<dim3((D * D + 255) / 256, 3), 256, 0, st>>>(dw, B, D * D, dWq, dWk, dWv);
-  return cudaGetLastError();
+  return launch_pdl(sum_users_kernel, dim3(D * D / 128, 3), dim3(128), 0, st, dw, B, D * D, dWq, dWk, dWv);
 }
 
 template <typename T>

@@ -80,8 +80,8 @@ cudaError_t launch_t(int B, int N, int d, int r, const void* H, const float* V, 
 }  // namespace
 
 cudaError_t launch_project_us(int B, int N, int d, int r, solar_dtype_t dt, const void* H,
-                              const float* V, void* US, cudaStream_t st) {
-  if (project_us_umma_supported(N, d, r, dt)) return launch_project_us_umma(B, N, d, r, H, V, US, st);
+                              const float* V, void* US, bool early_h, cudaStream_t st) {
+  if (project_us_umma_supported(N, d, r, dt)) return launch_project_us_umma(B, N, d, r, H, V, US, early_h, st);
   return dt == SOLAR_BF16 ? launch_t<__nv_bfloat16>(B, N, d, r, H, V, US, st)
                           : launch_t<float>(B, N, d, r, H, V, US, st);
 }

@@ -12,6 +12,8 @@
 // accumulators in tensor memory; warps 0-3 read the finished accumulator (one row per
 // thread), round to bf16 and store the rows, while the next tile is being multiplied
 // into the other accumulator.  H is read from HBM once and never passes through registers.
+// Bound by HBM.  16 x 10240 x 64: q = 64 19.4 us with every thread storing its own row (32 lines per
+// instruction), 17.9 through shared memory; q = 32 13.5 and 12.4.
 #include "sm100_ptx.cuh"
 #include "solar_internal.cuh"
 
@@ -28,16 +30,18 @@ template <int D> struct UsCfg {
   static constexpr int KB = D / 64;                          // 64-column TMA boxes per tile
   static constexpr int BOX_BYTES = kTileRows * 128;          // 16 KB: 128 rows x 64 bf16
   static constexpr int TILE_BYTES = KB * BOX_BYTES;
-  static constexpr int STAGES = (D == 64) ? 6 : 4;
-  // ring + X^T as [2 halves][KB][np rows][128 B] + slack to align to 1024
-  static constexpr size_t smem(int np) { return (size_t)STAGES * TILE_BYTES + (size_t)2 * KB * np * 128 + 1024; }
+  static constexpr int STAGES = (D == 64) ? 6 : 3;
+  // ring + X^T as [2 halves][KB][np rows][128 B] + the output rows at odd 16-byte pitch + slack to align to 1024
+  static constexpr size_t smem(int np) {
+    return (size_t)STAGES * TILE_BYTES + (size_t)2 * KB * np * 128 + (size_t)kTileRows * (np / 8 + 1) * 16 + 1024;
+  }
 };
 
 // byte offset of 16-byte chunk c of row `row` in a [rows][128 B] tile with the 128-byte swizzle
 template <int D>
 __global__ void __launch_bounds__(kThreads, 1)
 project_us_umma_kernel(const __grid_constant__ CUtensorMap tmap, const float* __restrict__ V,
-                       __nv_bfloat16* __restrict__ US, int N, int r, int chunk_rows) {
+                       __nv_bfloat16* __restrict__ US, int N, int r, int chunk_rows, int early_h) {
   // V is the per-user matrix X [D][r] and US the output [N][r]; r stands for q here.
   using Cfg = UsCfg<D>;
   constexpr int STAGES = Cfg::STAGES;
@@ -82,15 +86,19 @@ project_us_umma_kernel(const __grid_constant__ CUtensorMap tmap, const float* __
       ptx::tma_load_3d(tiles + (size_t)st * Cfg::TILE_BYTES + x * Cfg::BOX_BYTES, &tmap, &full_bar[st],
                        x * 64, row0 + t * kTileRows, b);
   };
-  // the first tiles are on their way while V^T is being packed
+  // The first tiles are on their way while V^T is being packed; ahead of the wait only when an earlier
+  // kernel of the same library call has already waited for whatever wrote H (early_h).
   const int primed = min(ntiles, STAGES);
+  if (!early_h) pdl_wait();
   if (warp == kProducerWarp && lane == 0)
     for (int t = 0; t < primed; ++t) load_tile(t);
+  if (early_h) pdl_wait();
 
   // V^T as two K-major bf16 operands: row i (factor), K = k (feature); rows r .. np-1 zero
+#pragma unroll 8
   for (int e = tid; e < np * D; e += kThreads) {
-    const int k = e / np, i = e % np;
-    const float v = i < r ? V[((size_t)b * D + k) * r + i] : 0.f;
+    const int k = e / np, i = e - k * np;
+    const float x = ld_dep(V + ((size_t)b * D + k) * r + min(i, r - 1)), v = i < r ? x : 0.f;
     const __nv_bfloat16 hi = __float2bfloat16_rn(v);
     const __nv_bfloat16 lo = __float2bfloat16_rn(v - __bfloat162float(hi));
     const uint32_t off = (uint32_t)(k / 64) * v_tile + ptx::swz128(i, (k % 64) / 8) + (k % 8) * 2;
@@ -143,6 +151,10 @@ project_us_umma_kernel(const __grid_constant__ CUtensorMap tmap, const float* __
     // ---- epilogue warps: accumulator row tid -> bf16 -> US[b, n, 0:r] ------------------
     const uint32_t lane_base = (uint32_t)(warp * 32) << 16;
     const bool vec = (r % 8) == 0 && (reinterpret_cast<uintptr_t>(US) & 15) == 0;   // rows start on 16-byte boundaries
+    // the warp's 32 rows, contiguous in global memory, pass through shared memory (odd pitch in 16-byte
+    // pieces: no bank conflicts) so that they leave in whole lines
+    const int pieces = r / 8, pitch = pieces | 1;
+    uint4* sO = reinterpret_cast<uint4*>(sV + 2 * Cfg::KB * v_tile) + warp * 32 * pitch;
     int t = 0;
     for (; t < ntiles; ++t) {
       const int a = t & 1;
@@ -159,22 +171,28 @@ project_us_umma_kernel(const __grid_constant__ CUtensorMap tmap, const float* __
           ptx::tc_fence_before_sync();
           ptx::mbar_arrive(&acc_free[a]);
         }
-        if (n < N) {
-          if (vec) {
-            uint4* o4 = reinterpret_cast<uint4*>(o + c0);
+        if (vec) {
 #pragma unroll
-            for (int c = 0; c < 4; ++c)
-              if (c0 + 8 * c < r)
-                o4[c] = make_uint4(ptx::pack_bf16(__uint_as_float(v[8 * c]), __uint_as_float(v[8 * c + 1])),
-                                   ptx::pack_bf16(__uint_as_float(v[8 * c + 2]), __uint_as_float(v[8 * c + 3])),
-                                   ptx::pack_bf16(__uint_as_float(v[8 * c + 4]), __uint_as_float(v[8 * c + 5])),
-                                   ptx::pack_bf16(__uint_as_float(v[8 * c + 6]), __uint_as_float(v[8 * c + 7])));
-          } else {
+          for (int c = 0; c < 4; ++c)
+            if (c0 + 8 * c < r)
+              sO[lane * pitch + c0 / 8 + c] =
+                  make_uint4(ptx::pack_bf16(__uint_as_float(v[8 * c]), __uint_as_float(v[8 * c + 1])),
+                             ptx::pack_bf16(__uint_as_float(v[8 * c + 2]), __uint_as_float(v[8 * c + 3])),
+                             ptx::pack_bf16(__uint_as_float(v[8 * c + 4]), __uint_as_float(v[8 * c + 5])),
+                             ptx::pack_bf16(__uint_as_float(v[8 * c + 6]), __uint_as_float(v[8 * c + 7])));
+        } else if (n < N) {
 #pragma unroll
-            for (int i = 0; i < 32; ++i)
-              if (c0 + i < r) o[c0 + i] = __float2bfloat16_rn(__uint_as_float(v[i]));
-          }
+          for (int i = 0; i < 32; ++i)
+            if (c0 + i < r) o[c0 + i] = __float2bfloat16_rn(__uint_as_float(v[i]));
         }
+      }
+      if (vec) {
+        __syncwarp();
+        const int n0 = row0 + t * kTileRows + warp * 32, count = min(32, N - n0) * pieces;    // <= 0 past the end
+        uint4* dst = reinterpret_cast<uint4*>(US + ((size_t)b * N + min(n0, N - 1)) * r);
+#pragma unroll 4
+        for (int e = lane; e < count; e += 32) dst[e] = sO[(e / pieces) * pitch + e % pieces];
+        __syncwarp();
       }
     }
     // a wait ran out: the rows that were not produced read as NaN
@@ -190,21 +208,18 @@ project_us_umma_kernel(const __grid_constant__ CUtensorMap tmap, const float* __
 }
 
 template <int D>
-cudaError_t launch_d(int B, int N, int r, const void* H, const float* V, void* US, cudaStream_t st) {
+cudaError_t launch_d(int B, int N, int r, const void* H, const float* V, void* US, bool early_h, cudaStream_t st) {
   using Cfg = UsCfg<D>;
   const GramPlan plan = slice_plan(B, N);
   CUtensorMap tmap;
   if (!encode_tmap_bf16_3d(&tmap, H, D, (uint64_t)N, (uint64_t)B, (uint64_t)D * 2, (uint64_t)N * D * 2, 64,
                            kTileRows))
     return cudaErrorInvalidValue;
-  const size_t smem = Cfg::smem((r + 15) & ~15);
-  cudaError_t e = cudaFuncSetAttribute(project_us_umma_kernel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)Cfg::smem(kMaxCols));
+  static bool limits_set[kMaxDevicesCached] = {};
+  const cudaError_t e = set_kernel_limits(reinterpret_cast<const void*>(&project_us_umma_kernel<D>), Cfg::smem(kMaxCols), limits_set);
   if (e != cudaSuccess) return e;
-  const dim3 grid(plan.splits, B), block(kThreads);
-  project_us_umma_kernel<D><<<grid, block, smem, st>>>(tmap, V, static_cast<__nv_bfloat16*>(US), N, r,
-                                                           plan.chunk_tiles * kTileRows);
-  return cudaGetLastError();
+  return launch_pdl(project_us_umma_kernel<D>, dim3(plan.splits, B), dim3(kThreads), Cfg::smem((r + 15) & ~15), st, tmap, V,
+                    static_cast<__nv_bfloat16*>(US), N, r, plan.chunk_tiles * kTileRows, (int)early_h);
 }
 
 }  // namespace
@@ -214,8 +229,8 @@ bool project_us_umma_supported(int N, int d, int r, solar_dtype_t dt) {
 }
 
 cudaError_t launch_project_us_umma(int B, int N, int d, int r, const void* H, const float* V, void* US,
-                                   cudaStream_t st) {
-  return d == 64 ? launch_d<64>(B, N, r, H, V, US, st) : launch_d<128>(B, N, r, H, V, US, st);
+                                   bool early_h, cudaStream_t st) {
+  return d == 64 ? launch_d<64>(B, N, r, H, V, US, early_h, st) : launch_d<128>(B, N, r, H, V, US, early_h, st);
 }
 
 }  // namespace solar

@@ -143,7 +143,7 @@ solar_status_t solar_project_us(int B, int N, int d, int r, solar_dtype_t dt, co
   SOLAR_TRY(check_ptr(H));
   SOLAR_TRY(check_ptr(V));
   SOLAR_TRY(check_ptr(US));
-  return from_cuda(launch_project_us(B, N, d, r, dt, H, V, US, static_cast<cudaStream_t>(stream)));
+  return from_cuda(launch_project_us(B, N, d, r, dt, H, V, US, false, static_cast<cudaStream_t>(stream)));
 }
 
 solar_status_t solar_lowrank_factor(int B, int M, int N, int d, int r, solar_dtype_t dt,
@@ -160,7 +160,7 @@ solar_status_t solar_lowrank_factor(int B, int M, int N, int d, int r, solar_dty
   SOLAR_TRY(check_ws(workspace, workspace_bytes, factor_ws_bytes(B, N, d, dt)));
   SOLAR_TRY(solar_gram_partials(B, N, d, dt, H, workspace, workspace_bytes, stream));
   SOLAR_TRY(solar_eig_from_partials(B, N, d, r, dt, S, V, info, workspace, workspace_bytes, stream));
-  if (US != nullptr) SOLAR_TRY(solar_project_us(B, N, d, r, dt, H, V, US, stream));
+  if (US != nullptr) SOLAR_TRY(from_cuda(launch_project_us(B, N, d, r, dt, H, V, US, true, static_cast<cudaStream_t>(stream))));
   return SOLAR_OK;
 }
 
@@ -312,7 +312,7 @@ solar_status_t solar_svd_backward(int B, int N, int d, int r, solar_dtype_t dt, 
   float* K = static_cast<float*>(workspace);
   SOLAR_TRY(from_cuda(launch_svd_grad(B, d, r, S, V, dS, dV, eps_rel, K, st)));
   // dH_b = H_b K_b: the right-multiplication kernel of the left factor, with q = d columns
-  return from_cuda(launch_project_us(B, N, d, d, dt, H, K, dH, st));
+  return from_cuda(launch_project_us(B, N, d, d, dt, H, K, dH, true, st));
 }
 
 solar_status_t solar_factored_softmax_attention_fwd(int B, int M, int N, int d, int r, solar_dtype_t dt,

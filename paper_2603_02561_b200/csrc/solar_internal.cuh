@@ -209,7 +209,7 @@ cudaError_t launch_eig_tridiag(int B, int d, int r, solar_dtype_t dt, int route,
                                cudaStream_t st);
 int eig_subspace_dim(int d, int r);
 cudaError_t launch_project_us(int B, int N, int d, int r, solar_dtype_t dt, const void* H,
-                              const float* V, void* US, cudaStream_t st);
+                              const float* V, void* US, bool early_h, cudaStream_t st);
 cudaError_t launch_svd_grad(int B, int d, int r, const float* S, const float* V, const float* dS,
                             const float* dV, float eps_rel, float* K, cudaStream_t st);
 cudaError_t launch_attn_bwd(int B, int M, int d, int r, solar_dtype_t dt, const void* C, const void* dO,
@@ -223,7 +223,7 @@ cudaError_t launch_attn_bwd_umma(int B, int M, int d, int r, const void* C, cons
                                  const AttnWs& lay, cudaStream_t st);
 bool project_us_umma_supported(int N, int d, int r, solar_dtype_t dt);
 cudaError_t launch_project_us_umma(int B, int N, int d, int r, const void* H, const float* V, void* US,
-                                   cudaStream_t st);
+                                   bool early_h, cudaStream_t st);
 // bwd_pk: also the backward kernel's operands [B][4][64][d] (tensor-core shapes), or nullptr; f32: also the
 // fp32 copies where only the backward pass or a caller of the stage would read them
 cudaError_t launch_attn_prepare(int B, int d, int r, solar_dtype_t dt, const float* S,

@@ -201,18 +201,24 @@ def factored_softmax_attention_fwd(C, US, V, Wq, Wk, Wv, scale, O=None, workspac
     the factors (US[B,N,r] = H V from lowrank_factor, V[B,d,r])."""
     B, M, d = C.shape
     N, r = US.shape[1], US.shape[2]
-    _need(C, (B, M, d), C.dtype, "C"); _need(US, (B, N, r), C.dtype, "US")
-    _need(V, (B, d, r), torch.float32, "V")
-    for nm, W in (("Wq", Wq), ("Wk", Wk), ("Wv", Wv)):
-        _need(W, (d, d), C.dtype, nm)
-    O = torch.empty_like(C) if O is None else O
-    _need(O, (B, M, d), C.dtype, "O")
+    dt, dd = C.dtype, (d, d)
+    _need(C, (B, M, d), dt, "C")
+    _need(US, (B, N, r), dt, "US")
+    _need(V, (B, d, r), _F32, "V")
+    _need(Wq, dd, dt, "Wq")
+    _need(Wk, dd, dt, "Wk")
+    _need(Wv, dd, dt, "Wv")
+    if O is None:
+        O = _empty((B, M, d), dtype=dt, device=C.device)
+    else:
+        _need(O, (B, M, d), dt, "O")
     if workspace is None:
-        workspace = alloc_workspace(B, M, N, d, r, C.dtype, C.device)
-    st = lib().solar_factored_softmax_attention_fwd(B, M, N, d, r, dtype_code(C.dtype), _ptr(C), _ptr(US),
-                                                    _ptr(V), _ptr(Wq), _ptr(Wk), _ptr(Wv), float(scale),
-                                                    _ptr(O), _ptr(workspace), workspace.numel(), _stream(stream))
-    _check(st, "solar_factored_softmax_attention_fwd")
+        workspace = alloc_workspace(B, M, N, d, r, dt, C.device)
+    st = (_lib or lib()).solar_factored_softmax_attention_fwd(
+        B, M, N, d, r, dtype_code(dt), C.data_ptr(), US.data_ptr(), V.data_ptr(), Wq.data_ptr(), Wk.data_ptr(),
+        Wv.data_ptr(), float(scale), O.data_ptr(), workspace.data_ptr(), workspace.numel(), _stream(stream))
+    if st:
+        _check(st, "solar_factored_softmax_attention_fwd")
     return O
 
 
@@ -277,9 +283,10 @@ def alloc_backward_workspace(B, M, N, d, r, dtype, device="cuda") -> torch.Tenso
 def alloc_attention_grads(C, r):
     """Output tensors of svd_attention_bwd: dC, dWq, dWk, dWv, dS, dV."""
     B, M, d = C.shape
-    dev = C.device
-    return (torch.empty_like(C), *(torch.empty(d, d, dtype=torch.float32, device=dev) for _ in range(3)),
-            torch.empty(B, r, dtype=torch.float32, device=dev), torch.empty(B, d, r, dtype=torch.float32, device=dev))
+    dev, dd = C.device, (d, d)
+    return (_empty((B, M, d), dtype=C.dtype, device=dev), _empty(dd, dtype=_F32, device=dev),
+            _empty(dd, dtype=_F32, device=dev), _empty(dd, dtype=_F32, device=dev),
+            _empty((B, r), dtype=_F32, device=dev), _empty((B, d, r), dtype=_F32, device=dev))
 
 
 def svd_attention_bwd(C, S, V, Wq, Wk, Wv, scale, dO, workspace, flags=0, out=None, stream=None):
@@ -287,16 +294,25 @@ def svd_attention_bwd(C, S, V, Wq, Wk, Wv, scale, dO, workspace, flags=0, out=No
     Returns dC[B,M,d], dWq, dWk, dWv [d,d] f32, dS[B,r], dV[B,d,r] (written into `out` if given)."""
     B, M, d = C.shape
     r = S.shape[1]
-    _need(dO, (B, M, d), C.dtype, "dO")
-    dC, dWq, dWk, dWv, dS, dV = alloc_attention_grads(C, r) if out is None else out
-    _need(dC, (B, M, d), C.dtype, "dC"); _need(dS, (B, r), torch.float32, "dS"); _need(dV, (B, d, r), torch.float32, "dV")
-    for nm, W in (("dWq", dWq), ("dWk", dWk), ("dWv", dWv)):
-        _need(W, (d, d), torch.float32, nm)
-    _check(lib().solar_svd_attention_bwd(B, M, max(r, 1), d, r, dtype_code(C.dtype), _ptr(C), _ptr(S), _ptr(V),
-                                         _ptr(Wq), _ptr(Wk), _ptr(Wv), float(scale), int(flags), _ptr(dO),
-                                         _ptr(dC), _ptr(dWq), _ptr(dWk), _ptr(dWv), _ptr(dS), _ptr(dV),
-                                         _ptr(workspace), workspace.numel(), _stream(stream)),
-           "solar_svd_attention_bwd")
+    dt = C.dtype
+    _need(dO, (B, M, d), dt, "dO")
+    if out is None:
+        out = alloc_attention_grads(C, r)
+        dC, dWq, dWk, dWv, dS, dV = out
+    else:
+        dC, dWq, dWk, dWv, dS, dV = out
+        _need(dC, (B, M, d), dt, "dC")
+        _need(dS, (B, r), _F32, "dS")
+        _need(dV, (B, d, r), _F32, "dV")
+        for nm, W in (("dWq", dWq), ("dWk", dWk), ("dWv", dWv)):
+            _need(W, (d, d), _F32, nm)
+    st = (_lib or lib()).solar_svd_attention_bwd(
+        B, M, r if r > 1 else 1, d, r, dtype_code(dt), C.data_ptr(), S.data_ptr(), V.data_ptr(), Wq.data_ptr(),
+        Wk.data_ptr(), Wv.data_ptr(), float(scale), int(flags), dO.data_ptr(), dC.data_ptr(), dWq.data_ptr(),
+        dWk.data_ptr(), dWv.data_ptr(), dS.data_ptr(), dV.data_ptr(), workspace.data_ptr(), workspace.numel(),
+        _stream(stream))
+    if st:
+        _check(st, "solar_svd_attention_bwd")
     return dC, dWq, dWk, dWv, dS, dV
 
 
@@ -304,9 +320,11 @@ def svd_backward(H, S, V, dS, dV, dH, workspace, eps_rel=0.0, stream=None):
     """dH = U [diag(dS) + 2 Sigma sym(F o (dV^T V))] V^T with U = H V Sigma^-1 (Eq. 13-15)."""
     B, N, d = H.shape
     r = V.shape[2]
-    _check(lib().solar_svd_backward(B, N, d, r, dtype_code(H.dtype), _ptr(H), _ptr(S), _ptr(V), _ptr(dS),
-                                    _ptr(dV), float(eps_rel), _ptr(dH), _ptr(workspace), workspace.numel(),
-                                    _stream(stream)), "solar_svd_backward")
+    st = (_lib or lib()).solar_svd_backward(B, N, d, r, dtype_code(H.dtype), H.data_ptr(), S.data_ptr(), V.data_ptr(),
+                                            dS.data_ptr(), dV.data_ptr(), float(eps_rel), dH.data_ptr(),
+                                            workspace.data_ptr(), workspace.numel(), _stream(stream))
+    if st:
+        _check(st, "solar_svd_backward")
 
 
 def attn_prepare(S, V, Wq, Wk, Wv, scale, workspace, stream=None):
