@@ -12,6 +12,9 @@
 //        the SAME shared-memory tiles read as MN-major operands (K = the 128 rows), both
 //        accumulating in tensor memory across the tiles of the chunk
 //   tcgen05.ld: dC -> bf16 -> shared memory -> TMA store
+// Bound by latency (a chain of loads, two rounds of GEMMs and the softmax per tile): what helps is two
+// CTAs per SM, which the 97 KB of r <= 32 at d = 64 allow since P and dS have 64-byte rows there (130 KB with
+// 128-byte rows: 16 x 2048 candidates took 17.8 us in two waves of CTAs, 12.9 in one now).
 // At the end the two accumulators go to the chunk's partial in the workspace.  Scores and
 // probabilities never leave the SM.  Every wait is bounded; if one runs out, the chunk's
 // dC rows and its partial are written as NaN.
@@ -32,9 +35,10 @@ template <int D> struct BwdCfg {
   static constexpr int TILE_BYTES = KB * kBoxBytes;                 // C, dO, dC tiles
   __host__ __device__ static constexpr int tok_bytes(int np) { return 2 * KB * np * 128; }   // [2][KB][np][128 B]
   static constexpr int TK_BYTES = 2 * D * 128;                      // T hi/lo as [2][D rows][128 B]
-  static constexpr int PD_BYTES = 2 * kBoxBytes;                    // P or dS, hi/lo
+  // P or dS, hi/lo halves: rows of 64 bytes (32 tokens, 64-byte swizzle) when np <= 32, else of 128
+  __host__ __device__ static constexpr int pd_half(int np) { return np <= 32 ? kBoxBytes / 2 : kBoxBytes; }
   static constexpr size_t smem(int np) {
-    return (size_t)2 * TILE_BYTES + 2 * tok_bytes(np) + TK_BYTES + 2 * PD_BYTES + 1024;
+    return (size_t)2 * TILE_BYTES + 2 * tok_bytes(np) + TK_BYTES + 4 * pd_half(np) + 1024;
   }
 };
 
@@ -70,8 +74,10 @@ attn_bwd_umma_kernel(const __grid_constant__ CUtensorMap tmC, const __grid_const
   uint8_t* sT = sG + Cfg::TILE_BYTES;          // [2][KB][np][128 B]  T^T hi/lo       (B of S = C T)
   uint8_t* sVk = sT + Cfg::tok_bytes(np);      // [2][KB][np][128 B]  Value_r hi/lo   (B of dP = dO Value_r^T)
   uint8_t* sTk = sVk + Cfg::tok_bytes(np);     // [2][D][128 B]       T hi/lo         (B of dC = dS T^T)
-  uint8_t* sP = sTk + Cfg::TK_BYTES;           // [2][128][128 B]     P hi/lo
-  uint8_t* sD = sP + Cfg::PD_BYTES;            // [2][128][128 B]     dS hi/lo
+  uint8_t* sP = sTk + Cfg::TK_BYTES;           // [2][128][128 B or 64 B]  P hi/lo
+  const int pd = Cfg::pd_half(np);             // bytes of one half of P or dS
+  const bool narrow = np <= 32;
+  uint8_t* sD = sP + 2 * pd;                   // [2][128][128 B or 64 B]  dS hi/lo
   __shared__ __align__(8) uint64_t bar_ops, bar_load, bar_s, bar_o;
   __shared__ uint32_t s_tmem;
   __shared__ int s_err;
@@ -222,12 +228,13 @@ attn_bwd_umma_kernel(const __grid_constant__ CUtensorMap tmC, const __grid_const
 #pragma unroll
         for (int c = 0; c < 4; ++c) {
           uint4 hi, lo;
+          const uint32_t off = narrow ? ptx::swz64(tid, c) : ptx::swz128(tid, c0 / 8 + c);
           split8(&p[c0 + 8 * c], hi, lo);
-          *reinterpret_cast<uint4*>(sP + ptx::swz128(tid, c0 / 8 + c)) = hi;
-          *reinterpret_cast<uint4*>(sP + kBoxBytes + ptx::swz128(tid, c0 / 8 + c)) = lo;
+          *reinterpret_cast<uint4*>(sP + off) = hi;
+          *reinterpret_cast<uint4*>(sP + pd + off) = lo;
           split8(&dsv[8 * c], hi, lo);
-          *reinterpret_cast<uint4*>(sD + ptx::swz128(tid, c0 / 8 + c)) = hi;
-          *reinterpret_cast<uint4*>(sD + kBoxBytes + ptx::swz128(tid, c0 / 8 + c)) = lo;
+          *reinterpret_cast<uint4*>(sD + off) = hi;
+          *reinterpret_cast<uint4*>(sD + pd + off) = lo;
         }
       }
     }
@@ -244,10 +251,10 @@ attn_bwd_umma_kernel(const __grid_constant__ CUtensorMap tmC, const __grid_const
           bool acc = false;
 #pragma unroll
           for (int term = 0; term < 3; ++term) {
-            const uint32_t a = ptx::smem_u32(sD) + (term == 2 ? kBoxBytes : 0);
+            const uint32_t a = ptx::smem_u32(sD) + (term == 2 ? pd : 0);
             const uint32_t bb = ptx::smem_u32(sTk) + (term == 1 ? D * 128 : 0);
             for (int kk = 0; kk < np / 16; ++kk) {
-              ptx::umma_bf16_ss(tmem + kColS, ptx::umma_smem_desc(a + kk * 32, 0, 1024),
+              ptx::umma_bf16_ss(tmem + kColS, ptx::umma_smem_desc_sw(a + kk * 32, 0, narrow ? 512 : 1024, narrow ? 4 : 2),
                                 ptx::umma_smem_desc(bb + kk * 32, 0, 1024), idesc, acc);
               acc = true;
             }
@@ -266,7 +273,8 @@ attn_bwd_umma_kernel(const __grid_constant__ CUtensorMap tmC, const __grid_const
               for (int ks = 0; ks < kRows / 16; ++ks) {
                 // 16 rows = two 8-row swizzle atoms of 1024 B; 64-column boxes are kBoxBytes apart
                 const uint64_t ad = ptx::umma_smem_desc(abase + ks * 2048, kBoxBytes, 1024);
-                const uint64_t bd = ptx::umma_smem_desc(bbase + h * kBoxBytes + ks * 2048, kBoxBytes, 1024);
+                const uint64_t bd = narrow ? ptx::umma_smem_desc_sw(bbase + h * pd + ks * 1024, 0, 512, 4)
+                                           : ptx::umma_smem_desc(bbase + h * pd + ks * 2048, kBoxBytes, 1024);
                 ptx::umma_bf16_ss(tmem + (g == 0 ? kColT : kColV), ad, bd, idesc, (it | h | ks) != 0);
               }
           }

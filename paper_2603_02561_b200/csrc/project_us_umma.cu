@@ -10,10 +10,10 @@
 // issues tcgen05.mma with the tile as the K-major A operand (M = 128 rows, K = d) and
 // X^T, split into a high and a low bf16 half, as the K-major B operand, into one of two
 // accumulators in tensor memory; warps 0-3 read the finished accumulator (one row per
-// thread), round to bf16 and store the rows, while the next tile is being multiplied
+// thread), round to bf16 and store the rows by TMA, while the next tile is being multiplied
 // into the other accumulator.  H is read from HBM once and never passes through registers.
 // Bound by HBM.  16 x 10240 x 64: q = 64 19.4 us with every thread storing its own row (32 lines per
-// instruction), 17.9 through shared memory; q = 32 13.5 and 12.4.
+// instruction) and X^T packed element by element, 13.5 now; q = 32 13.5 and 10.3.
 #include "sm100_ptx.cuh"
 #include "solar_internal.cuh"
 
@@ -31,16 +31,17 @@ template <int D> struct UsCfg {
   static constexpr int BOX_BYTES = kTileRows * 128;          // 16 KB: 128 rows x 64 bf16
   static constexpr int TILE_BYTES = KB * BOX_BYTES;
   static constexpr int STAGES = (D == 64) ? 6 : 3;
-  // ring + X^T as [2 halves][KB][np rows][128 B] + the output rows at odd 16-byte pitch + slack to align to 1024
+  // ring + X^T as [2 halves][KB][np rows][128 B] + two output tiles + slack to align to 1024
   static constexpr size_t smem(int np) {
-    return (size_t)STAGES * TILE_BYTES + (size_t)2 * KB * np * 128 + (size_t)kTileRows * (np / 8 + 1) * 16 + 1024;
+    return (size_t)STAGES * TILE_BYTES + ((size_t)2 * KB * np * 128 + 1023) / 1024 * 1024 + (size_t)2 * kTileRows * np * 2 + 1024;
   }
 };
 
 // byte offset of 16-byte chunk c of row `row` in a [rows][128 B] tile with the 128-byte swizzle
 template <int D>
 __global__ void __launch_bounds__(kThreads, 1)
-project_us_umma_kernel(const __grid_constant__ CUtensorMap tmap, const float* __restrict__ V,
+project_us_umma_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_constant__ CUtensorMap tmOut, int tma_out,
+                       const float* __restrict__ V,
                        __nv_bfloat16* __restrict__ US, int N, int r, int chunk_rows, int early_h) {
   // V is the per-user matrix X [D][r] and US the output [N][r]; r stands for q here.
   using Cfg = UsCfg<D>;
@@ -94,16 +95,26 @@ project_us_umma_kernel(const __grid_constant__ CUtensorMap tmap, const float* __
     for (int t = 0; t < primed; ++t) load_tile(t);
   if (early_h) pdl_wait();
 
-  // V^T as two K-major bf16 operands: row i (factor), K = k (feature); rows r .. np-1 zero
-#pragma unroll 8
-  for (int e = tid; e < np * D; e += kThreads) {
-    const int k = e / np, i = e - k * np;
-    const float x = ld_dep(V + ((size_t)b * D + k) * r + min(i, r - 1)), v = i < r ? x : 0.f;
-    const __nv_bfloat16 hi = __float2bfloat16_rn(v);
-    const __nv_bfloat16 lo = __float2bfloat16_rn(v - __bfloat162float(hi));
-    const uint32_t off = (uint32_t)(k / 64) * v_tile + ptx::swz128(i, (k % 64) / 8) + (k % 8) * 2;
-    *reinterpret_cast<__nv_bfloat16*>(sV + off) = hi;
-    *reinterpret_cast<__nv_bfloat16*>(sV + Cfg::KB * v_tile + off) = lo;
+  // V^T as two K-major bf16 operands: row i (factor), K = k (feature); rows r .. np-1 zero.  Eight features
+  // of a factor at a time, all loads of a thread before the first use.
+#pragma unroll 3
+  for (int e = tid; e < np * (D / 8); e += kThreads) {
+    const int kc = e / np, i = e - kc * np;
+    const float* src = V + ((size_t)b * D + 8 * kc) * r + min(i, r - 1);
+    float x[8];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) x[u] = ld_dep(src + (size_t)u * r);
+    uint32_t hi[4], lo[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const float x0 = i < r ? x[2 * q] : 0.f, x1 = i < r ? x[2 * q + 1] : 0.f;
+      const float h0 = __bfloat162float(__float2bfloat16_rn(x0)), h1 = __bfloat162float(__float2bfloat16_rn(x1));
+      hi[q] = ptx::pack_bf16(h0, h1);
+      lo[q] = ptx::pack_bf16(x0 - h0, x1 - h1);
+    }
+    uint8_t* dst = sV + (kc / 8) * v_tile + ptx::swz128(i, kc % 8);
+    *reinterpret_cast<uint4*>(dst) = make_uint4(hi[0], hi[1], hi[2], hi[3]);
+    *reinterpret_cast<uint4*>(dst + Cfg::KB * v_tile) = make_uint4(lo[0], lo[1], lo[2], lo[3]);
   }
   ptx::fence_proxy_async_smem();
   __syncthreads();
@@ -150,11 +161,10 @@ project_us_umma_kernel(const __grid_constant__ CUtensorMap tmap, const float* __
   } else {
     // ---- epilogue warps: accumulator row tid -> bf16 -> US[b, n, 0:r] ------------------
     const uint32_t lane_base = (uint32_t)(warp * 32) << 16;
-    const bool vec = (r % 8) == 0 && (reinterpret_cast<uintptr_t>(US) & 15) == 0;   // rows start on 16-byte boundaries
-    // the warp's 32 rows, contiguous in global memory, pass through shared memory (odd pitch in 16-byte
-    // pieces: no bank conflicts) so that they leave in whole lines
-    const int pieces = r / 8, pitch = pieces | 1;
-    uint4* sO = reinterpret_cast<uint4*>(sV + 2 * Cfg::KB * v_tile) + warp * 32 * pitch;
+    // A warp's 32 rows leave by TMA from one of its two staging buffers (r = 16, 32, 64 or 128: rows of a
+    // swizzle span, or two spans side by side); other widths are stored by the threads themselves.
+    const int span = r >= 64 ? 128 : 2 * r, boxes = r > 64 ? 2 : 1, rows_bytes = 32 * span;
+    uint8_t* sO = sV + (2 * Cfg::KB * v_tile + 1023) / 1024 * 1024 + warp * 2 * boxes * rows_bytes;
     int t = 0;
     for (; t < ntiles; ++t) {
       const int a = t & 1;
@@ -163,6 +173,11 @@ project_us_umma_kernel(const __grid_constant__ CUtensorMap tmap, const float* __
       ptx::tc_fence_after_sync();
       const int n = row0 + t * kTileRows + tid;
       __nv_bfloat16* o = US + ((size_t)b * N + (n < N ? n : 0)) * r;
+      uint8_t* buf = sO + a * boxes * rows_bytes;
+      if (tma_out) {                             // the store before the last has left this buffer
+        if (lane == 0) ptx::tma_store_wait_read_1();
+        __syncwarp();
+      }
       for (int c0 = 0; c0 < np; c0 += 32) {
         uint32_t v[32];
         ptx::tmem_ld_32x32(tmem + lane_base + a * acc_cols + c0, v);
@@ -171,30 +186,36 @@ project_us_umma_kernel(const __grid_constant__ CUtensorMap tmap, const float* __
           ptx::tc_fence_before_sync();
           ptx::mbar_arrive(&acc_free[a]);
         }
-        if (vec) {
+        if (tma_out) {
 #pragma unroll
           for (int c = 0; c < 4; ++c)
-            if (c0 + 8 * c < r)
-              sO[lane * pitch + c0 / 8 + c] =
+            if (c0 + 8 * c < r) {
+              const int ch = (c0 % 64) / 8 + c;
+              const uint32_t off = span == 128 ? ptx::swz128(lane, ch) : span == 64 ? ptx::swz64(lane, ch) : ptx::swz32(lane, ch);
+              *reinterpret_cast<uint4*>(buf + (c0 / 64) * rows_bytes + off) =
                   make_uint4(ptx::pack_bf16(__uint_as_float(v[8 * c]), __uint_as_float(v[8 * c + 1])),
                              ptx::pack_bf16(__uint_as_float(v[8 * c + 2]), __uint_as_float(v[8 * c + 3])),
                              ptx::pack_bf16(__uint_as_float(v[8 * c + 4]), __uint_as_float(v[8 * c + 5])),
                              ptx::pack_bf16(__uint_as_float(v[8 * c + 6]), __uint_as_float(v[8 * c + 7])));
+            }
         } else if (n < N) {
 #pragma unroll
           for (int i = 0; i < 32; ++i)
             if (c0 + i < r) o[c0 + i] = __float2bfloat16_rn(__uint_as_float(v[i]));
         }
       }
-      if (vec) {
+      if (tma_out) {
+        ptx::fence_proxy_async_smem();
         __syncwarp();
-        const int n0 = row0 + t * kTileRows + warp * 32, count = min(32, N - n0) * pieces;    // <= 0 past the end
-        uint4* dst = reinterpret_cast<uint4*>(US + ((size_t)b * N + min(n0, N - 1)) * r);
-#pragma unroll 4
-        for (int e = lane; e < count; e += 32) dst[e] = sO[(e / pieces) * pitch + e % pieces];
-        __syncwarp();
+        const int n0 = row0 + t * kTileRows + warp * 32;
+        if (lane == 0) {
+          if (n0 < N)                            // rows past N are clipped
+            for (int x = 0; x < boxes; ++x) ptx::tma_store_3d(&tmOut, buf + x * rows_bytes, x * 64, n0, b);
+          ptx::tma_store_commit();
+        }
       }
     }
+    if (tma_out && lane == 0) ptx::tma_store_wait_read();      // before the CTA's shared memory goes
     // a wait ran out: the rows that were not produced read as NaN
     for (; t < ntiles; ++t) {
       const int n = row0 + t * kTileRows + tid;
@@ -215,10 +236,17 @@ cudaError_t launch_d(int B, int N, int r, const void* H, const float* V, void* U
   if (!encode_tmap_bf16_3d(&tmap, H, D, (uint64_t)N, (uint64_t)B, (uint64_t)D * 2, (uint64_t)N * D * 2, 64,
                            kTileRows))
     return cudaErrorInvalidValue;
+  CUtensorMap tmOut = tmap;
+  const int span = r >= 64 ? 128 : 2 * r;                     // bytes of a box row
+  const bool tma_out = r == 16 || r == 32 || r == 64 || r == 128;
+  if (tma_out && !encode_tmap_bf16_3d_sw(&tmOut, US, r, (uint64_t)N, (uint64_t)B, (uint64_t)r * 2, (uint64_t)N * r * 2,
+                                         span / 2, 32, span))
+    return cudaErrorInvalidValue;
   static bool limits_set[kMaxDevicesCached] = {};
   const cudaError_t e = set_kernel_limits(reinterpret_cast<const void*>(&project_us_umma_kernel<D>), Cfg::smem(kMaxCols), limits_set);
   if (e != cudaSuccess) return e;
-  return launch_pdl(project_us_umma_kernel<D>, dim3(plan.splits, B), dim3(kThreads), Cfg::smem((r + 15) & ~15), st, tmap, V,
+  return launch_pdl(project_us_umma_kernel<D>, dim3(plan.splits, B), dim3(kThreads), Cfg::smem((r + 15) & ~15), st, tmap, tmOut,
+                    (int)tma_out, V,
                     static_cast<__nv_bfloat16*>(US), N, r, plan.chunk_tiles * kTileRows, (int)early_h);
 }
 

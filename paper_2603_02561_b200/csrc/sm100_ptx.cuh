@@ -105,6 +105,9 @@ __device__ __forceinline__ void tma_store_wait_all() { asm volatile("cp.async.bu
 // leave or reuse the buffer); the global writes complete on their own before the grid ends.
 __device__ __forceinline__ void tma_store_wait_read() { asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory"); }
 
+// The same with the youngest store still on its way (two buffers in turn).
+__device__ __forceinline__ void tma_store_wait_read_1() { asm volatile("cp.async.bulk.wait_group.read 1;" ::: "memory"); }
+
 // ---- tensor memory ---------------------------------------------------------------------
 // One full warp allocates `ncols` (power of two >= 32) columns; the base address lands in *dst.
 __device__ __forceinline__ void tmem_alloc(uint32_t* dst_smem, uint32_t ncols) {
@@ -191,6 +194,10 @@ __device__ __forceinline__ uint32_t swz128(int row, int c) {
 // XORed with bits 7-8, i.e. with row / 2).
 __device__ __forceinline__ uint32_t swz64(int row, int c) {
   return (uint32_t)row * 64u + (uint32_t)((c ^ ((row >> 1) & 3)) << 4);
+}
+// The same for a 32-byte-swizzled tile of 32-byte rows (2 chunks per row; bit 4 XORed with bit 7).
+__device__ __forceinline__ uint32_t swz32(int row, int c) {
+  return (uint32_t)row * 32u + (uint32_t)((c ^ ((row >> 2) & 1)) << 4);
 }
 // Two fp32 values rounded to bf16 (nearest even), `lo` in the low half of the word.
 __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
