@@ -3,10 +3,9 @@
 //   Value_r = (V Sigma)^T W_V   [r,d]
 // and the folded score operand T_b = scale * W_Q Key_r^T [d,r], so that the
 // scores of Eq. 12 are  scale * (C W_Q) Key_r^T = C T_b.
-// Written to the workspace in fp32 (for the FFMA attention kernel) and as packed bf16
-// operand images for the tensor-core attention kernel: T^T and Value_r^T, each split
-// into a high and a low bf16 half so that both GEMMs keep ~16 mantissa bits, zero padded
-// to 64 token slots.
+// Written to the workspace in fp32 for the FFMA attention kernels (fp32 storage, d = 32) and as packed
+// bf16 operand images for the tensor-core ones: T^T and Value_r^T, each split into a high and a low
+// bf16 half so that both GEMMs keep ~16 mantissa bits, zero padded to a multiple of 16 tokens.
 //
 // Two CTAs per user: one computes Key_r^T and T (W_K, W_Q), the other Value_r (W_V).
 // Each weight matrix is staged once in shared memory with coalesced 16-byte loads; the small
@@ -47,9 +46,6 @@ attn_prepare_kernel(const float* __restrict__ S, const float* __restrict__ V,
   char* wsb = ws + (size_t)b * lay.per_user;
   float* Tf = reinterpret_cast<float*>(wsb + lay.tf_off);
   float* Vr = reinterpret_cast<float*>(wsb + lay.vr_off);
-  __nv_bfloat16* Tpk = reinterpret_cast<__nv_bfloat16*>(wsb + lay.tpk_off);
-  __nv_bfloat16* Vpk = reinterpret_cast<__nv_bfloat16*>(wsb + lay.vpk_off);
-  const __nv_bfloat16 zero = __float2bfloat16_rn(0.f);
 
   // S and V come from the eigensolver, the weights from the caller (a kernel earlier on the
   // stream may have written them), and the workspace may still be in use: nothing is read or
@@ -60,18 +56,6 @@ attn_prepare_kernel(const float* __restrict__ S, const float* __restrict__ V,
   for (int e = tid; e < D * rp; e += kPrepThreads) {
     const int k = e / rp, i = e % rp;
     VS[e] = i < r ? V[((size_t)b * D + k) * r + i] * (S != nullptr ? S[(size_t)b * r + i] : 1.f) : 0.f;
-  }
-  // zero padding of the packed operands: token slots r .. 63
-  if (role == 0) {
-    for (int e = tid; e < 2 * (kTokenSlots - r) * D; e += kPrepThreads) {
-      const int h = e / ((kTokenSlots - r) * D), rem = e % ((kTokenSlots - r) * D);
-      Tpk[((size_t)h * kTokenSlots + r) * D + rem] = zero;
-    }
-  } else {
-    for (int e = tid; e < 2 * D * (kTokenSlots - r); e += kPrepThreads) {
-      const int row = e / (kTokenSlots - r), i = r + e % (kTokenSlots - r);
-      Vpk[(size_t)row * kTokenSlots + i] = zero;      // row runs over [2][D]
-    }
   }
   __syncthreads();
   pdl_trigger();       // the next kernel may start launching while the products run
@@ -90,7 +74,6 @@ attn_prepare_kernel(const float* __restrict__ S, const float* __restrict__ V,
   };
 
   if (role == 1) {
-    // Value_r (fp32) and Value_r^T (packed bf16 halves)
     for (int t = tid; t < (rp / 4) * D; t += kPrepThreads) {
       const int j = t % D, i0 = (t / D) * 4;
       float acc[4];
@@ -98,12 +81,7 @@ attn_prepare_kernel(const float* __restrict__ S, const float* __restrict__ V,
 #pragma unroll
       for (int m = 0; m < 4; ++m) {
         const int i = i0 + m;
-        if (i < r) {
-          Vr[i * D + j] = acc[m];
-          const __nv_bfloat16 hi = __float2bfloat16_rn(acc[m]);
-          Vpk[(size_t)j * kTokenSlots + i] = hi;
-          Vpk[(size_t)(D + j) * kTokenSlots + i] = __float2bfloat16_rn(acc[m] - __bfloat162float(hi));
-        }
+        if (i < r) Vr[i * D + j] = acc[m];
       }
     }
     return;
@@ -131,13 +109,7 @@ attn_prepare_kernel(const float* __restrict__ S, const float* __restrict__ V,
 #pragma unroll
     for (int m = 0; m < 4; ++m) {
       const int i = i0 + m;
-      if (i < r) {
-        const float v = acc[m] * scale;
-        Tf[k * r + i] = v;
-        const __nv_bfloat16 hi = __float2bfloat16_rn(v);
-        Tpk[(size_t)i * D + k] = hi;
-        Tpk[((size_t)kTokenSlots + i) * D + k] = __float2bfloat16_rn(v - __bfloat162float(hi));
-      }
+      if (i < r) Tf[k * r + i] = acc[m] * scale;
     }
   }
 }

@@ -1178,70 +1178,15 @@ struct FuseArgs {
   char* ws;            // attention workspace (all users)
   AttnWs lay;
   int mode;            // 0: no epilogue; 1: weights are bf16; 2: weights are fp32
-  int write_f32;       // also write the fp32 copies T and Value_r (read by the FFMA attention kernel)
   int late_trigger;    // release the next kernel after the certificate instead of before the residuals
 };
 
-// Stages W[D][D] (bf16 or fp32 in global memory) as fp32 in shared memory, as it is or
-// transposed.  All loads of a thread are issued before the first store.
-template <int D, int NT, bool TRANSPOSE>
-__device__ __forceinline__ void stage_weight_any(const void* __restrict__ W, int mode, float* __restrict__ Ws,
-                                                 int tid) {
-  constexpr int NV = D * D / 8 / NT;              // 8-element pieces per thread
-  static_assert(NV * NT * 8 == D * D, "whole pieces");
-  float x[NV][8];
-  if (mode == 1) {
-    const uint4* w = static_cast<const uint4*>(W);
-    uint4 raw[NV];
-#pragma unroll
-    for (int n = 0; n < NV; ++n) raw[n] = __ldg(w + tid + n * NT);
-#pragma unroll
-    for (int n = 0; n < NV; ++n) {
-      const uint32_t u[4] = {raw[n].x, raw[n].y, raw[n].z, raw[n].w};
-#pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        x[n][2 * q] = __uint_as_float(u[q] << 16);
-        x[n][2 * q + 1] = __uint_as_float(u[q] & 0xffff0000u);
-      }
-    }
-  } else {
-    const float4* w = static_cast<const float4*>(W);
-#pragma unroll
-    for (int n = 0; n < NV; ++n) {
-      const float4 lo = __ldg(w + 2 * (tid + n * NT)), hi = __ldg(w + 2 * (tid + n * NT) + 1);
-      x[n][0] = lo.x; x[n][1] = lo.y; x[n][2] = lo.z; x[n][3] = lo.w;
-      x[n][4] = hi.x; x[n][5] = hi.y; x[n][6] = hi.z; x[n][7] = hi.w;
-    }
-  }
-#pragma unroll
-  for (int n = 0; n < NV; ++n) {
-    const int e0 = (tid + n * NT) * 8;            // element e0 = row * D + col
-    if (!TRANSPOSE) {
-      *reinterpret_cast<float4*>(Ws + e0) = make_float4(x[n][0], x[n][1], x[n][2], x[n][3]);
-      *reinterpret_cast<float4*>(Ws + e0 + 4) = make_float4(x[n][4], x[n][5], x[n][6], x[n][7]);
-    } else {
-      const int row = e0 / D, col = e0 % D;
-#pragma unroll
-      for (int u = 0; u < 8; ++u) Ws[(col + u) * D + row] = x[n][u];
-    }
-  }
-}
-
-// 16-byte pieces of a packed bf16 operand row: eight fp32 values as their high halves (h = 0)
-// or as what the high halves leave over (h = 1).
-__device__ __forceinline__ uint4 pack8_bf16(const float (&x)[8], int h) {
-  uint32_t w[4];
-#pragma unroll
-  for (int q = 0; q < 4; ++q) {
-    float a = x[2 * q], c = x[2 * q + 1];
-    if (h) {
-      a -= __bfloat162float(__float2bfloat16_rn(a));
-      c -= __bfloat162float(__float2bfloat16_rn(c));
-    }
-    const __nv_bfloat162 v = __floats2bfloat162_rn(a, c);
-    w[q] = *reinterpret_cast<const uint32_t*>(&v);
-  }
-  return make_uint4(w[0], w[1], w[2], w[3]);
+// Four consecutive elements of a weight matrix as fp32.
+__device__ __forceinline__ float4 weight4(const void* __restrict__ W, int mode, int e4) {
+  if (mode != 1) return ld_dep(static_cast<const float4*>(W) + e4);
+  const uint2 u = __ldg(static_cast<const uint2*>(W) + e4);
+  return make_float4(__uint_as_float(u.x << 16), __uint_as_float(u.x & 0xffff0000u), __uint_as_float(u.y << 16),
+                     __uint_as_float(u.y & 0xffff0000u));
 }
 
 // vs_ready: V Sigma of this user already lies at sm[0 .. D * rp) (pitch rp = r rounded up to 4,
@@ -1252,166 +1197,132 @@ __device__ __forceinline__ void prepare_epilogue(float* __restrict__ sm, int b, 
                                                  int tid) {
   const int rp = (r + 3) & ~3;          // token pitch: rows of VS / KrT are read 4 at a time
   float* VS = sm;                       // [D][rp]  V Sigma (zero in the padding)
-  float* KrT = VS + D * rp;             // [D][rp]  Key_r^T; later Value_r^T
-  float* W0 = KrT + D * rp;             // [D][D]   W_K, then W_V
-  float* W1 = W0 + D * D;               // [D][D]   W_Q^T; later T^T [r][D]
+  float* KrT = VS + D * rp;             // [D][rp]  Key_r^T
+  float* W0 = KrT + D * rp;             // [D][D]   W_K; later W_Q with row pitch D + 4
+  float* W1 = W0 + D * D;               // [D][D]   W_V
   char* wsb = fa.ws + (size_t)b * fa.lay.per_user;
-  float* Tf = reinterpret_cast<float*>(wsb + fa.lay.tf_off);
-  float* Vr = reinterpret_cast<float*>(wsb + fa.lay.vr_off);
-  __nv_bfloat16* Tpk = reinterpret_cast<__nv_bfloat16*>(wsb + fa.lay.tpk_off);
-  __nv_bfloat16* Vpk = reinterpret_cast<__nv_bfloat16*>(wsb + fa.lay.vpk_off);
-  const int nt4 = rp / 4;               // groups of four tokens
-  const int ntile = nt4 * (D / 4);      // 4 x 4 output tiles of each of the three products
-  constexpr int MAXT = 2;               // tiles per thread (kept in registers across a barrier)
-  const uint4 z4 = make_uint4(0u, 0u, 0u, 0u);
-
-  if (D >= 64 && fa.mode == 1 && !fa.write_f32) {
-    // bf16 weights: the three products on the tensor cores
-    if (!vs_ready) {
-      for (int e = tid; e < D * rp; e += NT) {
-        const int k = e / rp, i = e % rp;
-        VS[e] = i < r ? __ldcg(V + ((size_t)b * D + k) * r + i) * __ldcg(S + (size_t)b * r + i) : 0.f;
-      }
-      __syncthreads();
+  const bool mma = D >= 64 && fa.mode == 1;
+  if (!mma && fa.mode == 2) {
+#pragma unroll 4
+    for (int e = tid; e < D * D / 4; e += NT) {
+      cp_async16(W0 + 4 * e, static_cast<const float*>(fa.Wk) + 4 * e);
+      cp_async16(W1 + 4 * e, static_cast<const float*>(fa.Wv) + 4 * e);
     }
-    constexpr int DP = D >= 64 ? D : 64;
-    pmma::Weights<DP, NT, 3> w;
-    w.load(fa.Wq, fa.Wk, fa.Wv, tid);
-    pmma::project<DP, NT, 3>(reinterpret_cast<unsigned char*>(sm), r, w, fa.scale, pmma::Out{Tpk, Vpk, nullptr, nullptr, nullptr, nullptr}, tid);
-    return;
   }
-  stage_weight_any<D, NT, false>(fa.Wk, fa.mode, W0, tid);
-  stage_weight_any<D, NT, true>(fa.Wq, fa.mode, W1, tid);
-  if (!vs_ready)
+  if (!vs_ready) {
     for (int e = tid; e < D * rp; e += NT) {
       const int k = e / rp, i = e % rp;
       // written earlier by this CTA: read through the L2, not the non-coherent path
       VS[e] = i < r ? __ldcg(V + ((size_t)b * D + k) * r + i) * __ldcg(S + (size_t)b * r + i) : 0.f;
     }
-  // Zero padding of the packed operands, 16 bytes at a time.  The tensor-core attention kernel
-  // multiplies over np = 16 ceil(r / 16) token slots only (slots r .. r8-1, r8 = r rounded up to
-  // 8, are written as zeros with the data below); the FFMA kernels' callers want all 64.
-  const int r8 = (r + 7) & ~7;
-  const int pad_to = fa.write_f32 ? kTokenSlots : ((r + 15) & ~15);
-  for (int e = tid; e < 2 * (pad_to - r8) * (D / 8); e += NT) {
-    const int h = e / ((pad_to - r8) * (D / 8)), rem = e % ((pad_to - r8) * (D / 8));
-    reinterpret_cast<uint4*>(Tpk + ((size_t)h * kTokenSlots + r8) * D)[rem] = z4;
+    if (mma) __syncthreads();
   }
-  for (int e = tid; e < 2 * D * ((pad_to - r8) / 8); e += NT) {
-    const int row = e / ((pad_to - r8) / 8), c = e % ((pad_to - r8) / 8);
-    reinterpret_cast<uint4*>(Vpk + (size_t)row * kTokenSlots + r8)[c] = z4;      // row runs over [2][D]
+  if constexpr (D >= 64) {
+    if (mma) {
+      // bf16 weights: the three products on the tensor cores
+      pmma::Weights<D, NT, 3> w;
+      w.load(fa.Wq, fa.Wk, fa.Wv, tid);
+      pmma::project<D, NT, 3>(reinterpret_cast<unsigned char*>(sm), r, w, fa.scale,
+                              pmma::Out{reinterpret_cast<__nv_bfloat16*>(wsb + fa.lay.tpk_off),
+                                        reinterpret_cast<__nv_bfloat16*>(wsb + fa.lay.vpk_off), nullptr, nullptr, nullptr, nullptr}, tid);
+      return;
+    }
   }
+  // FFMA form (fp32 weights, d = 32): the fp32 operands of the FFMA attention kernel, T [D][r] and
+  // Value_r [r][D].  Bound by latency and issue of the CTA's four (eight) warps: Key_r and Value_r in one
+  // loop over the rows of V Sigma, W_Q on its way meanwhile and read by rows, not transposed, results
+  // straight from registers.  A pass over 16 x 5000 x 64 with r = 24 took 82.2 us with one product after the
+  // other and the packed operands (which only the tensor-core kernels read) written beside the fp32 ones,
+  // 76.9 now; one user of 256 x 32 with r = 8: 23.8 and 22.1.
+  float* Tf = reinterpret_cast<float*>(wsb + fa.lay.tf_off);
+  float* Vr = reinterpret_cast<float*>(wsb + fa.lay.vr_off);
+  const int nt4 = rp / 4;               // groups of four tokens
+  constexpr int CT = D == 32 ? 1 : 4;   // columns (rows of T) of a thread's tile: a small user still has work for the threads
+  constexpr int NV = D * D / 4 / NT, LQ = D + 4;
+  if (fa.mode == 1) {
+#pragma unroll
+    for (int n = 0; n < NV; ++n) {
+      reinterpret_cast<float4*>(W0)[tid + n * NT] = weight4(fa.Wk, 1, tid + n * NT);
+      reinterpret_cast<float4*>(W1)[tid + n * NT] = weight4(fa.Wv, 1, tid + n * NT);
+    }
+  }
+  float4 wq[NV];
+#pragma unroll
+  for (int n = 0; n < NV; ++n) wq[n] = weight4(fa.Wq, fa.mode, tid + n * NT);
+  cp_async_wait_all();
   __syncthreads();
-  // acc[a][c] = sum_k VS[k][i0 + a] W0[k][j0 + c]: a 4 x 4 tile per thread, two 16-byte reads per
-  // 16 FMAs, every output summed over k in ascending order
-  auto project = [&](float (&acc)[4][4], int i0, int j0) {
+  // Key_r and Value_r: every output summed over k in ascending order
+  for (int t = tid; t < nt4 * (D / CT); t += NT) {
+    const int j0 = (t % (D / CT)) * CT, i0 = (t / (D / CT)) * 4;
+    float ka[4][CT], va[4][CT];
 #pragma unroll
     for (int a = 0; a < 4; ++a)
 #pragma unroll
-      for (int c = 0; c < 4; ++c) acc[a][c] = 0.f;
+      for (int c = 0; c < CT; ++c) ka[a][c] = va[a][c] = 0.f;
 #pragma unroll 4
     for (int k = 0; k < D; ++k) {
-      const float4 w = *reinterpret_cast<const float4*>(W0 + k * D + j0);
-      const float4 v = *reinterpret_cast<const float4*>(VS + k * rp + i0);
-      const float ww[4] = {w.x, w.y, w.z, w.w}, vv[4] = {v.x, v.y, v.z, v.w};
+      float v[4], wk[CT], wv[CT];
+      ld4(VS + k * rp + i0, v);
+      if constexpr (CT == 4) {
+        ld4(W0 + k * D + j0, wk);
+        ld4(W1 + k * D + j0, wv);
+      } else {
+        wk[0] = W0[k * D + j0];
+        wv[0] = W1[k * D + j0];
+      }
 #pragma unroll
       for (int a = 0; a < 4; ++a)
 #pragma unroll
-        for (int c = 0; c < 4; ++c) acc[a][c] = fmaf(vv[a], ww[c], acc[a][c]);
+        for (int c = 0; c < CT; ++c) {
+          ka[a][c] = fmaf(v[a], wk[c], ka[a][c]);
+          va[a][c] = fmaf(v[a], wv[c], va[a][c]);
+        }
     }
-  };
-  // Key_r^T [j][i]
-  for (int t = tid; t < ntile; t += NT) {
-    const int j0 = (t % (D / 4)) * 4, i0 = (t / (D / 4)) * 4;
-    float acc[4][4];
-    project(acc, i0, j0);
 #pragma unroll
-    for (int c = 0; c < 4; ++c)
-      *reinterpret_cast<float4*>(KrT + (j0 + c) * rp + i0) = make_float4(acc[0][c], acc[1][c], acc[2][c], acc[3][c]);
-  }
-  __syncthreads();
-  // T[k][i] = scale * sum_j Wq[k][j] Key_r[i][j]: tile of four rows k and four tokens i; kept in
-  // registers until W_Q is done with, then laid down over it as T^T [i][D] (the packed rows)
-  float tacc[MAXT][4][4];
+    for (int c = 0; c < CT; ++c)
+      *reinterpret_cast<float4*>(KrT + (j0 + c) * rp + i0) = make_float4(ka[0][c], ka[1][c], ka[2][c], ka[3][c]);
 #pragma unroll
-  for (int n = 0; n < MAXT; ++n) {
-    const int t = tid + n * NT;
-#pragma unroll
-    for (int a = 0; a < 4; ++a)
-#pragma unroll
-      for (int c = 0; c < 4; ++c) tacc[n][a][c] = 0.f;
-    if (t < ntile) {
-      const int i0 = (t % nt4) * 4, k0 = (t / nt4) * 4;
-#pragma unroll 4
-      for (int j = 0; j < D; ++j) {
-        const float4 w = *reinterpret_cast<const float4*>(W1 + j * D + k0);      // W_Q[k0 ..][j]
-        const float4 kr = *reinterpret_cast<const float4*>(KrT + j * rp + i0);
-        const float ww[4] = {w.x, w.y, w.z, w.w}, kk[4] = {kr.x, kr.y, kr.z, kr.w};
-#pragma unroll
-        for (int a = 0; a < 4; ++a)
-#pragma unroll
-          for (int c = 0; c < 4; ++c) tacc[n][a][c] = fmaf(ww[a], kk[c], tacc[n][a][c]);
-      }
+    for (int a = 0; a < 4; ++a) {
+      if (i0 + a >= r) continue;
+      if constexpr (CT == 4) *reinterpret_cast<float4*>(Vr + (size_t)(i0 + a) * D + j0) = make_float4(va[a][0], va[a][1], va[a][2], va[a][3]);
+      else Vr[(size_t)(i0 + a) * D + j0] = va[a][0];
     }
   }
   __syncthreads();
-  stage_weight_any<D, NT, false>(fa.Wv, fa.mode, W0, tid);       // W_K is done with
 #pragma unroll
-  for (int n = 0; n < MAXT; ++n) {
-    const int t = tid + n * NT;
-    if (t < ntile) {
-      const int i0 = (t % nt4) * 4, k0 = (t / nt4) * 4;
+  for (int n = 0; n < NV; ++n) {
+    const int e = tid + n * NT;
+    *reinterpret_cast<float4*>(W0 + (e / (D / 4)) * LQ + (e % (D / 4)) * 4) = wq[n];
+  }
+  __syncthreads();
+  // T[k][i] = scale * sum_j Wq[k][j] Key_r[i][j]: rows k0 + (D / CT) x, four tokens i
+  for (int t = tid; t < nt4 * (D / CT); t += NT) {
+    const int i0 = (t % nt4) * 4, k0 = t / nt4;
+    float acc[CT][4];
+#pragma unroll
+    for (int x = 0; x < CT; ++x)
+#pragma unroll
+      for (int c = 0; c < 4; ++c) acc[x][c] = 0.f;
+#pragma unroll 2
+    for (int j = 0; j < D; j += 4) {
+      float w[CT][4], kr[4][4];
+#pragma unroll
+      for (int x = 0; x < CT; ++x) ld4(W0 + (k0 + x * (D / CT)) * LQ + j, w[x]);
+#pragma unroll
+      for (int u = 0; u < 4; ++u) ld4(KrT + (j + u) * rp + i0, kr[u]);
+#pragma unroll
+      for (int u = 0; u < 4; ++u)
+#pragma unroll
+        for (int x = 0; x < CT; ++x)
+#pragma unroll
+          for (int c = 0; c < 4; ++c) acc[x][c] = fmaf(w[x][u], kr[u][c], acc[x][c]);
+    }
+#pragma unroll
+    for (int x = 0; x < CT; ++x)
 #pragma unroll
       for (int c = 0; c < 4; ++c)
-        *reinterpret_cast<float4*>(W1 + (i0 + c) * D + k0) =
-            make_float4(tacc[n][0][c] * fa.scale, tacc[n][1][c] * fa.scale, tacc[n][2][c] * fa.scale,
-                        tacc[n][3][c] * fa.scale);
-    }
+        if (i0 + c < r) Tf[(size_t)(k0 + x * (D / CT)) * r + i0 + c] = acc[x][c] * fa.scale;
   }
-  __syncthreads();
-  // T^T out: 16-byte pieces of the packed rows (tokens r .. r8-1 are zero rows), and the fp32 copy
-  for (int e = tid; e < 2 * r8 * (D / 8); e += NT) {
-    const int h = e / (r8 * (D / 8)), rem = e % (r8 * (D / 8)), i = rem / (D / 8), c = rem % (D / 8);
-    const float4 lo = *reinterpret_cast<const float4*>(W1 + i * D + 8 * c);
-    const float4 hi = *reinterpret_cast<const float4*>(W1 + i * D + 8 * c + 4);
-    float x[8] = {lo.x, lo.y, lo.z, lo.w, hi.x, hi.y, hi.z, hi.w};
-    if (i >= r) {
-#pragma unroll
-      for (int u = 0; u < 8; ++u) x[u] = 0.f;
-    }
-    reinterpret_cast<uint4*>(Tpk + ((size_t)h * kTokenSlots + i) * D)[c] = pack8_bf16(x, h);
-  }
-  if (fa.write_f32)
-    for (int e = tid; e < D * r; e += NT) Tf[e] = W1[(e % r) * D + e / r];
-  // Value_r, kept in registers until Key_r^T is done with, then laid down over it as
-  // Value_r^T [j][rp] (the packed operand's rows)
-#pragma unroll
-  for (int n = 0; n < MAXT; ++n) {
-    const int t = tid + n * NT;
-    if (t < ntile) project(tacc[n], (t / (D / 4)) * 4, (t % (D / 4)) * 4);
-  }
-  __syncthreads();
-#pragma unroll
-  for (int n = 0; n < MAXT; ++n) {
-    const int t = tid + n * NT;
-    if (t < ntile) {
-      const int j0 = (t % (D / 4)) * 4, i0 = (t / (D / 4)) * 4;
-#pragma unroll
-      for (int c = 0; c < 4; ++c)
-        *reinterpret_cast<float4*>(KrT + (j0 + c) * rp + i0) =
-            make_float4(tacc[n][0][c], tacc[n][1][c], tacc[n][2][c], tacc[n][3][c]);
-    }
-  }
-  __syncthreads();
-  for (int e = tid; e < 2 * D * (r8 / 8); e += NT) {
-    const int h = e / (D * (r8 / 8)), rem = e % (D * (r8 / 8)), j = rem / (r8 / 8), c = rem % (r8 / 8);
-    float x[8];
-#pragma unroll
-    for (int u = 0; u < 8; ++u) x[u] = (8 * c + u < r) ? KrT[j * rp + 8 * c + u] : 0.f;
-    reinterpret_cast<uint4*>(Vpk + ((size_t)h * D + j) * kTokenSlots)[c] = pack8_bf16(x, h);
-  }
-  if (fa.write_f32)
-    for (int e = tid; e < r * D; e += NT) Vr[e] = KrT[(e % D) * rp + e / D];
 }
 
 template <int D, int RP>
@@ -1453,7 +1364,6 @@ cudaError_t launch_eig_tridiag(int B, int d, int r, solar_dtype_t dt, int route,
     fa.Wq = fuse->Wq; fa.Wk = fuse->Wk; fa.Wv = fuse->Wv; fa.scale = fuse->scale;
     fa.ws = fuse->attn_ws; fa.lay = attn_ws_layout(d, r);
     fa.mode = (dt == SOLAR_BF16) ? 1 : 2;
-    fa.write_f32 = !attn_umma_supported(d, dt);
     fa.late_trigger = slice_limit() > 0;
   }
   TriTol tol;
