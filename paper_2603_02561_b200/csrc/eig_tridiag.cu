@@ -34,9 +34,12 @@
 // directions), or the certificate fails, the CTA runs the same chain with steps 2-4 in fp64, where
 // the angle is eps_64 |T| / gap; the fp32 eigenvalues are its starting brackets.  Only what that
 // cannot certify either (vectors of equal eigenvalues) goes to the parallel Jacobi solve on the
-// whole matrix, which is valid for any spectrum.  Forward pass of 8 users, d = 128, r = 64 of a power
-// law (every user takes the fp64 chain): 3075 us with Jacobi in its place, 384 now; 64 users, d = r =
-// 64, one or none of them: 440 and 134 us.
+// whole matrix, which is valid for any spectrum.  Where SMs are idle (r > 32, few users) the user has two
+// CTAs, a cluster: one runs the fp32 chain, the other starts the fp64 chain at once; when the fp32
+// eigenvalues are there, the first either sends them across and leaves the user to the second, or sends
+// the second home.  Forward pass of 8 users, d = 128, r = 64 of a power
+// law (every user takes the fp64 chain): 3075 us with Jacobi in its place, 374 with the fp64 chain behind
+// the fp32 one, 281 beside it; 64 users, d = r = 64, one or none of them: 440, 148 and 112 us.
 //
 // What bounds it: the dependency chain (d steps of a matrix-vector product, an inner product and a
 // barrier, then the recurrences over the rows of T), not work or bandwidth: 16 users keep 16 of
@@ -187,6 +190,18 @@ __device__ __forceinline__ void cp_async16(float* dst, const float* src) {
 }
 __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 
+// Two CTAs for one user: which chain a CTA runs, and what the fp32 one tells the other.
+constexpr int kAlone = 0, kFp32Half = 1, kFp64Half = 2;
+constexpr int kNotNeeded = 1, kCarryOn = 2;
+__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
+// Store to the same place in the other CTA's shared memory.
+__device__ __forceinline__ void st_peer(void* local, uint32_t v, uint32_t rank) {
+  uint32_t remote;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(remote) : "r"((uint32_t)__cvta_generic_to_shared(local)), "r"(rank));
+  asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(remote), "r"(v) : "memory");
+}
+
 // What a thread carries through the Householder steps.
 template <typename T, int D, bool KEEP> struct TriState {
   using C = TriCfg<D>;
@@ -203,6 +218,7 @@ template <typename T> struct TriOut {
   T *dg, *eo, *yv, *xp;
   float *betas, *hv;
   float* stop;                  // [2] (0 or 1) for warps without unfinished rows: the reduction ended in the step before
+  const volatile int* verdict;  // fp64 beside an fp32 partner: what it says, looked at every eight steps; else nullptr
   int r;
 };
 
@@ -266,6 +282,7 @@ __device__ __forceinline__ void tri_stage(TriState<T, D, KEEP>& s, const TriOut<
     const int k1 = k + 1, par = k & 1, kc = k1 - CW * M;
     const T* const yv = o.yv + par * D;
     const T* const xp = o.xp + par * D;
+    if (F64 && o.verdict != nullptr && (k & 7) == 7 && __syncthreads_or(*o.verdict == kNotNeeded)) { s.k_stop = D; return; }
     __syncthreads();
     if (!KEEP && (warp + 1) * WR <= k1) {                    // only finished rows
       if (!F64 && *(volatile float*)(o.stop + par) != 0.f) { s.k_stop = k - 1; return; }
@@ -489,16 +506,18 @@ struct TriShared {
   float stop[2];
   int flags[4];
   int why;
+  int verdict;       // written by the other CTA of the user's pair
 };
 
 // Steps 2-7 in T for the user of this CTA; acc: the thread's tile of G in fp32.  Returns whether the
 // result is certified; Vc: where the vectors are ([D][RP]).  theta[] holds the eigenvalues of sc * G,
 // part[NW ..] the largest component of every vector per warp.  Without force, nothing is finished
-// that cannot be certified any more.
+// that cannot be certified any more.  With two CTAs for the user (half) `not_mine` comes back true where
+// the other one has the result.
 template <typename T, int D, int RP>
 __device__ __forceinline__ bool tri_chain(const float (&acc)[TriCfg<D>::RT][TriCfg<D>::NCH][4], float* __restrict__ smem,
                                           TriShared& sh, const float* __restrict__ gout, float sc, int r, bool force,
-                                          const TriTol& tol, bool trigger_early, float*& Vc_out, int& passes, int tid) {
+                                          const TriTol& tol, bool trigger_early, int half, bool& not_mine, float*& Vc_out, int& passes, int tid) {
   using C = TriCfg<D>;
   using L = TriSmem<D, RP>;
   constexpr int GX = C::GX, RT = C::RT, NT = C::NT, NW = C::NW, NCH = C::NCH, CW = C::CW, LD = C::LD;
@@ -514,6 +533,7 @@ __device__ __forceinline__ bool tri_chain(const float (&acc)[TriCfg<D>::RT][TriC
   float* const part = smem + L::PART;
   bool ok = true;
   passes = 0;
+  not_mine = false;
 
   // ---- 2. Householder tridiagonalisation, the matrix in registers ------------------------------
   int k_stop;
@@ -524,6 +544,7 @@ __device__ __forceinline__ bool tri_chain(const float (&acc)[TriCfg<D>::RT][TriC
     o.xp = reinterpret_cast<T*>(smem + L::XP);
     o.betas = smem + L::BE; o.hv = smem + L::R0;
     o.stop = sh.stop; o.r = r;
+    o.verdict = F64 && half == kFp64Half ? &sh.verdict : nullptr;
     TriState<T, D, KEEP> s;
     const float trs = (float)((double)sc * sh.trace);
     s.tr_rest = trs; s.tr_comp = 0.f;
@@ -577,6 +598,11 @@ __device__ __forceinline__ bool tri_chain(const float (&acc)[TriCfg<D>::RT][TriC
           for (int c = 0; c < 4; ++c) Qt[(CW * m + 4 * g + c) * LD + row0 + rr] = s.q[KEEP ? rr : 0][KEEP ? m : 0][c];
     }
     k_stop = s.k_stop;
+  }
+  if (F64 && half == kFp64Half) {            // the fp32 chain is long past its eigenvalues; they lie in lam32[]
+    cluster_arrive();
+    cluster_wait();
+    if (sh.verdict == kNotNeeded) { not_mine = true; return false; }
   }
   // T has `de` rows (all D unless the reduction stopped early), padded with zero rows to a multiple of 8
   const int de = k_stop >= 0 ? k_stop + 1 : D, de8 = (de + 7) & ~7;
@@ -662,7 +688,15 @@ __device__ __forceinline__ bool tri_chain(const float (&acc)[TriCfg<D>::RT][TriC
   __syncthreads();
   if (!F64) {                            // gaps too small for the angle the storage type needs
     const int tight = tid < r - 1 && (float)(lamv[tid] - lamv[tid + 1]) < tol.gap_min * (float)lamv[0];
-    if (__syncthreads_or(tight)) {
+    const bool gap = __syncthreads_or(tight);
+    if (half == kFp32Half) {
+      if (gap && tid < RP) st_peer(lam32 + tid, __float_as_uint(lam32[tid]), 1);
+      if (tid == 0) st_peer(&sh.verdict, gap ? kCarryOn : kNotNeeded, 1);
+      __syncwarp();
+      cluster_arrive();
+      not_mine = gap;
+    }
+    if (gap) {
       ok = false;
       if (tid == 0) sh.why |= kWhyGap;
       if (!force) return false;
@@ -992,11 +1026,12 @@ __device__ __forceinline__ bool tri_chain(const float (&acc)[TriCfg<D>::RT][TriC
   return ok;
 }
 
-// The eigensolve of user blockIdx.x; every thread of the CTA calls it and all leave together.
+// The eigensolve of user b; every thread of the CTA calls it and all leave together.
 // With want_vs, a certified tridiagonal result also leaves V Sigma at the start of the dynamic
-// shared memory ([D][rp], rp = r rounded up to 4, zero in the padding) and true is returned.
+// shared memory ([D][rp], rp = r rounded up to 4, zero in the padding).
+enum EigEnd { kEnded, kEndedVs, kOtherHalf };      // S and V written; V Sigma in shared memory too; the pair's other CTA does it
 template <int D, int RP>
-__device__ __forceinline__ bool eig_user(const float* __restrict__ gpart, const int* __restrict__ gram_status,
+__device__ __forceinline__ EigEnd eig_user(int b, int half, bool& joined, const float* __restrict__ gpart, const int* __restrict__ gram_status,
                                          int parts, int splits, float* __restrict__ gsum, int r, int route, int sweep_cap,
                                          const TriTol& tol, bool want_vs, bool late_trigger, float* __restrict__ S,
                                          float* __restrict__ V, int* __restrict__ info,
@@ -1006,10 +1041,17 @@ __device__ __forceinline__ bool eig_user(const float* __restrict__ gpart, const 
   constexpr int GX = C::GX, RT = C::RT, NT = C::NT, NW = C::NW, NCH = C::NCH, CW = C::CW, LD = C::LD, NE = RP / 32;
   extern __shared__ __align__(16) float smem[];
   __shared__ TriShared sh;
-  const int b = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int g = lane & (GX - 1), row0 = (tid / GX) * RT;
   float* const theta = smem + L::TH;
   float* const part = smem + L::PART;
+  joined = false;
+  if (half != kAlone) {
+    if (tid == 0) sh.verdict = 0;
+    __syncwarp();
+    cluster_arrive();
+    cluster_wait();
+  }
   pdl_wait();          // everything below reads what the Gram kernel wrote
 
   // ---- 1. G = sum of the slices' partial Grams, in a fixed order, in the registers' layout ---------
@@ -1072,7 +1114,7 @@ __device__ __forceinline__ bool eig_user(const float* __restrict__ gpart, const 
       for (int e = tid; e < r; e += NT) S[(size_t)b * r + e] = qnan;
       if (tid == 0 && info) info[b] = lost ? SOLAR_INFO_DEVICE_WAIT : SOLAR_INFO_NONFINITE;
       if (tid == 0 && route_taken) route_taken[b] = 0;
-      return false;
+      return half == kFp64Half ? kOtherHalf : kEnded;
     }
   }
   float gmax = 0.f;
@@ -1097,7 +1139,14 @@ __device__ __forceinline__ bool eig_user(const float* __restrict__ gpart, const 
   if (route != kRouteFull && gmax > 0.f) {
     float* Vc = nullptr;
     int passes = 0, wide = 0;            // wide: the fp64 chain gave the result
-    bool ok = tri_chain<float, D, RP>(acc, smem, sh, gout, sc, r, route == kRouteTridiag, tol, !late_trigger, Vc, passes, tid);
+    bool ok = false, not_mine = false;
+    if (half != kFp64Half) {
+      ok = tri_chain<float, D, RP>(acc, smem, sh, gout, sc, r, route == kRouteTridiag, tol, !late_trigger, half, not_mine, Vc, passes, tid);
+      joined = half != kAlone;
+      if (not_mine) return kOtherHalf;
+    } else if (tid == 0) {
+      sh.why = kWhyGap;
+    }
     if (!ok && route != kRouteTridiag) {
       __syncthreads();
 #pragma unroll
@@ -1105,7 +1154,8 @@ __device__ __forceinline__ bool eig_user(const float* __restrict__ gpart, const 
 #pragma unroll
         for (int m = 0; m < NCH; ++m) ld4(gout + (row0 + rr) * D + CW * m + 4 * g, acc[rr][m]);
       wide = 1;
-      ok = tri_chain<double, D, RP>(acc, smem, sh, gout, sc, r, false, tol, false, Vc, passes, tid);
+      ok = tri_chain<double, D, RP>(acc, smem, sh, gout, sc, r, false, tol, false, half, not_mine, Vc, passes, tid);
+      if (not_mine) return kOtherHalf;
     }
     if (ok || route == kRouteTridiag) {
       if (late_trigger || wide) pdl_trigger();
@@ -1149,10 +1199,11 @@ __device__ __forceinline__ bool eig_user(const float* __restrict__ gpart, const 
         if (info) info[b] = ok ? 0 : SOLAR_INFO_NOT_CERTIFIED;
         if (route_taken) route_taken[b] = (wide ? kRouteFull | (kDetailWide << 8) : kRouteTridiag) | (passes << 16) | (sh.why << 24);
       }
-      return want_vs;
+      return want_vs ? kEndedVs : kEnded;
     }
     __syncthreads();
   }
+  if (half == kFp64Half && !(gmax > 0.f)) return kOtherHalf;
 
   // ---- last resort (or the caller's choice): Jacobi on the whole matrix ----------------------------
   for (int e = tid; e < D * D / 4; e += NT) {
@@ -1164,7 +1215,7 @@ __device__ __forceinline__ bool eig_user(const float* __restrict__ gpart, const 
   const float thr_abs2 = (kTolAbs * gmax * sc) * (kTolAbs * gmax * sc);
   full_jacobi_route<D, NT>(smem, sh.flags, b, tid, r, sc, thr_abs2, tol.sweep_stop * tol.sweep_stop, sh.why,
                            sweep_cap, S, V, info, route_taken);
-  return false;
+  return kEnded;
 }
 
 // ---- optional epilogue: the factor-token projections of Eq. 11 for this user ---------------
@@ -1330,27 +1381,40 @@ __global__ void __launch_bounds__(TriCfg<D>::NT, TriCfg<D>::CTAS)
 eig_tridiag_kernel(const float* __restrict__ gpart, const int* __restrict__ gram_status, int parts, int splits,
                    float* __restrict__ gsum, int r, int route, int sweep_cap, TriTol tol,
                    float* __restrict__ S, float* __restrict__ V, int* __restrict__ info,
-                   int* __restrict__ route_taken, FuseArgs fa) {
-  const bool vs_ready = eig_user<D, RP>(gpart, gram_status, parts, splits, gsum, r, route, sweep_cap, tol, fa.mode != 0, fa.late_trigger != 0, S, V,
-                                        info, route_taken);
-  if (fa.mode != 0) {
+                   int* __restrict__ route_taken, FuseArgs fa, int pairs) {
+  const bool two = RP > 32 && pairs;
+  const int b = two ? blockIdx.x >> 1 : blockIdx.x, half = !two ? kAlone : (blockIdx.x & 1) ? kFp64Half : kFp32Half;
+  bool joined;                          // this CTA has arrived at the pair's second barrier and not yet waited
+  const EigEnd end = eig_user<D, RP>(b, half, joined, gpart, gram_status, parts, splits, gsum, r, route, sweep_cap, tol, fa.mode != 0,
+                                     fa.late_trigger != 0, S, V, info, route_taken);
+  if (fa.mode != 0 && end != kOtherHalf) {
     extern __shared__ __align__(16) float smem[];
     __syncthreads();                    // S and V of this user are written (and visible to the CTA)
-    prepare_epilogue<D, TriCfg<D>::NT>(smem, blockIdx.x, r, S, V, fa, vs_ready, threadIdx.x);
+    prepare_epilogue<D, TriCfg<D>::NT>(smem, b, r, S, V, fa, end == kEndedVs, threadIdx.x);
   }
+  __syncwarp();
+  if (RP > 32 && joined) cluster_wait();
 }
 
 template <int D, int RP>
 cudaError_t launch_tri(int B, int r, int route, int sweep_cap, TriTol tol, const float* gpart,
                        const int* gram_status, int parts, int splits, float* gsum, float* S, float* V, int* info,
-                       int* route_taken, const FuseArgs& fa, cudaStream_t st) {
+                       int* route_taken, const FuseArgs& fa, bool pairs, cudaStream_t st) {
   using L = TriSmem<D, RP>;
   static bool limits_set[kMaxDevicesCached] = {};
   const cudaError_t e = set_kernel_limits(reinterpret_cast<const void*>(&eig_tridiag_kernel<D, RP>), L::BYTES,
                                           limits_set);
   if (e != cudaSuccess) return e;
-  return launch_pdl(eig_tridiag_kernel<D, RP>, dim3(B), dim3(TriCfg<D>::NT), L::BYTES, st, gpart, gram_status,
-                    parts, splits, gsum, r, route, sweep_cap, tol, S, V, info, route_taken, fa);
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(pairs ? 2 * B : B); cfg.blockDim = dim3(TriCfg<D>::NT); cfg.dynamicSmemBytes = L::BYTES; cfg.stream = st;
+  cudaLaunchAttribute attr[2];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  attr[1].id = cudaLaunchAttributeClusterDimension;
+  attr[1].val.clusterDim.x = 2; attr[1].val.clusterDim.y = 1; attr[1].val.clusterDim.z = 1;
+  cfg.attrs = attr; cfg.numAttrs = pairs ? 2 : 1;
+  return cudaLaunchKernelEx(&cfg, eig_tridiag_kernel<D, RP>, gpart, gram_status, parts, splits, gsum, r, route, sweep_cap, tol, S, V,
+                            info, route_taken, fa, (int)pairs);
 }
 
 }  // namespace
@@ -1377,15 +1441,20 @@ cudaError_t launch_eig_tridiag(int B, int d, int r, solar_dtype_t dt, int route,
     tol.stop_trace = 1.1920929e-07f; tol.stop_couple = 2.9802322e-08f;     // 2^-23, 2^-25
   }
   const bool wide = r > 32;
+  // Two CTAs per user where the fp64 chain is likely (gaps among 33 and more kept eigenvalues), half of the
+  // SMs would stay idle anyway and no slice limit says that other requests use them.  For smaller ranks
+  // the second chain is hardly ever needed, and it costs: 16 x 10240 x 64 with r = 32 51.8 -> 52.8 us per
+  // pass, one user of 256 x 32 with r = 8 22.1 -> 24.6.
+  const bool pairs = route == SOLAR_ROUTE_AUTO && wide && B <= kNumSMs / 2 && slice_limit() == 0;
   switch (d) {
     case 32:
-      return launch_tri<32, 32>(B, r, route, sweep_cap, tol, gpart, gram_status, parts, splits, gsum, S, V, info, route_taken, fa, st);
+      return launch_tri<32, 32>(B, r, route, sweep_cap, tol, gpart, gram_status, parts, splits, gsum, S, V, info, route_taken, fa, pairs, st);
     case 64:
-      return wide ? launch_tri<64, 64>(B, r, route, sweep_cap, tol, gpart, gram_status, parts, splits, gsum, S, V, info, route_taken, fa, st)
-                  : launch_tri<64, 32>(B, r, route, sweep_cap, tol, gpart, gram_status, parts, splits, gsum, S, V, info, route_taken, fa, st);
+      return wide ? launch_tri<64, 64>(B, r, route, sweep_cap, tol, gpart, gram_status, parts, splits, gsum, S, V, info, route_taken, fa, pairs, st)
+                  : launch_tri<64, 32>(B, r, route, sweep_cap, tol, gpart, gram_status, parts, splits, gsum, S, V, info, route_taken, fa, pairs, st);
     case 128:
-      return wide ? launch_tri<128, 64>(B, r, route, sweep_cap, tol, gpart, gram_status, parts, splits, gsum, S, V, info, route_taken, fa, st)
-                  : launch_tri<128, 32>(B, r, route, sweep_cap, tol, gpart, gram_status, parts, splits, gsum, S, V, info, route_taken, fa, st);
+      return wide ? launch_tri<128, 64>(B, r, route, sweep_cap, tol, gpart, gram_status, parts, splits, gsum, S, V, info, route_taken, fa, pairs, st)
+                  : launch_tri<128, 32>(B, r, route, sweep_cap, tol, gpart, gram_status, parts, splits, gsum, S, V, info, route_taken, fa, pairs, st);
     default: return cudaErrorInvalidValue;
   }
 }
