@@ -647,13 +647,40 @@ __device__ __forceinline__ bool tri_chain(const float (&acc)[TriCfg<D>::RT][TriC
   {
     constexpr int PT = NT / RP < 8 ? NT / RP : 8;               // lanes per eigenvalue
     constexpr int CH = NW == 4 ? 2 : 1, NPT = PT * CH;          // points per lane (one warp per scheduler: two)
-    constexpr int STEPS = (NPT == 8 ? 9 : 12);                  // (NPT + 1)^STEPS >= 2^27
-    constexpr int STEPS64 = (NPT == 8 ? 14 : 19);               // ... >= 2^44, from the Gershgorin interval in fp64
-    static_assert(PT * RP == NT && (NPT == 8 || NPT == 4), "every lane has points");
+    constexpr int NP0 = 256, PRB = 16 / PT;                     // points of the first step, all threads together
+    constexpr int STEPS = (NPT == 8 ? 6 : 9);                   // (NP0 + 1) (NPT + 1)^STEPS >= 2^27
+    constexpr int STEPS64 = (NPT == 8 ? 14 : 19);               // fp64: (NPT + 1)^STEPS64 >= 2^44 from the Gershgorin interval
+    constexpr int STEPS_B = (NPT == 8 ? 9 : 12);                // ... and from a bracket of 2^-14 |T|
+    static_assert(PT * RP == NT && (NPT == 8 || NPT == 4) && CH * NT == NP0 && NP0 <= 3 * NW * RP, "every lane has points");
     const int j = tid / PT, pt = tid % PT, jj = j < r ? j : r - 1;     // surplus lanes shadow column r-1
     const int target = de8 - 1 - jj;    // lambda_(jj-th largest) >= x  <=>  #(eigenvalues < x) <= target
     int steps = STEPS;
-    if (F64) {
+    if (!F64) {
+      // The first step starts from one interval for all eigenvalues, so they share its points: 256 instead
+      // of NPT; every eigenvalue finds its place among their counts by two 16-ary searches.
+      const T w = (hi - lo) * T(1.0 / (NP0 + 1));
+      T x[CH];
+      int n[CH];
+#pragma unroll
+      for (int h = 0; h < CH; ++h) x[h] = fma_t(T(tid + h * NT + 1), w, lo);
+      sturm<T, CH>(dg, e2s, x, n, de8 >> 3);
+      int* const cnt = reinterpret_cast<int*>(part);
+#pragma unroll
+      for (int h = 0; h < CH; ++h) cnt[tid + h * NT] = n[h];
+      __syncthreads();
+      int a = 0, c = 0;
+#pragma unroll
+      for (int q = 0; q < PRB; ++q)
+        a += __popc((__ballot_sync(kFull, cnt[16 * (PT * q + pt) + 15] <= target) >> (lane & ~(PT - 1))) & ((1u << PT) - 1));
+      const int a0 = min(a, NP0 / 16 - 1) * 16;
+#pragma unroll
+      for (int q = 0; q < PRB; ++q)
+        c += __popc((__ballot_sync(kFull, cnt[a0 + PT * q + pt] <= target) >> (lane & ~(PT - 1))) & ((1u << PT) - 1));
+      const int idx = a0 + c;                                   // points at or below the eigenvalue
+      const T nlo = fma_t(T(idx), w, lo), nhi = fma_t(T(idx + 1), w, lo);
+      lo = idx == 0 ? lo : nlo;
+      hi = idx == NP0 ? hi : nhi;
+    } else {
       // bracket: the fp32 chain's eigenvalue +- 2^-15 |T| where the counts confirm it
       const T c0 = (T)lam32[j], dl = tnorm * T(3.0517578125e-05);
       T x[CH];
@@ -665,7 +692,7 @@ __device__ __forceinline__ bool tri_chain(const float (&acc)[TriCfg<D>::RT][TriC
       const unsigned all = __ballot_sync(kFull, in);
       const bool mine = ((~all >> (lane & ~(PT - 1))) & ((1u << PT) - 1)) == 0;
       lo = mine ? c0 - dl : lo; hi = mine ? c0 + dl : hi;
-      steps = all == kFull ? STEPS : STEPS64;
+      steps = all == kFull ? STEPS_B : STEPS64;
     }
 #pragma unroll 1
     for (int step = 0; step < steps; ++step) {
