@@ -4,8 +4,9 @@
 //
 //   1. G = sum of the slices' partial Grams (fixed order), scaled by a power of two.
 //   2. Householder tridiagonalisation T = Q^T G Q with the matrix in REGISTERS, in tiles of d/32
-//      rows x 16 columns per thread (at d = 64 rows 32 apart, so that half of them leave the later stages
-//      for all threads: 43.9 thousand cycles for the 62 steps with adjacent rows, 37.6 now); the vectors of a step live in registers too, at the thread's
+//      rows x 16 columns per thread (rows 32 apart, so that finished ones leave the later stages for all
+//      threads: at d = 64 43.9 thousand cycles for the 62 steps with adjacent rows, 37.6 now; at d = 128
+//      165 and 138, in fp64 319 and 297); the vectors of a step live in registers too, at the thread's
 //      columns and at its rows, so the norm, the inner product and a row of A x are each complete
 //      after the two (three) shuffles over the threads of a row.  The product is taken with the
 //      column x itself and corrected to the reflector v = x - alpha e_1 afterwards, so that the
@@ -60,17 +61,17 @@ constexpr unsigned kFull = 0xffffffffu;
 
 template <int D> struct TriCfg {
   static constexpr int GX = (D == 128) ? 8 : 4;       // threads across a row; 32 groups of them
-  static constexpr int RT = D / 32;                   // rows of a thread: RG * group + RS * 0, 1, ..
-  // d = 64: the second row 32 further down, so that half of the rows are finished for all threads at once
-  // and the later stages leave them out.  d = 128: next to each other, and whole warps finish.
-  static constexpr int RG = (D == 128) ? RT : 1, RS = (D == 128) ? 1 : 32;
+  // rows of a thread: group, group + 32, ..: they are finished for all threads at once, and the later stages
+  // leave them out
+  static constexpr int RT = D / 32;
   static constexpr int NT = 32 * GX;                  // threads of the CTA
   static constexpr int NW = NT / 32;
   static constexpr int CW = 4 * GX;                   // columns of a chunk: thread g of a group has 4 g .. 4 g + 3
   static constexpr int NCH = D / CW;                  // chunks of a row
   static constexpr int WG = 32 / NW;                  // groups of a warp
-  __device__ static constexpr int first_row(int m) { return RS == 1 ? 0 : CW * m / 32; }   // first unfinished one in chunk m's stage
-  __device__ static constexpr int rows_end(int warp) { return RG * (WG * (warp + 1) - 1) + RS * (RT - 1) + 1; }   // behind a warp's last row
+  __device__ static constexpr int first_row(int m) { return CW * m / 32; }                 // a thread's first unfinished row in chunk m's stage
+  __device__ static constexpr int last_next(int m) { return CW * (m + 1) / 32 < RT && RT > 2 ? CW * (m + 1) / 32 : RT - 1; }   // row k+1 is among the rows to this one (of two, both are tried: not slower)
+  __device__ static constexpr int rows_end(int warp) { return WG * (warp + 1) + 32 * (RT - 1); }   // behind a warp's last row
   static constexpr int CTAS = (D == 128) ? 1 : 3;     // resident CTAs that the register count has to allow
   static constexpr int LD = D + 4;                    // pitch of Q^T and of the row-major G
 };
@@ -234,7 +235,7 @@ template <int M, typename T, int D, bool KEEP>
 __device__ __forceinline__ void tri_prepare(TriState<T, D, KEEP>& s, const TriOut<T>& o, int k, int tid) {
   using C = TriCfg<D>;
   constexpr int GX = C::GX, RT = C::RT, NCH = C::NCH, CW = C::CW, M2 = M + 1 < NCH ? M + 1 : M, R0 = C::first_row(M);
-  const int lane = tid & 31, g = lane & (GX - 1), row0 = (tid / GX) * C::RG;
+  const int lane = tid & 31, g = lane & (GX - 1), row0 = tid / GX;
   const int k1 = k + 1, par = k & 1, kc = k1 - CW * M;      // column k+1 within the chunk (CW: it opens the next one)
   // the entries k and k+1 of the column
   const T dkl = (k & 2) ? ((k & 1) ? s.x[M][3] : s.x[M][2]) : ((k & 1) ? s.x[M][1] : s.x[M][0]);
@@ -244,12 +245,12 @@ __device__ __forceinline__ void tri_prepare(TriState<T, D, KEEP>& s, const TriOu
 #pragma unroll
   for (int c = 0; c < 4; ++c) s.x[M][c] = (4 * g + c >= kc) ? s.x[M][c] : T(0);
 #pragma unroll
-  for (int rr = R0; rr < RT; ++rr) s.xr[rr] = (row0 + C::RS * rr >= k1) ? s.xr[rr] : T(0);
+  for (int rr = R0; rr < RT; ++rr) s.xr[rr] = (row0 + 32 * rr >= k1) ? s.xr[rr] : T(0);
   // row k+1 of the matrix (predicated stores: no index into the registers may depend on k)
 #pragma unroll
-  for (int rr = R0; rr < RT; ++rr)
+  for (int rr = R0; rr <= C::last_next(M); ++rr)
 #pragma unroll
-    for (int m = M; m < NCH; ++m) st4_if(o.xp + par * D + CW * m + 4 * g, s.a[rr][m], row0 + C::RS * rr == k1);
+    for (int m = M; m < NCH; ++m) st4_if(o.xp + par * D + CW * m + 4 * g, s.a[rr][m], row0 + 32 * rr == k1);
   T n0 = 0, n1 = 0;
 #pragma unroll
   for (int rr = R0; rr < RT; ++rr) {
@@ -268,7 +269,7 @@ __device__ __forceinline__ void tri_prepare(TriState<T, D, KEEP>& s, const TriOu
   }
   s.s2 = row_sum<GX>(n0 + n1);
 #pragma unroll
-  for (int rr = R0; rr < RT; ++rr) st_if(o.yv + par * D + row0 + C::RS * rr, s.y[rr], g == 0);
+  for (int rr = R0; rr < RT; ++rr) st_if(o.yv + par * D + row0 + 32 * rr, s.y[rr], g == 0);
 }
 
 // ---- Householder steps k whose column k+1 lies in chunk M ---------------------------------------
@@ -281,7 +282,7 @@ __device__ __forceinline__ void tri_stage(TriState<T, D, KEEP>& s, const TriOut<
   constexpr int R0 = C::first_row(M);
   constexpr int K0 = CW * M > 0 ? CW * M - 1 : 0, K1 = CW * (M + 1) - 1 < D - 2 ? CW * (M + 1) - 1 : D - 2;
   constexpr bool F64 = sizeof(T) == 8;
-  const int lane = tid & 31, warp = tid >> 5, g = lane & (GX - 1), row0 = (tid / GX) * C::RG;
+  const int lane = tid & 31, warp = tid >> 5, g = lane & (GX - 1), row0 = tid / GX;
   if (s.k_stop >= 0) return;
   int kend = K1;
 #pragma unroll 1
@@ -363,7 +364,7 @@ __device__ __forceinline__ void tri_stage(TriState<T, D, KEEP>& s, const TriOut<
     T bv[RT], bw[RT];
 #pragma unroll
     for (int rr = R0; rr < RT; ++rr) {
-      const int row = row0 + C::RS * rr;
+      const int row = row0 + 32 * rr;
       const T xpi = xp[row], v = row == k1 ? vk1 : s.xr[rr];
       T w = fma_t(-kap, v, fma_t(-alpha, xpi, s.y[rr]));
       w = row >= k1 ? w : T(0);
@@ -530,7 +531,7 @@ __device__ __forceinline__ bool tri_chain(const float (&acc)[TriCfg<D>::RT][TriC
   constexpr int GX = C::GX, RT = C::RT, NT = C::NT, NW = C::NW, NCH = C::NCH, CW = C::CW, LD = C::LD;
   constexpr bool F64 = sizeof(T) == 8, KEEP = !F64 && D <= 64;
   constexpr int NE = RP / 32;                 // groups of 32 eigenvalues (columns)
-  const int lane = tid & 31, warp = tid >> 5, g = lane & (GX - 1), row0 = (tid / GX) * C::RG;
+  const int lane = tid & 31, warp = tid >> 5, g = lane & (GX - 1), row0 = tid / GX;
   T* const dg = reinterpret_cast<T*>(smem + L::DG);
   T* const eo = reinterpret_cast<T*>(smem + L::EO);
   T* const e2s = reinterpret_cast<T*>(smem + L::E2);
@@ -565,7 +566,7 @@ __device__ __forceinline__ bool tri_chain(const float (&acc)[TriCfg<D>::RT][TriC
 #pragma unroll
         for (int c = 0; c < 4; ++c) {
           s.a[rr][m][c] = (T)(acc[rr][m][c] * sc);
-          if (KEEP) s.q[KEEP ? rr : 0][KEEP ? m : 0][c] = (CW * m + 4 * g + c == row0 + C::RS * rr) ? 1.f : 0.f;
+          if (KEEP) s.q[KEEP ? rr : 0][KEEP ? m : 0][c] = (CW * m + 4 * g + c == row0 + 32 * rr) ? 1.f : 0.f;
         }
     // column 0 (= row 0), by way of the buffer that step 1 writes
 #pragma unroll
@@ -576,7 +577,7 @@ __device__ __forceinline__ bool tri_chain(const float (&acc)[TriCfg<D>::RT][TriC
 #pragma unroll
     for (int m = 0; m < NCH; ++m) ld4(o.xp + D + CW * m + 4 * g, s.x[m]);
 #pragma unroll
-    for (int rr = 0; rr < RT; ++rr) s.xr[rr] = o.xp[D + row0 + C::RS * rr];
+    for (int rr = 0; rr < RT; ++rr) s.xr[rr] = o.xp[D + row0 + 32 * rr];
     tri_prepare<0, T, D, KEEP>(s, o, 0, tid);
     tri_stage<0, T, D, KEEP>(s, o, tid);
     tri_stage<1, T, D, KEEP>(s, o, tid);
@@ -602,7 +603,7 @@ __device__ __forceinline__ bool tri_chain(const float (&acc)[TriCfg<D>::RT][TriC
 #pragma unroll
         for (int m = 0; m < NCH; ++m)
 #pragma unroll
-          for (int c = 0; c < 4; ++c) Qt[(CW * m + 4 * g + c) * LD + row0 + C::RS * rr] = s.q[KEEP ? rr : 0][KEEP ? m : 0][c];
+          for (int c = 0; c < 4; ++c) Qt[(CW * m + 4 * g + c) * LD + row0 + 32 * rr] = s.q[KEEP ? rr : 0][KEEP ? m : 0][c];
     }
     k_stop = s.k_stop;
   }
@@ -1076,7 +1077,7 @@ __device__ __forceinline__ EigEnd eig_user(int b, int half, bool& joined, const 
   extern __shared__ __align__(16) float smem[];
   __shared__ TriShared sh;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int g = lane & (GX - 1), row0 = (tid / GX) * C::RG;
+  const int g = lane & (GX - 1), row0 = tid / GX;
   float* const theta = smem + L::TH;
   float* const part = smem + L::PART;
   joined = false;
@@ -1113,7 +1114,7 @@ __device__ __forceinline__ EigEnd eig_user(int b, int half, bool& joined, const 
         for (int rr = 0; rr < RT; ++rr)
 #pragma unroll
           for (int m = 0; m < NCH; ++m)
-            v[s][rr][m] = (s0 + s < parts) ? ld_dep(gp + (size_t)(s0 + s) * (D * D / 4) + (row0 + C::RS * rr) * (D / 4) + GX * m + g)
+            v[s][rr][m] = (s0 + s < parts) ? ld_dep(gp + (size_t)(s0 + s) * (D * D / 4) + (row0 + 32 * rr) * (D / 4) + GX * m + g)
                                            : make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
       for (int s = 0; s < SCN; ++s)
@@ -1133,10 +1134,10 @@ __device__ __forceinline__ EigEnd eig_user(int b, int half, bool& joined, const 
 #pragma unroll
         for (int c = 0; c < 4; ++c) {
           zero = fmaf(acc[rr][m][c], 0.f, zero);             // NaN where an entry is not finite
-          st_if(part + row0 + C::RS * rr, acc[rr][m][c], CW * m + 4 * g + c == row0 + C::RS * rr);
+          st_if(part + row0 + 32 * rr, acc[rr][m][c], CW * m + 4 * g + c == row0 + 32 * rr);
         }
         if (parts > 1)                                        // read back by the residual check and the fallback
-          reinterpret_cast<float4*>(gsum + (size_t)b * D * D)[(row0 + C::RS * rr) * (D / 4) + GX * m + g] =
+          reinterpret_cast<float4*>(gsum + (size_t)b * D * D)[(row0 + 32 * rr) * (D / 4) + GX * m + g] =
               make_float4(acc[rr][m][0], acc[rr][m][1], acc[rr][m][2], acc[rr][m][3]);
       }
     if (tid < 4) sh.flags[tid] = 0;
@@ -1186,7 +1187,7 @@ __device__ __forceinline__ EigEnd eig_user(int b, int half, bool& joined, const 
 #pragma unroll
       for (int rr = 0; rr < RT; ++rr)
 #pragma unroll
-        for (int m = 0; m < NCH; ++m) ld4(gout + (row0 + C::RS * rr) * D + CW * m + 4 * g, acc[rr][m]);
+        for (int m = 0; m < NCH; ++m) ld4(gout + (row0 + 32 * rr) * D + CW * m + 4 * g, acc[rr][m]);
       wide = 1;
       ok = tri_chain<double, D, RP>(acc, smem, sh, gout, sc, r, false, tol, false, half, not_mine, Vc, passes, tid);
       if (not_mine) return kOtherHalf;
