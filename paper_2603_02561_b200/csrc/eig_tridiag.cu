@@ -133,19 +133,32 @@ __device__ __forceinline__ float lg2(float x) {
   asm("lg2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
   return y;
 }
-// 1 / sqrt(x) and 1 / x to the accuracy of the type (fp32: approximation plus one Newton step):
+// 1 / sqrt(x) and 1 / x to the accuracy of the type for normal x (the hardware's approximation plus one
+// Newton step in fp32, two in fp64; without the library functions' branches for special values):
 // the reflector I - beta v v^T is orthogonal only as far as beta v^T v = 2 holds.
 __device__ __forceinline__ float rsqrt_t(float x) {
   float y;
   asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
   return y * fmaf(-0.5f * x * y, y, 1.5f);
 }
-__device__ __forceinline__ double rsqrt_t(double x) { return rsqrt(x); }
+__device__ __forceinline__ double rsqrt_t(double x) {
+  double y;
+  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+#pragma unroll
+  for (int i = 0; i < 2; ++i) y = fma(0.5 * y, fma(-x * y, y, 1.0), y);
+  return y;
+}
 __device__ __forceinline__ float rcp_t(float x) {
   const float y = rcp_fast(x);
   return y * fmaf(-x, y, 2.f);
 }
-__device__ __forceinline__ double rcp_t(double x) { return 1.0 / x; }
+__device__ __forceinline__ double rcp_t(double x) {
+  double y;
+  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+#pragma unroll
+  for (int i = 0; i < 2; ++i) y = fma(y, fma(-x, y, 1.0), y);
+  return y;
+}
 // the word that holds the sign and the exponent
 __device__ __forceinline__ unsigned top_word(float x) { return __float_as_uint(x); }
 __device__ __forceinline__ unsigned top_word(double x) { return (unsigned)__double2hiint(x); }
