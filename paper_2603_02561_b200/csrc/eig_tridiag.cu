@@ -6,7 +6,7 @@
 //   2. Householder tridiagonalisation T = Q^T G Q with the matrix in REGISTERS, in tiles of d/32
 //      rows x 16 columns per thread (rows 32 apart, so that finished ones leave the later stages for all
 //      threads: at d = 64 43.9 thousand cycles for the 62 steps with adjacent rows, 37.6 now; at d = 128
-//      165 and 138, in fp64 319 and 297); the vectors of a step live in registers too, at the thread's
+//      165 and 138, in fp64 319 and 297, 260 with the reciprocals and A x as below); the vectors of a step live in registers too, at the thread's
 //      columns and at its rows, so the norm, the inner product and a row of A x are each complete
 //      after the two (three) shuffles over the threads of a row.  The product is taken with the
 //      column x itself and corrected to the reflector v = x - alpha e_1 afterwards, so that the
@@ -311,10 +311,12 @@ __device__ __forceinline__ void tri_stage(TriState<T, D, KEEP>& s, const TriOut<
     }
     // x^T A x; meanwhile the reflector's scalars
     const T yk1 = yv[k1], xpk1 = xp[k1];
-    T d0 = 0, d1 = 0, d2 = 0, d3 = 0;
+    // A x at the thread's columns; kept for the update where Q leaves registers for it (d = 128, fp64: a
+    // read of 16 bytes takes the SM's shared memory four cycles a warp)
+    T d0 = 0, d1 = 0, d2 = 0, d3 = 0, yc[KEEP ? 1 : NCH][4];
 #pragma unroll
     for (int m = M; m < NCH; ++m) {
-      T t[4];
+      T (&t)[4] = yc[KEEP ? 0 : m];
       ld4(yv + CW * m + 4 * g, t);
       d0 = fma_t(s.x[m][0], t[0], d0); d1 = fma_t(s.x[m][1], t[1], d1);
       d2 = fma_t(s.x[m][2], t[2], d2); d3 = fma_t(s.x[m][3], t[3], d3);
@@ -386,8 +388,9 @@ __device__ __forceinline__ void tri_stage(TriState<T, D, KEEP>& s, const TriOut<
     }
 #pragma unroll
     for (int m = M; m < NCH; ++m) {
-      T yy[4], pp[4];
-      ld4(yv + CW * m + 4 * g, yy);
+      T pp[4];
+      T (&yy)[4] = yc[KEEP ? 0 : m];
+      if (KEEP) ld4(yv + CW * m + 4 * g, yy);
       ld4(xp + CW * m + 4 * g, pp);
 #pragma unroll
       for (int c = 0; c < 4; ++c) {
