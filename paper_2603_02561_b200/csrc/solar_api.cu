@@ -85,12 +85,12 @@ int solar_set_slice_limit(int max_slices) {
 
 int solar_gram_splits(int B, int N, int d, solar_dtype_t dt) {
   if (check_dims(B, 0, N, d, 1, dt) != SOLAR_OK) return 0;
-  return gram_plan(B, N, gram_is_clustered(N, d, dt)).parts;
+  return gram_plan(B, N, gram_cluster_limit(N, d, dt)).parts;
 }
 
 int solar_gram_slices(int B, int N, int d, solar_dtype_t dt) {
   if (check_dims(B, 0, N, d, 1, dt) != SOLAR_OK) return 0;
-  return gram_plan(B, N, gram_is_clustered(N, d, dt)).splits;
+  return gram_plan(B, N, gram_cluster_limit(N, d, dt)).splits;
 }
 
 solar_status_t solar_gram_partials(int B, int N, int d, solar_dtype_t dt, const void* H,
@@ -99,7 +99,7 @@ solar_status_t solar_gram_partials(int B, int N, int d, solar_dtype_t dt, const 
   if (B == 0) return SOLAR_OK;
   SOLAR_TRY(check_ptr(H));
   SOLAR_TRY(check_ws(workspace, workspace_bytes, factor_ws_bytes(B, N, d, dt)));
-  const GramPlan plan = gram_plan(B, N, gram_is_clustered(N, d, dt));
+  const GramPlan plan = gram_plan(B, N, gram_cluster_limit(N, d, dt));
   float* gpart = static_cast<float*>(workspace);
   int* status = reinterpret_cast<int*>(static_cast<char*>(workspace) + gram_status_offset(B, N, d, dt));
   const cudaStream_t st = static_cast<cudaStream_t>(stream);
@@ -120,7 +120,7 @@ solar_status_t solar_eig_from_partials_ex(int B, int N, int d, int r, solar_dtyp
   if (route_taken != nullptr && (reinterpret_cast<uintptr_t>(route_taken) & 3u))
     return SOLAR_ERR_INVALID_ARG;
   SOLAR_TRY(check_ws(workspace, workspace_bytes, factor_ws_bytes(B, N, d, dt)));
-  const GramPlan plan = gram_plan(B, N, gram_is_clustered(N, d, dt));
+  const GramPlan plan = gram_plan(B, N, gram_cluster_limit(N, d, dt));
   const int* status =
       reinterpret_cast<const int*>(static_cast<const char*>(workspace) + gram_status_offset(B, N, d, dt));
   float* gsum = reinterpret_cast<float*>(static_cast<char*>(workspace) + gram_sum_offset(B, N, d, dt));
@@ -245,7 +245,7 @@ solar_status_t solar_svd_attention_fused(int B, int M, int N, int d, int r, sola
   // streaming pass over H (the first kernel of the call: it waits for what ran before)
   SOLAR_TRY(solar_gram_partials(B, N, d, dt, H, workspace, factor_ws_bytes(B, N, d, dt), stream));
   // eigensolve; every user's CTA ends with that user's factor-token projections
-  const GramPlan plan = gram_plan(B, N, gram_is_clustered(N, d, dt));
+  const GramPlan plan = gram_plan(B, N, gram_cluster_limit(N, d, dt));
   const int* status = reinterpret_cast<const int*>(ws + gram_status_offset(B, N, d, dt));
   float* gsum = reinterpret_cast<float*>(ws + gram_sum_offset(B, N, d, dt));
   const EigFuse fuse = {Wq, Wk, Wv, scale, attn_ws};

@@ -58,37 +58,28 @@ inline GramPlan slice_plan(int B, int N) {
   return p;
 }
 
-// The plan of the tensor-core Gram kernel.  Its CTAs can form thread-block clusters of
-// kMaxCluster slices of a user that add up their accumulators through distributed shared
-// memory, so that a user leaves splits / cluster partial matrices.  Measured on the headline
-// shape (B = 16, N = 10240: nine slices), clusters of 3 and of 8 both lose more in the Gram
-// kernel (gang-scheduled CTAs, two cluster barriers: 3.3 -> 3.95 us per launch with 24 requests
-// in flight, 7.4 -> 9.9 us alone) than the eigensolver gains from reading one matrix instead
-// of nine (45 -> 44 us), so the cluster size is 1 and every slice writes its own partial.
-constexpr int kMaxCluster = 1;
-inline GramPlan gram_plan(int B, int N, bool clustered) {
-  if (!clustered) return slice_plan(B, N);
-  GramPlan p;
-  p.tiles = (N + kGramTileRows - 1) / kGramTileRows;
-  long best_cost = -1;
-  int smax = p.tiles < kMaxSplits ? p.tiles : kMaxSplits;
-  const int cap = slice_limit();
-  if (cap > 0 && cap < smax) smax = cap;
-  p.splits = 1; p.chunk_tiles = p.tiles;
-  for (int s = 1; s <= smax; ++s) {
-    int s_eff, chunk;
-    const long cost = slice_cost(B, p.tiles, s, &s_eff, &chunk);
-    if (best_cost < 0 || cost < best_cost) { best_cost = cost; p.splits = s_eff; p.chunk_tiles = chunk; }
-  }
-  // the largest cluster size (<= kMaxCluster) that divides the slice count
-  p.cluster = 1;
-  for (int c = 2; c <= kMaxCluster; ++c)
+// The plan of the tensor-core Gram kernel.  Its CTAs can form thread-block clusters of slices of a user
+// that add up their accumulators through distributed shared memory, so that a user leaves splits /
+// cluster partial matrices, which the one CTA of the eigensolver reads.
+//   d = 64 (16 KB a matrix): no clusters.  On the headline shape (B = 16, N = 10240: nine slices), clusters
+// of 3 and of 8 both lose more in the Gram kernel (gang-scheduled CTAs, two cluster barriers: 3.3 -> 3.95 us
+// per launch with 24 requests in flight, 7.4 -> 9.9 us alone) than the eigensolver gains from reading one
+// matrix instead of nine (45 -> 44 us).
+//   d = 128 (64 KB): clusters of up to four, unless a slice limit keeps the slices few anyway: the
+// eigensolver's CTA reads a matrix at 44 bytes a clock, and 16 of them are 12 us of a pass over 8 x 16384 x
+// 128 (four: 3 us; the Gram kernel 9.6 -> 11.1 us, with clusters of eight 19.8).
+constexpr int kMaxCluster = 4;
+inline int gram_cluster_limit(int N, int d, solar_dtype_t dt) {      // 0: not the tensor-core kernel's shape
+  if (dt != SOLAR_BF16 || (d != 64 && d != 128) || N < kGramTileRows) return 0;
+  return d == 128 && slice_limit() == 0 ? kMaxCluster : 1;
+}
+inline GramPlan gram_plan(int B, int N, int cluster_limit) {
+  GramPlan p = slice_plan(B, N);
+  // the largest cluster size within the limit that divides the slice count
+  for (int c = 2; c <= cluster_limit; ++c)
     if (p.splits % c == 0) p.cluster = c;
   p.parts = p.splits / p.cluster;
   return p;
-}
-inline bool gram_is_clustered(int N, int d, solar_dtype_t dt) {
-  return dt == SOLAR_BF16 && (d == 64 || d == 128) && N >= kGramTileRows;   // the tensor-core kernel's shapes
 }
 
 // Workspace of the factorization: partial Grams [B][parts][d][d] fp32, then one status word per
@@ -96,14 +87,14 @@ inline bool gram_is_clustered(int N, int d, solar_dtype_t dt) {
 // device-side wait that ran out.
 constexpr int kGramStatusOk = 0x600D;
 inline size_t gram_status_offset(int B, int N, int d, solar_dtype_t dt) {
-  const GramPlan p = gram_plan(B, N, gram_is_clustered(N, d, dt));
+  const GramPlan p = gram_plan(B, N, gram_cluster_limit(N, d, dt));
   return align_up((size_t)B * p.parts * d * d * sizeof(float), 256);
 }
 // Behind the status words: the summed Gram matrices [B][d][d] fp32, written by the eigensolver
 // when a user has more than one partial (its residual check and its Jacobi fallback read the
 // sum back; a single partial is the sum).
 inline size_t gram_sum_offset(int B, int N, int d, solar_dtype_t dt) {
-  const GramPlan p = gram_plan(B, N, gram_is_clustered(N, d, dt));
+  const GramPlan p = gram_plan(B, N, gram_cluster_limit(N, d, dt));
   return gram_status_offset(B, N, d, dt) + align_up((size_t)B * p.splits * sizeof(int), 256);
 }
 inline size_t factor_ws_bytes(int B, int N, int d, solar_dtype_t dt) {
