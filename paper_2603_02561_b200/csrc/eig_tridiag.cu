@@ -180,6 +180,19 @@ __device__ __forceinline__ void ld4(const double* p, double (&o)[4]) {
   const double2 t = *reinterpret_cast<const double2*>(p), u = *reinterpret_cast<const double2*>(p + 2);
   o[0] = t.x; o[1] = t.y; o[2] = u.x; o[3] = u.y;
 }
+// N consecutive floats
+template <int N> __device__ __forceinline__ void ldn(const float* p, float (&o)[N]) {
+  if constexpr (N == 2) {
+    const float2 t = *reinterpret_cast<const float2*>(p);
+    o[0] = t.x; o[1] = t.y;
+  } else {
+#pragma unroll
+    for (int q = 0; q < N; q += 4) {
+      const float4 t = *reinterpret_cast<const float4*>(p + q);
+      o[q] = t.x; o[q + 1] = t.y; o[q + 2] = t.z; o[q + 3] = t.w;
+    }
+  }
+}
 __device__ __forceinline__ void st4(float* p, const float (&v)[4]) { *reinterpret_cast<float4*>(p) = make_float4(v[0], v[1], v[2], v[3]); }
 __device__ __forceinline__ void st4(double* p, const double (&v)[4]) {
   *reinterpret_cast<double2*>(p) = make_double2(v[0], v[1]);
@@ -311,12 +324,12 @@ __device__ __forceinline__ void tri_stage(TriState<T, D, KEEP>& s, const TriOut<
     }
     // x^T A x; meanwhile the reflector's scalars
     const T yk1 = yv[k1], xpk1 = xp[k1];
-    // A x at the thread's columns; kept for the update where Q leaves registers for it (d = 128, fp64: a
+    // A x at the thread's columns; kept for the update where there are registers for it (d = 128: a
     // read of 16 bytes takes the SM's shared memory four cycles a warp)
-    T d0 = 0, d1 = 0, d2 = 0, d3 = 0, yc[KEEP ? 1 : NCH][4];
+    T d0 = 0, d1 = 0, d2 = 0, d3 = 0, yc[D == 128 ? NCH : 1][4];
 #pragma unroll
     for (int m = M; m < NCH; ++m) {
-      T (&t)[4] = yc[KEEP ? 0 : m];
+      T (&t)[4] = yc[D == 128 ? m : 0];
       ld4(yv + CW * m + 4 * g, t);
       d0 = fma_t(s.x[m][0], t[0], d0); d1 = fma_t(s.x[m][1], t[1], d1);
       d2 = fma_t(s.x[m][2], t[2], d2); d3 = fma_t(s.x[m][3], t[3], d3);
@@ -389,8 +402,8 @@ __device__ __forceinline__ void tri_stage(TriState<T, D, KEEP>& s, const TriOut<
 #pragma unroll
     for (int m = M; m < NCH; ++m) {
       T pp[4];
-      T (&yy)[4] = yc[KEEP ? 0 : m];
-      if (KEEP) ld4(yv + CW * m + 4 * g, yy);
+      T (&yy)[4] = yc[D == 128 ? m : 0];
+      if (D != 128) ld4(yv + CW * m + 4 * g, yy);
       ld4(xp + CW * m + 4 * g, pp);
 #pragma unroll
       for (int c = 0; c < 4; ++c) {
@@ -902,44 +915,54 @@ __device__ __forceinline__ bool tri_chain(const float (&acc)[TriCfg<D>::RT][TriC
   float* const Gsm = smem + L::R0;
   for (int e = tid; e < D * D / 4; e += NT) cp_async16(Gsm + 4 * e, gout + 4 * e);
 
+  // The products of steps 6 and 7 are bound by shared-memory reads (16 bytes a lane take four cycles a warp,
+  // whatever the lanes share), so every thread has a tile of at least 4 x 4 outputs (2 x 4 at d = 32): column
+  // group fastest, so that the eight lanes of a read's phase share the other operand.  A column per lane and
+  // 16 rows per thread: 25.7 thousand cycles for both steps at d = 64, r = 64, 20.2 so; 9.3 and 7.3 at r = 32.
+  constexpr int CG = RP / 4, TR = D * RP / (4 * NT);        // tile of V: TR rows, 4 columns
+  constexpr int UN = RP == 32 ? 8 : 4;                      // rows fetched ahead of their FMAs, as far as registers go
+  const int r0 = (tid / CG) * TR, c0 = (tid % CG) * 4;
+
   // ---- 6. orthogonalisation passes while V^T V - I is above the rounding level ---------------------
-  // Column-parallel: lane = column(s) c, c + 32; a warp takes RP / NW rows a of E.
-  constexpr int AW = RP / NW;
-  float* const Em = smem + L::A4;
+  constexpr int TA = RP == 64 ? 8 : 4, SPL = NT / (RP / TA * CG), LPS = 32 / SPL;      // tile of E: TA x 4, SPL lanes share its sum
+  static_assert(SPL >= 1 && LPS >= 8, "a read's phase has one row of V");
+  float* const Em = smem + L::A4;                            // strict upper triangle of E
+  float* const diag = part + RP;
+  float* const scol = part + 2 * RP;
   for (;;) {
-    float ev[NE][AW];
+    const int sp = lane / LPS, tile = warp * LPS + lane % LPS, xa = tile / CG * TA, xc = tile % CG * 4;
+    float ev[TA][4];
 #pragma unroll
-    for (int h = 0; h < NE; ++h)
+    for (int u = 0; u < TA; ++u)
 #pragma unroll
-      for (int u = 0; u < AW; ++u) ev[h][u] = 0.f;
-    const int a0 = warp * AW;
-#pragma unroll 8
-    for (int n = 0; n < D; ++n) {
-      float av[AW];
+      for (int c = 0; c < 4; ++c) ev[u][c] = 0.f;
+#pragma unroll UN
+    for (int n = sp * (D / SPL); n < (sp + 1) * (D / SPL); ++n) {
+      float va[TA], vc[4];
+      ldn(Vc + n * RP + xa, va);
+      ld4(Vc + n * RP + xc, vc);
 #pragma unroll
-      for (int u = 0; u < AW; u += 4) {
-        float t[4];
-        ld4(Vc + n * RP + a0 + u, t);
-        av[u] = t[0]; av[u + 1] = t[1]; av[u + 2] = t[2]; av[u + 3] = t[3];
-      }
+      for (int u = 0; u < TA; ++u)
 #pragma unroll
-      for (int h = 0; h < NE; ++h) {
-        const float vc = Vc[n * RP + 32 * h + lane];
-#pragma unroll
-        for (int u = 0; u < AW; ++u) ev[h][u] = fmaf(av[u], vc, ev[h][u]);
-      }
+        for (int c = 0; c < 4; ++c) ev[u][c] = fmaf(va[u], vc[c], ev[u][c]);
     }
     float emax = 0.f;
 #pragma unroll
-    for (int h = 0; h < NE; ++h)
+    for (int u = 0; u < TA; ++u) {
+      float up[4];
+      const int x = xa + u;
 #pragma unroll
-      for (int u = 0; u < AW; ++u) {
-        const int x = a0 + u, c = 32 * h + lane;
-        float e = ev[h][u] - (x == c ? 1.f : 0.f);
-        e = ((int)(x >= r) | (int)(c >= r)) ? 0.f : e;       // surplus columns are copies of column r-1
-        Em[x * RP + c] = e;
+      for (int c = 0; c < 4; ++c) {
+#pragma unroll
+        for (int o = LPS; o < 32; o <<= 1) ev[u][c] += __shfl_xor_sync(kFull, ev[u][c], o);
+        float e = ev[u][c] - (x == xc + c ? 1.f : 0.f);
+        e = ((int)(x >= r) | (int)(xc + c >= r)) ? 0.f : e;  // surplus columns are copies of column r-1
+        up[c] = x < xc + c ? e : 0.f;
+        st_if(diag + x, e, x == xc + c);
         emax = (fabsf(e) <= emax) ? emax : fabsf(e);         // a NaN stays
       }
+      st4_if(Em + x * RP + xc, up, sp == 0);
+    }
 #pragma unroll
     for (int o = 16; o; o >>= 1) {
       const float e2 = __shfl_xor_sync(kFull, emax, o);
@@ -957,28 +980,48 @@ __device__ __forceinline__ bool tri_chain(const float (&acc)[TriCfg<D>::RT][TriC
     // better determined vectors): v_c <- (v_c - sum_{a<c} E_ac v_a) / |.|.  A later column never
     // changes an earlier one, so a poorly separated pair cannot damage its neighbours; for
     // two vectors the pass is exact, for more it converges quadratically like the symmetric
-    // form.  Rows n of V' for this warp: D / NW of them; lane = column.
-#pragma unroll 1
-    for (int h = 0; h < NE; ++h) {
-      const int c = 32 * h + lane;
-      float ecol[RP], nn = 1.f;
-#pragma unroll
-      for (int x = 0; x < RP; ++x) {
-        const float e = Em[x * RP + c];
-        ecol[x] = x < c ? e : 0.f;
-        nn += x < c ? -e * e : (x == c ? e : 0.f);
+    // form.
+    if (tid < RP) {
+      float n0 = 1.f + diag[tid], n1 = 0.f;
+#pragma unroll 8
+      for (int x = 0; x < RP; x += 2) {
+        const float e0 = Em[x * RP + tid], e1 = Em[(x + 1) * RP + tid];
+        n0 = fmaf(-e0, e0, n0);
+        n1 = fmaf(-e1, e1, n1);
       }
-      const float scol = rsqrtf(fmaxf(nn, 1e-6f));
-#pragma unroll 2
-      for (int n = warp; n < D; n += NW) {
-        float o0 = 0.f, o1 = 0.f;
+      scol[tid] = rsqrtf(fmaxf(n0 + n1, 1e-6f));
+    }
+    __syncthreads();
+    {
+      float o[TR][4];
 #pragma unroll
-        for (int x = 0; x < RP; x += 4) {
-          const float4 t = *reinterpret_cast<const float4*>(Vc + n * RP + x);
-          o0 = fmaf(t.x, ecol[x], o0);     o1 = fmaf(t.y, ecol[x + 1], o1);
-          o0 = fmaf(t.z, ecol[x + 2], o0); o1 = fmaf(t.w, ecol[x + 3], o1);
+      for (int u = 0; u < TR; ++u)
+#pragma unroll
+        for (int c = 0; c < 4; ++c) o[u][c] = 0.f;
+#pragma unroll 2
+      for (int x = 0; x < RP; x += 4) {
+        float e[4][4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) ld4(Em + (x + q) * RP + c0, e[q]);
+#pragma unroll
+        for (int u = 0; u < TR; ++u) {
+          float v[4];
+          ld4(Vc + (r0 + u) * RP + x, v);
+#pragma unroll
+          for (int q = 0; q < 4; ++q)
+#pragma unroll
+            for (int c = 0; c < 4; ++c) o[u][c] = fmaf(v[q], e[q][c], o[u][c]);
         }
-        Vn[n * RP + c] = (Vc[n * RP + c] - (o0 + o1)) * scol;
+      }
+      float sc4[4];
+      ld4(scol + c0, sc4);
+#pragma unroll
+      for (int u = 0; u < TR; ++u) {
+        float v[4];
+        ld4(Vc + (r0 + u) * RP + c0, v);
+#pragma unroll
+        for (int c = 0; c < 4; ++c) v[c] = (v[c] - o[u][c]) * sc4[c];
+        st4(Vn + (r0 + u) * RP + c0, v);
       }
     }
     __syncthreads();
@@ -995,65 +1038,82 @@ __device__ __forceinline__ bool tri_chain(const float (&acc)[TriCfg<D>::RT][TriC
 
   // ---- 7. Rayleigh quotients and residuals against G; certification; the largest components -------
   {
-    constexpr int RW = D / NW;        // rows of Y = G V per warp
-    float y[NE][RW];
+    // Y = G V (row k of G in the place of column k)
+    float y[TR][4], v[TR][4], t[4];
 #pragma unroll
-    for (int h = 0; h < NE; ++h)
+    for (int u = 0; u < TR; ++u)
 #pragma unroll
-      for (int u = 0; u < RW; ++u) y[h][u] = 0.f;
-    const int i0 = warp * RW;
-#pragma unroll 2
-    for (int k = 0; k < D; k += 4) {
-      float vk[NE][4];
+      for (int c = 0; c < 4; ++c) y[u][c] = 0.f;
+#pragma unroll UN
+    for (int k = 0; k < D; ++k) {
+      float gg[TR], vk[4];
+      ldn(Gsm + k * D + r0, gg);
+      ld4(Vc + k * RP + c0, vk);
 #pragma unroll
-      for (int h = 0; h < NE; ++h)
+      for (int u = 0; u < TR; ++u)
 #pragma unroll
-        for (int u = 0; u < 4; ++u) vk[h][u] = Vc[(k + u) * RP + 32 * h + lane];
+        for (int c = 0; c < 4; ++c) y[u][c] = fmaf(gg[u], vk[c], y[u][c]);
+    }
+    // sum over the rows of the warp; every column group's first lane stores
+    auto column_sums = [&](float* dst) {
 #pragma unroll
-      for (int u = 0; u < RW; ++u) {
-        const float4 gg = *reinterpret_cast<const float4*>(Gsm + (i0 + u) * D + k);
+      for (int c = 0; c < 4; ++c)
 #pragma unroll
-        for (int h = 0; h < NE; ++h) {
-          y[h][u] = fmaf(gg.x, vk[h][0], y[h][u]); y[h][u] = fmaf(gg.y, vk[h][1], y[h][u]);
-          y[h][u] = fmaf(gg.z, vk[h][2], y[h][u]); y[h][u] = fmaf(gg.w, vk[h][3], y[h][u]);
-        }
+        for (int o = CG; o < 32; o <<= 1) t[c] += __shfl_xor_sync(kFull, t[c], o);
+      st4_if(dst + warp * RP + c0, t, lane < CG);
+    };
+#pragma unroll
+    for (int c = 0; c < 4; ++c) t[c] = 0.f;
+#pragma unroll
+    for (int u = 0; u < TR; ++u) {
+      ld4(Vc + (r0 + u) * RP + c0, v[u]);
+#pragma unroll
+      for (int c = 0; c < 4; ++c) {
+        y[u][c] *= sc;
+        t[c] = fmaf(v[u][c], y[u][c], t[c]);
       }
     }
-    float* const lead = part + NW * RP;                // [NW][RP] the largest component of the warp's rows
+    column_sums(part);
+    {
+      constexpr int RW = D / NW;                       // the largest component of the warp's rows, a column per lane
+      float* const lead = part + NW * RP;              // [NW][RP]
 #pragma unroll
-    for (int h = 0; h < NE; ++h) {
-      float t = 0.f, best = -1.f, lv = 1.f;
-#pragma unroll
-      for (int u = 0; u < RW; ++u) {
-        const float v = Vc[(i0 + u) * RP + 32 * h + lane];
-        y[h][u] *= sc;
-        t = fmaf(v, y[h][u], t);
-        lv = fabsf(v) > best ? v : lv;                          // strict: lowest index wins a tie
-        best = fmaxf(fabsf(v), best);
+      for (int h = 0; h < NE; ++h) {
+        float best = -1.f, lv = 1.f;
+#pragma unroll 8
+        for (int u = 0; u < RW; ++u) {
+          const float x = Vc[(warp * RW + u) * RP + 32 * h + lane];
+          lv = fabsf(x) > best ? x : lv;               // strict: lowest index wins a tie
+          best = fmaxf(fabsf(x), best);
+        }
+        lead[warp * RP + 32 * h + lane] = lv;
       }
-      part[warp * RP + 32 * h + lane] = t;
-      lead[warp * RP + 32 * h + lane] = lv;
     }
     __syncthreads();
+    float th[4] = {0.f, 0.f, 0.f, 0.f};
+    if (F64) {
 #pragma unroll
-    for (int h = 0; h < NE; ++h) {
-      const int c = 32 * h + lane;
-      float th = 0.f;
-      if (F64) {
-        th = (float)lamv[c];             // accurate relative to the eigenvalue itself, unlike an fp32 quotient
-      } else {
+      for (int c = 0; c < 4; ++c) th[c] = (float)lamv[c0 + c];   // accurate relative to the eigenvalue itself, unlike an fp32 quotient
+    } else {
 #pragma unroll
-        for (int w = 0; w < NW; ++w) th += part[w * RP + c];
+      for (int w = 0; w < NW; ++w) {
+        float q[4];
+        ld4(part + w * RP + c0, q);
+#pragma unroll
+        for (int c = 0; c < 4; ++c) th[c] += q[c];
       }
-      if (warp == 0) theta[c] = th;
-      float t = 0.f;
-#pragma unroll
-      for (int u = 0; u < RW; ++u) {
-        const float d = fmaf(-th, Vc[(i0 + u) * RP + c], y[h][u]);
-        t = fmaf(d, d, t);
-      }
-      part[(2 * NW + warp) * RP + c] = t;
     }
+    st4_if(theta + c0, th, tid < CG);
+#pragma unroll
+    for (int c = 0; c < 4; ++c) t[c] = 0.f;
+#pragma unroll
+    for (int u = 0; u < TR; ++u)
+#pragma unroll
+      for (int c = 0; c < 4; ++c) {
+        const float d = fmaf(-th[c], v[u][c], y[u][c]);
+        t[c] = fmaf(d, d, t[c]);
+      }
+    column_sums(part + 2 * NW * RP);
     __syncthreads();
     int good = 1;
     if (tid < r) {
