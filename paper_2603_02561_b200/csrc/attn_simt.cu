@@ -1,10 +1,11 @@
 // SVD-Attention over the r factor tokens (Eq. 12), FFMA version (fp32 storage, and bf16 at d = 32).
-// One candidate row per thread: its scores stay in registers (R = r rounded up to the template's
-// token count), so the softmax needs no shuffles, and the operands T and Value_r are read from shared
-// memory as 16-byte broadcasts, four FMAs each.  The candidate tile comes in and the output tile goes
-// out coalesced through one shared buffer of odd 16-byte pitch.  Bound by shared-memory reads and
-// FMAs alike (2 d r of each row's lanes), then by HBM.  16 x 1000 candidates, d = 64, r = 24, fp32:
-// 33 us with a warp per row over 64 padded tokens, 15 now.
+// Two neighbouring lanes have two candidate rows: each the scores of half of the tokens (R = r rounded up
+// to the template's token count) and, once the probabilities are exchanged, half of the output columns.
+// The operands T and Value_r are read from shared memory as 16-byte broadcasts, eight FMAs each: such a
+// read takes four cycles a warp, so with a row per lane and four FMAs the reads were the bound.  The
+// candidate tile comes in and the output tile goes out coalesced through one shared buffer of odd 16-byte
+// pitch.  16 x 1000 candidates, d = 64, r = 24, fp32: 33 us with a warp per row over 64 padded tokens, 15
+// with a row per lane; two rows and longer Gram stages: 71.8 -> 69.8 us per pass over 5000 x 64 histories.
 #include <math.h>
 
 #include "solar_internal.cuh"
@@ -58,56 +59,87 @@ attn_simt_kernel(const T* __restrict__ C, T* __restrict__ O, const char* __restr
   for (int e = tid; e < R * D / 4; e += kRows)
     reinterpret_cast<float4*>(Vs)[e] = e / (D / 4) < r ? ld_dep(reinterpret_cast<const float4*>(Vr) + e) : make_float4(0.f, 0.f, 0.f, 0.f);
   __syncthreads();
-  pdl_trigger();
+  // A large grid releases the next kernel only behind its work: the next call's first kernel would be packed
+  // onto the SMs that are free (two of its CTAs on one: 16 x 5000 x 64 in fp32 70 -> 81 us per pass).  A small
+  // one leaves most SMs free, and an early release hides the launch (one user: 22.5 -> 22.0 us).
+  const bool few = gridDim.x * gridDim.y <= kNumSMs / 2;
+  if (few) pdl_trigger();
 
-  if (tid < rows) {
-    float* row = Cs + tid * LC;
-    float p[R];
+  if ((tid & ~31) < rows) {              // (rows past the end compute on what lies there and are not stored)
+    constexpr int RH = R / 2, DH = D / 2;
+    const int half = tid & 1, i0 = half * RH;
+    float* const row = Cs + (tid & ~1) * LC;           // rows tid & ~1 and the next
+    float p[2][R];                                      // p[.][i]: this lane's tokens i0 + i first, the partner's behind
 #pragma unroll
-    for (int i = 0; i < R; ++i) p[i] = 0.f;
+    for (int q = 0; q < 2; ++q)
+#pragma unroll
+      for (int i = 0; i < RH; ++i) p[q][i] = 0.f;
 #pragma unroll 1
     for (int k = 0; k < D; k += 4) {
-      const float4 c4 = *reinterpret_cast<const float4*>(row + k);
-      const float c[4] = {c4.x, c4.y, c4.z, c4.w};
+      const float4 a4 = *reinterpret_cast<const float4*>(row + k), b4 = *reinterpret_cast<const float4*>(row + LC + k);
+      const float a[4] = {a4.x, a4.y, a4.z, a4.w}, b[4] = {b4.x, b4.y, b4.z, b4.w};
 #pragma unroll
       for (int u = 0; u < 4; ++u)
 #pragma unroll
-        for (int i = 0; i < R; i += 4) {
-          const float4 t = *reinterpret_cast<const float4*>(Ts + (k + u) * R + i);
-          p[i] = fmaf(c[u], t.x, p[i]);         p[i + 1] = fmaf(c[u], t.y, p[i + 1]);
-          p[i + 2] = fmaf(c[u], t.z, p[i + 2]); p[i + 3] = fmaf(c[u], t.w, p[i + 3]);
+        for (int i = 0; i < RH; i += 4) {
+          const float4 t4 = *reinterpret_cast<const float4*>(Ts + (k + u) * R + i0 + i);
+          const float t[4] = {t4.x, t4.y, t4.z, t4.w};
+#pragma unroll
+          for (int c = 0; c < 4; ++c) {
+            p[0][i + c] = fmaf(a[u], t[c], p[0][i + c]);
+            p[1][i + c] = fmaf(b[u], t[c], p[1][i + c]);
+          }
         }
     }
     if (!(flags & SOLAR_FLAG_NO_SOFTMAX)) {
-      float mx = -INFINITY;
 #pragma unroll
-      for (int i = 0; i < R; ++i) mx = fmaxf(mx, i < r ? p[i] : -INFINITY);
-      float sum = 0.f;
+      for (int q = 0; q < 2; ++q) {
+        float mx = -INFINITY;
 #pragma unroll
-      for (int i = 0; i < R; ++i) {
-        p[i] = i < r ? expf(p[i] - mx) : 0.f;
-        sum += p[i];
+        for (int i = 0; i < RH; ++i) mx = fmaxf(mx, i0 + i < r ? p[q][i] : -INFINITY);
+        mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 1));
+        float sum = 0.f;
+#pragma unroll
+        for (int i = 0; i < RH; ++i) {
+          p[q][i] = i0 + i < r ? expf(p[q][i] - mx) : 0.f;
+          sum += p[q][i];
+        }
+        sum += __shfl_xor_sync(0xffffffffu, sum, 1);
+        const float inv = 1.f / sum;
+#pragma unroll
+        for (int i = 0; i < RH; ++i) p[q][i] *= inv;
       }
-      const float inv = 1.f / sum;
-#pragma unroll
-      for (int i = 0; i < R; ++i) p[i] *= inv;
     }                                     // without it: padded tokens have zero scores and zero Value_r rows
-#pragma unroll 1
-    for (int j = 0; j < D; j += 8) {
-      float o[8];
 #pragma unroll
-      for (int u = 0; u < 8; ++u) o[u] = 0.f;
+    for (int q = 0; q < 2; ++q)
+#pragma unroll
+      for (int i = 0; i < RH; ++i) p[q][RH + i] = __shfl_xor_sync(0xffffffffu, p[q][i], 1);
+    __syncwarp();                         // the rows have been read: they take the output
+    const float* const mine = Vs + i0 * D + half * DH, * const theirs = Vs + (RH - i0) * D + half * DH;
+#pragma unroll 1
+    for (int j4 = 0; j4 < DH; j4 += 4) {
+      const int j = (j4 + 4 * half) & (DH - 1);        // the partner's 16 bytes lie in other banks
+      float o[2][4];
+#pragma unroll
+      for (int q = 0; q < 2; ++q)
+#pragma unroll
+        for (int u = 0; u < 4; ++u) o[q][u] = 0.f;
 #pragma unroll
       for (int i = 0; i < R; ++i) {
-        const float4 v = *reinterpret_cast<const float4*>(Vs + i * D + j), w = *reinterpret_cast<const float4*>(Vs + i * D + j + 4);
-        o[0] = fmaf(p[i], v.x, o[0]); o[1] = fmaf(p[i], v.y, o[1]); o[2] = fmaf(p[i], v.z, o[2]); o[3] = fmaf(p[i], v.w, o[3]);
-        o[4] = fmaf(p[i], w.x, o[4]); o[5] = fmaf(p[i], w.y, o[5]); o[6] = fmaf(p[i], w.z, o[6]); o[7] = fmaf(p[i], w.w, o[7]);
+        const float4 v = *reinterpret_cast<const float4*>((i < RH ? mine + i * D : theirs + (i - RH) * D) + j);
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {
+          o[q][0] = fmaf(p[q][i], v.x, o[q][0]); o[q][1] = fmaf(p[q][i], v.y, o[q][1]);
+          o[q][2] = fmaf(p[q][i], v.z, o[q][2]); o[q][3] = fmaf(p[q][i], v.w, o[q][3]);
+        }
       }
-      *reinterpret_cast<float4*>(row + j) = make_float4(o[0], o[1], o[2], o[3]);
-      *reinterpret_cast<float4*>(row + j + 4) = make_float4(o[4], o[5], o[6], o[7]);
+#pragma unroll
+      for (int q = 0; q < 2; ++q)
+        *reinterpret_cast<float4*>(row + q * LC + half * DH + j) = make_float4(o[q][0], o[q][1], o[q][2], o[q][3]);
     }
   }
   __syncthreads();
+  if (!few) pdl_trigger();
   T* Ob = O + ((size_t)b * M + m0) * D;
 #pragma unroll 4
   for (int v = tid; v < rows * VPR; v += kRows) {

@@ -8,7 +8,8 @@
 // shared-memory reads, most of them broadcasts; KG groups of such threads fill the CTA and their
 // tiles are added up in group order at the end.  Rows arrive by cp.async in a ring of three stages,
 // in the storage type.  16 x 5000 x 64 fp32: 54 us with 4 x 4 tiles of the full matrix and one
-// synchronous stage, 21 now (8 of them FMA time).  The next kernel is not released early: its few
+// synchronous stage, 19.6 with stages of 56 rows, 18.8 now (112 rows, the last stage only as long as it has
+// rows; 8 of them FMA time).  The next kernel is not released early: its few
 // CTAs would be packed onto the SMs that are free first and slow each other down.
 #include "solar_internal.cuh"
 
@@ -20,8 +21,8 @@ template <int D> struct SimtGram {
   static constexpr int NB = D / 8, TILES = NB * (NB + 1) / 2;            // 8 x 8 tiles on and above the diagonal
   static constexpr int NT = D == 128 ? 288 : 256;                         // threads: KG groups of TILES, a few idle
   static constexpr int KG = NT / TILES;                                   // 25, 7, 2
-  static constexpr int IT = D == 32 ? 4 : D == 64 ? 8 : 16;               // rows of a group per stage
-  static constexpr int TR = KG * IT;                                      // rows per stage: 100, 56, 32
+  static constexpr int IT = D == 32 ? 4 : 16;                             // rows of a group per stage
+  static constexpr int TR = KG * IT;                                      // rows per stage: 100, 112, 32
   static constexpr int STAGES = 3;
   template <typename T> static constexpr size_t smem() {
     const size_t ring = (size_t)STAGES * TR * D * sizeof(T), red = (size_t)KG * TILES * 64 * sizeof(float);
@@ -60,7 +61,8 @@ gram_simt_kernel(const T* __restrict__ H, float* __restrict__ gpart, int* __rest
   pdl_wait();            // H is the caller's: whatever wrote it earlier on the stream has completed
   auto fetch = [&](int st) {
     T* dst = ring + (size_t)(st % C::STAGES) * TR * D;
-    for (int v = tid; v < TR * VPR; v += NT) {
+    const int want = min(TR, (rows - st * TR + KG - 1) / KG * KG);        // whole rounds of the groups
+    for (int v = tid; v < want * VPR; v += NT) {
       const int rr = st * TR + v / VPR;
       const int bytes = rr < rows ? 16 : 0;                               // rows past the end arrive as zeros
       const T* src = Hb + (size_t)min(rr, rows - 1) * D + (v % VPR) * VE;
@@ -82,8 +84,9 @@ gram_simt_kernel(const T* __restrict__ H, float* __restrict__ gpart, int* __rest
     __syncthreads();                       // stage st is there; everybody is done with stage st - 1
     if (st + 2 < nst) fetch(st + 2); else asm volatile("cp.async.commit_group;" ::: "memory");
     const T* rowp = ring + (size_t)(st % C::STAGES) * TR * D + (size_t)grp * D;
+    const int rounds = min(C::IT, (rows - st * TR + KG - 1) / KG);
 #pragma unroll 2
-    for (int it = 0; it < C::IT; ++it) {
+    for (int it = 0; it < rounds; ++it) {
       float a[8], c[8];
       load8(rowp + (size_t)it * KG * D + 8 * ti, a);
       load8(rowp + (size_t)it * KG * D + 8 * tj, c);
