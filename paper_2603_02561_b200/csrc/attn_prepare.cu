@@ -143,7 +143,8 @@ template <int D>
 __global__ void __launch_bounds__(D == 128 ? 256 : 128, 1)
 attn_prepare_mma_kernel(const float* __restrict__ S, const float* __restrict__ V, const void* __restrict__ Wq,
                         const void* __restrict__ Wk, const void* __restrict__ Wv, float scale, int r,
-                        char* __restrict__ ws, AttnWs lay, int f32, __nv_bfloat16* __restrict__ bwd_pk) {
+                        char* __restrict__ ws, AttnWs lay, int f32, __nv_bfloat16* __restrict__ bwd_pk,
+                        int* __restrict__ zero, int zeros) {
   extern __shared__ __align__(16) unsigned char smb[];
   const int b = blockIdx.x, tid = threadIdx.x;
   char* wsb = ws + (size_t)b * lay.per_user;
@@ -155,20 +156,23 @@ attn_prepare_mma_kernel(const float* __restrict__ S, const float* __restrict__ V
   o.Tkm = bwd_pk != nullptr ? bwd_pk + (size_t)b * 4 * kTokenSlots * D : nullptr;
   o.Vkm = bwd_pk != nullptr ? o.Tkm + 2 * kTokenSlots * D : nullptr;
   pdl_wait();                                    // as in the kernel above
+  if (zero != nullptr && blockIdx.y == 1)
+    for (int e = tid; e < zeros; e += blockDim.x) zero[(size_t)b * zeros + e] = 0;
   if (blockIdx.y == 0) prepare_kinds<D, 1>(smb, S, V, Wq, Wk, Wv, scale, r, o, b, tid);
   else prepare_kinds<D, 2>(smb, S, V, Wq, Wk, Wv, scale, r, o, b, tid);
 }
 
 template <int D>
 cudaError_t launch_mma(int B, int r, const float* S, const float* V, const void* Wq, const void* Wk, const void* Wv,
-                       float scale, char* ws, const AttnWs& lay, bool f32, void* bwd_pk, cudaStream_t st) {
+                       float scale, char* ws, const AttnWs& lay, bool f32, void* bwd_pk, cudaStream_t st, int* zero,
+                       int zeros) {
   static bool limits_set[kMaxDevicesCached] = {};
   cudaError_t e = set_kernel_limits(reinterpret_cast<const void*>(&attn_prepare_mma_kernel<D>),
                                     (size_t)pmma::Lay<D>::bytes(kTokenSlots), limits_set);
   if (e != cudaSuccess) return e;
   return launch_pdl(attn_prepare_mma_kernel<D>, dim3(B, 2), dim3(D == 128 ? 256 : 128),
                     (size_t)pmma::Lay<D>::bytes((r + 15) & ~15), st, S, V, Wq, Wk, Wv, scale, r, ws, lay, (int)f32,
-                    static_cast<__nv_bfloat16*>(bwd_pk));
+                    static_cast<__nv_bfloat16*>(bwd_pk), zero, zeros);
 }
 
 template <typename T>
@@ -204,9 +208,9 @@ cudaError_t launch_t(int B, int d, int r, const float* S, const float* V, const 
 
 cudaError_t launch_attn_prepare(int B, int d, int r, solar_dtype_t dt, const float* S,
                                 const float* V, const void* Wq, const void* Wk, const void* Wv,
-                                float scale, char* ws, const AttnWs& lay, bool f32, void* bwd_pk, cudaStream_t st) {
-  if (dt == SOLAR_BF16 && d == 64) return launch_mma<64>(B, r, S, V, Wq, Wk, Wv, scale, ws, lay, f32, bwd_pk, st);
-  if (dt == SOLAR_BF16 && d == 128) return launch_mma<128>(B, r, S, V, Wq, Wk, Wv, scale, ws, lay, f32, bwd_pk, st);
+                                float scale, char* ws, const AttnWs& lay, bool f32, void* bwd_pk, cudaStream_t st, int* zero, int zeros) {
+  if (dt == SOLAR_BF16 && d == 64) return launch_mma<64>(B, r, S, V, Wq, Wk, Wv, scale, ws, lay, f32, bwd_pk, st, zero, zeros);
+  if (dt == SOLAR_BF16 && d == 128) return launch_mma<128>(B, r, S, V, Wq, Wk, Wv, scale, ws, lay, f32, bwd_pk, st, zero, zeros);
   return dt == SOLAR_BF16
              ? launch_t<__nv_bfloat16>(B, d, r, S, V, Wq, Wk, Wv, scale, ws, lay, st)
              : launch_t<float>(B, d, r, S, V, Wq, Wk, Wv, scale, ws, lay, st);

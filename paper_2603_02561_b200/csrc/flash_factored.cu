@@ -17,6 +17,10 @@
 //                                       MN-major operand; accumulates in tensor memory and overlaps the
 //                                       next tile's exponentials
 //   O [128 x d] = (Y / l) B1  (B1 = V^T W_V, hi/lo halves), tcgen05.mma, TMA store.
+// Where the candidates do not fill the GPU, the positions are split as well (flash_split): a CTA then leaves
+// Y, l and m of its range, and the one that arrives last adds up the ranges in their order.  128 candidates,
+// 32768 positions, d = 64, r = 32: 281 us a call with one CTA, 35 now; 8 x 512 candidates,
+// 10240 positions: 98 and 44.
 // The reference m of a row is the maximum of its first tile and is raised (Y and l rescaled) only when a
 // score passes it by more than 2^8: any m gives the same quotient, and bf16 keeps its relative accuracy
 // at every magnitude.  The N x M score matrix never exists outside tensor memory.  Every wait is bounded;
@@ -104,7 +108,8 @@ template <int D, int R>
 __global__ void __launch_bounds__(kThreads, 2)
 flash_factored_kernel(const __grid_constant__ CUtensorMap tmC, const __grid_constant__ CUtensorMap tmO,
                       const __grid_constant__ CUtensorMap tmT, const __grid_constant__ CUtensorMap tmV,
-                      const __grid_constant__ CUtensorMap tmUS, int N, int M, __nv_bfloat16* __restrict__ O) {
+                      const __grid_constant__ CUtensorMap tmUS, int N, int M, __nv_bfloat16* __restrict__ O,
+                      int tiles_per_range, float* __restrict__ part, int* __restrict__ counters) {
   using Cfg = FlashCfg<D, R>;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* base = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
@@ -115,14 +120,15 @@ flash_factored_kernel(const __grid_constant__ CUtensorMap tmC, const __grid_cons
   uint8_t* sUS = sC + Cfg::C_BYTES;           // [kStages][128][RB]
   __shared__ __align__(8) uint64_t bar_load, bar_q, bar_qs, bar_s, bar_sf, bar_p, bar_y, bar_o, us_full[kStages], us_free[kStages];
   __shared__ uint32_t s_tmem;
-  __shared__ int s_err;
+  __shared__ int s_err, s_last;
 
   const int b = blockIdx.y, m0 = blockIdx.x * kRows;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int ntiles = (N + kPos - 1) / kPos;
+  const int ranges = gridDim.z, t0 = blockIdx.z * tiles_per_range;     // this CTA's tiles: t0 ..
+  const int ntiles = min((N + kPos - 1) / kPos - t0, tiles_per_range), p0 = t0 * kPos;
 
   if (tid == 0) {
-    s_err = 0;
+    s_err = 0; s_last = 1;
     ptx::mbar_init(&bar_load, 1); ptx::mbar_init(&bar_q, 1); ptx::mbar_init(&bar_qs, kRowWarps);
     ptx::mbar_init(&bar_s, 1); ptx::mbar_init(&bar_sf, kRowWarps); ptx::mbar_init(&bar_p, kRowWarps);
     ptx::mbar_init(&bar_y, 1); ptx::mbar_init(&bar_o, 1);
@@ -157,7 +163,7 @@ flash_factored_kernel(const __grid_constant__ CUtensorMap tmC, const __grid_cons
         const int st = t % kStages;
         if (t >= kStages && !ptx::mbar_wait(&us_free[st], (t / kStages - 1) & 1, err, kErrTile)) break;
         ptx::mbar_arrive_expect_tx(&us_full[st], Cfg::US_TILE);
-        ptx::tma_load_3d(sUS + st * Cfg::US_TILE, &tmUS, &us_full[st], 0, t * kPos, b);
+        ptx::tma_load_3d(sUS + st * Cfg::US_TILE, &tmUS, &us_full[st], 0, p0 + t * kPos, b);
         issued = t + 1;
       }
       // the copies still in flight land before the CTA leaves, whatever happened
@@ -230,7 +236,7 @@ flash_factored_kernel(const __grid_constant__ CUtensorMap tmC, const __grid_cons
       }
       // ---- O = (y / l) B1 : M = 128, N = D, K = R, hi*hi + hi*lo + lo*hi ---------------------
       ok = ok && ptx::mbar_wait(&bar_p, ntiles & 1, err, kErrP);
-      if (ok) {
+      if (ok && *(volatile int*)&s_last) {
         ptx::tc_fence_after_sync();
         const uint32_t idesc = ptx::umma_idesc_bf16(kRows, D, false, false);
         bool acc = false;
@@ -284,7 +290,7 @@ flash_factored_kernel(const __grid_constant__ CUtensorMap tmC, const __grid_cons
       }
       ptx::tc_fence_before_sync();
       ptx::mbar_arrive_warp(&bar_sf, lane);          // the next tile's scores may be formed
-      const int valid = N - t * kPos;                // positions past N hold zero-filled rows
+      const int valid = N - p0 - t * kPos;           // positions past N hold zero-filled rows
       if (valid < kPos) {
 #pragma unroll
         for (int j = 0; j < kPos; ++j) s[j] = (j < valid) ? s[j] : -INFINITY;
@@ -355,6 +361,39 @@ flash_factored_kernel(const __grid_constant__ CUtensorMap tmC, const __grid_cons
     {
       float y[R];
       tmem_row<R>(tm_y + lane_base, y);
+      if (ranges > 1) {
+        // ---- the ranges' sums: whoever comes last adds them up, in their order ----------------------
+        pdl_wait();                                  // the counters were set by the kernel before
+        const size_t item = (size_t)b * gridDim.x + blockIdx.x;
+        float* mine = part + (item * ranges + blockIdx.z) * (R + 2) * kRows + tid;
+        const float bad = *err != 0 ? __int_as_float(0x7fc00000) : 0.f;
+#pragma unroll
+        for (int i = 0; i < R; ++i) mine[i * kRows] = y[i];
+        mine[R * kRows] = l_run + bad;               // after a lost wait the rows come out as NaN
+        mine[(R + 1) * kRows] = m_ref;
+        __threadfence();
+        asm volatile("bar.sync 1, %0;" ::"n"(kRowThreads) : "memory");
+        if (tid == 0) s_last = atomicAdd(counters + item, 1) == ranges - 1;
+        asm volatile("bar.sync 1, %0;" ::"n"(kRowThreads) : "memory");
+        if (s_last) {
+          __threadfence();
+          const float* all = part + item * ranges * (R + 2) * kRows + tid;
+          float m = -INFINITY;
+#pragma unroll 8
+          for (int z = 0; z < ranges; ++z) m = fmaxf(m, __ldcg(all + ((size_t)z * (R + 2) + R + 1) * kRows));
+          l_run = 0.f;
+#pragma unroll
+          for (int i = 0; i < R; ++i) y[i] = 0.f;
+#pragma unroll 1
+          for (int z = 0; z < ranges; ++z) {
+            const float* from = all + (size_t)z * (R + 2) * kRows;
+            const float f = ptx::fast_exp2(__ldcg(from + (R + 1) * kRows) - m);
+            l_run = fmaf(f, __ldcg(from + R * kRows), l_run);
+#pragma unroll
+            for (int i = 0; i < R; ++i) y[i] = fmaf(f, __ldcg(from + i * kRows), y[i]);
+          }
+        }
+      }
       const float inv = 1.f / l_run;
 #pragma unroll
       for (int i = 0; i < R; ++i) y[i] *= inv;
@@ -385,7 +424,8 @@ flash_factored_kernel(const __grid_constant__ CUtensorMap tmC, const __grid_cons
   }
   ptx::tc_fence_before_sync();
   __syncthreads();
-  if (s_err == 0) {
+  if (!s_last) {
+  } else if (s_err == 0) {
     if (tid == 0) {
 #pragma unroll
       for (int x = 0; x < Cfg::KB; ++x) ptx::tma_store_3d(&tmO, sC + x * kBox, x * 64, m0, b);
@@ -409,8 +449,8 @@ flash_factored_kernel(const __grid_constant__ CUtensorMap tmC, const __grid_cons
 }
 
 template <int D, int R>
-cudaError_t launch_dr(int B, int M, int N, const void* C, const void* US, void* O, const char* ws,
-                      const AttnWs& lay, cudaStream_t st) {
+cudaError_t launch_dr(int B, int M, int N, const void* C, const void* US, void* O, char* ws,
+                      const AttnWs& lay, const FlashSplit& split, cudaStream_t st) {
   using Cfg = FlashCfg<D, R>;
   CUtensorMap tmC, tmO, tmT, tmV, tmUS;
   const uint64_t pu = lay.per_user;
@@ -426,9 +466,10 @@ cudaError_t launch_dr(int B, int M, int N, const void* C, const void* US, void* 
   const cudaError_t e = set_kernel_limits(reinterpret_cast<const void*>(&flash_factored_kernel<D, R>), Cfg::SMEM,
                                           limits_set);
   if (e != cudaSuccess) return e;
-  const dim3 grid((M + kRows - 1) / kRows, B), block(kThreads);
+  const dim3 grid((M + kRows - 1) / kRows, B, split.ranges), block(kThreads);
   return launch_pdl(flash_factored_kernel<D, R>, grid, block, Cfg::SMEM, st, tmC, tmO, tmT, tmV, tmUS, N, M,
-                    static_cast<__nv_bfloat16*>(O));
+                    static_cast<__nv_bfloat16*>(O), split.tiles_per_range, reinterpret_cast<float*>(ws + split.part_off),
+                    reinterpret_cast<int*>(ws + split.counter_off));
 }
 
 }  // namespace
@@ -437,10 +478,34 @@ bool flash_factored_supported(int d, int r, solar_dtype_t dt) {
   return dt == SOLAR_BF16 && (d == 64 || d == 128) && (r == 16 || r == 32 || r == 64);
 }
 
+// Few candidates: the positions of 128 candidates are split into ranges, a CTA each, so that the CTAs fill the
+// SMs once (twice where two fit).  Ranges of at least four tiles (a CTA's start costs about two), and no more
+// than 3 sqrt(tiles) of them: the last CTA reads every range's sums, about a sixth of a tile's time each, so
+// the sum of both is smallest near sqrt(6 tiles).  The sums lie behind the operands in the workspace, which
+// the factorization of the same sizes makes large enough; a smaller one means fewer ranges.
+FlashSplit flash_split(int B, int M, int N, int d, int r, size_t workspace_bytes) {
+  FlashSplit s = {};
+  const int tiles = (N + kPos - 1) / kPos;
+  s.items_per_user = (M + kRows - 1) / kRows;
+  const size_t items = (size_t)B * s.items_per_user, part = (size_t)(r + 2) * kRows * sizeof(float);
+  s.counter_off = align_up(attn_ws_bytes(B, d, r), 256);
+  s.part_off = s.counter_off + align_up(items * sizeof(int), 256);
+  const int per_sm = (d == 64 && r <= 32) || r == 16 ? 2 : 1;                    // by shared memory
+  size_t k = (size_t)(kNumSMs * per_sm) / items;
+  if (k > (size_t)tiles / 4) k = (size_t)tiles / 4;
+  while (k > 1 && k * k > (size_t)9 * tiles) --k;
+  const size_t room = workspace_bytes > s.part_off ? (workspace_bytes - s.part_off) / (items * part) : 0;
+  if (k > room) k = room;
+  if (k < 1) k = 1;
+  s.tiles_per_range = (int)((tiles + k - 1) / k);
+  s.ranges = (tiles + s.tiles_per_range - 1) / s.tiles_per_range;
+  return s;
+}
+
 cudaError_t launch_flash_factored(int B, int M, int N, int d, int r, const void* C, const void* US, void* O,
-                                  const char* ws, const AttnWs& lay, cudaStream_t st) {
+                                  char* ws, const AttnWs& lay, const FlashSplit& split, cudaStream_t st) {
 #define SOLAR_FF(DD, RR) \
-  if (d == DD && r == RR) return launch_dr<DD, RR>(B, M, N, C, US, O, ws, lay, st);
+  if (d == DD && r == RR) return launch_dr<DD, RR>(B, M, N, C, US, O, ws, lay, split, st);
   SOLAR_FF(64, 16) SOLAR_FF(64, 32) SOLAR_FF(64, 64) SOLAR_FF(128, 16) SOLAR_FF(128, 32) SOLAR_FF(128, 64)
 #undef SOLAR_FF
   return cudaErrorInvalidValue;

@@ -335,10 +335,12 @@ solar_status_t solar_factored_softmax_attention_fwd(int B, int M, int N, int d, 
   const AttnWs lay = attn_ws_layout(d, r);
   // The packed operands of the kernel are the prepare kernel's with unit singular values:
   // T^T becomes (scale log2e W_Q W_K^T V)^T and Value_r^T becomes (V^T W_V)^T.
-  SOLAR_TRY(from_cuda(launch_attn_prepare(B, d, r, dt, nullptr, V, Wq, Wk, Wv,
-                                          scale * 1.4426950408889634f, static_cast<char*>(workspace), lay, false,
-                                          nullptr, st)));
-  return from_cuda(launch_flash_factored(B, M, N, d, r, C, US, O, static_cast<const char*>(workspace), lay, st));
+  char* ws = static_cast<char*>(workspace);
+  const FlashSplit split = flash_split(B, M, N, d, r, workspace_bytes);
+  int* counters = split.ranges > 1 ? reinterpret_cast<int*>(ws + split.counter_off) : nullptr;
+  SOLAR_TRY(from_cuda(launch_attn_prepare(B, d, r, dt, nullptr, V, Wq, Wk, Wv, scale * 1.4426950408889634f, ws, lay, false,
+                                          nullptr, st, counters, split.items_per_user)));
+  return from_cuda(launch_flash_factored(B, M, N, d, r, C, US, O, ws, lay, split, st));
 }
 
 }  // extern "C"

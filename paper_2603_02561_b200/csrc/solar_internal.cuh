@@ -217,15 +217,24 @@ cudaError_t launch_project_us_umma(int B, int N, int d, int r, const void* H, co
                                    bool early_h, cudaStream_t st);
 // bwd_pk: also the backward kernel's operands [B][4][64][d] (tensor-core shapes), or nullptr; f32: also the
 // fp32 copies where only the backward pass or a caller of the stage would read them
+// zero: zeros [B][zeros] words (tensor-core shapes), or nullptr
 cudaError_t launch_attn_prepare(int B, int d, int r, solar_dtype_t dt, const float* S,
                                 const float* V, const void* Wq, const void* Wk, const void* Wv,
-                                float scale, char* ws, const AttnWs& lay, bool f32, void* bwd_pk, cudaStream_t st);
+                                float scale, char* ws, const AttnWs& lay, bool f32, void* bwd_pk, cudaStream_t st,
+                                int* zero = nullptr, int zeros = 0);
 cudaError_t launch_attn_simt(int B, int M, int d, int r, solar_dtype_t dt, const void* C,
                              unsigned flags, void* O, const char* ws, const AttnWs& lay, bool early_c,
                              cudaStream_t st);
 bool flash_factored_supported(int d, int r, solar_dtype_t dt);
+// How the positions are split over CTAs where the candidates alone do not fill the GPU: ranges per 128
+// candidates, and where in the workspace the ranges' sums and their arrival counters lie.
+struct FlashSplit {
+  int ranges, tiles_per_range, items_per_user;
+  size_t counter_off, part_off;
+};
+FlashSplit flash_split(int B, int M, int N, int d, int r, size_t workspace_bytes);
 cudaError_t launch_flash_factored(int B, int M, int N, int d, int r, const void* C, const void* US, void* O,
-                                  const char* ws, const AttnWs& lay, cudaStream_t st);
+                                  char* ws, const AttnWs& lay, const FlashSplit& split, cudaStream_t st);
 bool attn_umma_supported(int d, solar_dtype_t dt);
 // Throughput form of the tensor-core attention kernel: long CTAs that overlap the candidate
 // stream, the GEMMs and the softmax of consecutive tiles (chosen under a slice limit).
