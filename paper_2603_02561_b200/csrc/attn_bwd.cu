@@ -170,7 +170,7 @@ __device__ __forceinline__ void small_gemm(int rows, int K, FA a, FB b, FS store
     for (int x = 0; x < 4; ++x)
 #pragma unroll
       for (int c = 0; c < NC; ++c) acc[x][c] = 0.f;
-#pragma unroll 4
+#pragma unroll 8
     for (int k = 0; k < K; ++k) {
       float av[4], bv[NC];
 #pragma unroll
@@ -195,7 +195,8 @@ __device__ __forceinline__ void small_gemm(int rows, int K, FA a, FB b, FS store
 // Bound by latency: a round of global loads, then two small products (three for role 2) with a barrier
 // each; a weight that is needed later is fetched into registers while the product before runs.  Weights
 // sit in shared memory as fp32 at odd pitch, dT and dValue_r^T are read along both indices.
-// 16 users, d = 64, r = 32: 24 us as one chain on one CTA of 1024 threads, 12 now.
+// A has odd pitch too (it is written along its columns), and role 2 has V and Sigma on chip before it needs
+// them.  16 users, d = 64, r = 32: 24 us as one chain on one CTA of 1024 threads, 16 on four CTAs, 14 now.
 template <typename T, int D>
 __global__ void __launch_bounds__(kUserThreads)
 attn_bwd_user_kernel(const float* __restrict__ part, int chunks, const float* __restrict__ S,
@@ -204,12 +205,13 @@ attn_bwd_user_kernel(const float* __restrict__ part, int chunks, const float* __
                      float* __restrict__ dV, float* __restrict__ dw) {
   extern __shared__ __align__(16) float sm[];
   constexpr int LR = kRP + 1;           // odd pitch
-  constexpr int LW = D + 1;
+  constexpr int LW = D + 1, LA = D + 1;
   float* dT = sm;                       // [D][LR]    dT[k][i]
   float* dVT = dT + D * LR;             // [D][LR]    dValue_r^T[j][i]
-  float* A = dVT + D * LR;              // [kRP][D]   Sigma V^T; role 2: dA
-  float* X = A + kRP * D;               // [kRP][D]   Key_r or dKey_r
+  float* A = dVT + D * LR;              // [kRP][LA]  Sigma V^T; role 2: dA
+  float* X = A + kRP * LA;              // [kRP][D]   Key_r or dKey_r
   float* Ws = X + kRP * D;              // [D][LW]    the weight matrix in use
+  __shared__ float Ss[kRP];             // role 2: Sigma
   const int b = blockIdx.x, role = blockIdx.y, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   constexpr int VE = Vec16<T>::kElems, PCS = D * D / VE, NV = (PCS + kUserThreads - 1) / kUserThreads;
 
@@ -242,7 +244,7 @@ attn_bwd_user_kernel(const float* __restrict__ part, int chunks, const float* __
 #pragma unroll 8
     for (int e = tid; e < D * r; e += kUserThreads) {          // V is read along its rows
       const int k = e / r, i = e - k * r;
-      A[i * D + k] = ld_dep(S + (size_t)b * r + i) * ld_dep(V + (size_t)b * D * r + e);
+      A[i * LA + k] = ld_dep(S + (size_t)b * r + i) * ld_dep(V + (size_t)b * D * r + e);
     }
   };
   float* dWq = dw + (size_t)b * 3 * D * D;
@@ -256,21 +258,31 @@ attn_bwd_user_kernel(const float* __restrict__ part, int chunks, const float* __
     load_sum(dVT, 1);
     __syncthreads();
     pdl_trigger();
-    small_gemm<D>(D, r, [&](int k, int i) { return A[i * D + k]; }, [&](int i, int j) { return dVT[j * LR + i]; },
+    small_gemm<D>(D, r, [&](int k, int i) { return A[i * LA + k]; }, [&](int i, int j) { return dVT[j * LR + i]; },
                   [&](int k, int j, float v) { dWv[k * D + j] = v; }, warp, lane, kUserWarps);
     return;
   }
   fetch(role == 0 ? Wk : Wq);
   load_sum(dT, 0);
-  if (role == 2) load_sum(dVT, 1); else load_a();
+  constexpr int VR = D * kRP / kUserThreads;
+  float vreg[VR];                       // role 2: V, to lie over dT (as [D][LR]) once that has been read
+  if (role == 2) {
+    load_sum(dVT, 1);
+#pragma unroll
+    for (int n = 0; n < VR; ++n) vreg[n] = ld_dep(V + (size_t)b * D * r + min(tid + n * kUserThreads, D * r - 1));
+    if (tid < r) Ss[tid] = ld_dep(S + (size_t)b * r + tid);
+  } else {
+    load_a();
+  }
   stage();
   if (role == 2) fetch(Wk);
   // rows past r that a tile of four reads
-  for (int e = tid; e < kRP * D - r * D; e += kUserThreads) { X[r * D + e] = 0.f; A[r * D + e] = 0.f; }
+  for (int e = tid; e < kRP * D - r * D; e += kUserThreads) X[r * D + e] = 0.f;
+  for (int e = tid; e < (kRP - r) * LA; e += kUserThreads) A[r * LA + e] = 0.f;
   __syncthreads();
   if (role == 0) {
     // Key_r[i][j] = sum_k A[i][k] W_K[k][j];  dW_Q[k][j] = scale sum_i dT[k][i] Key_r[i][j]
-    small_gemm<D>(r, D, [&](int i, int k) { return A[i * D + k]; }, [&](int k, int j) { return Ws[k * LW + j]; },
+    small_gemm<D>(r, D, [&](int i, int k) { return A[i * LA + k]; }, [&](int k, int j) { return Ws[k * LW + j]; },
                   [&](int i, int j, float v) { X[i * D + j] = v; }, warp, lane, kUserWarps);
     __syncthreads();
     pdl_trigger();
@@ -285,22 +297,28 @@ attn_bwd_user_kernel(const float* __restrict__ part, int chunks, const float* __
   if (role == 1) {
     pdl_trigger();
     // dW_K[k][j] = sum_i A[i][k] dKey_r[i][j]
-    small_gemm<D>(D, r, [&](int k, int i) { return A[i * D + k]; }, [&](int i, int j) { return X[i * D + j]; },
+    small_gemm<D>(D, r, [&](int k, int i) { return A[i * LA + k]; }, [&](int i, int j) { return X[i * D + j]; },
                   [&](int k, int j, float v) { dWk[k * D + j] = v; }, warp, lane, kUserWarps);
     return;
   }
   // dA[i][k] = sum_j dKey_r[i][j] W_K[k][j] + dValue_r[i][j] W_V[k][j]
   stage();
   fetch(Wv);
+  float* Vs = dT;
+#pragma unroll
+  for (int n = 0; n < VR; ++n) {
+    const int e = tid + n * kUserThreads;
+    if (e < D * r) Vs[(e / r) * LR + e % r] = vreg[n];
+  }
   __syncthreads();
   small_gemm<D>(r, D, [&](int i, int j) { return X[i * D + j]; }, [&](int j, int k) { return Ws[k * LW + j]; },
-                [&](int i, int k, float v) { A[i * D + k] = v; }, warp, lane, kUserWarps);
+                [&](int i, int k, float v) { A[i * LA + k] = v; }, warp, lane, kUserWarps);
   __syncthreads();
   stage();
   __syncthreads();
   pdl_trigger();
   small_gemm<D>(r, D, [&](int i, int j) { return dVT[j * LR + i]; }, [&](int j, int k) { return Ws[k * LW + j]; },
-                [&](int i, int k, float v) { A[i * D + k] += v; }, warp, lane, kUserWarps);
+                [&](int i, int k, float v) { A[i * LA + k] += v; }, warp, lane, kUserWarps);
   __syncthreads();
   const float* dA = A;
   // dSigma_i = sum_k dA[i][k] V[k][i],  dV[k][i] = dA[i][k] sigma_i
@@ -308,7 +326,7 @@ attn_bwd_user_kernel(const float* __restrict__ part, int chunks, const float* __
   for (int i = warp; i < r; i += kUserWarps) {
     float acc = 0.f;
 #pragma unroll
-    for (int k = lane; k < D; k += 32) acc = fmaf(dA[i * D + k], V[((size_t)b * D + k) * r + i], acc);
+    for (int k = lane; k < D; k += 32) acc = fmaf(dA[i * LA + k], Vs[k * LR + i], acc);
 #pragma unroll
     for (int o = 16; o; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
     if (lane == 0) dS[(size_t)b * r + i] = acc;
@@ -316,7 +334,7 @@ attn_bwd_user_kernel(const float* __restrict__ part, int chunks, const float* __
 #pragma unroll 4
   for (int e = tid; e < D * r; e += kUserThreads) {
     const int k = e / r, i = e - k * r;
-    dV[(size_t)b * D * r + e] = dA[i * D + k] * S[(size_t)b * r + i];
+    dV[(size_t)b * D * r + e] = dA[i * LA + k] * Ss[i];
   }
 }
 
@@ -381,7 +399,7 @@ cudaError_t launch_td(int B, int M, int r, const void* C, const void* dO, const 
     e = launch_pdl(sum_chunks_kernel, dim3(n / 256, B), dim3(256), 0, st, part, chunks, n);
     if (e != cudaSuccess) return e;
   }
-  constexpr size_t smem_user = (size_t)(2 * D * (kRP + 1) + 2 * kRP * D + D * (D + 1)) * sizeof(float);
+  constexpr size_t smem_user = (size_t)(2 * D * (kRP + 1) + kRP * (D + 1) + kRP * D + D * (D + 1)) * sizeof(float);
   static bool limits_set[kMaxDevicesCached] = {};
   e = set_kernel_limits(reinterpret_cast<const void*>(&attn_bwd_user_kernel<T, D>), smem_user, limits_set);
   if (e != cudaSuccess) return e;
