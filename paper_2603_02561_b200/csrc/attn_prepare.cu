@@ -118,11 +118,11 @@ attn_prepare_kernel(const float* __restrict__ S, const float* __restrict__ V,
 // cores (the routine the eigensolver's epilogue uses, so a forward pass gives the same bits either
 // way).  Bound by latency: one round of global loads (weights, factors and singular values together),
 // two barriers and the chained products.  8 users, d = 64, r = 27: 14.6 us with one CTA per user and the
-// weights loaded behind the factors, 5.7 now.
+// weights loaded behind the factors, 5.7 with two of 128 threads, 5.4 of 256 (training step 97.9 -> 96.8).
 template <int D, int KINDS>
 __device__ __forceinline__ void prepare_kinds(unsigned char* smb, const float* S, const float* V, const void* Wq, const void* Wk,
                                               const void* Wv, float scale, int r, const pmma::Out& o, int b, int tid) {
-  constexpr int NT = D == 128 ? 256 : 128;
+  constexpr int NT = 256;
   const int rp = (r + 3) & ~3;
   float* VS = reinterpret_cast<float*>(smb);     // [D][rp]  V Sigma (zero in the padding)
   pmma::Weights<D, NT, KINDS> w;
@@ -140,7 +140,7 @@ __device__ __forceinline__ void prepare_kinds(unsigned char* smb, const float* S
 }
 
 template <int D>
-__global__ void __launch_bounds__(D == 128 ? 256 : 128, 1)
+__global__ void __launch_bounds__(256, 1)
 attn_prepare_mma_kernel(const float* __restrict__ S, const float* __restrict__ V, const void* __restrict__ Wq,
                         const void* __restrict__ Wk, const void* __restrict__ Wv, float scale, int r,
                         char* __restrict__ ws, AttnWs lay, int f32, __nv_bfloat16* __restrict__ bwd_pk,
@@ -170,7 +170,7 @@ cudaError_t launch_mma(int B, int r, const float* S, const float* V, const void*
   cudaError_t e = set_kernel_limits(reinterpret_cast<const void*>(&attn_prepare_mma_kernel<D>),
                                     (size_t)pmma::Lay<D>::bytes(kTokenSlots), limits_set);
   if (e != cudaSuccess) return e;
-  return launch_pdl(attn_prepare_mma_kernel<D>, dim3(B, 2), dim3(D == 128 ? 256 : 128),
+  return launch_pdl(attn_prepare_mma_kernel<D>, dim3(B, 2), dim3(256),
                     (size_t)pmma::Lay<D>::bytes((r + 15) & ~15), st, S, V, Wq, Wk, Wv, scale, r, ws, lay, (int)f32,
                     static_cast<__nv_bfloat16*>(bwd_pk), zero, zeros);
 }
