@@ -135,7 +135,7 @@ def alloc_workspace(B, M, N, d, r, dtype, device="cuda") -> torch.Tensor:
     return torch.empty(max(workspace_bytes(B, M, N, d, r, dtype), 256), dtype=torch.uint8, device=device)
 
 
-_F32, _BF16, _I32, _empty = torch.float32, torch.bfloat16, torch.int32, torch.empty
+_F32, _BF16, _I32, _empty, _empty_like = torch.float32, torch.bfloat16, torch.int32, torch.empty, torch.empty_like
 
 
 def _need(t, shape, dtype, name):
@@ -182,7 +182,7 @@ def svd_attention_fwd(C, S, V, Wq, Wk, Wv, scale, flags=0, O=None, workspace=Non
     _need(Wk, dd, dt, "Wk")
     _need(Wv, dd, dt, "Wv")
     if O is None:
-        O = _empty((B, M, d), dtype=dt, device=C.device)
+        O = _empty_like(C)
     else:
         _need(O, (B, M, d), dt, "O")
     N = N if N > r else r
@@ -209,7 +209,7 @@ def factored_softmax_attention_fwd(C, US, V, Wq, Wk, Wv, scale, O=None, workspac
     _need(Wk, dd, dt, "Wk")
     _need(Wv, dd, dt, "Wv")
     if O is None:
-        O = _empty((B, M, d), dtype=dt, device=C.device)
+        O = _empty_like(C)
     else:
         _need(O, (B, M, d), dt, "O")
     if workspace is None:
@@ -374,7 +374,7 @@ def svd_attention_fused(H, C, Wq, Wk, Wv, r, scale, flags=0, S=None, V=None, O=N
     else:
         _need(V, (B, d, r), _F32, "V")
     if O is None:
-        O = _empty((B, M, d), dtype=dt, device=dev)
+        O = _empty_like(C)
     else:
         _need(O, (B, M, d), dt, "O")
     if info is not None:
