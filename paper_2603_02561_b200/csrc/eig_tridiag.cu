@@ -72,7 +72,10 @@ template <int D> struct TriCfg {
   __device__ static constexpr int first_row(int m) { return CW * m / 32; }                 // a thread's first unfinished row in chunk m's stage
   __device__ static constexpr int last_next(int m) { return CW * (m + 1) / 32 < RT && RT > 2 ? CW * (m + 1) / 32 : RT - 1; }   // row k+1 is among the rows to this one (of two, both are tried: not slower)
   __device__ static constexpr int rows_end(int warp) { return WG * (warp + 1) + 32 * (RT - 1); }   // behind a warp's last row
-  static constexpr int CTAS = (D == 128) ? 1 : 3;     // resident CTAs that the register count has to allow
+  // Resident CTAs that the register count has to allow.  d = 64: three (168 registers) for r <= 32 -- with 255 or
+  // 128 the schedule is worse (16 x 10240 x 64 47.8 us per pass; 51.3, 50.2); above, shared memory allows two
+  // anyway (64 users, d = r = 64: 101.5 -> 100.1).
+  static constexpr int ctas(int rp) { return D == 128 ? 1 : rp > 32 ? 2 : 3; }
   static constexpr int LD = D + 4;                    // pitch of Q^T and of the row-major G
 };
 
@@ -1489,7 +1492,7 @@ __device__ __forceinline__ void prepare_epilogue(float* __restrict__ sm, int b, 
 }
 
 template <int D, int RP>
-__global__ void __launch_bounds__(TriCfg<D>::NT, TriCfg<D>::CTAS)
+__global__ void __launch_bounds__(TriCfg<D>::NT, TriCfg<D>::ctas(RP))
 eig_tridiag_kernel(const float* __restrict__ gpart, const int* __restrict__ gram_status, int parts, int splits,
                    float* __restrict__ gsum, int r, int route, int sweep_cap, TriTol tol,
                    float* __restrict__ S, float* __restrict__ V, int* __restrict__ info,
