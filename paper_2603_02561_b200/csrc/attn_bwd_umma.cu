@@ -197,7 +197,8 @@ attn_bwd_umma_kernel(const __grid_constant__ CUtensorMap tmC, const __grid_const
       const float inv = 1.f / sum;
 #pragma unroll
       for (int i = 0; i < kTokenSlots; ++i) p[i] *= inv;
-      // rowsum(P o dP): first pass over dP
+      // rowsum(P o dP): first pass over dP.  Only np columns are dP; behind them lies what another CTA left in
+      // tensor memory, a NaN perhaps, which a product with a zero probability would keep
 #pragma unroll
       for (int c0 = 0; c0 < kTokenSlots; c0 += 32) {
         if (c0 < np) {
@@ -205,7 +206,7 @@ attn_bwd_umma_kernel(const __grid_constant__ CUtensorMap tmC, const __grid_const
           ptx::tmem_ld_32x32(tmem + lane_base + kColP + c0, v);
           ptx::tmem_ld_wait();
 #pragma unroll
-          for (int i = 0; i < 32; ++i) dot = fmaf(p[c0 + i], __uint_as_float(v[i]), dot);
+          for (int i = 0; i < 32; ++i) dot = (c0 + i < r) ? fmaf(p[c0 + i], __uint_as_float(v[i]), dot) : dot;
         }
       }
     } else {
@@ -223,7 +224,7 @@ attn_bwd_umma_kernel(const __grid_constant__ CUtensorMap tmC, const __grid_const
 #pragma unroll
         for (int i = 0; i < 32; ++i) {
           const float dp = __uint_as_float(v[i]);
-          dsv[i] = use_softmax ? p[c0 + i] * (dp - dot) : ((c0 + i < r) ? dp : 0.f);
+          dsv[i] = (c0 + i < r) ? (use_softmax ? p[c0 + i] * (dp - dot) : dp) : 0.f;
         }
 #pragma unroll
         for (int c = 0; c < 4; ++c) {
@@ -323,7 +324,7 @@ attn_bwd_umma_kernel(const __grid_constant__ CUtensorMap tmC, const __grid_const
   }
   if (tid == 0) ptx::tma_store_wait_all();
 
-  // ---- the chunk's partial: [2][D][64] fp32, columns >= np zero --------------------------------
+  // ---- the chunk's partial: [2][D][64] fp32; columns >= np are not read -------------------------
   // (the last tile's wait on bar_o covered every MMA into the two accumulators)
   float* out = part + ((size_t)b * gridDim.x + chunk) * 2 * D * kTokenSlots;
   const bool good = (s_err == 0) && (t_end > t_begin);

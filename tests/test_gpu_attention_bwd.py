@@ -180,3 +180,39 @@ def test_attention_bwd_argument_checks():
     with pytest.raises(solar.SolarError) as e:
         solar.svd_attention_bwd(C, S, V, Wq, Wk, Wv, inp["scale"], dO, bws, flags=2)
     assert e.value.status == solar.ERR_UNSUPPORTED
+
+
+@pytest.mark.parametrize("d", [64, 128])
+def test_gradients_after_calls_on_non_finite_data(d):
+    """Earlier calls, and other users of the same call, leave NaN in the columns of tensor memory that a call
+    with fewer tokens does not write: its gradients are those of a run without them, bit for bit."""
+    g = torch.Generator().manual_seed(d)
+    B, M = 200, 300                                # more CTAs than the GPU holds at a time
+    C, dO = ((torch.randn(B, M, d, generator=g) * d ** -0.5).bfloat16().cuda() for _ in range(2))
+    W = [(torch.randn(d, d, generator=g) * d ** -0.5).bfloat16().cuda() for _ in range(3)]
+
+    def call(r, users, c, do):
+        h = torch.Generator().manual_seed(r)
+        V = torch.linalg.qr(torch.randn(B, d, r, generator=h))[0].contiguous().cuda()[users].contiguous()
+        S = (torch.rand(B, r, generator=h) * 4 + 1).cuda()[users].contiguous()
+        ws = solar.alloc_backward_workspace(len(users), M, r, d, r, c.dtype)
+        out = solar.svd_attention_bwd(c[users].contiguous(), S, V, *W, d ** -0.5, do[users].contiguous(), ws)
+        torch.cuda.synchronize()
+        return out
+
+    bad = torch.full_like(dO, float("nan"))
+    everyone = list(range(B))
+    for r in (1, 16, 33, 48):
+        call(64, everyone, C, dO)                  # finite everywhere
+        clean = call(r, everyone, C, dO)
+        for poison in (32, 64):
+            call(poison, everyone, C, bad)
+            got = call(r, everyone, C, dO)
+            for a, b in zip(got, clean):
+                assert torch.equal(a, b), (r, poison)      # (a NaN is not equal to itself)
+        mixed = dO.clone()
+        mixed[::3] = float("nan")                  # healthy users beside the others
+        got = call(r, everyone, C, mixed)
+        for i in (0, 4, 5):                        # dC, dS, dV are the user's own
+            for k in range(B):
+                assert k % 3 == 0 or torch.equal(got[i][k], clean[i][k]), (r, i, k)
