@@ -109,7 +109,12 @@ attn_simt_kernel(const T* __restrict__ C, T* __restrict__ O, const char* __restr
 #pragma unroll
         for (int i = 0; i < RH; ++i) p[q][i] *= inv;
       }
-    }                                     // without it: padded tokens have zero scores and zero Value_r rows
+    } else {                              // an infinite candidate times the zeros of a padded token is a NaN
+#pragma unroll
+      for (int q = 0; q < 2; ++q)
+#pragma unroll
+        for (int i = 0; i < RH; ++i) p[q][i] = i0 + i < r ? p[q][i] : 0.f;
+    }
 #pragma unroll
     for (int q = 0; q < 2; ++q)
 #pragma unroll

@@ -47,3 +47,25 @@ def test_attention_rows_and_tokens(d, dtype, flags):
             ref = P @ (A @ Wv.double())
             tol = 1e-5 if dtype == torch.float32 else 2.0 ** -8      # fp32 sums of up to 3 d products; bf16 output rounding
             assert float((O.cpu().double() - ref).abs().max()) <= tol * float(ref.abs().max()), (r, M)
+
+
+@pytest.mark.parametrize("d,dtype", [(32, torch.float32), (32, torch.bfloat16), (64, torch.float32), (128, torch.float32)])
+def test_infinite_candidates_without_softmax(d, dtype):
+    """A row with an infinity: infinite scores on the tokens there are, nothing from the padded ones."""
+    g = torch.Generator().manual_seed(d)
+    B, M = 2, 9
+    Wq, Wk, Wv = ((torch.randn(d, d, generator=g) * d ** -0.5).to(dtype) for _ in range(3))
+    for r in (1, 2, 3, 7, 8, 15):
+        C = (torch.randn(B, M, d, generator=g) * d ** -0.5).to(dtype)
+        C[0, 4, 5] = float("inf")
+        C[1, 0, 0] = -float("inf")
+        V = torch.linalg.qr(torch.randn(B, d, r, generator=g))[0].contiguous()
+        S = torch.rand(B, r, generator=g) * 10 + 1
+        O = solar.svd_attention_fwd(*(t.cuda() for t in (C, S, V, Wq, Wk, Wv)), d ** -0.5, solar.FLAG_NO_SOFTMAX).cpu()
+        A = (V.double() * S.double()[:, None]).transpose(1, 2)
+        P = C.double() @ (d ** -0.5 * Wq.double() @ (A @ Wk.double()).transpose(1, 2))       # scores through T
+        ref = P @ (A @ Wv.double())
+        assert torch.equal(torch.isnan(O), torch.isnan(ref)), r
+        assert torch.equal(torch.isinf(O), torch.isinf(ref)), r
+        assert torch.equal(O[torch.isinf(O)] > 0, ref[torch.isinf(ref)] > 0), r
+        assert r > 2 or bool(torch.isinf(O).any()), r
