@@ -182,9 +182,10 @@ solar_status_t solar_svd_attention_fused(int B, int M, int N, int d, int r, sola
  * bits in O -- and the eigensolver releases it a little later; together 7.6 us per request in
  * flight and about 100 us for a lone call.
  * Results agree to rounding (the partial sums are grouped differently), not bit for bit.
- * Set it before sizing workspaces: the *_workspace_bytes functions follow the current value,
- * and a call made under a higher cap than its workspace was sized for returns
- * SOLAR_ERR_WORKSPACE.  Keep it unchanged between a stage call that writes a workspace
+ * Set it before sizing workspaces: the *_workspace_bytes functions follow the current value.  A
+ * workspace sized without a cap serves every cap, one sized under a cap that cap and smaller ones;
+ * a call made under a higher cap whose workspace is too small for it returns SOLAR_ERR_WORKSPACE.
+ * A call reads the cap once, when it is made.  Keep it unchanged between a stage call that writes a workspace
  * (solar_gram_partials) and the stage calls that read it.  Returns the previous value.  Safe to
  * call from any thread; calls already enqueued are not affected. */
 int solar_set_slice_limit(int max_slices);
@@ -337,9 +338,9 @@ solar_status_t solar_factored_softmax_attention_fwd(int B, int M, int N, int d, 
  *   - Same arguments, outputs, info bits and rules as solar_lowrank_factor,
  *     minus US and the workspace.  Calls no cudaMalloc / cudaFree and no
  *     allocating library routine.
- *   - Sizes whose scratch need, solar_workspace_bytes(B, 0, N, d, r, dt) bytes,
- *     exceeds the array return SOLAR_ERR_WORKSPACE before anything is launched
- *     (the headline shape B=16, N=10240, d=64 needs 2.25 MiB).
+ *   - Sizes whose scratch need, at most solar_workspace_bytes(B, 0, N, d, r, dt)
+ *     bytes, exceeds the array return SOLAR_ERR_WORKSPACE before anything is
+ *     launched (the headline shape B=16, N=10240, d=64 needs 2.25 MiB).
  *   - The first call on each device looks up the array's device address (with
  *     that device current) and caches it; make that first call outside any
  *     stream capture.  The array is chosen by the CURRENT device: the device

@@ -53,8 +53,23 @@ solar_status_t attn_apply_impl(int B, int M, int d, int r, solar_dtype_t dt, con
   return from_cuda(launch_attn_simt(B, M, d, r, dt, C, flags, O, ws, attn_ws_layout(d, r), early_c, st));
 }
 
-// Workspace of the fused forward call: the factorization's, then the attention's.
-size_t fused_attn_offset(int B, int N, int d, solar_dtype_t dt) { return align_up(factor_ws_bytes(B, N, d, dt), 256); }
+// The streaming pass and the eigensolve of one call, on a workspace laid out by `plan`.
+solar_status_t gram_impl(int B, int N, int d, solar_dtype_t dt, const void* H, void* workspace, const GramPlan& plan,
+                         cudaStream_t st) {
+  float* gpart = static_cast<float*>(workspace);
+  int* status = reinterpret_cast<int*>(static_cast<char*>(workspace) + gram_status_offset(B, d, plan));
+  if (gram_umma_supported(N, d, dt)) return from_cuda(launch_gram_umma(B, N, d, H, gpart, status, plan, st));
+  return from_cuda(launch_gram_simt(B, N, d, dt, H, gpart, status, plan, st));
+}
+
+solar_status_t eig_impl(int B, int d, int r, solar_dtype_t dt, int route, int sweep_cap, int force_iters, float* S,
+                        float* V, int* info, int* route_taken, void* workspace, const GramPlan& plan, cudaStream_t st) {
+  char* ws = static_cast<char*>(workspace);
+  const int* status = reinterpret_cast<const int*>(ws + gram_status_offset(B, d, plan));
+  float* gsum = reinterpret_cast<float*>(ws + gram_sum_offset(B, d, plan));
+  return from_cuda(launch_eig(B, d, r, dt, route, sweep_cap, force_iters, reinterpret_cast<const float*>(ws), status,
+                              plan.parts, plan.splits, gsum, S, V, info, route_taken, st));
+}
 
 }  // namespace
 
@@ -73,7 +88,7 @@ const char* solar_status_string(solar_status_t st) {
 
 size_t solar_workspace_bytes(int B, int M, int N, int d, int r, solar_dtype_t dt) {
   if (check_dims(B, M, N, d, r, dt) != SOLAR_OK) return 0;
-  const size_t f = factor_ws_bytes(B, N, d, dt), a = attn_ws_bytes(B, d, r);
+  const size_t f = factor_ws_reserve(B, N, d, slice_limit()), a = attn_ws_bytes(B, d, r);
   const size_t need = f > a ? f : a;
   return need ? need : 256;
 }
@@ -85,12 +100,12 @@ int solar_set_slice_limit(int max_slices) {
 
 int solar_gram_splits(int B, int N, int d, solar_dtype_t dt) {
   if (check_dims(B, 0, N, d, 1, dt) != SOLAR_OK) return 0;
-  return gram_plan(B, N, gram_cluster_limit(N, d, dt)).parts;
+  return gram_plan(B, N, d, dt, slice_limit()).parts;
 }
 
 int solar_gram_slices(int B, int N, int d, solar_dtype_t dt) {
   if (check_dims(B, 0, N, d, 1, dt) != SOLAR_OK) return 0;
-  return gram_plan(B, N, gram_cluster_limit(N, d, dt)).splits;
+  return gram_plan(B, N, d, dt, slice_limit()).splits;
 }
 
 solar_status_t solar_gram_partials(int B, int N, int d, solar_dtype_t dt, const void* H,
@@ -98,13 +113,9 @@ solar_status_t solar_gram_partials(int B, int N, int d, solar_dtype_t dt, const 
   SOLAR_TRY(check_dims(B, 0, N, d, 1, dt));
   if (B == 0) return SOLAR_OK;
   SOLAR_TRY(check_ptr(H));
-  SOLAR_TRY(check_ws(workspace, workspace_bytes, factor_ws_bytes(B, N, d, dt)));
-  const GramPlan plan = gram_plan(B, N, gram_cluster_limit(N, d, dt));
-  float* gpart = static_cast<float*>(workspace);
-  int* status = reinterpret_cast<int*>(static_cast<char*>(workspace) + gram_status_offset(B, N, d, dt));
-  const cudaStream_t st = static_cast<cudaStream_t>(stream);
-  if (gram_umma_supported(N, d, dt)) return from_cuda(launch_gram_umma(B, N, d, H, gpart, status, plan, st));
-  return from_cuda(launch_gram_simt(B, N, d, dt, H, gpart, status, plan, st));
+  const GramPlan plan = gram_plan(B, N, d, dt, slice_limit());
+  SOLAR_TRY(check_ws(workspace, workspace_bytes, factor_ws_bytes(B, d, plan)));
+  return gram_impl(B, N, d, dt, H, workspace, plan, static_cast<cudaStream_t>(stream));
 }
 
 solar_status_t solar_eig_from_partials_ex(int B, int N, int d, int r, solar_dtype_t dt, int route,
@@ -119,14 +130,10 @@ solar_status_t solar_eig_from_partials_ex(int B, int N, int d, int r, solar_dtyp
   if (info != nullptr && (reinterpret_cast<uintptr_t>(info) & 3u)) return SOLAR_ERR_INVALID_ARG;
   if (route_taken != nullptr && (reinterpret_cast<uintptr_t>(route_taken) & 3u))
     return SOLAR_ERR_INVALID_ARG;
-  SOLAR_TRY(check_ws(workspace, workspace_bytes, factor_ws_bytes(B, N, d, dt)));
-  const GramPlan plan = gram_plan(B, N, gram_cluster_limit(N, d, dt));
-  const int* status =
-      reinterpret_cast<const int*>(static_cast<const char*>(workspace) + gram_status_offset(B, N, d, dt));
-  float* gsum = reinterpret_cast<float*>(static_cast<char*>(workspace) + gram_sum_offset(B, N, d, dt));
-  return from_cuda(launch_eig(B, d, r, dt, base_route, sweep_cap, force_iters, static_cast<const float*>(workspace),
-                              status, plan.parts, plan.splits, gsum, S, V, info, route_taken,
-                              static_cast<cudaStream_t>(stream)));
+  const GramPlan plan = gram_plan(B, N, d, dt, slice_limit());
+  SOLAR_TRY(check_ws(workspace, workspace_bytes, factor_ws_bytes(B, d, plan)));
+  return eig_impl(B, d, r, dt, base_route, sweep_cap, force_iters, S, V, info, route_taken, workspace, plan,
+                  static_cast<cudaStream_t>(stream));
 }
 
 solar_status_t solar_eig_from_partials(int B, int N, int d, int r, solar_dtype_t dt, float* S,
@@ -157,10 +164,12 @@ solar_status_t solar_lowrank_factor(int B, int M, int N, int d, int r, solar_dty
   SOLAR_TRY(check_ptr(V));
   if (US != nullptr) SOLAR_TRY(check_ptr(US));
   if (info != nullptr && (reinterpret_cast<uintptr_t>(info) & 3u)) return SOLAR_ERR_INVALID_ARG;
-  SOLAR_TRY(check_ws(workspace, workspace_bytes, factor_ws_bytes(B, N, d, dt)));
-  SOLAR_TRY(solar_gram_partials(B, N, d, dt, H, workspace, workspace_bytes, stream));
-  SOLAR_TRY(solar_eig_from_partials(B, N, d, r, dt, S, V, info, workspace, workspace_bytes, stream));
-  if (US != nullptr) SOLAR_TRY(from_cuda(launch_project_us(B, N, d, r, dt, H, V, US, true, static_cast<cudaStream_t>(stream))));
+  const GramPlan plan = gram_plan(B, N, d, dt, slice_limit());
+  SOLAR_TRY(check_ws(workspace, workspace_bytes, factor_ws_bytes(B, d, plan)));
+  const cudaStream_t st = static_cast<cudaStream_t>(stream);
+  SOLAR_TRY(gram_impl(B, N, d, dt, H, workspace, plan, st));
+  SOLAR_TRY(eig_impl(B, d, r, dt, SOLAR_ROUTE_AUTO, 0, 0, S, V, info, nullptr, workspace, plan, st));
+  if (US != nullptr) SOLAR_TRY(from_cuda(launch_project_us(B, N, d, r, dt, H, V, US, true, st)));
   return SOLAR_OK;
 }
 
@@ -219,7 +228,7 @@ solar_status_t solar_svd_attention_fwd(int B, int M, int N, int d, int r, solar_
 
 size_t solar_fused_workspace_bytes(int B, int M, int N, int d, int r, solar_dtype_t dt) {
   if (check_dims(B, M, N, d, r, dt) != SOLAR_OK) return 0;
-  return fused_attn_offset(B, N, d, dt) + align_up(attn_ws_bytes(B, d, r), 256);
+  return align_up(factor_ws_reserve(B, N, d, slice_limit()), 256) + align_up(attn_ws_bytes(B, d, r), 256);
 }
 
 solar_status_t solar_svd_attention_fused(int B, int M, int N, int d, int r, solar_dtype_t dt,
@@ -238,16 +247,18 @@ solar_status_t solar_svd_attention_fused(int B, int M, int N, int d, int r, sola
   SOLAR_TRY(check_ptr(Wv));
   if (M > 0) { SOLAR_TRY(check_ptr(C)); SOLAR_TRY(check_ptr(O)); }
   if (info != nullptr && (reinterpret_cast<uintptr_t>(info) & 3u)) return SOLAR_ERR_INVALID_ARG;
-  SOLAR_TRY(check_ws(workspace, workspace_bytes, solar_fused_workspace_bytes(B, M, N, d, r, dt)));
+  // the factorization's workspace, then the attention's
+  const GramPlan plan = gram_plan(B, N, d, dt, slice_limit());
+  const size_t attn_off = align_up(factor_ws_bytes(B, d, plan), 256);
+  SOLAR_TRY(check_ws(workspace, workspace_bytes, attn_off + align_up(attn_ws_bytes(B, d, r), 256)));
   const cudaStream_t st = static_cast<cudaStream_t>(stream);
   char* ws = static_cast<char*>(workspace);
-  char* attn_ws = ws + fused_attn_offset(B, N, d, dt);
+  char* attn_ws = ws + attn_off;
   // streaming pass over H (the first kernel of the call: it waits for what ran before)
-  SOLAR_TRY(solar_gram_partials(B, N, d, dt, H, workspace, factor_ws_bytes(B, N, d, dt), stream));
+  SOLAR_TRY(gram_impl(B, N, d, dt, H, workspace, plan, st));
   // eigensolve; every user's CTA ends with that user's factor-token projections
-  const GramPlan plan = gram_plan(B, N, gram_cluster_limit(N, d, dt));
-  const int* status = reinterpret_cast<const int*>(ws + gram_status_offset(B, N, d, dt));
-  float* gsum = reinterpret_cast<float*>(ws + gram_sum_offset(B, N, d, dt));
+  const int* status = reinterpret_cast<const int*>(ws + gram_status_offset(B, d, plan));
+  float* gsum = reinterpret_cast<float*>(ws + gram_sum_offset(B, d, plan));
   const EigFuse fuse = {Wq, Wk, Wv, scale, attn_ws};
   SOLAR_TRY(from_cuda(launch_eig_tridiag(B, d, r, dt, SOLAR_ROUTE_AUTO, kMaxSweeps, reinterpret_cast<const float*>(ws),
                                          status, plan.parts, plan.splits, gsum, S, V, info, nullptr, &fuse, st)));

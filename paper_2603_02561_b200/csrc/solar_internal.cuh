@@ -37,15 +37,15 @@ inline long slice_cost(int B, int tiles, int s, int* s_eff_out, int* chunk_out) 
   return waves * (chunk + 2);
 }
 
-// Process-wide cap on the slices per user (solar_set_slice_limit; 0 = none).
+// Process-wide cap on the slices per user (solar_set_slice_limit; 0 = none).  It may change at any time: a
+// call reads it once for its Gram plan, which everything about the factorization's workspace follows.
 int slice_limit();
 
-inline GramPlan slice_plan(int B, int N) {
+inline GramPlan slice_plan(int B, int N, int cap) {
   GramPlan p;
   p.tiles = (N + kGramTileRows - 1) / kGramTileRows;
   long best_cost = -1;
   int smax = p.tiles < kMaxSplits ? p.tiles : kMaxSplits;
-  const int cap = slice_limit();
   if (cap > 0 && cap < smax) smax = cap;
   p.splits = 1; p.chunk_tiles = p.tiles;
   for (int s = 1; s <= smax; ++s) {
@@ -58,7 +58,7 @@ inline GramPlan slice_plan(int B, int N) {
   return p;
 }
 
-// The plan of the tensor-core Gram kernel.  Its CTAs can form thread-block clusters of slices of a user
+// The plan of the Gram pass.  The tensor-core kernel's CTAs can form thread-block clusters of slices of a user
 // that add up their accumulators through distributed shared memory, so that a user leaves splits /
 // cluster partial matrices, which the one CTA of the eigensolver reads.
 //   d = 64 (16 KB a matrix): no clusters.  On the headline shape (B = 16, N = 10240: nine slices), clusters
@@ -69,14 +69,11 @@ inline GramPlan slice_plan(int B, int N) {
 // eigensolver's CTA reads a matrix at 44 bytes a clock, and 16 of them are 12 us of a pass over 8 x 16384 x
 // 128 (four: 3 us; the Gram kernel 9.6 -> 11.1 us, with clusters of eight 19.8).
 constexpr int kMaxCluster = 4;
-inline int gram_cluster_limit(int N, int d, solar_dtype_t dt) {      // 0: not the tensor-core kernel's shape
-  if (dt != SOLAR_BF16 || (d != 64 && d != 128) || N < kGramTileRows) return 0;
-  return d == 128 && slice_limit() == 0 ? kMaxCluster : 1;
-}
-inline GramPlan gram_plan(int B, int N, int cluster_limit) {
-  GramPlan p = slice_plan(B, N);
+inline GramPlan gram_plan(int B, int N, int d, solar_dtype_t dt, int cap) {
+  GramPlan p = slice_plan(B, N, cap);
+  const bool clusters = dt == SOLAR_BF16 && d == 128 && N >= kGramTileRows && cap == 0;
   // the largest cluster size within the limit that divides the slice count
-  for (int c = 2; c <= cluster_limit; ++c)
+  for (int c = 2; clusters && c <= kMaxCluster; ++c)
     if (p.splits % c == 0) p.cluster = c;
   p.parts = p.splits / p.cluster;
   return p;
@@ -86,19 +83,22 @@ inline GramPlan gram_plan(int B, int N, int cluster_limit) {
 // (user, slice), written by every Gram CTA: kGramStatusOk, or the code of the bounded
 // device-side wait that ran out.
 constexpr int kGramStatusOk = 0x600D;
-inline size_t gram_status_offset(int B, int N, int d, solar_dtype_t dt) {
-  const GramPlan p = gram_plan(B, N, gram_cluster_limit(N, d, dt));
+inline size_t gram_status_offset(int B, int d, const GramPlan& p) {
   return align_up((size_t)B * p.parts * d * d * sizeof(float), 256);
 }
 // Behind the status words: the summed Gram matrices [B][d][d] fp32, written by the eigensolver
 // when a user has more than one partial (its residual check and its Jacobi fallback read the
 // sum back; a single partial is the sum).
-inline size_t gram_sum_offset(int B, int N, int d, solar_dtype_t dt) {
-  const GramPlan p = gram_plan(B, N, gram_cluster_limit(N, d, dt));
-  return gram_status_offset(B, N, d, dt) + align_up((size_t)B * p.splits * sizeof(int), 256);
+inline size_t gram_sum_offset(int B, int d, const GramPlan& p) {
+  return gram_status_offset(B, d, p) + align_up((size_t)B * p.splits * sizeof(int), 256);
 }
-inline size_t factor_ws_bytes(int B, int N, int d, solar_dtype_t dt) {
-  return gram_sum_offset(B, N, d, dt) + align_up((size_t)B * d * d * sizeof(float), 256);
+inline size_t factor_ws_bytes(int B, int d, const GramPlan& p) {
+  return gram_sum_offset(B, d, p) + align_up((size_t)B * d * d * sizeof(float), 256);
+}
+// What callers are told to reserve: a partial for every slice, so that the workspace is large enough under any
+// smaller cap too, where the slices are fewer but each leaves its own.
+inline size_t factor_ws_reserve(int B, int N, int d, int cap) {
+  return factor_ws_bytes(B, d, slice_plan(B, N, cap));
 }
 
 // Workspace of the attention call, per user (all segments 256-byte aligned):

@@ -139,3 +139,32 @@ def test_slice_limit_is_a_host_side_setting():
         assert L.solar_gram_slices(16, 10240, 64, solar.BF16) == n0
     finally:
         L.solar_set_slice_limit(old)
+
+
+@pytest.mark.parametrize("d,dtype", [(32, solar.F32), (64, solar.BF16), (64, solar.F32), (128, solar.BF16), (128, solar.F32)])
+def test_a_workspace_sized_without_a_limit_serves_every_limit(L, d, dtype):
+    """The sizes fall with the limit, and the size without one holds what each limit's plan lays down."""
+    old = L.solar_set_slice_limit(0)
+    limits = (0, 64, 33, 16, 9, 8, 7, 5, 4, 3, 2, 1)
+    vp = ctypes.c_void_p
+    p = vp(0x1000)
+    try:
+        for B in (1, 2, 3, 8, 16, 24, 32, 37, 48, 64, 74, 150):
+            for N in (100, 128, 1000, 5000, 8192, 16384, 50000):
+                for bytes_of in (L.solar_workspace_bytes, L.solar_fused_workspace_bytes):
+                    sizes = []
+                    for lim in limits:
+                        L.solar_set_slice_limit(lim)
+                        sizes.append(bytes_of(B, 8, N, d, 16, dtype))
+                    assert sizes == sorted(sizes, reverse=True), (B, N, sizes)
+                L.solar_set_slice_limit(0)
+                size, fused = L.solar_workspace_bytes(B, 8, N, d, 16, dtype), L.solar_fused_workspace_bytes(B, 8, N, d, 16, dtype)
+                for lim in limits:
+                    L.solar_set_slice_limit(lim)
+                    need = B * L.solar_gram_splits(B, N, d, dtype) * d * d * 4
+                    assert need + B * d * d * 4 <= size < fused, (B, N, lim)
+                    # one byte less than the partials take: refused before anything is launched
+                    args = (B, N, d, dtype, p, p, need - 1, None)
+                    assert L.solar_gram_partials(*args) == solar.ERR_WORKSPACE, (B, N, lim)
+    finally:
+        L.solar_set_slice_limit(old)

@@ -175,3 +175,65 @@ def test_throughput_attention_kernel_gives_the_same_bits(M, r, flags):
         del O1, guard
     finally:
         solar.set_slice_limit(old)
+
+
+def _wide_case():
+    g = torch.Generator().manual_seed(5)
+    B, N, d, r, M = 8, 8192, 128, 16, 130
+    H = (torch.randn(B, N, r, generator=g) @ torch.randn(B, r, d, generator=g) + 0.1 * torch.randn(B, N, d, generator=g)).bfloat16().cuda()
+    C = (torch.randn(B, M, d, generator=g) * d ** -0.5).bfloat16().cuda()
+    W = [(torch.randn(d, d, generator=g) * d ** -0.5).bfloat16().cuda() for _ in range(3)]
+    return (B, M, N, d, r, torch.bfloat16), H, C, W, r, d ** -0.5
+
+
+def test_default_workspace_under_a_slice_limit():
+    """Workspaces sized without a limit, at d = 128, where a limit means more partial matrices."""
+    size, H, C, W, r, scale = _wide_case()
+    old = solar.set_slice_limit(0)
+    try:
+        fused, two = solar.alloc_fused_workspace(*size), solar.alloc_workspace(*size)
+        O0, S0, V0 = solar.svd_attention_fused(H, C, *W, r, scale, workspace=fused)
+        for limit in (1, 2, 3, 8, 13, 64):
+            solar.set_slice_limit(limit)
+            fused.fill_(0xFF); two.fill_(0xFF)
+            O, S, V = solar.svd_attention_fused(H, C, *W, r, scale, workspace=fused)
+            S2, V2 = solar.lowrank_factor(H, r, workspace=two)
+            torch.cuda.synchronize()
+            assert torch.equal(S, S2) and torch.equal(V, V2), limit
+            # the same sums of N products in another grouping: about sqrt(N) roundings of 2^-24 of theta_1
+            assert float((S - S0).abs().max()) <= 1e-5 * float(S0.max()), limit
+            assert float((O - O0).float().abs().max()) <= 2.0 ** -6 * float(O0.float().abs().max()), limit
+    finally:
+        solar.set_slice_limit(old)
+
+
+def test_slice_limit_changed_by_another_thread():
+    """Calls on default-sized workspaces while the limit flips: each gives the bits of one setting."""
+    import threading
+    size, H, C, W, r, scale = _wide_case()
+    old = solar.set_slice_limit(0)
+    stop = threading.Event()
+
+    def flip():
+        while not stop.is_set():
+            solar.set_slice_limit(2)
+            solar.set_slice_limit(0)
+
+    try:
+        want = []
+        for limit in (0, 2):
+            solar.set_slice_limit(limit)
+            want.append(solar.svd_attention_fused(H, C, *W, r, scale))
+        torch.cuda.synchronize()
+        solar.set_slice_limit(0)
+        wss = [solar.alloc_fused_workspace(*size).fill_(0xFF) for _ in range(20)]
+        t = threading.Thread(target=flip)
+        t.start()
+        got = [solar.svd_attention_fused(H, C, *W, r, scale, workspace=ws) for ws in wss for _ in range(10)]
+        stop.set(); t.join()
+        torch.cuda.synchronize()
+        for x in got:
+            assert any(all(torch.equal(a, b) for a, b in zip(x, y)) for y in want)
+    finally:
+        stop.set()
+        solar.set_slice_limit(old)
