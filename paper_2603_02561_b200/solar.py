@@ -135,12 +135,19 @@ def alloc_workspace(B, M, N, d, r, dtype, device="cuda") -> torch.Tensor:
     return torch.empty(max(workspace_bytes(B, M, N, d, r, dtype), 256), dtype=torch.uint8, device=device)
 
 
-_F32, _BF16, _I32, _empty, _empty_like = torch.float32, torch.bfloat16, torch.int32, torch.empty, torch.empty_like
+_F32, _I32, _empty, _empty_like = torch.float32, torch.int32, torch.empty, torch.empty_like
 
 
 def _need(t, shape, dtype, name):
     if t.dtype is not dtype or t.shape != shape or not t.is_contiguous() or not t.is_cuda:
         raise ValueError(f"{name}: want contiguous CUDA {dtype} {tuple(shape)}, got {t.dtype} {tuple(t.shape)}")
+
+
+# The backward calls pass a missing tensor on as NULL, which the library refuses, and take any shape of enough
+# elements; what they cannot see is a tensor that is too small, of another type, strided or not on the GPU.
+def _need_buf(t, n, dtype, name):
+    if t is not None and n and (t.dtype is not dtype or t.numel() < n or not t.is_contiguous() or not t.is_cuda):
+        raise ValueError(f"{name}: want contiguous CUDA {dtype} of {n} elements, got {t.dtype} {tuple(t.shape)}")
 
 
 def lowrank_factor(H, r, S=None, V=None, US=None, info=None, workspace=None, M=0, stream=None):
@@ -294,8 +301,14 @@ def svd_attention_bwd(C, S, V, Wq, Wk, Wv, scale, dO, workspace, flags=0, out=No
     Returns dC[B,M,d], dWq, dWk, dWv [d,d] f32, dS[B,r], dV[B,d,r] (written into `out` if given)."""
     B, M, d = C.shape
     r = S.shape[1]
-    dt = C.dtype
+    dt, dd = C.dtype, d * d
+    _need_buf(C, B * M * d, dt, "C")
     _need(dO, (B, M, d), dt, "dO")
+    _need_buf(S, B * r, _F32, "S")
+    _need_buf(V, B * d * r, _F32, "V")
+    _need_buf(Wq, dd, dt, "Wq")
+    _need_buf(Wk, dd, dt, "Wk")
+    _need_buf(Wv, dd, dt, "Wv")
     if out is None:
         out = alloc_attention_grads(C, r)
         dC, dWq, dWk, dWv, dS, dV = out
@@ -307,8 +320,8 @@ def svd_attention_bwd(C, S, V, Wq, Wk, Wv, scale, dO, workspace, flags=0, out=No
         for nm, W in (("dWq", dWq), ("dWk", dWk), ("dWv", dWv)):
             _need(W, (d, d), _F32, nm)
     st = (_lib or lib()).solar_svd_attention_bwd(
-        B, M, r if r > 1 else 1, d, r, dtype_code(dt), C.data_ptr(), S.data_ptr(), V.data_ptr(), Wq.data_ptr(),
-        Wk.data_ptr(), Wv.data_ptr(), float(scale), int(flags), dO.data_ptr(), dC.data_ptr(), dWq.data_ptr(),
+        B, M, r if r > 1 else 1, d, r, dtype_code(dt), C.data_ptr(), S.data_ptr(), _ptr(V), _ptr(Wq),
+        _ptr(Wk), _ptr(Wv), float(scale), int(flags), dO.data_ptr(), dC.data_ptr(), dWq.data_ptr(),
         dWk.data_ptr(), dWv.data_ptr(), dS.data_ptr(), dV.data_ptr(), workspace.data_ptr(), workspace.numel(),
         _stream(stream))
     if st:
@@ -320,9 +333,16 @@ def svd_backward(H, S, V, dS, dV, dH, workspace, eps_rel=0.0, stream=None):
     """dH = U [diag(dS) + 2 Sigma sym(F o (dV^T V))] V^T with U = H V Sigma^-1 (Eq. 13-15)."""
     B, N, d = H.shape
     r = V.shape[2]
-    st = (_lib or lib()).solar_svd_backward(B, N, d, r, dtype_code(H.dtype), H.data_ptr(), S.data_ptr(), V.data_ptr(),
-                                            dS.data_ptr(), dV.data_ptr(), float(eps_rel), dH.data_ptr(),
-                                            workspace.data_ptr(), workspace.numel(), _stream(stream))
+    dt, n = H.dtype, B * d * r
+    _need_buf(H, B * N * d, dt, "H")
+    _need_buf(S, B * r, _F32, "S")
+    _need_buf(V, n, _F32, "V")
+    _need_buf(dS, B * r, _F32, "dS")
+    _need_buf(dV, n, _F32, "dV")
+    _need_buf(dH, B * N * d, dt, "dH")
+    st = (_lib or lib()).solar_svd_backward(B, N, d, r, dtype_code(dt), H.data_ptr(), _ptr(S), V.data_ptr(), _ptr(dS),
+                                            _ptr(dV), float(eps_rel), _ptr(dH), workspace.data_ptr(), workspace.numel(),
+                                            _stream(stream))
     if st:
         _check(st, "solar_svd_backward")
 
