@@ -22,10 +22,15 @@ constexpr int kPrepThreads = 512;
 // Stages W[D][D] (storage type T) as fp32 in shared memory.
 template <typename T, int D>
 __device__ __forceinline__ void stage_weight(const T* __restrict__ W, float* __restrict__ Ws, int tid) {
-  constexpr int VE = Vec16<T>::kElems;
-  for (int v = tid; v < D * D / VE; v += kPrepThreads) {
+  constexpr int VE = Vec16<T>::kElems, PCS = D * D / VE, NV = (PCS + kPrepThreads - 1) / kPrepThreads;
+  uint4 raw[NV];
+#pragma unroll
+  for (int n = 0; n < NV; ++n) raw[n] = ld_dep(reinterpret_cast<const uint4*>(W) + min(tid + n * kPrepThreads, PCS - 1));
+#pragma unroll
+  for (int n = 0; n < NV; ++n) {
+    const int v = min(tid + n * kPrepThreads, PCS - 1);
     float tmp[VE];
-    Vec16<T>::load(W + (size_t)v * VE, tmp);
+    Vec16<T>::load(reinterpret_cast<const T*>(&raw[n]), tmp);
 #pragma unroll
     for (int e = 0; e < VE; ++e) Ws[v * VE + e] = tmp[e];
   }
@@ -53,9 +58,11 @@ attn_prepare_kernel(const float* __restrict__ S, const float* __restrict__ V,
   pdl_wait();
   stage_weight<T, D>(role == 0 ? Wk : Wv, Ws, tid);
   if (role == 0) stage_weight<T, D>(Wq, Wq_s, tid);
+#pragma unroll 4
   for (int e = tid; e < D * rp; e += kPrepThreads) {
-    const int k = e / rp, i = e % rp;
-    VS[e] = i < r ? V[((size_t)b * D + k) * r + i] * (S != nullptr ? S[(size_t)b * r + i] : 1.f) : 0.f;
+    const int k = e / rp, i = e - k * rp, ic = min(i, r - 1);
+    const float v = ld_dep(V + ((size_t)b * D + k) * r + ic), s = S != nullptr ? ld_dep(S + (size_t)b * r + ic) : 1.f;
+    VS[e] = i < r ? v * s : 0.f;
   }
   __syncthreads();
   pdl_trigger();       // the next kernel may start launching while the products run

@@ -43,8 +43,9 @@ attn_simt_kernel(const T* __restrict__ C, T* __restrict__ O, const char* __restr
   const T* Cb = C + ((size_t)b * M + m0) * D;
 #pragma unroll 4
   for (int v = tid; v < rows * VPR; v += kRows) {
+    const uint4 raw = ld_dep(reinterpret_cast<const uint4*>(Cb) + v);
     float x[VE];
-    Vec16<T>::load(Cb + (size_t)v * VE, x);
+    Vec16<T>::load(reinterpret_cast<const T*>(&raw), x);
     float* dst = Cs + (v / VPR) * LC + (v % VPR) * VE;
 #pragma unroll
     for (int e = 0; e < VE; e += 4) *reinterpret_cast<float4*>(dst + e) = make_float4(x[e], x[e + 1], x[e + 2], x[e + 3]);

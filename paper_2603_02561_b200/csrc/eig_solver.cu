@@ -354,7 +354,7 @@ eig_kernel(const float* __restrict__ gpart, const int* __restrict__ gram_status,
   const float4* gp = reinterpret_cast<const float4*>(gpart + (size_t)b * parts * D * D);
   // a Gram CTA whose bounded wait ran out leaves a code other than kGramStatusOk
   int lost = 0;
-  for (int s = tid; s < splits; s += NT) lost |= (gram_status[b * splits + s] != kGramStatusOk);
+  for (int s = tid; s < splits; s += NT) lost |= (ld_dep(gram_status + b * splits + s) != kGramStatusOk);
   int bad = 0;
   for (int e = tid; e < D * D / 4; e += NT) {
     // fp32 sums in a fixed order (GW slices at a time, pairwise within the group): the
@@ -366,7 +366,7 @@ eig_kernel(const float* __restrict__ gpart, const int* __restrict__ gram_status,
       float4 v[GW];
 #pragma unroll
       for (int u = 0; u < GW; ++u)
-        v[u] = (s + u < parts) ? __ldg(gp + (size_t)(s + u) * (D * D / 4) + e)
+        v[u] = (s + u < parts) ? ld_dep(gp + (size_t)(s + u) * (D * D / 4) + e)
                                 : make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
       for (int h = GW / 2; h >= 1; h >>= 1)

@@ -1176,7 +1176,7 @@ __device__ __forceinline__ EigEnd eig_user(int b, int half, bool& joined, const 
   {
     const float4* gp = reinterpret_cast<const float4*>(gpart + (size_t)b * parts * D * D);
     int lost = 0;
-    for (int s = tid; s < splits; s += NT) lost |= (gram_status[b * splits + s] != kGramStatusOk);
+    for (int s = tid; s < splits; s += NT) lost |= (ld_dep(gram_status + b * splits + s) != kGramStatusOk);
     // fp32 sums in slice order; the loads of SCN slices are issued before the first add: the
     // phase is bound by their latency
     constexpr int SCN = RT * NCH >= 16 ? 2 : RT * NCH >= 8 ? 3 : 8;
@@ -1267,7 +1267,10 @@ __device__ __forceinline__ EigEnd eig_user(int b, int half, bool& joined, const 
 #pragma unroll
       for (int rr = 0; rr < RT; ++rr)
 #pragma unroll
-        for (int m = 0; m < NCH; ++m) ld4(gout + (row0 + 32 * rr) * D + CW * m + 4 * g, acc[rr][m]);
+        for (int m = 0; m < NCH; ++m) {
+          const float4 t = ld_dep(reinterpret_cast<const float4*>(gout + (row0 + 32 * rr) * D + CW * m + 4 * g));
+          acc[rr][m][0] = t.x; acc[rr][m][1] = t.y; acc[rr][m][2] = t.z; acc[rr][m][3] = t.w;
+        }
       wide = 1;
       ok = tri_chain<double, D, RP>(acc, smem, sh, gout, sc, r, false, tol, false, half, not_mine, Vc, passes, tid);
       if (not_mine) return kOtherHalf;
@@ -1322,7 +1325,7 @@ __device__ __forceinline__ EigEnd eig_user(int b, int half, bool& joined, const 
 
   // ---- last resort (or the caller's choice): Jacobi on the whole matrix ----------------------------
   for (int e = tid; e < D * D / 4; e += NT) {
-    float4 t = reinterpret_cast<const float4*>(gout)[e];
+    float4 t = ld_dep(reinterpret_cast<const float4*>(gout) + e);
     t.x *= sc; t.y *= sc; t.z *= sc; t.w *= sc;
     *reinterpret_cast<float4*>(smem + (e / (D / 4)) * LD + (e % (D / 4)) * 4) = t;
   }
@@ -1350,7 +1353,7 @@ struct FuseArgs {
 // Four consecutive elements of a weight matrix as fp32.
 __device__ __forceinline__ float4 weight4(const void* __restrict__ W, int mode, int e4) {
   if (mode != 1) return ld_dep(static_cast<const float4*>(W) + e4);
-  const uint2 u = __ldg(static_cast<const uint2*>(W) + e4);
+  const uint2 u = ld_dep(static_cast<const uint2*>(W) + e4);
   return make_float4(__uint_as_float(u.x << 16), __uint_as_float(u.x & 0xffff0000u), __uint_as_float(u.y << 16),
                      __uint_as_float(u.y & 0xffff0000u));
 }

@@ -287,8 +287,19 @@ inline cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, s
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
-// Loads of what the kernel before wrote, after pdl_wait(): volatile, because a load that the compiler
-// takes for a read of constant memory (__ldg, a const __restrict__ pointer) may be moved above the wait.
+// Loads of what an earlier kernel may have written (its results, the caller's tensors), after pdl_wait():
+// volatile, because a load that the compiler takes for a read of constant memory (__ldg, a const
+// __restrict__ pointer) may be moved above the wait.
+__device__ __forceinline__ int ld_dep(const int* p) {
+  int v;
+  asm volatile("ld.global.s32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+  return v;
+}
+__device__ __forceinline__ uint2 ld_dep(const uint2* p) {
+  uint2 v;
+  asm volatile("ld.global.v2.u32 {%0, %1}, [%2];" : "=r"(v.x), "=r"(v.y) : "l"(p) : "memory");
+  return v;
+}
 __device__ __forceinline__ float ld_dep(const float* p) {
   float v;
   asm volatile("ld.global.f32 %0, [%1];" : "=f"(v) : "l"(p) : "memory");

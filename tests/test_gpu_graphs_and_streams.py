@@ -67,3 +67,44 @@ def test_random_shapes_agree_with_the_oracle(seed):
     for k in range(B):
         res = ph.compare_user(w, inp, got, k)
         assert res["o_err"] <= ph.TOL[dtype], (w, k, res["o_err"])
+
+
+@pytest.mark.parametrize("d,dtype", [(32, torch.float32), (32, torch.bfloat16), (64, torch.float32), (64, torch.bfloat16), (128, torch.float32)])
+def test_outputs_of_a_call_are_inputs_of_the_next(d, dtype):
+    """Calls that start while the one before is draining, each reading what that one writes: the attention's
+    output as candidates, gradients as factors, through the whole calls and the single stages."""
+    g = torch.Generator().manual_seed(d)
+    B, M, N, r = 4, 500, 600, 12
+    C0, dO = ((torch.randn(B, M, d, generator=g) * d ** -0.5).to(dtype).cuda() for _ in range(2))
+    H = (torch.randn(B, N, r, generator=g) @ torch.randn(B, r, d, generator=g) + 0.1 * torch.randn(B, N, d, generator=g)).to(dtype).cuda()
+    W = [(torch.randn(d, d, generator=g) * d ** -0.5).to(dtype).cuda() for _ in range(3)]
+    ws, bws = solar.alloc_workspace(B, M, N, d, r, dtype), solar.alloc_backward_workspace(B, M, N, d, r, dtype)
+
+    def chain(wait):
+        out = []
+
+        def done(*t):
+            out.extend(x.clone() for x in t if wait)               # (a copy would stand between the calls)
+            if wait:
+                torch.cuda.synchronize()
+            else:
+                out.extend(t)
+        S, V = solar.lowrank_factor(H, r, workspace=ws); done(S, V)
+        C = C0
+        for _ in range(3):
+            C = solar.svd_attention_fwd(C, S, V, *W, d ** -0.5, workspace=ws); done(C)
+        grads = solar.svd_attention_bwd(C, S, V, *W, d ** -0.5, dO, bws); done(*grads)
+        O = torch.empty_like(C)
+        solar.attn_prepare(grads[4], grads[5], *W, 0.3, ws)        # S and V from the kernel just before
+        solar.attn_apply(C, r, 0, O, ws); done(O)
+        P = torch.empty_like(C)
+        solar.attn_apply(O, r, 0, P, ws); done(P)
+        dH = torch.empty_like(H)
+        solar.svd_backward(H, S, V, grads[4], grads[5], dH, bws, eps_rel=1e-6); done(dH)
+        torch.cuda.synchronize()
+        return out
+
+    ref = chain(True)
+    for _ in range(5):
+        for a, b in zip(chain(False), ref):
+            assert torch.equal(a.view(torch.uint8), b.view(torch.uint8))
