@@ -37,10 +37,9 @@ template <int D> struct UsCfg {
   }
 };
 
-// byte offset of 16-byte chunk c of row `row` in a [rows][128 B] tile with the 128-byte swizzle
-template <int D>
+template <int D, bool TMA>
 __global__ void __launch_bounds__(kThreads, 1)
-project_us_umma_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_constant__ CUtensorMap tmOut, int tma_out,
+project_us_umma_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_constant__ CUtensorMap tmOut,
                        const float* __restrict__ V,
                        __nv_bfloat16* __restrict__ US, int N, int r, int chunk_rows, int early_h) {
   // V is the per-user matrix X [D][r] and US the output [N][r]; r stands for q here.
@@ -162,7 +161,9 @@ project_us_umma_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_co
     // ---- epilogue warps: accumulator row tid -> bf16 -> US[b, n, 0:r] ------------------
     const uint32_t lane_base = (uint32_t)(warp * 32) << 16;
     // A warp's 32 rows leave by TMA from one of its two staging buffers (r = 16, 32, 64 or 128: rows of a
-    // swizzle span, or two spans side by side); other widths are stored by the threads themselves.
+    // swizzle span, or two spans side by side); other widths are stored by the threads themselves, a row each,
+    // in pieces of 16 bytes where r is a multiple of 8 (16 x 10240 x 64, r = 56: 9.9 us, 94 in pieces of 2;
+    // r = 64 without TMA 11.4, with it 9.6).
     const int span = r >= 64 ? 128 : 2 * r, boxes = r > 64 ? 2 : 1, rows_bytes = 32 * span;
     uint8_t* sO = sV + (2 * Cfg::KB * v_tile + 1023) / 1024 * 1024 + warp * 2 * boxes * rows_bytes;
     int t = 0;
@@ -174,7 +175,7 @@ project_us_umma_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_co
       const int n = row0 + t * kTileRows + tid;
       __nv_bfloat16* o = US + ((size_t)b * N + (n < N ? n : 0)) * r;
       uint8_t* buf = sO + a * boxes * rows_bytes;
-      if (tma_out) {                             // the store before the last has left this buffer
+      if constexpr (TMA) {                       // the store before the last has left this buffer
         if (lane == 0) ptx::tma_store_wait_read_1();
         __syncwarp();
       }
@@ -186,7 +187,7 @@ project_us_umma_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_co
           ptx::tc_fence_before_sync();
           ptx::mbar_arrive(&acc_free[a]);
         }
-        if (tma_out) {
+        if constexpr (TMA) {
 #pragma unroll
           for (int c = 0; c < 4; ++c)
             if (c0 + 8 * c < r) {
@@ -198,13 +199,22 @@ project_us_umma_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_co
                              ptx::pack_bf16(__uint_as_float(v[8 * c + 4]), __uint_as_float(v[8 * c + 5])),
                              ptx::pack_bf16(__uint_as_float(v[8 * c + 6]), __uint_as_float(v[8 * c + 7])));
             }
+        } else if (n < N && r % 8 == 0) {        // rows start on 16-byte boundaries
+#pragma unroll
+          for (int c = 0; c < 4; ++c)
+            if (c0 + 8 * c < r)
+              reinterpret_cast<uint4*>(o + c0)[c] =
+                  make_uint4(ptx::pack_bf16(__uint_as_float(v[8 * c]), __uint_as_float(v[8 * c + 1])),
+                             ptx::pack_bf16(__uint_as_float(v[8 * c + 2]), __uint_as_float(v[8 * c + 3])),
+                             ptx::pack_bf16(__uint_as_float(v[8 * c + 4]), __uint_as_float(v[8 * c + 5])),
+                             ptx::pack_bf16(__uint_as_float(v[8 * c + 6]), __uint_as_float(v[8 * c + 7])));
         } else if (n < N) {
 #pragma unroll
           for (int i = 0; i < 32; ++i)
             if (c0 + i < r) o[c0 + i] = __float2bfloat16_rn(__uint_as_float(v[i]));
         }
       }
-      if (tma_out) {
+      if constexpr (TMA) {
         ptx::fence_proxy_async_smem();
         __syncwarp();
         const int n0 = row0 + t * kTileRows + warp * 32;
@@ -215,7 +225,7 @@ project_us_umma_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_co
         }
       }
     }
-    if (tma_out && lane == 0) ptx::tma_store_wait_read();      // before the CTA's shared memory goes
+    if (TMA && lane == 0) ptx::tma_store_wait_read();          // before the CTA's shared memory goes
     // a wait ran out: the rows that were not produced read as NaN
     for (; t < ntiles; ++t) {
       const int n = row0 + t * kTileRows + tid;
@@ -242,12 +252,14 @@ cudaError_t launch_d(int B, int N, int r, const void* H, const float* V, void* U
   if (tma_out && !encode_tmap_bf16_3d_sw(&tmOut, US, r, (uint64_t)N, (uint64_t)B, (uint64_t)r * 2, (uint64_t)N * r * 2,
                                          span / 2, 32, span))
     return cudaErrorInvalidValue;
-  static bool limits_set[kMaxDevicesCached] = {};
-  const cudaError_t e = set_kernel_limits(reinterpret_cast<const void*>(&project_us_umma_kernel<D>), Cfg::smem(kMaxCols), limits_set);
-  if (e != cudaSuccess) return e;
-  return launch_pdl(project_us_umma_kernel<D>, dim3(plan.splits, B), dim3(kThreads), Cfg::smem((r + 15) & ~15), st, tmap, tmOut,
-                    (int)tma_out, V,
-                    static_cast<__nv_bfloat16*>(US), N, r, plan.chunk_tiles * kTileRows, (int)early_h);
+  auto launch = [&](auto kernel, bool (&limits_set)[kMaxDevicesCached]) {
+    const cudaError_t e = set_kernel_limits(reinterpret_cast<const void*>(kernel), Cfg::smem(kMaxCols), limits_set);
+    if (e != cudaSuccess) return e;
+    return launch_pdl(kernel, dim3(plan.splits, B), dim3(kThreads), Cfg::smem((r + 15) & ~15), st, tmap, tmOut, V,
+                      static_cast<__nv_bfloat16*>(US), N, r, plan.chunk_tiles * kTileRows, (int)early_h);
+  };
+  static bool limits_tma[kMaxDevicesCached] = {}, limits_set[kMaxDevicesCached] = {};
+  return tma_out ? launch(project_us_umma_kernel<D, true>, limits_tma) : launch(project_us_umma_kernel<D, false>, limits_set);
 }
 
 }  // namespace

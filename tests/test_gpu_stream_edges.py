@@ -12,7 +12,7 @@ pytestmark = pytest.mark.gpu
 @pytest.mark.parametrize("d", [64, 128])
 def test_left_factor_rows(d):
     g = torch.Generator().manual_seed(d)
-    for r in (15, 16, 24, 32, 64):
+    for r in (8, 15, 16, 24, 32, 40, 48, 56, 64):
         for N in (128, 129, 159, 160, 161, 385):
             H = torch.randn(3, N, d, generator=g).bfloat16()
             V = torch.linalg.qr(torch.randn(3, d, r, generator=g))[0].contiguous()
@@ -24,6 +24,27 @@ def test_left_factor_rows(d):
             # one rounding to bf16 (2^-9 of the value) and 2^-16 halves of V
             assert float((got - ref).abs().max()) <= 2.0 ** -8 * float(ref.abs().max()), (r, N)
             assert bool(torch.isnan(buf[3 * N * r:]).all())
+
+
+@pytest.mark.parametrize("d", [64, 128])
+def test_left_factor_rows_of_whole_16_bytes_are_stored_as_such(d):
+    """A width that TMA does not store takes about as long as the next one that it does (2-byte stores: four to
+    seven times as long)."""
+    H = torch.randn(16, 8192, d, device="cuda").bfloat16()
+    us = {}
+    for r in (40, 56, 64):
+        V, US = torch.randn(16, d, r, device="cuda"), torch.empty(16, 8192, r, dtype=H.dtype, device="cuda")
+        best = []
+        for _ in range(6):
+            a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            a.record()
+            for _ in range(20):
+                solar.project_us(H, V, US)
+            b.record()
+            b.synchronize()
+            best.append(a.elapsed_time(b))
+        us[r] = min(best)
+    assert max(us[40], us[56]) <= 2.5 * us[64], us
 
 
 @pytest.mark.parametrize("d", [64, 128])
