@@ -1267,10 +1267,7 @@ __device__ __forceinline__ EigEnd eig_user(int b, int half, bool& joined, const 
 #pragma unroll
       for (int rr = 0; rr < RT; ++rr)
 #pragma unroll
-        for (int m = 0; m < NCH; ++m) {
-          const float4 t = ld_dep(reinterpret_cast<const float4*>(gout + (row0 + 32 * rr) * D + CW * m + 4 * g));
-          acc[rr][m][0] = t.x; acc[rr][m][1] = t.y; acc[rr][m][2] = t.z; acc[rr][m][3] = t.w;
-        }
+        for (int m = 0; m < NCH; ++m) ld4(gout + (row0 + 32 * rr) * D + CW * m + 4 * g, acc[rr][m]);
       wide = 1;
       ok = tri_chain<double, D, RP>(acc, smem, sh, gout, sc, r, false, tol, false, half, not_mine, Vc, passes, tid);
       if (not_mine) return kOtherHalf;
@@ -1325,7 +1322,7 @@ __device__ __forceinline__ EigEnd eig_user(int b, int half, bool& joined, const 
 
   // ---- last resort (or the caller's choice): Jacobi on the whole matrix ----------------------------
   for (int e = tid; e < D * D / 4; e += NT) {
-    float4 t = ld_dep(reinterpret_cast<const float4*>(gout) + e);
+    float4 t = reinterpret_cast<const float4*>(gout)[e];
     t.x *= sc; t.y *= sc; t.z *= sc; t.w *= sc;
     *reinterpret_cast<float4*>(smem + (e / (D / 4)) * LD + (e % (D / 4)) * 4) = t;
   }
