@@ -510,11 +510,20 @@ __device__ __forceinline__ void minors(const T* __restrict__ dg, const T* __rest
     float mu[4], lg[4];
 #pragma unroll
     for (int u = 0; u < 4; ++u) {
-      lg[u] = lg2(fabsf((float)p)) + (float)ex;
+      if constexpr (sizeof(T) == 4) lg[u] = lg2(fabsf(p)) + (float)ex;
       T np = fma_t(d[u] - lam, p, -(e2[u] * po));
       const T fl = pfl * abs_t(p);
       np = abs_t(np) >= fl ? np : -fl;
-      mu[u] = -(float)e1[u] * ((float)p * rcp_fast((float)np));
+      if constexpr (sizeof(T) == 4) {
+        mu[u] = -e1[u] * (p * rcp_fast(np));
+      } else {
+        // The fp64 minors of four rows can shrink past the range of fp32, which takes their ratio and logarithm:
+        // both are brought near 1 by their exponents (they differ by 2^61 at most).
+        const int m = max(__double2hiint(p) & 0x7ff00000, __double2hiint(np) & 0x7ff00000) - 0x3ff00000;
+        const float pf = (float)__hiloint2double(__double2hiint(p) - m, __double2loint(p));
+        lg[u] = lg2(fabsf(pf)) + (float)(ex + (m >> 20));
+        mu[u] = -(float)e1[u] * (pf * rcp_fast((float)__hiloint2double(__double2hiint(np) - m, __double2loint(np))));
+      }
       po = p; p = np;
     }
 #pragma unroll

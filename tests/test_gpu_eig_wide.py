@@ -43,3 +43,34 @@ def test_graded_spectra_take_the_double_precision_chain(d, r):
         sine = np.sqrt(np.maximum(0.0, 1 - np.abs(np.sum(V[b] * vec[:, :r], axis=0)).clip(0, 1) ** 2))
         clear = gap > 8 * eps
         assert clear[0] and np.all(sine[clear] <= 2 * eps / gap[clear] + 2e-3), (sine[clear], eps / gap[clear])
+
+
+@pytest.mark.parametrize("kind", ["rank r/2", "orthogonal columns"])
+@pytest.mark.parametrize("d,r", [(64, 16), (64, 32), (64, 64), (128, 16), (128, 64)])
+def test_eigenvalues_apart_by_rounding_errors_only(d, r, kind):
+    """Kept eigenvalues that are zero, or all the same, but for the rounding errors of the Gram matrix: the
+    minors of T - lambda I shrink by those errors from row to row, and the fp64 chain has to follow them."""
+    rng = np.random.default_rng(d + 3 * r)
+    B, N = 6, 1000
+    H = np.empty((B, N, d), np.float32)
+    for b in range(B):
+        if kind == "rank r/2":
+            H[b] = rng.standard_normal((N, r // 2)) @ rng.standard_normal((r // 2, d))
+        else:
+            H[b] = np.linalg.qr(rng.standard_normal((N, d)))[0] * np.sqrt(N)
+    ws = solar.alloc_workspace(B, 1, N, d, r, torch.float32)
+    S = torch.empty(B, r, device="cuda"); V = torch.empty(B, d, r, device="cuda")
+    info = torch.full((B,), -1, dtype=torch.int32, device="cuda"); taken = torch.zeros_like(info)
+    solar.gram_partials(torch.from_numpy(H).cuda(), ws)
+    solar.eig_from_partials_ex(B, N, d, r, torch.float32, solar.ROUTE_AUTO, S, V, info, taken, ws)
+    torch.cuda.synchronize()
+    assert info.tolist() == [0] * B
+    assert [t & 0xffff for t in taken.tolist()] == [2 | (1 << 8)] * B, [hex(t & 0xffffffff) for t in taken.tolist()]
+    S, V = S.cpu().numpy().astype(np.float64), V.cpu().numpy().astype(np.float64)
+    for b in range(B):
+        G = H[b].astype(np.float64).T @ H[b].astype(np.float64)
+        lam = np.linalg.eigvalsh(G)[::-1]
+        eps = 16 * 2.0 ** -24 * lam[0]                 # the kernel's Gram matrix: a few 2^-24 lambda_1
+        assert np.all(np.abs(S[b] ** 2 - lam[:r]) <= eps)
+        assert np.abs(V[b].T @ V[b] - np.eye(r)).max() <= 2e-5
+        assert np.linalg.norm(G @ V[b] - V[b] * lam[:r], axis=0).max() <= 2e-5 * lam[0]
