@@ -23,7 +23,10 @@ namespace solar {
 namespace {
 
 constexpr int kGradThreads = 256;
-constexpr int kGradParts = 4;        // CTAs per user: each forms W (small) and a share of K's rows
+// CTAs per user: each forms W and a share of K's rows.  As many as stay within one per SM: every further one
+// forms W again (64 users, d = r = 64, with dH over 100 rows: 37.2, 31.7 and 37.1 us on one, two and four; 128
+// users 43.3, 47.4, 61.7; 16 users 37.2, 31.0, 29.0).
+inline int grad_parts(int B) { return 4 * B <= kNumSMs ? 4 : 2 * B <= kNumSMs ? 2 : 1; }
 
 // out(i, j) = sum_k a(i, k) b(k, j) for i < rows, j < cols, in tiles of 2 x 2 (four reads for four FMAs).
 template <typename FA, typename FB, typename FS>
@@ -58,11 +61,11 @@ svd_grad_kernel(const float* __restrict__ S, const float* __restrict__ V, const 
   float* dVs = Vs + D * lw;             // [D][lw]  Vbar
   float* Pt = dVs + D * lw;             // [r+1][lw]  Vbar^T V
   float* W = Pt + (r + 1) * lw;         // [r+1][lw]
-  float* T1 = W + (r + 1) * lw;         // [D / kGradParts][lw]  a share of V W
-  float* ss = T1 + D / kGradParts * lw; // [r] sigma
+  const int KR = D / (int)gridDim.y;    // rows of K of a CTA
+  float* T1 = W + (r + 1) * lw;         // [KR][lw]  a share of V W
+  float* ss = T1 + KR * lw;             // [r] sigma
   float* ds = ss + r;                   // [r] dL/dsigma
   const int b = blockIdx.x, tid = threadIdx.x;
-  constexpr int KR = D / kGradParts;
   const int k0 = blockIdx.y * KR;       // this CTA's rows of K
 
   pdl_wait();          // the first kernel of its entry point: everything below reads the caller's buffers
@@ -117,14 +120,15 @@ svd_grad_kernel(const float* __restrict__ S, const float* __restrict__ V, const 
 template <int D>
 cudaError_t launch_d(int B, int r, const float* S, const float* V, const float* dS, const float* dV,
                      float eps_rel, float* K, cudaStream_t st) {
-  auto smem = [](int rank) {
+  const int parts = grad_parts(B);
+  auto smem = [](int rank, int shares) {
     const int lw = (rank | 1) + 2;
-    return (size_t)(2 * D * lw + 2 * (rank + 1) * lw + D / kGradParts * lw + 2 * rank) * sizeof(float);
+    return (size_t)(2 * D * lw + 2 * (rank + 1) * lw + D / shares * lw + 2 * rank) * sizeof(float);
   };
   static bool limits_set[kMaxDevicesCached] = {};
-  const cudaError_t e = set_kernel_limits(reinterpret_cast<const void*>(&svd_grad_kernel<D>), smem(D < 64 ? D : 64), limits_set);
+  const cudaError_t e = set_kernel_limits(reinterpret_cast<const void*>(&svd_grad_kernel<D>), smem(D < 64 ? D : 64, 1), limits_set);
   if (e != cudaSuccess) return e;
-  return launch_pdl(svd_grad_kernel<D>, dim3(B, kGradParts), dim3(kGradThreads), smem(r), st, S, V, dS, dV, eps_rel, r, K);
+  return launch_pdl(svd_grad_kernel<D>, dim3(B, parts), dim3(kGradThreads), smem(r, parts), st, S, V, dS, dV, eps_rel, r, K);
 }
 
 }  // namespace

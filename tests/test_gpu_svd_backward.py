@@ -101,3 +101,31 @@ def test_argument_checks():
     with pytest.raises(solar.SolarError) as e:
         solar.svd_backward(H, S, V, S, V, dH, ws, eps_rel=-1.0)
     assert e.value.status == solar.ERR_INVALID_ARG
+
+
+@pytest.mark.parametrize("d,r", [(32, 32), (64, 9), (64, 64), (128, 64)])
+def test_gradient_of_a_user_does_not_depend_on_the_batch(d, r):
+    """The work of a user is split over four, two or one CTA by the size of the batch."""
+    g = torch.Generator().manual_seed(d + r)
+    B, N = 150, 70
+    H = torch.randn(B, N, d, generator=g).cuda()
+    V = torch.linalg.qr(torch.randn(B, d, r, generator=g))[0].contiguous().cuda()
+    S = (torch.arange(r, 0, -1).float() + 3).repeat(B, 1).cuda()
+    dS, dV = torch.randn(B, r, generator=g).cuda(), torch.randn(B, d, r, generator=g).cuda()
+
+    def run(n):
+        dH = torch.full((n, N, d), float("nan"), device="cuda")
+        ws = solar.alloc_backward_workspace(n, 1, N, d, r, H.dtype).fill_(0xFF)
+        solar.svd_backward(H[:n], S[:n], V[:n], dS[:n], dV[:n], dH, ws, eps_rel=1e-6)
+        return dH
+
+    whole = run(B)
+    s, v = S.double(), V.double()
+    D = s[:, :, None] ** 2 - s[:, None, :] ** 2
+    F = D / (D ** 2 + (1e-6 * s[:, :1, None] ** 2) ** 2)
+    X = F * (dV.double().transpose(1, 2) @ v)
+    K = v @ ((torch.diag_embed(dS.double()) + s[:, :, None] * (X + X.transpose(1, 2))) / s[:, :, None]) @ v.transpose(1, 2)
+    ref = H.double() @ K
+    assert float((whole.double() - ref).abs().max()) <= 2e-4 * float(ref.abs().max())
+    for n in (1, 37, 38, 74, 75):
+        assert torch.equal(run(n), whole[:n]), n
