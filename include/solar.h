@@ -202,9 +202,9 @@ int solar_gram_slices(int B, int N, int d, solar_dtype_t dt);
  * solar_eig_from_partials).  H_b^T H_b (the matrix whose eigenvectors are V of Eq. 9) is
  * the sum over p.  bf16 storage with d = 64 or 128 and N >= 128 runs on the tensor cores
  * (TMA tiles, tcgen05.mma, fp32 accumulation in tensor memory); other shapes use FFMA.
- * P = solar_gram_splits() divides the slice count solar_gram_slices(): the CTAs of P-th
- * parts of the slices may add up their results on chip (thread-block clusters); as built,
- * every slice leaves its own partial. */
+ * P = solar_gram_splits() divides the slice count solar_gram_slices(): on the tensor cores at
+ * d = 128 the CTAs of up to four slices may add up their results on chip (thread-block clusters);
+ * otherwise every slice leaves its own partial. */
 solar_status_t solar_gram_partials(int B, int N, int d, solar_dtype_t dt, const void* H,
                                    void* workspace, size_t workspace_bytes, void* stream);
 

@@ -9,11 +9,11 @@
 // accumulating the d x d result in tensor memory.  H is read from HBM exactly once and never
 // passes through registers.
 //
-// The CTAs of up to eight slices of a user form a thread-block cluster: each lays its
-// accumulator down in its own shared memory, and after a cluster barrier every CTA adds up
+// The CTAs of a user can form thread-block clusters of several slices (gram_plan: up to four, at d = 128): each lays
+// its accumulator down in its own shared memory, and after a cluster barrier every CTA adds up
 // one share of the matrix over all of them through distributed shared memory (plain loads, in
 // rank order: the sum is reproducible) and stores it.  A user so leaves splits / cluster
-// partial matrices in global memory -- one in the usual case -- instead of one per slice.
+// partial matrices in global memory instead of one per slice.
 #include "sm100_ptx.cuh"
 #include "solar_internal.cuh"
 

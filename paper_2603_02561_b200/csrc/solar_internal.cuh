@@ -65,16 +65,20 @@ inline GramPlan slice_plan(int B, int N, int cap) {
 // of 3 and of 8 both lose more in the Gram kernel (gang-scheduled CTAs, two cluster barriers: 3.3 -> 3.95 us
 // per launch with 24 requests in flight, 7.4 -> 9.9 us alone) than the eigensolver gains from reading one
 // matrix instead of nine (45 -> 44 us).
-//   d = 128 (64 KB): clusters of up to four, unless a slice limit keeps the slices few anyway: the
-// eigensolver's CTA reads a matrix at 44 bytes a clock, and 16 of them are 12 us of a pass over 8 x 16384 x
-// 128 (four: 3 us; the Gram kernel 9.6 -> 11.1 us, with clusters of eight 19.8).
-constexpr int kMaxCluster = 4;
+//   d = 128 (64 KB): the largest cluster of up to four that divides the slices and with which all CTAs still run
+// at once, unless a slice limit keeps the slices few anyway.  The eigensolver's CTA reads a matrix at 44 bytes a
+// clock, 64 of them 48 us of a pass, 16 of them 12; adding them up costs the Gram kernel 2 to 4 us, but as much
+// as a second wave where its clusters do not all fit (148 CTAs in pairs, 135 in threes, 132 in fours do; 144 in
+// threes 12.7 -> 28.5 us, 136 in fours 13.4 -> 26.1).  us per pass without and with: 2 x 8192 x 128 (64
+// slices) 184 and 152, 1 x 40000 (63) 185 and 161, 5 x 16384 (26) 162 and 156, 8 x 16384 (16) 157 and 150, 16 x
+// 8192 (8) 151 and 148, 70 x 4096 (2) 160 and 156; where they do not fit, 16 x 16384 (9) 156 and 173, 37 x
+// 8192 (4) 158 and 168.  Clusters of eight lose against four (8 x 16384: the Gram kernel 10.7 and 19.4 us).
 inline GramPlan gram_plan(int B, int N, int d, solar_dtype_t dt, int cap) {
   GramPlan p = slice_plan(B, N, cap);
+  constexpr int kAtOnce[] = {0, 0, kNumSMs, 135, 132};
   const bool clusters = dt == SOLAR_BF16 && d == 128 && N >= kGramTileRows && cap == 0;
-  // the largest cluster size within the limit that divides the slice count
-  for (int c = 2; clusters && c <= kMaxCluster; ++c)
-    if (p.splits % c == 0) p.cluster = c;
+  for (int c = 2; clusters && c <= 4; ++c)
+    if (p.splits % c == 0 && (long)B * p.splits <= kAtOnce[c]) p.cluster = c;
   p.parts = p.splits / p.cluster;
   return p;
 }

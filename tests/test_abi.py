@@ -168,3 +168,25 @@ def test_a_workspace_sized_without_a_limit_serves_every_limit(L, d, dtype):
                     assert L.solar_gram_partials(*args) == solar.ERR_WORKSPACE, (B, N, lim)
     finally:
         L.solar_set_slice_limit(old)
+
+
+def test_clusters_of_the_gram_pass(L):
+    """At d = 128 up to four slices leave one partial, where all clusters run at once."""
+    bf = solar.BF16
+    old = L.solar_set_slice_limit(0)
+    try:
+        plan = lambda B, N, d=128, dt=bf: (L.solar_gram_slices(B, N, d, dt), L.solar_gram_splits(B, N, d, dt))
+        assert plan(8, 16384) == (16, 4) and plan(2, 8192) == (64, 16) and plan(16, 8192) == (8, 2)
+        assert plan(1, 40000) == (63, 21) and plan(5, 16384) == (26, 13) and plan(64, 4096) == (2, 1)
+        assert plan(15, 16384) == (9, 3) and plan(16, 16384) == (9, 9)          # 135 and 144 CTAs in threes
+        assert plan(33, 8192) == (4, 1) and plan(37, 8192) == (4, 2)            # 132 in fours; 148 in pairs
+        assert plan(48, 4096) == (3, 3)
+        assert plan(8, 16384, 64)[0] == plan(8, 16384, 64)[1] and plan(8, 16384, 128, solar.F32) == (16, 16)
+        for B in range(1, 150):
+            for N in (128, 1000, 4096, 16384, 50000):
+                s, p = plan(B, N)
+                assert s % p == 0 and s // p <= 4 and B * s <= (10 ** 9, 148, 135, 132)[s // p - 1], (B, N)
+        L.solar_set_slice_limit(64)
+        assert plan(8, 16384) == (16, 16)
+    finally:
+        L.solar_set_slice_limit(old)

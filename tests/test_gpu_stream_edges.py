@@ -1,4 +1,4 @@
-"""The streaming kernels of the left factor and of the backward pass where their layouts change: output
+"""The clusters of the Gram pass.  The streaming kernels of the left factor and of the backward pass where their layouts change: output
 rows of one, two and four swizzle spans and rows that end inside a warp's 32; token counts around 32,
 where the probabilities' shared-memory rows widen."""
 import pytest
@@ -87,3 +87,21 @@ def test_attention_gradients_by_token_count(r):
         # dC: one rounding to bf16; the fp32 outputs: products of bf16 halves, about 2^-16 each
         tol = 2.0 ** -7 if name == "dC" else 2e-4
         assert float((a.cpu().double() - b).abs().max()) <= tol * max(float(b.abs().max()), 1e-3), name
+
+
+@pytest.mark.parametrize("B,N,slices,parts", [(2, 8192, 64, 16), (8, 16384, 16, 4), (16, 8190, 8, 2), (1, 40000, 63, 21), (9, 16300, 16, 8), (15, 16384, 9, 3),
+                                              (16, 16384, 9, 9), (3, 1000, 8, 2), (1, 130, 2, 1)])
+def test_partial_matrices_of_clustered_slices(B, N, slices, parts):
+    d = 128
+    H = torch.randn(B, N, d, generator=torch.Generator().manual_seed(N)).bfloat16().cuda()
+    assert (solar.gram_slices(B, N, d, H.dtype), solar.gram_splits(B, N, d, H.dtype)) == (slices, parts)
+    ws = solar.alloc_workspace(B, 1, N, d, 1, H.dtype).fill_(0xFF)
+    solar.gram_partials(H, ws)
+    torch.cuda.synchronize()
+    got = ws[: B * parts * d * d * 4].view(torch.float32).view(B, parts, d, d).double()
+    rows = -(-(-(-N // 128)) // slices) * 128 * (slices // parts)          # rows of a partial: whole tiles of 128
+    for p in range(parts):
+        x = H[:, p * rows: (p + 1) * rows].double()
+        ref = x.transpose(1, 2) @ x
+        # a sum of `rows` exact products in fp32: at most one rounding (or truncation) of 2^-23 of the sum per product
+        assert float((got[:, p] - ref).abs().max()) <= x.shape[1] * 2.0 ** -23 * float(ref.abs().max()), p
