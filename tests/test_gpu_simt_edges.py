@@ -33,7 +33,7 @@ def test_gram_rows(d, dtype):
 def test_attention_rows_and_tokens(d, dtype, flags):
     g = torch.Generator().manual_seed(d)
     Wq, Wk, Wv = ((torch.randn(d, d, generator=g) * d ** -0.5).to(dtype) for _ in range(3))
-    for r in sorted({1, 7, 8, 9, 16, 17, 24, 25, 32} | ({33, 48, 49, 63, 64} if d > 32 else set())):
+    for r in sorted({1, 7, 8, 9, 16, 17, 24, 25, 32} | ({33, 40, 41, 48, 49, 63, 64} if d > 32 else set())):
         for M in (1, 127, 128, 129, 300):
             B = 2
             C = (torch.randn(B, M, d, generator=g) * d ** -0.5).to(dtype)
