@@ -1184,8 +1184,8 @@ __device__ __forceinline__ EigEnd eig_user(int b, int half, bool& joined, const 
   float acc[RT][NCH][4];
   {
     const float4* gp = reinterpret_cast<const float4*>(gpart + (size_t)b * parts * D * D);
-    int lost = 0;
-    for (int s = tid; s < splits; s += NT) lost |= (ld_dep(gram_status + b * splits + s) != kGramStatusOk);
+    static_assert(kMaxSplits <= NT, "a status word per thread");
+    const int word = tid < splits ? ld_dep(gram_status + b * splits + tid) : kGramStatusOk;      // looked at behind the sum
     // fp32 sums in slice order; the loads of SCN slices are issued before the first add: the
     // phase is bound by their latency
     constexpr int SCN = RT * NCH >= 16 ? 2 : RT * NCH >= 8 ? 3 : 8;
@@ -1231,6 +1231,7 @@ __device__ __forceinline__ EigEnd eig_user(int b, int half, bool& joined, const 
       }
     if (tid < 4) sh.flags[tid] = 0;
     if (tid == 0) sh.why = 0;
+    int lost = word != kGramStatusOk;
     if (__syncthreads_or(lost | (int)!(zero == 0.f))) {
       lost = __syncthreads_or(lost);
       const float qnan = __int_as_float(0x7fc00000);
