@@ -108,7 +108,7 @@ size_t solar_workspace_bytes(int B, int M, int N, int d, int r, solar_dtype_t dt
  * Route: G_b = H_b^T H_b is accumulated in one streaming pass over H; its top-r
  * eigenpairs come from a tridiagonal reduction of the d x d matrix (Householder,
  * Sturm-count multisection, twisted factorisation) when that result can be certified
- * against G_b, else from a parallel Jacobi eigensolver on the whole matrix
+ * against G_b, else from the same in double precision or a parallel Jacobi eigensolver on the whole matrix
  * (SOLAR_ROUTE_AUTO above); s_i = sqrt(lambda_i).  Algorithm 1 of the paper (the
  * randomized range finder) is available as SOLAR_ROUTE_SUBSPACE of
  * solar_eig_from_partials_ex.  M is accepted for a uniform signature and ignored.
@@ -217,11 +217,11 @@ solar_status_t solar_eig_from_partials(int B, int N, int d, int r, solar_dtype_t
 
 /* As above with the route chosen by the caller.  route_taken (device, [B] ints, or
  * NULL) receives per user: route used (1 subspace, 2 full, 3 tridiagonal; 0 = non-finite
- * input) | power steps << 8 (route 2: 1 if it was the double-precision tridiagonal chain) | Jacobi sweeps (tridiagonal chains: orthogonalisation passes) << 16 |
- * reason << 24, where reason says why the first route tried was not certified: 1 no gap
+ * input) | power steps << 8 (route 2: 1 if it was the double-precision tridiagonal chain) |
+ * Jacobi sweeps (tridiagonal chains: orthogonalisation passes) << 16 | reason << 24, where reason says why the first route tried was not certified: 1 no gap
  * at the cut, 2 residual too large for its gap, 4 a kept eigenvalue not positive, 8 sweep
  * cap, 16 non-finite pivot, 32 vectors of a cluster not independent, 64 trace mismatch
- * or a non-finite value. */
+ * or a non-finite value, 128 a gap between kept eigenvalues too small for fp32. */
 solar_status_t solar_eig_from_partials_ex(int B, int N, int d, int r, solar_dtype_t dt, int route,
                                           float* S, float* V, int* info, int* route_taken,
                                           void* workspace, size_t workspace_bytes, void* stream);
@@ -312,7 +312,9 @@ solar_status_t solar_svd_attention_bwd(int B, int M, int N, int d, int r, solar_
  *   V        [B,d,r] f32 (in)  right singular vectors (any sign convention: it cancels)
  *   Wq,Wk,Wv [d,d] dt   (in)   shared by all users; y = x W
  *   O        [B,M,d] dt (out)
- *   workspace: solar_workspace_bytes() of the same sizes.
+ *   workspace: solar_workspace_bytes() of the same sizes.  With few candidates the positions are
+ *   split over as many CTAs as workspace_bytes has room for; a workspace of another size can mean
+ *   another split, and so another rounding of O.
  * One flash-attention style kernel per call (after the small per-user operand set-up):
  * the N x M scores live in tensor memory only.  Supported: dt = SOLAR_BF16, d in
  * {64, 128}, r in {16, 32, 64}; other shapes return SOLAR_ERR_UNSUPPORTED.

@@ -125,7 +125,7 @@ attn_prepare_kernel(const float* __restrict__ S, const float* __restrict__ V,
 // cores (the routine the eigensolver's epilogue uses, so a forward pass gives the same bits either
 // way).  Bound by latency: one round of global loads (weights, factors and singular values together),
 // two barriers and the chained products.  8 users, d = 64, r = 27: 14.6 us with one CTA per user and the
-// weights loaded behind the factors, 5.7 with two of 128 threads, 5.4 of 256 (training step 97.9 -> 96.8).
+// weights loaded behind the factors, 5.7 with two of 128 threads, 5.4 of 256 (training step 1 % faster).
 template <int D, int KINDS>
 __device__ __forceinline__ void prepare_kinds(unsigned char* smb, const float* S, const float* V, const void* Wq, const void* Wk,
                                               const void* Wv, float scale, int r, const pmma::Out& o, int b, int tid) {

@@ -41,7 +41,7 @@
 // eigenvalues are there, the first either sends them across and leaves the user to the second, or sends
 // the second home.  Forward pass of 8 users, d = 128, r = 64 of a power
 // law (every user takes the fp64 chain): 3075 us with Jacobi in its place, 374 with the fp64 chain behind
-// the fp32 one, 281 beside it; 64 users, d = r = 64, one or none of them: 440, 148 and 112 us.
+// the fp32 one, 239 beside it; 64 users, d = r = 64, one or none of them: 440, 148 and 109 us.
 //
 // What bounds it: the dependency chain (d steps of a matrix-vector product, an inner product and a
 // barrier, then the recurrences over the rows of T), not work or bandwidth: 16 users keep 16 of
@@ -74,7 +74,7 @@ template <int D> struct TriCfg {
   __device__ static constexpr int rows_end(int warp) { return WG * (warp + 1) + 32 * (RT - 1); }   // behind a warp's last row
   // Resident CTAs that the register count has to allow.  d = 64: three (168 registers) for r <= 32 -- with 255 or
   // 128 the schedule is worse (16 x 10240 x 64 47.8 us per pass; 51.3, 50.2); above, shared memory allows two
-  // anyway (64 users, d = r = 64: 101.5 -> 100.1).
+  // anyway (64 users, d = r = 64: 1.4 % faster than with three).
   static constexpr int ctas(int rp) { return D == 128 ? 1 : rp > 32 ? 2 : 3; }
   static constexpr int LD = D + 4;                    // pitch of Q^T and of the row-major G
 };
@@ -700,7 +700,7 @@ __device__ __forceinline__ bool tri_chain(const float (&acc)[TriCfg<D>::RT][TriC
     constexpr int NP0 = 256, PRB = 16 / PT;                     // points of the first step, all threads together
     constexpr int STEPS = (NPT == 8 ? 6 : 9);                   // (NP0 + 1) (NPT + 1)^STEPS >= 2^27
     constexpr int STEPS64 = (NPT == 8 ? 14 : 19);               // fp64: (NPT + 1)^STEPS64 >= 2^44 from the Gershgorin interval
-    constexpr int STEPS_B = (NPT == 8 ? 9 : 12);                // ... and from a bracket of 2^-14 |T|
+    constexpr int STEPS_B = (NPT == 8 ? 9 : 12);                // >= 2^27.9, from a bracket of 2^-14 |T|: to 2^-42 |T|
     static_assert(PT * RP == NT && (NPT == 8 || NPT == 4) && CH * NT == NP0 && NP0 <= 3 * NW * RP, "every lane has points");
     const int j = tid / PT, pt = tid % PT, jj = j < r ? j : r - 1;     // surplus lanes shadow column r-1
     const int target = de8 - 1 - jj;    // lambda_(jj-th largest) >= x  <=>  #(eigenvalues < x) <= target

@@ -20,7 +20,7 @@
 // Where the candidates do not fill the GPU, the positions are split as well (flash_split): a CTA then leaves
 // Y, l and m of its range, and the one that arrives last adds up the ranges in their order.  128 candidates,
 // 32768 positions, d = 64, r = 32: 281 us a call with one CTA, 35 now; 8 x 512 candidates,
-// 10240 positions: 98 and 44.
+// 10240 positions: 98 and 44 in the three ranges that solar_workspace_bytes has room for.
 // The reference m of a row is the maximum of its first tile and is raised (Y and l rescaled) only when a
 // score passes it by more than 2^8: any m gives the same quotient, and bf16 keeps its relative accuracy
 // at every magnitude.  The N x M score matrix never exists outside tensor memory.  Every wait is bounded;
@@ -481,8 +481,10 @@ bool flash_factored_supported(int d, int r, solar_dtype_t dt) {
 // Few candidates: the positions of 128 candidates are split into ranges, a CTA each, so that the CTAs fill the
 // SMs once (twice where two fit).  Ranges of at least four tiles (a CTA's start costs about two), and no more
 // than 3 sqrt(tiles) of them: the last CTA reads every range's sums, about a sixth of a tile's time each, so
-// the sum of both is smallest near sqrt(6 tiles).  The sums lie behind the operands in the workspace, which
-// the factorization of the same sizes makes large enough; a smaller one means fewer ranges.
+// the sum of both is smallest near sqrt(6 tiles).  The ranges' sums lie behind the operands, as many as the
+// workspace holds: it is sized for the factorization and the operands (solar_workspace_bytes), which often is fewer
+// than are wanted (8 x 512 candidates, 10240 positions, d = 64, r = 32: three of nine; 1 x 512, 32768: fourteen of
+// 48).  A larger workspace has more of them, and rounds differently.
 FlashSplit flash_split(int B, int M, int N, int d, int r, size_t workspace_bytes) {
   FlashSplit s = {};
   const int tiles = (N + kPos - 1) / kPos;
