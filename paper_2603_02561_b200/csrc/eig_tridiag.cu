@@ -1155,7 +1155,7 @@ __device__ __forceinline__ bool tri_chain(const float (&acc)[TriCfg<D>::RT][TriC
 // shared memory ([D][rp], rp = r rounded up to 4, zero in the padding).
 enum EigEnd { kEnded, kEndedVs, kOtherHalf };      // S and V written; V Sigma in shared memory too; the pair's other CTA does it
 template <int D, int RP>
-__device__ __forceinline__ EigEnd eig_user(int b, int half, bool& joined, const float* __restrict__ gpart, const int* __restrict__ gram_status,
+__device__ __forceinline__ EigEnd eig_user(int b, int half, bool& joined, const float* __restrict__ gpart, const int* gram_status,
                                          int parts, int splits, float* __restrict__ gsum, int r, int route, int sweep_cap,
                                          const TriTol& tol, bool want_vs, bool late_trigger, float* __restrict__ S,
                                          float* __restrict__ V, int* __restrict__ info,
@@ -1184,8 +1184,8 @@ __device__ __forceinline__ EigEnd eig_user(int b, int half, bool& joined, const 
   float acc[RT][NCH][4];
   {
     const float4* gp = reinterpret_cast<const float4*>(gpart + (size_t)b * parts * D * D);
-    static_assert(kMaxSplits <= NT, "a status word per thread");
-    const int word = tid < splits ? ld_dep(gram_status + b * splits + tid) : kGramStatusOk;      // looked at behind the sum
+    int lost = 0;                        // (gram_status is no __restrict__ pointer: its loads stay behind the wait)
+    for (int s = tid; s < splits; s += NT) lost |= (gram_status[b * splits + s] != kGramStatusOk);
     // fp32 sums in slice order; the loads of SCN slices are issued before the first add: the
     // phase is bound by their latency
     constexpr int SCN = RT * NCH >= 16 ? 2 : RT * NCH >= 8 ? 3 : 8;
@@ -1231,7 +1231,6 @@ __device__ __forceinline__ EigEnd eig_user(int b, int half, bool& joined, const 
       }
     if (tid < 4) sh.flags[tid] = 0;
     if (tid == 0) sh.why = 0;
-    int lost = word != kGramStatusOk;
     if (__syncthreads_or(lost | (int)!(zero == 0.f))) {
       lost = __syncthreads_or(lost);
       const float qnan = __int_as_float(0x7fc00000);
@@ -1503,7 +1502,7 @@ __device__ __forceinline__ void prepare_epilogue(float* __restrict__ sm, int b, 
 
 template <int D, int RP>
 __global__ void __launch_bounds__(TriCfg<D>::NT, TriCfg<D>::ctas(RP))
-eig_tridiag_kernel(const float* __restrict__ gpart, const int* __restrict__ gram_status, int parts, int splits,
+eig_tridiag_kernel(const float* __restrict__ gpart, const int* gram_status, int parts, int splits,
                    float* __restrict__ gsum, int r, int route, int sweep_cap, TriTol tol,
                    float* __restrict__ S, float* __restrict__ V, int* __restrict__ info,
                    int* __restrict__ route_taken, FuseArgs fa, int pairs) {
