@@ -3,7 +3,7 @@
 // dense-symmetric chain, one CTA per user (128 threads; 256 at d = 128):
 //
 //   1. G = sum of the slices' partial Grams (fixed order), scaled by a power of two.
-//   2. Householder tridiagonalisation T = Q^T G Q with the matrix in REGISTERS, in tiles of d/32
+//   2. Householder tridiagonalisation T = Q^T G Q (only as far as the kept vectors reach) with the matrix in REGISTERS, in tiles of d/32
 //      rows x 16 columns per thread (rows 32 apart, so that finished ones leave the later stages for all
 //      threads: at d = 64 43.9 thousand cycles for the 62 steps with adjacent rows, 37.6 now; at d = 128
 //      165 and 138, in fp64 319 and 297, 260 with the reciprocals and A x as below); the vectors of a step live in registers too, at the thread's
@@ -238,6 +238,10 @@ __device__ __forceinline__ void st_peer(void* local, uint32_t v, uint32_t rank) 
   asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(remote), "r"(v) : "memory");
 }
 
+// log2 of the residual that an early end of T may leave, the largest diagonal entry being in [1, 2): 2^-4 of what
+// rounding does anyway
+constexpr float kTailBits = -28.f;
+
 // What a thread carries through the Householder steps.
 template <typename T, int D, bool KEEP> struct TriState {
   using C = TriCfg<D>;
@@ -248,6 +252,10 @@ template <typename T, int D, bool KEEP> struct TriState {
   T s2, x1, dk;                 // |x|^2, the subdiagonal entry, the diagonal entry
   float tr_rest, tr_comp, stop_tr, stop_x2;   // trace not yet reduced, compensated; the stop
   int k_stop;                   // step at which the reduction stopped early (uniform), or -1
+  // for the lane's shift x (fp32): 2 log2(x / 2), e^2 over the last pivot of x - T, its negative pivots so far, and
+  // 2 log2 of the bound on what a vector of an eigenvalue above x leaves behind the last row
+  float sx, lx, cpl, left;
+  int above;
 };
 // Where the steps exchange and leave their results.
 template <typename T> struct TriOut {
@@ -355,6 +363,19 @@ __device__ __forceinline__ void tri_stage(TriState<T, D, KEEP>& s, const TriOut<
       s.tr_comp = (t - s.tr_rest) - d;
       s.tr_rest = t;
       stop = (int)(k1 >= o.r) & (int)(t <= s.stop_tr) & (int)((float)s.s2 <= s.stop_x2);   // no branches
+      // Or the kept vectors do not reach the rows below k.  Those behind row j have trace t_j, so no eigenvalue of
+      // theirs, reduced or not, is above that, and the pivots of x - T_{j+1..k} are above x - t_j for a shift
+      // x >= 2 t_j.  Entry k of a vector of an eigenvalue above x is then at most prod_{j <= i < k} |e_i| / (x / 2)^(k-j),
+      // and times |e_k| that is the residual (for a norm of 1) that ending T at row k adds.  So T may end there once
+      // it has r eigenvalues above some x for which that is below the rounding level.  Every lane watches an x.
+      // A history of rank r plus noise, whose other rows never become negligible, so ends after about r + 5 steps
+      // instead of d - 2: 32 x 1024 x 64 with r = 16 50.9 -> 35.5 us per pass, 8 x 4096 x 128 with r = 32 148 -> 82;
+      // 0.3 us (d = 128: 2) more where a spectrum has no gap behind r.
+      const float pv = (s.sx - (float)s.dk) - s.cpl, s2 = (float)s.s2;
+      s.above += (int)(__float_as_uint(pv) >> 31);
+      s.cpl = s2 * rcp_fast(pv);
+      s.left = t + t <= s.sx ? s.left + (lg2(s2) - s.lx) : s.lx;
+      stop = (int)stop | __any_sync(kFull, (int)(s.above >= o.r) & (int)(s.left <= 2.f * kTailBits));
     }
     const bool last = tid == C::NT - 1;
     st_if(o.dg + k, s.dk, last);
@@ -601,6 +622,8 @@ __device__ __forceinline__ bool tri_chain(const float (&acc)[TriCfg<D>::RT][TriC
     s.stop_tr = trs * tol.stop_trace;
     s.stop_x2 = (trs * tol.stop_couple) * (trs * tol.stop_couple);
     s.k_stop = -1;
+    s.sx = trs * exp2f(-1.f - 0.5f * (float)lane); s.lx = 2.f * lg2(s.sx) - 2.f;     // trace / 2 .. trace / 2^16.5
+    s.cpl = 0.f; s.left = s.lx; s.above = 0;
 #pragma unroll
     for (int rr = 0; rr < RT; ++rr)
 #pragma unroll
@@ -632,6 +655,18 @@ __device__ __forceinline__ bool tri_chain(const float (&acc)[TriCfg<D>::RT][TriC
     if (!KEEP && !F64 && (s.k_stop < 0 || C::rows_end(warp) > s.k_stop + 1)) {
       __syncthreads();
       if (s.k_stop < 0 && *(volatile float*)(sh.stop + (D & 1)) != 0.f) s.k_stop = D - 3;
+    }
+    // the diagonal of the rows left out by an early end, for the comparison of the traces
+    if (!F64 && s.k_stop >= 0) {
+#pragma unroll
+      for (int rr = 0; rr < RT; ++rr) {
+        const int row = row0 + 32 * rr;
+        float t[4];
+#pragma unroll
+        for (int c = 0; c < 4; ++c) t[c] = (float)(CW == 32 || row0 < 16 ? s.a[rr][32 * rr / CW][c] : s.a[rr][(32 * rr + 16) / CW][c]);
+        const float v = (row & 2) ? ((row & 1) ? t[3] : t[2]) : ((row & 1) ? t[1] : t[0]);
+        st_if(part + row, v, (int)(row > s.k_stop) & (int)(((row & (CW - 1)) >> 2) == g));
+      }
     }
     // the last 2 x 2 block
     if (s.k_stop < 0 && tid == NT - 1) {
@@ -674,6 +709,7 @@ __device__ __forceinline__ bool tri_chain(const float (&acc)[TriCfg<D>::RT][TriC
       l = ((int)in & (int)(dd - rad < l)) ? dd - rad : l;
       h = ((int)in & (int)(dd + rad > h)) ? dd + rad : h;
       tr += dd;
+      if (!F64 && n >= de) tr += (T)part[n];
     }
 #pragma unroll
     for (int o = 16; o; o >>= 1) {

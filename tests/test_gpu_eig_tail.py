@@ -1,0 +1,54 @@
+"""Where the tridiagonal reduction ends because the kept vectors do not reach the rows behind (a history of
+rank R plus noise, whose remaining rows stay far above the rounding level): R at the edges of the kernel's
+stages of live columns and near the end of the matrix, noise from just above the rounding level to a
+twentieth of the smallest kept singular value, and R below r, where nothing may end early on the noise."""
+import numpy as np
+import pytest
+import torch
+
+from paper_2603_02561_b200 import solar
+
+pytestmark = pytest.mark.gpu
+
+
+def _histories(d, ranks, noises, N, seed):
+    rng = np.random.default_rng(seed)
+    H = []
+    for R in ranks:
+        for noise in noises:
+            U, _ = np.linalg.qr(rng.standard_normal((N, d)))
+            W, _ = np.linalg.qr(rng.standard_normal((d, d)))
+            s = noise * (2.0 - np.arange(d) / d)                  # the noise directions are apart from each other too
+            s[:R] = 3.0 - 2.0 * np.arange(R) / R
+            H.append((U * s) @ W.T)
+    return np.stack(H).astype(np.float32)
+
+
+@pytest.mark.parametrize("d", [32, 64, 128])
+def test_the_reduction_may_end_on_a_tail(d):
+    ranks = sorted({R for e in range(8, d, 16) for R in (e - 1, e, e + 1)} | {2, d - 12, d - 9, d - 7, d - 4, d - 2})
+    H = _histories(d, ranks, (0.05, 3e-3, 1e-4), 300, d)
+    exact = [np.linalg.svd(h.astype(np.float64), full_matrices=False) for h in H]
+    for r in sorted({1, 8, min(d, 32) - 3, min(d, 64) - 3}):
+        keep = [i for i in range(len(H)) if ranks[i // 3] >= r]
+        info = torch.full((len(keep),), -1, dtype=torch.int32, device="cuda")
+        S, V = solar.lowrank_factor(torch.from_numpy(H[keep]).cuda(), r, info=info)
+        torch.cuda.synchronize()
+        S, V = S.cpu().numpy().astype(np.float64), V.cpu().numpy().astype(np.float64)
+        assert torch.all(info == 0)
+        # the bounds of the test of the reduction's other early end
+        assert np.abs(S - np.stack([exact[i][1][:r] for i in keep])).max() <= 1e-5 * 3.0
+        assert np.abs(np.einsum("bki,bkj->bij", V, V) - np.eye(r)).max() <= 2e-5
+        G = np.einsum("bni,bnj->bij", H[keep].astype(np.float64), H[keep].astype(np.float64))
+        assert np.abs(G @ V - V * (S ** 2)[:, None, :]).max() <= 2e-5 * 9.0
+
+
+@pytest.mark.parametrize("d,R,r", [(64, 8, 16), (64, 16, 17), (128, 20, 32), (32, 4, 8)])
+def test_a_tail_that_holds_kept_directions_is_reduced_too(d, R, r):
+    H = _histories(d, [R], (0.05, 0.02), 300, 7 * d + r)
+    S, V = solar.lowrank_factor(torch.from_numpy(H).cuda(), r)
+    S = S.cpu().numpy().astype(np.float64)
+    for b in range(len(H)):
+        # fp32 Gram matrix: eigenvalues to 2^-22 of the largest (9), singular values of the noise (0.02 and more) to
+        # 9 * 2^-22 / (2 * 0.02) = 5.4e-5
+        assert np.abs(S[b] - np.linalg.svd(H[b].astype(np.float64), compute_uv=False)[:r]).max() <= 5.4e-5
