@@ -113,14 +113,18 @@ __device__ __forceinline__ void project(unsigned char* __restrict__ sm, int r, c
     if (KINDS & 2) *reinterpret_cast<uint4*>(wvs + row * P + c * 16) = w.v[n];
   }
   // (V Sigma)^T as bf16 halves, token-major; token rows >= rp are zero rows
+  // (no division by rp16, which is known at run time only)
+  for (int i = tid & 15; i < rp16; i += 16) {
+    const int ic = min(i, rp - 1);
+    const float* col = VS + ic;
 #pragma unroll 4
-  for (int e = tid; e < rp16 * (D / 2); e += NT) {
-    const int kp = e / rp16, i = e - kp * rp16, ic = min(i, rp - 1);
-    const float a0 = VS[(2 * kp) * rp + ic], c0 = VS[(2 * kp + 1) * rp + ic];
-    uint32_t hi, lo;
-    split2(i < rp ? a0 : 0.f, i < rp ? c0 : 0.f, hi, lo);
-    *reinterpret_cast<uint32_t*>(vsh + i * P + kp * 4) = hi;
-    *reinterpret_cast<uint32_t*>(vsl + i * P + kp * 4) = lo;
+    for (int kp = tid >> 4; kp < D / 2; kp += NT / 16) {
+      const float a0 = col[(2 * kp) * rp], c0 = col[(2 * kp + 1) * rp];
+      uint32_t hi, lo;
+      split2(i < rp ? a0 : 0.f, i < rp ? c0 : 0.f, hi, lo);
+      *reinterpret_cast<uint32_t*>(vsh + i * P + kp * 4) = hi;
+      *reinterpret_cast<uint32_t*>(vsl + i * P + kp * 4) = lo;
+    }
   }
   __syncthreads();
 
@@ -254,8 +258,10 @@ __device__ __forceinline__ void project(unsigned char* __restrict__ sm, int r, c
   if ((KINDS & 2) || dst != nullptr) {
     __syncthreads();
     const int pc = (KINDS & 2) ? rp16 / 8 : kTokenSlots / 8;
+    const unsigned inv = pc == 2 ? 32768u : pc == 4 ? 16384u : pc == 6 ? 10923u : 8192u;    // 2^16 / pc, up: exact for e < 2048
+#pragma unroll 4
     for (int e = tid; e < 2 * D * pc; e += NT) {
-      const int row = e / pc, c = e % pc;                                                  // row runs over [2][D]
+      const int row = (int)((unsigned)e * inv >> 16), c = e - row * pc;                    // row runs over [2][D]
       reinterpret_cast<uint4*>(dst + (size_t)row * kTokenSlots)[c] =
           c < rp16 / 8 ? *reinterpret_cast<const uint4*>(stage + ((size_t)row * (rp16 + 8) + 8 * c) * 2) : make_uint4(0u, 0u, 0u, 0u);
     }
