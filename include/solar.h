@@ -163,7 +163,8 @@ solar_status_t solar_svd_attention_fused(int B, int M, int N, int d, int r, sola
  * Stage-level entry points.  The two calls above are exactly
  *   solar_lowrank_factor    = solar_gram_partials ; solar_eig_from_partials [; solar_project_us]
  *   solar_svd_attention_fwd = solar_attn_prepare  ; solar_attn_apply
- * on the same workspace.  They exist so that each kernel can be timed and
+ * on the same workspace.  (The second is one kernel where its CTAs are few; results and workspace are
+ * the same.)  They exist so that each kernel can be timed and
  * checked on its own; argument meaning and rules are those given above.
  * ------------------------------------------------------------------------- */
 

@@ -12,8 +12,7 @@
 // the output tile after that; the output accumulator takes the scores' columns -- so that five
 // CTAs (d = 64, r <= 32) share an SM and keep enough bytes in flight for the HBM.  Every wait is bounded; if one runs out the
 // tile's output rows are written as NaN.
-#include "sm100_ptx.cuh"
-#include "solar_internal.cuh"
+#include "project_mma.cuh"
 
 namespace solar {
 
@@ -38,13 +37,23 @@ template <int D> struct AttnCfg {
     return (size_t)C_BYTES + t_bytes(np) + V_BYTES + (p_over_c(np) ? 0 : p_bytes(np)) + 1024;
   }
   static constexpr int TMEM_COLS = D;                             // scores (<= 64 columns), then the output (D)
+  // OWN: the projections' working space behind that
+  static constexpr size_t own_smem(int np) { return smem(np) + pmma::Lay<D>::vout(np); }
 };
 
-template <int D>
-__global__ void __launch_bounds__(128)
+// OWN: the factors and weights of a call whose CTAs make their user's operands themselves.
+struct OwnArgs { const float *S, *V; const void *Wq, *Wk, *Wv; float scale; char* ws; AttnWs lay; };
+constexpr int kOwnThreads = 256;           // the second half helps with the projections only
+
+// OWN (factors kept from an earlier call, d = 64, r <= 32, few CTAs): every CTA makes T^T and
+// Value_r^T of its user in shared memory, by the routine of the projection kernel (the same bits).  The two
+// launches were the bound of such a call: 8 x 3000 candidates, r = 27: 13.3 us per call with two launches (3.2 us of
+// the host's time each), 11.0 with one.
+template <int D, bool OWN>
+__global__ void __launch_bounds__(OWN ? kOwnThreads : 128)
 attn_umma_kernel(const __grid_constant__ CUtensorMap tmC, const __grid_constant__ CUtensorMap tmO,
                  const __grid_constant__ CUtensorMap tmT, const __grid_constant__ CUtensorMap tmV,
-                 int r, unsigned flags, __nv_bfloat16* __restrict__ O, int M, int early_c) {
+                 int r, unsigned flags, __nv_bfloat16* __restrict__ O, int M, int early_c, OwnArgs own) {
   using Cfg = AttnCfg<D>;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* base = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
@@ -67,8 +76,8 @@ attn_umma_kernel(const __grid_constant__ CUtensorMap tmC, const __grid_constant_
     s_err = 0;
     ptx::mbar_init(&bar_load, 1); ptx::mbar_init(&bar_s, 1); ptx::mbar_init(&bar_o, 1);
     ptx::fence_mbar_init();
-    ptx::prefetch_tensormap(&tmC); ptx::prefetch_tensormap(&tmT);
-    ptx::prefetch_tensormap(&tmV); ptx::prefetch_tensormap(&tmO);
+    ptx::prefetch_tensormap(&tmC); ptx::prefetch_tensormap(&tmO);
+    if (!OWN) { ptx::prefetch_tensormap(&tmT); ptx::prefetch_tensormap(&tmV); }
   }
   if (warp == 1) ptx::tmem_alloc(&s_tmem, Cfg::TMEM_COLS);
   ptx::tc_fence_before_sync();
@@ -78,26 +87,46 @@ attn_umma_kernel(const __grid_constant__ CUtensorMap tmC, const __grid_constant_
   volatile int* err = &s_err;
 
   if (tid == 0) {
-    ptx::mbar_arrive_expect_tx(&bar_load, Cfg::C_BYTES + Cfg::t_bytes(np) + Cfg::V_BYTES);
+    ptx::mbar_arrive_expect_tx(&bar_load, Cfg::C_BYTES + (OWN ? 0 : Cfg::t_bytes(np) + Cfg::V_BYTES));
     // The packed operands come from the kernel before this one.  The candidate tile is the
     // caller's: it may be fetched ahead of the wait only when an earlier kernel of the same
     // library call has already waited for whatever ran before the call (early_c).
     if (!early_c) pdl_wait();
 #pragma unroll
     for (int x = 0; x < Cfg::KB; ++x) ptx::tma_load_3d(sC + x * kBoxBytes, &tmC, &bar_load, x * 64, m0, b);
-    if (early_c) pdl_wait();
+    if (!OWN && early_c) pdl_wait();
 #pragma unroll
-    for (int x = 0; x < Cfg::KB; ++x) {
+    for (int x = 0; x < (OWN ? 0 : Cfg::KB); ++x) {
 #pragma unroll
       for (int h = 0; h < 2; ++h)     // rows h*64 .. h*64+63 of the packed T^T (hi, then lo)
         ptx::tma_load_3d(sT + (h * Cfg::KB + x) * t_tile, &tmT, &bar_load, x * 64,
                          h * kTokenSlots, b);
     }
 #pragma unroll
-    for (int h = 0; h < 2; ++h)
+    for (int h = 0; h < (OWN ? 0 : 2); ++h)
       ptx::tma_load_3d(sV + h * (D * 128), &tmV, &bar_load, 0, h * D, b);
   }
 
+  if constexpr (OWN) {
+    pdl_wait();                                  // the factors and weights are the caller's
+    unsigned char* const sw = sP == sC ? sV + Cfg::V_BYTES : sP + Cfg::p_bytes(np);
+    float* const VS = reinterpret_cast<float*>(sw);                                // [D][rp] V Sigma, zero in the padding
+    const int rp = (r + 3) & ~3;
+    pmma::Weights<D, kOwnThreads, 3> w;
+    w.load(own.Wq, own.Wk, own.Wv, tid);
+    const float* Vb = own.V + (size_t)b * D * r;
+    const unsigned inv = ((1u << 20) + rp - 1) / rp;                               // 2^20 / rp, up: exact for e < D rp
+#pragma unroll 8
+    for (int e = tid; e < D * rp; e += kOwnThreads) {
+      const int k = (int)((unsigned)e * inv >> 20), i = e - k * rp, ic = min(i, r - 1);
+      const float v = ld_dep(Vb + (size_t)k * r + ic), s = ld_dep(own.S + (size_t)b * r + ic);
+      VS[e] = i < r ? v * s : 0.f;
+    }
+    __syncthreads();
+    pmma::project<D, kOwnThreads, 3>(sw, r, w, own.scale, pmma::Tiles{sT, sV}, tid);
+    ptx::fence_proxy_async_smem();
+    __syncthreads();
+  }
   if (tid == 32) {
     // ---- scores = C T_hi + C T_lo : M = 128, N = np, K = D -------------------------------
     if (ptx::mbar_wait(&bar_load, 0, err, kErrLoad)) {
@@ -118,6 +147,26 @@ attn_umma_kernel(const __grid_constant__ CUtensorMap tmC, const __grid_constant_
   }
   __syncwarp();
 
+  if (OWN && tid >= 128) {                       // the row work is the first half's; its two barriers are met here
+    pdl_trigger();
+    if (blockIdx.x == 0) {                       // a user's first CTA leaves the operands in the workspace, as the projection kernel does
+      char* const wsb = own.ws + (size_t)b * own.lay.per_user;
+      for (int e = tid - 128; e < 2 * np * 8; e += 128) {
+        const int row = e >> 3, c = e & 7, h = row >= np;                          // row runs over [2][np]
+        *reinterpret_cast<uint4*>(wsb + own.lay.tpk_off + ((size_t)(row + h * (kTokenSlots - np)) * D + 8 * c) * 2) =
+            *reinterpret_cast<const uint4*>(sT + h * t_tile + ptx::swz128(row - h * np, c));
+      }
+      for (int e = tid - 128; e < 2 * D * 4; e += 128) {
+        const int row = e >> 2, c = e & 3;                                         // row runs over [2][D]
+        if (8 * c < np)
+          *reinterpret_cast<uint4*>(wsb + own.lay.vpk_off + ((size_t)row * kTokenSlots + 8 * c) * 2) =
+              *reinterpret_cast<const uint4*>(sV + ptx::swz128(row, c));
+      }
+    }
+    __syncthreads();
+    __syncthreads();
+    return;
+  }
   // ---- softmax over the r tokens, one candidate row per thread -------------------------
   const bool have_s = ptx::mbar_wait(&bar_s, 0, err, kErrScores);
   pdl_trigger();       // loads and the score GEMM are done: the next kernel may start launching
@@ -257,15 +306,44 @@ cudaError_t launch_d(int B, int M, int r, const void* C, unsigned flags, void* O
                                  kTokenSlots, D);
   if (!ok) return cudaErrorInvalidValue;
   static bool limits_set[kMaxDevicesCached] = {};
-  const cudaError_t e = set_kernel_limits(reinterpret_cast<const void*>(&attn_umma_kernel<D>), Cfg::smem(kTokenSlots),
+  const cudaError_t e = set_kernel_limits(reinterpret_cast<const void*>(&attn_umma_kernel<D, false>), Cfg::smem(kTokenSlots),
                                           limits_set);
   if (e != cudaSuccess) return e;
   const dim3 grid((M + kRows - 1) / kRows, B), block(128);
-  return launch_pdl(attn_umma_kernel<D>, grid, block, Cfg::smem(np), st, tmC, tmO, tmT, tmV, r, flags,
-                    static_cast<__nv_bfloat16*>(O), M, early_c ? 1 : 0);
+  return launch_pdl(attn_umma_kernel<D, false>, grid, block, Cfg::smem(np), st, tmC, tmO, tmT, tmV, r, flags,
+                    static_cast<__nv_bfloat16*>(O), M, early_c ? 1 : 0, OwnArgs{});
 }
 
+constexpr int kOwnTokens = 32;
+
 }  // namespace
+
+// As long as no more than every second SM has two of these CTAs.  us per call, one launch and two (as queued calls,
+// which the host's launches bound, and in a graph): 8 x 2048 candidates (128 CTAs) 10.2 / 8.5 and 12.3 / 8.7,
+// 128 x 120 (128) 10.3 / 8.6 and 13.5 / 12.8, 8 x 3000 (192) 10.2 / 9.6 and 12.4 / 9.3, 16 x 1536 (192) 10.3 / 9.6 and
+// 12.2 / 8.3, 16 x 2048 (256) 10.4 / 9.6 and 12.2 / 8.7 -- and there the training step, whose kernels are the bound, is 1 us
+// slower.  Under a slice limit other requests want the SMs.
+bool attn_own_supported(int B, int M, int d, int r, solar_dtype_t dt) {
+  return dt == SOLAR_BF16 && d == 64 && r <= kOwnTokens && slice_limit() == 0 &&
+         (long)B * ((M + kRows - 1) / kRows) <= kNumSMs * 3 / 2;
+}
+
+cudaError_t launch_attn_own(int B, int M, int r, const void* C, const float* S, const float* V, const void* Wq, const void* Wk,
+                            const void* Wv, float scale, unsigned flags, void* O, char* ws, const AttnWs& lay, cudaStream_t st) {
+  constexpr int D = 64;
+  using Cfg = AttnCfg<D>;
+  CUtensorMap tmC, tmO;
+  if (!encode_tmap_bf16_3d(&tmC, C, D, (uint64_t)M, (uint64_t)B, (uint64_t)D * 2, (uint64_t)M * D * 2, 64, kRows) ||
+      !encode_tmap_bf16_3d(&tmO, O, D, (uint64_t)M, (uint64_t)B, (uint64_t)D * 2, (uint64_t)M * D * 2, 64, kRows))
+    return cudaErrorInvalidValue;
+  const int np = (r + 15) & ~15;
+  static bool limits_set[kMaxDevicesCached] = {};
+  const cudaError_t e = set_kernel_limits(reinterpret_cast<const void*>(&attn_umma_kernel<D, true>), Cfg::own_smem(kOwnTokens),
+                                          limits_set);
+  if (e != cudaSuccess) return e;
+  return launch_pdl(attn_umma_kernel<D, true>, dim3((M + kRows - 1) / kRows, B), dim3(kOwnThreads), Cfg::own_smem(np), st, tmC, tmO,
+                    tmC, tmC, r, flags, static_cast<__nv_bfloat16*>(O), M, 0, OwnArgs{S, V, Wq, Wk, Wv, scale, ws, lay});
+}
 
 bool attn_umma_supported(int d, solar_dtype_t dt) { return dt == SOLAR_BF16 && (d == 64 || d == 128); }
 

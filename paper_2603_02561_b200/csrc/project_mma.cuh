@@ -16,6 +16,9 @@
 
 #include <cuda_bf16.h>
 
+#include <type_traits>
+
+#include "sm100_ptx.cuh"
 #include "solar_internal.cuh"
 
 namespace solar {
@@ -83,13 +86,18 @@ struct Out {
   __nv_bfloat16 *Tpk, *Vpk, *Tkm, *Vkm;
   float *Tf, *Vr;
 };
+// Or, in the kernel that uses them (d = 64), straight to the tiles that its MMAs read: T^T [2][rp16 rows][128 B] and
+// Value_r^T [2][64 rows][128 B], 128-byte swizzle.
+struct Tiles { unsigned char *T, *V; };
 
 // Every thread of the CTA (NT threads) calls this after a barrier behind the writes of the fp32
 // factor at sm[0 ..).  The MMAs of a job run as four independent accumulator chains; where the CTA has
 // more warps than jobs, two warps share the columns of T or Value_r.
-template <int D, int NT, int KINDS>
+template <int D, int NT, int KINDS, typename DST = Out>
 __device__ __forceinline__ void project(unsigned char* __restrict__ sm, int r, const Weights<D, NT, KINDS>& w, float scale,
-                                        const Out& o, int tid) {
+                                        const DST& o, int tid) {
+  constexpr bool TILES = std::is_same<DST, Tiles>::value;
+  static_assert(!TILES || (D == 64 && KINDS == 3), "both operands, one 64-wide box");
   using L = Lay<D>;
   constexpr int P = L::P, NW = NT / 32, KS = D / 16, NTL = D / 8, NV = Weights<D, NT, KINDS>::NV;
   constexpr int NK = KINDS == 3 ? 2 : 1;
@@ -168,6 +176,13 @@ __device__ __forceinline__ void project(unsigned char* __restrict__ sm, int r, c
 #pragma unroll
       for (int q = 0; q < 4; ++q) {
         const __nv_bfloat16 hi = __float2bfloat16_rn(x[q]);
+        if constexpr (TILES) {
+          const int tok = i0 + 8 * (q >> 1);
+          unsigned char* at = o.V + ptx::swz128(j + (q & 1), tok >> 3) + 2 * (tok & 7);
+          *reinterpret_cast<__nv_bfloat16*>(at) = hi;
+          *reinterpret_cast<__nv_bfloat16*>(at + D * 128) = __float2bfloat16_rn(x[q] - __bfloat162float(hi));
+          continue;
+        }
         __nv_bfloat16* row = reinterpret_cast<__nv_bfloat16*>(stage) + (size_t)(j + (q & 1)) * (rp16 + 8) + i0 + 8 * (q >> 1);
         row[0] = hi;
         row[(size_t)D * (rp16 + 8)] = __float2bfloat16_rn(x[q] - __bfloat162float(hi));
@@ -182,18 +197,20 @@ __device__ __forceinline__ void project(unsigned char* __restrict__ sm, int r, c
         for (int c = 0; c < 4; ++c) {
           const int j = 8 * (nt0 + c) + 2 * t;
           put(acc[c], j);
-          if (o.Vr != nullptr) {
-            if (i0 < r) *reinterpret_cast<float2*>(o.Vr + (size_t)i0 * D + j) = make_float2(acc[c][0], acc[c][1]);
-            if (i0 + 8 < r) *reinterpret_cast<float2*>(o.Vr + (size_t)(i0 + 8) * D + j) = make_float2(acc[c][2], acc[c][3]);
-          }
-          if (o.Vkm != nullptr) {                             // zero rows come out of zero rows of V Sigma
-            uint32_t hi, lo;
-            split2(acc[c][0], acc[c][1], hi, lo);
-            *reinterpret_cast<uint32_t*>(o.Vkm + (size_t)i0 * D + j) = hi;
-            *reinterpret_cast<uint32_t*>(o.Vkm + (size_t)(kTokenSlots + i0) * D + j) = lo;
-            split2(acc[c][2], acc[c][3], hi, lo);
-            *reinterpret_cast<uint32_t*>(o.Vkm + (size_t)(i0 + 8) * D + j) = hi;
-            *reinterpret_cast<uint32_t*>(o.Vkm + (size_t)(kTokenSlots + i0 + 8) * D + j) = lo;
+          if constexpr (!TILES) {
+            if (o.Vr != nullptr) {
+              if (i0 < r) *reinterpret_cast<float2*>(o.Vr + (size_t)i0 * D + j) = make_float2(acc[c][0], acc[c][1]);
+              if (i0 + 8 < r) *reinterpret_cast<float2*>(o.Vr + (size_t)(i0 + 8) * D + j) = make_float2(acc[c][2], acc[c][3]);
+            }
+            if (o.Vkm != nullptr) {                             // zero rows come out of zero rows of V Sigma
+              uint32_t hi, lo;
+              split2(acc[c][0], acc[c][1], hi, lo);
+              *reinterpret_cast<uint32_t*>(o.Vkm + (size_t)i0 * D + j) = hi;
+              *reinterpret_cast<uint32_t*>(o.Vkm + (size_t)(kTokenSlots + i0) * D + j) = lo;
+              split2(acc[c][2], acc[c][3], hi, lo);
+              *reinterpret_cast<uint32_t*>(o.Vkm + (size_t)(i0 + 8) * D + j) = hi;
+              *reinterpret_cast<uint32_t*>(o.Vkm + (size_t)(kTokenSlots + i0 + 8) * D + j) = lo;
+            }
           }
         }
       }
@@ -238,32 +255,44 @@ __device__ __forceinline__ void project(unsigned char* __restrict__ sm, int r, c
           for (int q = 0; q < 4; ++q) tc[c][q] *= scale;
           const int k0 = 8 * (nt0 + c) + 2 * t;
           uint32_t hi, lo;
-          split2(tc[c][0], tc[c][1], hi, lo);
-          *reinterpret_cast<uint32_t*>(o.Tpk + (size_t)i0 * D + k0) = hi;
-          *reinterpret_cast<uint32_t*>(o.Tpk + ((size_t)kTokenSlots + i0) * D + k0) = lo;
-          split2(tc[c][2], tc[c][3], hi, lo);
-          *reinterpret_cast<uint32_t*>(o.Tpk + (size_t)(i0 + 8) * D + k0) = hi;
-          *reinterpret_cast<uint32_t*>(o.Tpk + ((size_t)kTokenSlots + i0 + 8) * D + k0) = lo;
-          if (KINDS == 1 && o.Tkm != nullptr) put(tc[c], k0);
-          if (o.Tf != nullptr) {
-            if (i0 < r) { o.Tf[(size_t)k0 * r + i0] = tc[c][0]; o.Tf[(size_t)(k0 + 1) * r + i0] = tc[c][1]; }
-            if (i0 + 8 < r) { o.Tf[(size_t)k0 * r + i0 + 8] = tc[c][2]; o.Tf[(size_t)(k0 + 1) * r + i0 + 8] = tc[c][3]; }
+          if constexpr (TILES) {
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {                        // token rows i0, i0 + 8
+              split2(tc[c][2 * h], tc[c][2 * h + 1], hi, lo);
+              unsigned char* at = o.T + ptx::swz128(i0 + 8 * h, k0 >> 3) + 2 * (k0 & 7);
+              *reinterpret_cast<uint32_t*>(at) = hi;
+              *reinterpret_cast<uint32_t*>(at + rp16 * 128) = lo;
+            }
+          } else {
+            split2(tc[c][0], tc[c][1], hi, lo);
+            *reinterpret_cast<uint32_t*>(o.Tpk + (size_t)i0 * D + k0) = hi;
+            *reinterpret_cast<uint32_t*>(o.Tpk + ((size_t)kTokenSlots + i0) * D + k0) = lo;
+            split2(tc[c][2], tc[c][3], hi, lo);
+            *reinterpret_cast<uint32_t*>(o.Tpk + (size_t)(i0 + 8) * D + k0) = hi;
+            *reinterpret_cast<uint32_t*>(o.Tpk + ((size_t)kTokenSlots + i0 + 8) * D + k0) = lo;
+            if (KINDS == 1 && o.Tkm != nullptr) put(tc[c], k0);
+            if (o.Tf != nullptr) {
+              if (i0 < r) { o.Tf[(size_t)k0 * r + i0] = tc[c][0]; o.Tf[(size_t)(k0 + 1) * r + i0] = tc[c][1]; }
+              if (i0 + 8 < r) { o.Tf[(size_t)k0 * r + i0 + 8] = tc[c][2]; o.Tf[(size_t)(k0 + 1) * r + i0 + 8] = tc[c][3]; }
+            }
           }
         }
       }
     }
   }
-  // what was staged, as 16-byte pieces of the rows [h][j][0 .. rp16); Tkm is read to its 64th column
-  __nv_bfloat16* dst = (KINDS & 2) ? o.Vpk : o.Tkm;
-  if ((KINDS & 2) || dst != nullptr) {
-    __syncthreads();
-    const int pc = (KINDS & 2) ? rp16 / 8 : kTokenSlots / 8;
-    const unsigned inv = pc == 2 ? 32768u : pc == 4 ? 16384u : pc == 6 ? 10923u : 8192u;    // 2^16 / pc, up: exact for e < 2048
+  if constexpr (!TILES) {
+    // what was staged, as 16-byte pieces of the rows [h][j][0 .. rp16); Tkm is read to its 64th column
+    __nv_bfloat16* dst = (KINDS & 2) ? o.Vpk : o.Tkm;
+    if ((KINDS & 2) || dst != nullptr) {
+      __syncthreads();
+      const int pc = (KINDS & 2) ? rp16 / 8 : kTokenSlots / 8;
+      const unsigned inv = pc == 2 ? 32768u : pc == 4 ? 16384u : pc == 6 ? 10923u : 8192u;    // 2^16 / pc, up: exact for e < 2048
 #pragma unroll 4
-    for (int e = tid; e < 2 * D * pc; e += NT) {
-      const int row = (int)((unsigned)e * inv >> 16), c = e - row * pc;                    // row runs over [2][D]
-      reinterpret_cast<uint4*>(dst + (size_t)row * kTokenSlots)[c] =
-          c < rp16 / 8 ? *reinterpret_cast<const uint4*>(stage + ((size_t)row * (rp16 + 8) + 8 * c) * 2) : make_uint4(0u, 0u, 0u, 0u);
+      for (int e = tid; e < 2 * D * pc; e += NT) {
+        const int row = (int)((unsigned)e * inv >> 16), c = e - row * pc;                    // row runs over [2][D]
+        reinterpret_cast<uint4*>(dst + (size_t)row * kTokenSlots)[c] =
+            c < rp16 / 8 ? *reinterpret_cast<const uint4*>(stage + ((size_t)row * (rp16 + 8) + 8 * c) * 2) : make_uint4(0u, 0u, 0u, 0u);
+      }
     }
   }
 }

@@ -220,6 +220,9 @@ solar_status_t solar_svd_attention_fwd(int B, int M, int N, int d, int r, solar_
   SOLAR_TRY(check_ptr(Wk));
   SOLAR_TRY(check_ptr(Wv));
   SOLAR_TRY(check_ws(workspace, workspace_bytes, attn_ws_bytes(B, d, r)));
+  if (attn_own_supported(B, M, d, r, dt))
+    return from_cuda(launch_attn_own(B, M, r, C, S, V, Wq, Wk, Wv, scale, flags, O, static_cast<char*>(workspace),
+                                     attn_ws_layout(d, r), static_cast<cudaStream_t>(stream)));
   SOLAR_TRY(from_cuda(launch_attn_prepare(B, d, r, dt, S, V, Wq, Wk, Wv, scale, static_cast<char*>(workspace),
                                           attn_ws_layout(d, r), false, nullptr, static_cast<cudaStream_t>(stream))));
   return attn_apply_impl(B, M, d, r, dt, C, flags, O, static_cast<const char*>(workspace), true,

@@ -240,6 +240,10 @@ FlashSplit flash_split(int B, int M, int N, int d, int r, size_t workspace_bytes
 cudaError_t launch_flash_factored(int B, int M, int N, int d, int r, const void* C, const void* US, void* O,
                                   char* ws, const AttnWs& lay, const FlashSplit& split, cudaStream_t st);
 bool attn_umma_supported(int d, solar_dtype_t dt);
+// The attention kernel whose CTAs make the operands from S, V and the weights themselves.
+bool attn_own_supported(int B, int M, int d, int r, solar_dtype_t dt);
+cudaError_t launch_attn_own(int B, int M, int r, const void* C, const float* S, const float* V, const void* Wq, const void* Wk,
+                            const void* Wv, float scale, unsigned flags, void* O, char* ws, const AttnWs& lay, cudaStream_t st);
 // Throughput form of the tensor-core attention kernel: long CTAs that overlap the candidate
 // stream, the GEMMs and the softmax of consecutive tiles (chosen under a slice limit).
 bool attn_pipe_supported(int M, int d, int r, solar_dtype_t dt);
