@@ -77,6 +77,13 @@ template <int D> struct TriCfg {
   // anyway (64 users, d = r = 64: 1.4 % faster than with three).
   static constexpr int ctas(int rp) { return D == 128 ? 1 : rp > 32 ? 2 : 3; }
   static constexpr int LD = D + 4;                    // pitch of Q^T and of the row-major G
+  // of a thread's tile: the entry at(m, c) on the diagonal in row row0 + 32 rr, where its columns have it
+  template <typename F> __device__ static __forceinline__ auto diagonal(F at, int rr, int row0) {
+    const bool up = CW < 32 && (row0 & 16);
+    auto four = [&](int c) { return up ? at((32 * rr + 16) / CW, c) : at(32 * rr / CW, c); };
+    const auto a = (row0 & 1) ? four(1) : four(0), b = (row0 & 1) ? four(3) : four(2);
+    return (row0 & 2) ? b : a;
+  }
 };
 
 // Shared-memory layout (floats) for subspace width RP = 32 * ceil(r / 32).
@@ -136,6 +143,11 @@ __device__ __forceinline__ float lg2(float x) {
   asm("lg2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
   return y;
 }
+__device__ __forceinline__ float ex2(float x) {
+  float y;
+  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+  return y;
+}
 // 1 / sqrt(x) and 1 / x to the accuracy of the type for normal x (the hardware's approximation plus one
 // Newton step in fp32, two in fp64; without the library functions' branches for special values):
 // the reflector I - beta v v^T is orthogonal only as far as beta v^T v = 2 holds.
@@ -173,6 +185,7 @@ __device__ __forceinline__ double pow2_scale(double p, double q) {
   const int m = max(__double2hiint(p) & 0x7ff00000, __double2hiint(q) & 0x7ff00000);
   return __hiloint2double(0x7fe00000 - m, 0);
 }
+__device__ __forceinline__ int log2_int(float x) { return (int)(__float_as_uint(x) >> 23) - 127; }       // of x >= 0, rounded down; denormals -127
 __device__ __forceinline__ int exponent(float pow2) { return (int)(__float_as_uint(pow2) >> 23) - 127; }
 __device__ __forceinline__ int exponent(double pow2) { return (__double2hiint(pow2) >> 20) - 1023; }
 __device__ __forceinline__ void ld4(const float* p, float (&o)[4]) {
@@ -622,7 +635,7 @@ __device__ __forceinline__ bool tri_chain(const float (&acc)[TriCfg<D>::RT][TriC
     s.stop_tr = trs * tol.stop_trace;
     s.stop_x2 = (trs * tol.stop_couple) * (trs * tol.stop_couple);
     s.k_stop = -1;
-    s.sx = trs * exp2f(-1.f - 0.5f * (float)lane); s.lx = 2.f * lg2(s.sx) - 2.f;     // trace / 2 .. trace / 2^16.5
+    s.sx = trs * ex2(-1.f - 0.5f * (float)lane); s.lx = 2.f * lg2(s.sx) - 2.f;     // trace / 2 .. trace / 2^16.5
     s.cpl = 0.f; s.left = s.lx; s.above = 0;
 #pragma unroll
     for (int rr = 0; rr < RT; ++rr)
@@ -1172,11 +1185,11 @@ __device__ __forceinline__ bool tri_chain(const float (&acc)[TriCfg<D>::RT][TriC
       for (int w = 0; w < NW; ++w) rho2 += part[(2 * NW + w) * RP + tid];
       if (tid > 0) gap = fminf(gap, theta[tid - 1] - thi);
       if (tid < r - 1) gap = fminf(gap, thi - theta[tid + 1]);
-      const float resn = sqrtf(rho2);
-      const bool res_ok = resn <= fmaxf(tol.eps_vec * gap, tol.floor_rel * th1);
+      const float most = fmaxf(tol.eps_vec * gap, tol.floor_rel * th1);
+      const bool res_ok = (int)(most >= 0.f) & (int)(rho2 <= most * most);
       // T is similar to sc * G: the traces agree to rounding
       const float trG = (float)((double)sc * sh.trace);
-      const bool tr_ok = fabsf(sh.tr_t - trG) <= 1e-4f * fabsf(trG) && isfinite(thi) && isfinite(resn);
+      const bool tr_ok = fabsf(sh.tr_t - trG) <= 1e-4f * fabsf(trG) && isfinite(thi) && isfinite(rho2);
       if (!res_ok) atomicOr(&sh.why, kWhyResidual);
       if (!tr_ok) atomicOr(&sh.why, kWhyTrace);
       good = res_ok && tr_ok;
@@ -1259,12 +1272,16 @@ __device__ __forceinline__ EigEnd eig_user(int b, int half, bool& joined, const 
 #pragma unroll
         for (int c = 0; c < 4; ++c) {
           zero = fmaf(acc[rr][m][c], 0.f, zero);             // NaN where an entry is not finite
-          st_if(part + row0 + 32 * rr, acc[rr][m][c], CW * m + 4 * g + c == row0 + 32 * rr);
+          if (D == 128) st_if(part + row0 + 32 * rr, acc[rr][m][c], CW * m + 4 * g + c == row0 + 32 * rr);
         }
         if (parts > 1)                                        // read back by the residual check and the fallback
           reinterpret_cast<float4*>(gsum + (size_t)b * D * D)[(row0 + 32 * rr) * (D / 4) + GX * m + g] =
               make_float4(acc[rr][m][0], acc[rr][m][1], acc[rr][m][2], acc[rr][m][3]);
       }
+    // (d = 128: one store of these per row makes the steps' schedule worse, 149.8 -> 153.7 us for 8 x 4096 x 128)
+#pragma unroll
+    for (int rr = 0; rr < (D == 128 ? 0 : RT); ++rr)
+      st_if(part + row0 + 32 * rr, C::diagonal([&](int m, int c) { return acc[rr][m][c]; }, rr, row0), ((row0 & (CW - 1)) >> 2) == g);
     if (tid < 4) sh.flags[tid] = 0;
     if (tid == 0) sh.why = 0;
     if (__syncthreads_or(lost | (int)!(zero == 0.f))) {
@@ -1293,7 +1310,7 @@ __device__ __forceinline__ EigEnd eig_user(int b, int half, bool& joined, const 
   }
   // Power-of-two scale that brings the largest diagonal entry into [1, 2): everything below works
   // on sc * G (exact), and the eigenvalues are divided by sc at the end.
-  const float sc = gmax > 0.f ? exp2f(-(float)max(-100, min(100, ilogbf(gmax)))) : 1.f;
+  const float sc = gmax > 0.f ? __uint_as_float((unsigned)(127 - max(-100, min(100, log2_int(gmax)))) << 23) : 1.f;
   __syncthreads();
 
   if (route != kRouteFull && gmax > 0.f) {
