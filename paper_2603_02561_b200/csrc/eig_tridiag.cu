@@ -1309,8 +1309,10 @@ __device__ __forceinline__ EigEnd eig_user(int b, int half, bool& joined, const 
     if (tid == 0) sh.trace = tr;
   }
   // Power-of-two scale that brings the largest diagonal entry into [1, 2): everything below works
-  // on sc * G (exact), and the eigenvalues are divided by sc at the end.
-  const float sc = gmax > 0.f ? __uint_as_float((unsigned)(127 - max(-100, min(100, log2_int(gmax)))) << 23) : 1.f;
+  // on sc * G (exact), and the eigenvalues are divided by sc at the end.  The thresholds of the chain are absolute and
+  // the Sturm recurrence relies on the range, so it has to hold for every normal entry (the scale and 1 / scale are normal
+  // to 2^+-126; with a limit of 2^+-100 entries from 2^116 on, or below 2^-113, sent every user through the fp64 chain).
+  const float sc = gmax > 0.f ? __uint_as_float((unsigned)(127 - max(-126, min(126, log2_int(gmax)))) << 23) : 1.f;
   __syncthreads();
 
   if (route != kRouteFull && gmax > 0.f) {
