@@ -46,9 +46,8 @@ struct OwnArgs { const float *S, *V; const void *Wq, *Wk, *Wv; float scale; char
 constexpr int kOwnThreads = 256;           // the second half helps with the projections only
 
 // OWN (factors kept from an earlier call, d = 64, r <= 32, few CTAs): every CTA makes T^T and
-// Value_r^T of its user in shared memory, by the routine of the projection kernel (the same bits).  The two
-// launches were the bound of such a call: 8 x 3000 candidates, r = 27: 13.3 us per call with two launches (3.2 us of
-// the host's time each), 11.0 with one.
+// Value_r^T of its user in shared memory, by the routine of the projection kernel (the same bits).  Two
+// launches are the bound of such a call (3.2 us of the host's time each); figures at attn_own_supported().
 template <int D, bool OWN>
 __global__ void __launch_bounds__(OWN ? kOwnThreads : 128)
 attn_umma_kernel(const __grid_constant__ CUtensorMap tmC, const __grid_constant__ CUtensorMap tmO,
@@ -114,13 +113,17 @@ attn_umma_kernel(const __grid_constant__ CUtensorMap tmC, const __grid_constant_
     const int rp = (r + 3) & ~3;
     pmma::Weights<D, kOwnThreads, 3> w;
     w.load(own.Wq, own.Wk, own.Wv, tid);
-    const float* Vb = own.V + (size_t)b * D * r;
-    const unsigned inv = ((1u << 20) + rp - 1) / rp;                               // 2^20 / rp, up: exact for e < D rp
-#pragma unroll 8
-    for (int e = tid; e < D * rp; e += kOwnThreads) {
-      const int k = (int)((unsigned)e * inv >> 20), i = e - k * rp, ic = min(i, r - 1);
-      const float v = ld_dep(Vb + (size_t)k * r + ic), s = ld_dep(own.S + (size_t)b * r + ic);
-      VS[e] = i < r ? v * s : 0.f;
+    // A token per lane, every eighth row per warp, and all loads of a thread on their way before its first store: a load
+    // behind a store waits for it, eight of them in turn were 1.1 us (16 x 1536 candidates, r = 32, as graph nodes 9.5 -> 8.4).
+    const int i = tid & 31, ic = min(i, r - 1);
+    const float* Vb = own.V + (size_t)b * D * r + (size_t)warp * r + ic;
+    const float s = ld_dep(own.S + (size_t)b * r + ic);
+    float v[D * 32 / kOwnThreads];
+#pragma unroll
+    for (int n = 0; n < D * 32 / kOwnThreads; ++n) v[n] = ld_dep(Vb + n * (kOwnThreads / 32) * r);
+    if (i < rp) {
+#pragma unroll
+      for (int n = 0; n < D * 32 / kOwnThreads; ++n) VS[(warp + n * (kOwnThreads / 32)) * rp + i] = i < r ? v[n] * s : 0.f;
     }
     __syncthreads();
     pmma::project<D, kOwnThreads, 3>(sw, r, w, own.scale, pmma::Tiles{sT, sV}, tid);
@@ -169,7 +172,7 @@ attn_umma_kernel(const __grid_constant__ CUtensorMap tmC, const __grid_constant_
   }
   // ---- softmax over the r tokens, one candidate row per thread -------------------------
   const bool have_s = ptx::mbar_wait(&bar_s, 0, err, kErrScores);
-  pdl_trigger();       // loads and the score GEMM are done: the next kernel may start launching
+  pdl_trigger();       // loads and the score GEMM are done (OWN: so the last of the CTA's threads come here): the next kernel may start launching
   __syncwarp();
   ptx::tc_fence_after_sync();
   const uint32_t lane_base = (uint32_t)(warp * 32) << 16;
@@ -318,11 +321,15 @@ constexpr int kOwnTokens = 32;
 
 }  // namespace
 
-// As long as no more than every second SM has two of these CTAs.  us per call, one launch and two (as queued calls,
-// which the host's launches bound, and in a graph): 8 x 2048 candidates (128 CTAs) 10.2 / 8.5 and 12.3 / 8.7,
-// 128 x 120 (128) 10.3 / 8.6 and 13.5 / 12.8, 8 x 3000 (192) 10.2 / 9.6 and 12.4 / 9.3, 16 x 1536 (192) 10.3 / 9.6 and
-// 12.2 / 8.3, 16 x 2048 (256) 10.4 / 9.6 and 12.2 / 8.7 -- and there the training step, whose kernels are the bound, is 1 us
-// slower.  Under a slice limit other requests want the SMs.
+// As long as no more than every second SM has two of these CTAs.  us per call with one launch and with two, as queued calls
+// (where the host's launches bound two) and as nodes of a graph (where the device bounds both):
+//   1 x 128 candidates, r = 27     (1 CTA)  8.8 / 11.4   6.2 / 8.2      8 x 3000, r = 27  (192)  9.0 / 11.4  8.4 / 9.3
+//   8 x 2048, r = 27             (128 CTAs) 9.0 / 11.5   7.4 / 8.8      16 x 1536, r = 32 (192)  9.0 / 11.4  8.4 / 8.4
+//   128 x 120, r = 27                (128)  9.0 / 13.4   7.4 / 12.8     12 x 2048, r = 32 (192)  9.1 / 11.5  8.4 / 8.3
+//   12 x 1536, r = 32                (144)  9.0 / 11.2   7.7 / 7.7      222 x 128, r = 8  (222)  9.0 / 13.4  7.7 / 12.7
+// Training steps at 128 to 216 CTAs, queued: 0.1 to 2.8 us shorter with one.  Beyond the line the device is the bound: 256 CTAs
+// (16 x 2048, r = 32) 8.5 / 8.7 as nodes, 296 (37 x 1000) 45.3 / 45.0 for a forward call and the backward one behind it.
+// Under a slice limit other requests want the SMs.
 bool attn_own_supported(int B, int M, int d, int r, solar_dtype_t dt) {
   return dt == SOLAR_BF16 && d == 64 && r <= kOwnTokens && slice_limit() == 0 &&
          (long)B * ((M + kRows - 1) / kRows) <= kNumSMs * 3 / 2;
