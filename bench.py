@@ -626,7 +626,7 @@ def measure(args, w, torch, dist, solar, world, rank, local, light=False):
     dominant = max(stage_ms, key=stage_ms.get)
     tot = sum(stage_ms.values())
     routes = sorted(set(int(x) & 0xFF for x in route_words))
-    iters = float(np.mean([(int(x) >> 8) & 0xFF for x in route_words]))
+    iters = float(np.mean([(int(x) >> 8) & 0xFF if int(x) & 0xFF != 3 else 0 for x in route_words]))     # (route 3: rows of T)
     sweeps = float(np.mean([(int(x) >> 16) & 0xFF for x in route_words]))
     eflops = eig_flops(w, max(routes), iters, sweeps)
     per_kernel = {

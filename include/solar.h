@@ -218,11 +218,12 @@ solar_status_t solar_eig_from_partials(int B, int N, int d, int r, solar_dtype_t
 
 /* As above with the route chosen by the caller.  route_taken (device, [B] ints, or
  * NULL) receives per user: route used (1 subspace, 2 full, 3 tridiagonal; 0 = non-finite
- * input) | power steps << 8 (route 2: 1 if it was the double-precision tridiagonal chain) |
+ * input) | power steps << 8 (route 2: 1 if it was the double-precision tridiagonal chain;
+ * route 3: rows of the tridiagonal matrix, fewer than d where the reduction ended early) |
  * Jacobi sweeps (tridiagonal chains: orthogonalisation passes) << 16 | reason << 24, where reason says why the first route tried was not certified: 1 no gap
  * at the cut, 2 residual too large for its gap, 4 a kept eigenvalue not positive, 8 sweep
- * cap, 16 non-finite pivot, 32 vectors of a cluster not independent, 64 trace mismatch
- * or a non-finite value, 128 a gap between kept eigenvalues too small for fp32. */
+ * cap, 16 non-finite pivot, 32 vectors of a cluster not independent, 64 trace mismatch,
+ * rows left out that may hold a kept eigenvalue, or a non-finite value, 128 a gap between kept eigenvalues too small for fp32. */
 solar_status_t solar_eig_from_partials_ex(int B, int N, int d, int r, solar_dtype_t dt, int route,
                                           float* S, float* V, int* info, int* route_taken,
                                           void* workspace, size_t workspace_bytes, void* stream);

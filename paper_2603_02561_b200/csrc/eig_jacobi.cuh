@@ -20,7 +20,7 @@ constexpr float kTolRel = 2.3841858e-07f;  // 2^-22: |g_pq| <= tol*sqrt(g_pp g_q
 constexpr float kTolAbs = 7.4505806e-09f;  // 2^-27 of the largest diagonal entry
 constexpr float kUnit = 5.9604645e-08f;    // 2^-24, fp32 unit roundoff
 
-// route_taken[b] = route | detail << 8 | sweeps or passes << 16 | kWhy* bits << 24
+// route_taken[b] = route | detail << 8 | sweeps or passes << 16 | kWhy* bits << 24; detail of route 3: the rows of T
 constexpr int kRouteSubspace = 1, kRouteFull = 2, kRouteTridiag = 3;
 constexpr int kDetailWide = 1;      // route 2: the tridiagonal chain in double precision answered, not the Jacobi solve
 // Why a route's result was not certified (0 = it was, or it was not tried):
@@ -30,7 +30,7 @@ constexpr int kWhyNotPositive = 4;  // a kept Ritz value is not positive (rank(H
 constexpr int kWhySweepCap = 8;     // the Ritz Jacobi hit its sweep cap
 constexpr int kWhyCholesky = 16;    // non-finite pivot in the Cholesky-QR
 constexpr int kWhyOrtho = 32;       // tridiagonal route: vectors of a cluster came out dependent
-constexpr int kWhyTrace = 64;       // tridiagonal route: trace of T differs from trace of G, or not finite
+constexpr int kWhyTrace = 64;       // tridiagonal route: trace of T differs from trace of G, the rows left out may hold a kept eigenvalue, or not finite
 constexpr int kWhyGap = 128;        // tridiagonal route: a gap between kept eigenvalues is too small for fp32
 
 // Rotation J = [[c, s], [-s, c]] that annihilates g_pq of the 2x2 symmetric block

@@ -28,7 +28,8 @@
 //      the columns of larger eigenvalues.
 //   7. Rayleigh quotients theta_i = v_i^T G v_i and residuals G v_i - theta_i v_i against the
 //      ORIGINAL G: the result is accepted only if every residual is small against its gap (or
-//      at the rounding floor), V^T V = I to rounding, and trace(T) = trace(G).
+//      at the rounding floor), V^T V = I to rounding, trace(T) and the trace of the rows left out add up to
+//      trace(G), and those rows cannot hold an eigenvalue above the last kept one.
 //
 // The chain runs in fp32 first.  A reduction to tridiagonal form is backward stable in the norm of
 // G only: it fixes a kept vector to an angle of a few eps |T| / gap, whatever the size of its
@@ -51,6 +52,7 @@
 // with fixed live columns; conditions are predicates of single instructions), fetches ahead, and
 // keeps divisions off the dependency chains.
 #include "eig_jacobi.cuh"
+#include "eig_rest.cuh"
 #include "project_mma.cuh"
 
 namespace solar {
@@ -586,7 +588,8 @@ struct TriTol {
 
 struct TriShared {
   double trace;
-  float tr_t;
+  float tr_t, rest;  // traces of T and of the rows left out
+  int rows;          // of T
   float stop[2];
   int flags[4];
   int why;
@@ -669,7 +672,7 @@ __device__ __forceinline__ bool tri_chain(const float (&acc)[TriCfg<D>::RT][TriC
       __syncthreads();
       if (s.k_stop < 0 && *(volatile float*)(sh.stop + (D & 1)) != 0.f) s.k_stop = D - 3;
     }
-    // the diagonal of the rows left out by an early end, for the comparison of the traces
+    // the diagonal of the rows left out by an early end, for the certificate
     if (!F64 && s.k_stop >= 0) {
 #pragma unroll
       for (int rr = 0; rr < RT; ++rr) {
@@ -712,6 +715,7 @@ __device__ __forceinline__ bool tri_chain(const float (&acc)[TriCfg<D>::RT][TriC
   T lo, hi, tnorm;
   {
     T l = T(3.0e38), h = T(-3.0e38), tr = 0;
+    float rest = 0.f;
 #pragma unroll
     for (int q = 0; q < D / 32; ++q) {
       const int n = lane + 32 * q;
@@ -722,13 +726,14 @@ __device__ __forceinline__ bool tri_chain(const float (&acc)[TriCfg<D>::RT][TriC
       l = ((int)in & (int)(dd - rad < l)) ? dd - rad : l;
       h = ((int)in & (int)(dd + rad > h)) ? dd + rad : h;
       tr += dd;
-      if (!F64 && n >= de) tr += (T)part[n];
+      if (!F64 && n >= de) rest += part[n];
     }
 #pragma unroll
     for (int o = 16; o; o >>= 1) {
       const T l2 = __shfl_xor_sync(kFull, l, o), h2 = __shfl_xor_sync(kFull, h, o);
       l = l2 < l ? l2 : l; h = h2 > h ? h2 : h;
       tr += __shfl_xor_sync(kFull, tr, o);
+      if (!F64) rest += __shfl_xor_sync(kFull, rest, o);
     }
     const T span = h - l;
     lo = l - T(1e-6) * span - T(1e-30); hi = h + T(1e-6) * span + T(1e-30);
@@ -739,7 +744,7 @@ __device__ __forceinline__ bool tri_chain(const float (&acc)[TriCfg<D>::RT][TriC
         const T e = n > 0 ? eo[n - 1] : T(0);
         e2s[n] = n > 0 ? (e * e > fl * fl ? e * e : fl * fl) : T(0);
       }
-      if (lane == 0) sh.tr_t = (float)tr;
+      if (lane == 0) { sh.tr_t = (float)tr; sh.rest = rest; sh.rows = de; }
     }
   }
   __syncthreads();
@@ -1187,9 +1192,10 @@ __device__ __forceinline__ bool tri_chain(const float (&acc)[TriCfg<D>::RT][TriC
       if (tid < r - 1) gap = fminf(gap, thi - theta[tid + 1]);
       const float most = fmaxf(tol.eps_vec * gap, tol.floor_rel * th1);
       const bool res_ok = (int)(most >= 0.f) & (int)(rho2 <= most * most);
-      // T is similar to sc * G: the traces agree to rounding
+      // T and the rows left out are similar to sc * G: the traces agree to rounding; and nothing kept is among those rows
       const float trG = (float)((double)sc * sh.trace);
-      const bool tr_ok = fabsf(sh.tr_t - trG) <= 1e-4f * fabsf(trG) && isfinite(thi) && isfinite(rho2);
+      const bool tr_ok = fabsf(sh.tr_t + sh.rest - trG) <= 1e-4f * fabsf(trG) && rest_keeps_result(sh.rest, trG, theta[r - 1]) &&
+                         isfinite(thi) && isfinite(rho2);
       if (!res_ok) atomicOr(&sh.why, kWhyResidual);
       if (!tr_ok) atomicOr(&sh.why, kWhyTrace);
       good = res_ok && tr_ok;
@@ -1389,7 +1395,7 @@ __device__ __forceinline__ EigEnd eig_user(int b, int half, bool& joined, const 
       }
       if (tid == 0) {
         if (info) info[b] = ok ? 0 : SOLAR_INFO_NOT_CERTIFIED;
-        if (route_taken) route_taken[b] = (wide ? kRouteFull | (kDetailWide << 8) : kRouteTridiag) | (passes << 16) | (sh.why << 24);
+        if (route_taken) route_taken[b] = (wide ? kRouteFull | (kDetailWide << 8) : kRouteTridiag | (sh.rows << 8)) | (passes << 16) | (sh.why << 24);
       }
       return want_vs ? kEndedVs : kEnded;
     }
