@@ -677,10 +677,7 @@ __device__ __forceinline__ bool tri_chain(const float (&acc)[TriCfg<D>::RT][TriC
 #pragma unroll
       for (int rr = 0; rr < RT; ++rr) {
         const int row = row0 + 32 * rr;
-        float t[4];
-#pragma unroll
-        for (int c = 0; c < 4; ++c) t[c] = (float)(CW == 32 || row0 < 16 ? s.a[rr][32 * rr / CW][c] : s.a[rr][(32 * rr + 16) / CW][c]);
-        const float v = (row & 2) ? ((row & 1) ? t[3] : t[2]) : ((row & 1) ? t[1] : t[0]);
+        const float v = (float)C::diagonal([&](int m, int c) { return s.a[rr][m][c]; }, rr, row0);
         st_if(part + row, v, (int)(row > s.k_stop) & (int)(((row & (CW - 1)) >> 2) == g));
       }
     }
@@ -1284,7 +1281,9 @@ __device__ __forceinline__ EigEnd eig_user(int b, int half, bool& joined, const 
           reinterpret_cast<float4*>(gsum + (size_t)b * D * D)[(row0 + 32 * rr) * (D / 4) + GX * m + g] =
               make_float4(acc[rr][m][0], acc[rr][m][1], acc[rr][m][2], acc[rr][m][3]);
       }
-    // (d = 128: one store of these per row makes the steps' schedule worse, 149.8 -> 153.7 us for 8 x 4096 x 128)
+    // (d = 128: one store of these per row makes the steps' schedule worse, 149.8 -> 153.7 us for 8 x 4096 x 128.  d = 64, r <= 32:
+    // the selection costs one spilled pair of registers, here and not in the steps; four predicated stores a row need none
+    // and are as fast: 128 x 50 42.6 -> 42.5 us per pass, 32 x 1024 33.6 -> 33.8.)
 #pragma unroll
     for (int rr = 0; rr < (D == 128 ? 0 : RT); ++rr)
       st_if(part + row0 + 32 * rr, C::diagonal([&](int m, int c) { return acc[rr][m][c]; }, rr, row0), ((row0 & (CW - 1)) >> 2) == g);
