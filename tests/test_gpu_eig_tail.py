@@ -75,6 +75,8 @@ def test_where_the_reduction_ends(d, dtype):
         taken = torch.full_like(info, -1)
         ws = solar.alloc_workspace(B, 1, 300, d, r, dtype)
         solar.gram_partials(H[keep].contiguous(), ws)
+        parts = solar.gram_splits(B, 300, d, dtype)
+        G = ws[: B * parts * d * d * 4].view(torch.float32).reshape(B, parts, d, d).double().sum(1)
         solar.eig_from_partials_ex(B, 300, d, r, dtype, solar.ROUTE_AUTO, S, V, info, taken, ws)
         for i, word in zip(keep, taken.tolist()):
             R, tag = ranks[i // 3], (ranks[i // 3], noises[i % 3], r, hex(word & 0xFFFFFFFF))
@@ -84,6 +86,10 @@ def test_where_the_reduction_ends(d, dtype):
             if R + slack[i % 3] < d:
                 assert rows <= R + slack[i % 3], tag
         assert torch.all(info == 0)
+        # what the end leaves is below the rounding of the chain: a few 2^-24 of the largest eigenvalue (9), and far below
+        # what the certificate lets pass
+        left = (G @ V.double() - V.double() * (S.double() ** 2)[:, None, :]).norm(dim=1)
+        assert float(left.max()) <= 32 * 2.0 ** -24 * 9.0, r
 
 
 def test_a_noise_direction_that_is_kept_keeps_its_rows():
