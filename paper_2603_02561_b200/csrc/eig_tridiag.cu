@@ -327,7 +327,7 @@ __device__ __forceinline__ void tri_prepare(TriState<T, D, KEEP>& s, const TriOu
 // ---- Householder steps k whose column k+1 lies in chunk M ---------------------------------------
 // A <- H A H with H = I - beta v v^T: w = u - kappa v, u = A v, kappa = beta v^T u / 2,
 // A <- A - beta (v w^T + w v^T); Q <- Q H.
-template <int M, typename T, int D, bool KEEP>
+template <int M, int RP, typename T, int D, bool KEEP>
 __device__ __forceinline__ void tri_stage(TriState<T, D, KEEP>& s, const TriOut<T>& o, int tid) {
   using C = TriCfg<D>;
   constexpr int GX = C::GX, RT = C::RT, NCH = C::NCH, CW = C::CW, NW = C::NW;
@@ -348,6 +348,35 @@ __device__ __forceinline__ void tri_stage(TriState<T, D, KEEP>& s, const TriOut<
       if (!F64 && *(volatile float*)(o.stop + par) != 0.f) { s.k_stop = k - 1; return; }
       continue;
     }
+    // Whether T may end at row k.  The vote, and what the answer goes into, come behind the update: before it they held it up
+    // (8 power-law users, r = 8: d = 32 30.8 -> 29.9 us per pass, d = 64 51.3 -> 50.8, d = 128 147.3 -> 146.6; without
+    // the tail 30.5, 51.9 and 146.4).  The scalars for it are known already at this point.  They are worked out where a schedule
+    // measured best: at d = 128 here, beside the reads; at d = 64 for r > 32 between the reflector's scalars and the
+    // update (all 64 directions 100.9 -> 100.3); else behind the update (elsewhere registers spill at d = 64).
+    bool stop = false;
+    auto look = [&] {
+      if (F64) return;
+      // Rank-revealing stop: once the rows below k carry a negligible trace (G is positive
+      // semi-definite, so that bounds every entry of the block) and row k hardly couples to them,
+      // T ends at row k.  A history of low rank -- the premise of the method -- then costs its rank
+      // in Householder steps, and every later phase works on the shorter T.
+      const float d = -(float)s.dk - s.tr_comp, t = s.tr_rest + d;   // compensated: the trace is ~10^7 stop thresholds
+      s.tr_comp = (t - s.tr_rest) - d;
+      s.tr_rest = t;
+      stop = (int)(k1 >= o.r) & (int)(t <= s.stop_tr) & (int)((float)s.s2 <= s.stop_x2);   // no branches
+      // Or the kept vectors do not reach the rows below k.  Those behind row j have trace t_j, so no eigenvalue of
+      // theirs, reduced or not, is above that, and the pivots of x - T_{j+1..k} are above x - t_j for a shift
+      // x >= 2 t_j.  Entry k of a vector of an eigenvalue above x is then at most prod_{j <= i < k} |e_i| / (x / 2)^(k-j),
+      // and times |e_k| that is the residual (for a norm of 1) that ending T at row k adds.  So T may end there once
+      // it has r eigenvalues above some x for which that is below the rounding level.  Every lane watches an x.
+      // A history of rank r plus noise, whose other rows never become negligible, so ends after about r + 5 steps
+      // instead of d - 2: 32 x 1024 x 64 with r = 16 50.4 -> 33.2 us per pass, 8 x 4096 x 128 with r = 32 149 -> 82.
+      const float pv = (s.sx - (float)s.dk) - s.cpl, s2 = (float)s.s2;
+      s.above += (int)(__float_as_uint(pv) >> 31);
+      s.cpl = s2 * rcp_fast(pv);
+      s.left = t + t <= s.sx ? s.left + (lg2(s2) - s.lx) : s.lx;
+    };
+    if (D == 128) look();
     // x^T A x; meanwhile the reflector's scalars
     const T yk1 = yv[k1], xpk1 = xp[k1];
     // A x at the thread's columns; kept for the update where there are registers for it (d = 128: a
@@ -368,37 +397,7 @@ __device__ __forceinline__ void tri_stage(TriState<T, D, KEEP>& s, const TriOut<
     const T alpha = reflect ? (s.x1 < 0 ? nrm : -nrm) : s.x1;
     const T vk1 = reflect ? s.x1 - alpha : T(0);
     const T beta = reflect ? rcp_t(nrm * abs_t(vk1)) : T(0);
-    bool stop = false;
-    if (!F64) {
-      // Rank-revealing stop: once the rows below k carry a negligible trace (G is positive
-      // semi-definite, so that bounds every entry of the block) and row k hardly couples to them,
-      // T ends at row k.  A history of low rank -- the premise of the method -- then costs its rank
-      // in Householder steps, and every later phase works on the shorter T.
-      const float d = -(float)s.dk - s.tr_comp, t = s.tr_rest + d;   // compensated: the trace is ~10^7 stop thresholds
-      s.tr_comp = (t - s.tr_rest) - d;
-      s.tr_rest = t;
-      stop = (int)(k1 >= o.r) & (int)(t <= s.stop_tr) & (int)((float)s.s2 <= s.stop_x2);   // no branches
-      // Or the kept vectors do not reach the rows below k.  Those behind row j have trace t_j, so no eigenvalue of
-      // theirs, reduced or not, is above that, and the pivots of x - T_{j+1..k} are above x - t_j for a shift
-      // x >= 2 t_j.  Entry k of a vector of an eigenvalue above x is then at most prod_{j <= i < k} |e_i| / (x / 2)^(k-j),
-      // and times |e_k| that is the residual (for a norm of 1) that ending T at row k adds.  So T may end there once
-      // it has r eigenvalues above some x for which that is below the rounding level.  Every lane watches an x.
-      // A history of rank r plus noise, whose other rows never become negligible, so ends after about r + 5 steps
-      // instead of d - 2: 32 x 1024 x 64 with r = 16 50.9 -> 35.5 us per pass, 8 x 4096 x 128 with r = 32 148 -> 82;
-      // 0.3 us (d = 128: 2) more where a spectrum has no gap behind r.
-      const float pv = (s.sx - (float)s.dk) - s.cpl, s2 = (float)s.s2;
-      s.above += (int)(__float_as_uint(pv) >> 31);
-      s.cpl = s2 * rcp_fast(pv);
-      s.left = t + t <= s.sx ? s.left + (lg2(s2) - s.lx) : s.lx;
-      stop = (int)stop | __any_sync(kFull, (int)(s.above >= o.r) & (int)(s.left <= 2.f * kTailBits));
-    }
-    const bool last = tid == C::NT - 1;
-    st_if(o.dg + k, s.dk, last);
-    st_if(o.eo + k, stop ? T(0) : alpha, last);
-    if (!KEEP) st_if(o.betas + k, (float)beta, last);
-    if (!KEEP && !F64) st_if(o.stop + (par ^ 1), stop ? 1.f : 0.f, last);
-    kend = stop ? k1 : kend;
-    s.k_stop = stop ? k : -1;              // this step is still made: it touches nothing left of column k+1
+    if (D != 128 && RP > 32) look();
     // x becomes v
 #pragma unroll
     for (int c = 0; c < 4; ++c) s.x[M][c] = (4 * g + c == kc) ? vk1 : s.x[M][c];
@@ -459,6 +458,15 @@ __device__ __forceinline__ void tri_stage(TriState<T, D, KEEP>& s, const TriOut<
         s.x[m][c] = fma_t(-bw1, v, fma_t(-bv1, w, pp[c]));   // column k+1 of the updated matrix
       }
     }
+    if (D != 128 && RP <= 32) look();
+    if (!F64) stop = (int)stop | __any_sync(kFull, (int)(s.above >= o.r) & (int)(s.left <= 2.f * kTailBits));
+    const bool last = tid == C::NT - 1;
+    st_if(o.dg + k, s.dk, last);
+    st_if(o.eo + k, stop ? T(0) : alpha, last);
+    if (!KEEP) st_if(o.betas + k, (float)beta, last);
+    if (!KEEP && !F64) st_if(o.stop + (par ^ 1), stop ? 1.f : 0.f, last);
+    kend = stop ? k1 : kend;
+    s.k_stop = stop ? k : -1;              // this step is still made: it touches nothing left of column k+1
     tri_prepare<M, T, D, KEEP>(s, o, k1, tid);
   }
 }
@@ -660,11 +668,11 @@ __device__ __forceinline__ bool tri_chain(const float (&acc)[TriCfg<D>::RT][TriC
 #pragma unroll
     for (int rr = 0; rr < RT; ++rr) s.xr[rr] = o.xp[D + row0 + 32 * rr];
     tri_prepare<0, T, D, KEEP>(s, o, 0, tid);
-    tri_stage<0, T, D, KEEP>(s, o, tid);
-    tri_stage<1, T, D, KEEP>(s, o, tid);
+    tri_stage<0, RP, T, D, KEEP>(s, o, tid);
+    tri_stage<1, RP, T, D, KEEP>(s, o, tid);
     if constexpr (NCH > 2) {
-      tri_stage<2, T, D, KEEP>(s, o, tid);
-      tri_stage<3, T, D, KEEP>(s, o, tid);
+      tri_stage<2, RP, T, D, KEEP>(s, o, tid);
+      tri_stage<3, RP, T, D, KEEP>(s, o, tid);
     }
     // Finished warps learn of a stop one barrier later.  Those that did in the loop have passed that
     // barrier there; for all others (no stop, or one in the very last step) it is this one.
@@ -1281,9 +1289,7 @@ __device__ __forceinline__ EigEnd eig_user(int b, int half, bool& joined, const 
           reinterpret_cast<float4*>(gsum + (size_t)b * D * D)[(row0 + 32 * rr) * (D / 4) + GX * m + g] =
               make_float4(acc[rr][m][0], acc[rr][m][1], acc[rr][m][2], acc[rr][m][3]);
       }
-    // (d = 128: one store of these per row makes the steps' schedule worse, 149.8 -> 153.7 us for 8 x 4096 x 128.  d = 64, r <= 32:
-    // the selection costs one spilled pair of registers, here and not in the steps; four predicated stores a row need none
-    // and are as fast: 128 x 50 42.6 -> 42.5 us per pass, 32 x 1024 33.6 -> 33.8.)
+    // (d = 128: one store of these per row makes the steps' schedule worse, 149.8 -> 153.7 us for 8 x 4096 x 128.)
 #pragma unroll
     for (int rr = 0; rr < (D == 128 ? 0 : RT); ++rr)
       st_if(part + row0 + 32 * rr, C::diagonal([&](int m, int c) { return acc[rr][m][c]; }, rr, row0), ((row0 & (CW - 1)) >> 2) == g);
