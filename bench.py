@@ -46,7 +46,6 @@ from paper_2603_02561_b200 import bench_plan as bp  # noqa: E402
 from paper_2603_02561_b200 import workloads as wl  # noqa: E402
 
 L2_BYTES = 126 * 2 ** 20
-KERNELS_PER_STEP = {"fused": 3, "two_call": 4}   # gram, eigensolve (+ projections), [projections,] attention
 FP32_ALU_TFLOPS = 148 * 128 * 2 * 1.965e9 / 1e12   # 148 SMs x 128 FMA lanes x 2 flop at 1965 MHz
 SFU_TEXPS = 148 * 16 * 1.965e9 / 1e12              # 148 SMs x 16 special-function lanes at 1965 MHz
 def measured_traffic(workload: str, kernel: str):
@@ -684,7 +683,7 @@ def measure(args, w, torch, dist, solar, world, rank, local, light=False):
         "dominant_stage": dominant,
         "eig_route": {"routes": routes, "power_steps": iters, "sweeps_or_passes": sweeps,
                       "note": "route 3 = tridiagonal (orthogonalisation passes), 2 = Jacobi (sweeps), 1 = range finder"},
-        "gpu_launches": KERNELS_PER_STEP[args.path] * steps,
+        "gpu_launches": bp.kernels_per_step(args.path, w, args.slice_limit) * steps,
         "clocks": clocks,
         "factored_exact": factored,
         "backward": backward,

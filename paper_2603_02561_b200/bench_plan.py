@@ -34,6 +34,16 @@ def buffer_of_step(round_index: int, lane: int, in_flight: int, n_buffers: int) 
     return (round_index * in_flight + lane) % n_buffers
 
 
+def kernels_per_step(path: str, w, slice_limit: int) -> int:
+    """Kernels that one step launches: Gram, eigensolve (with the projections in the fused call) and attention;
+    in the two-call path the projections are a launch of their own unless the attention's few CTAs make them
+    (d = 64, r <= 32, bf16, at most 222 tiles of 128 candidates, no slice limit: attn_own_supported)."""
+    if path == "fused":
+        return 3
+    own = w.dtype == "bf16" and w.d == 64 and w.r <= 32 and slice_limit == 0 and w.B * math.ceil(w.M / 128) <= 222
+    return 3 if own else 4
+
+
 def replay_plan(steps_wanted: int, in_flight: int, ms_per_step_estimate: float, min_seconds: float = 0.5,
                 rounds_per_graph: int = 12, min_replays: int = 50, max_seconds: float = 3.0) -> tuple[int, int, int]:
     """(steps per graph, replays, steps actually timed).  A graph holds `rounds_per_graph` steps

@@ -59,3 +59,11 @@ def test_sweep_grid():
     s = wl.sweep_configs()
     assert len(s) == 20 and {x.r for x in s} == {8, 16, 32, 64}
     assert all(x.B == 64 and x.M == 1024 and x.d == 64 for x in s)
+
+
+def test_kernels_per_step_follows_the_form_of_the_attention():
+    from paper_2603_02561_b200 import bench_plan as bp
+    serve, c3 = wl.CONFIGS["serve27"], wl.CONFIGS["c3"]          # 192 and 256 tiles of candidates
+    assert [bp.kernels_per_step(p, w, lim) for p, w, lim in [
+        ("fused", c3, 2), ("two_call", c3, 0), ("two_call", serve, 0), ("two_call", serve, 2),
+        ("two_call", serve.with_(dtype="f32"), 0), ("two_call", serve.with_(r=33), 0)]] == [3, 4, 3, 4, 4, 4]
